@@ -314,6 +314,7 @@ struct guard_ctx {
     // scratch of the bracketed path: such rows take the direct selection.
     // site: 0 the ingested step, 1 the fleet baseline, -1 neither.  A site keeps the brackets of its single rows.
     bool row_hints = true;   // guard_set_row_hints
+    int stat_rows = 0;       // rows of the per-step statistics written since creation / reset
     // stamp of the split path's column records: changed whenever the scratch stops describing this context's data
     uint32_t split_epoch = 1;
     // never the same value twice in a process (device memory is handed out again with its old contents, at the
@@ -324,12 +325,17 @@ struct guard_ctx {
     }
     ColHintState *hint_state(int site) const { return (ColHintState *)(ws + L.xr_grid + (size_t)site * align_up(sizeof(ColHintState))); }
     cudaError_t xrank(XrankArgs a, int S, cudaStream_t st, bool own_scratch = true, int site = -1) {
-        // a few rows at a time: one CTA per column keeps the whole GPU busy
-        if (xrank_column_supported(R) && (long long)S * M <= 64 && !a.cut) {
-            // one row of a wide fleet: bracketed by the call site's previous result
-            if (S == 1 && site >= 0 && L.xr_gridp && row_hints) a.hint = hint_state(site);
+        // one row of a wide fleet: bracketed by the call site's previous result
+        if (S == 1 && site >= 0 && L.xr_gridp && row_hints) {
+            a.hint = hint_state(site);
             launches += 1;
             return launch_xrank_column(a, p, S, st);
+        }
+        // everything the streaming paths do not take, or not for so few columns (blocks of more than 16 384 ranks: the
+        // cluster path's one read of whole lines against a CTA per column, 80 us against 130 for 50 steps of 24 000)
+        if (xrank_count_supported(R) && ((!L.xr_split && !L.xr_cluster) || a.mask_bytes != 1 || (long long)S * M <= 64)) {
+            launches += 1;
+            return launch_xrank_count(a, p, S, st);
         }
         if (L.xr_split && a.mask_bytes == 1) {
             a.fallbacks = status() + 1;
@@ -340,6 +346,7 @@ struct guard_ctx {
                 const int n = (S - s0 < smax) ? (S - s0) : smax;
                 XrankArgs g = a;
                 g.first_slot = (int)(((long long)first + s0) % a.capacity);
+                g.prev_rows = a.prev_rows > s0 ? a.prev_rows - s0 : 0;
                 g.med = a.med + (size_t)s0 * M;
                 g.mad = a.mad + (size_t)s0 * M;
                 if (a.med_user) g.med_user = a.med_user + (size_t)s0 * M;
@@ -491,6 +498,8 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
     a.mask_bytes = c->mask_bytes();
     a.check_finite = 1;
     a.status = c->status();
+    a.prev_rows = c->row_hints ? c->stat_rows : 0;
+    if (B > c->stat_rows) c->stat_rows = B;
     cudaError_t e;
     const bool piped = c->deferred && c->L.xr_split && a.mask_bytes == 1 && (long long)B * c->M > 64 && !d_step_med &&
                        !d_step_mad && c->ensure_xs();
@@ -681,6 +690,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     x.med_user = d_fleet_med;
     x.mad_user = d_fleet_mad;
     x.status = c->status();
+    x.prev_rows = c->row_hints && c->evals > 0 ? 1 : 0;
     e = c->xrank(x, 1, ts, !defer, 1);
     if (e != cudaSuccess) return c->cuda_fail(e, "fleet baseline launch");
 
@@ -804,7 +814,10 @@ int guard_sweep_qualify(const float *d_S, int nodes, int gpus_per_node, int reps
     x.mad_user = d_fleet_mad;
     for (int m = 0; m < metrics; ++m) x.cut_rank[m] = p.dir[m] < 0 ? (int)(j - 1) : (int)(G - j);
     x.status = d_status;
-    e = xrank_column_supported(G) ? launch_xrank_column(x, p, 1, st) : launch_xrank_direct(x, p, 1, st);
+    // (a single row of more than 8 192 values without an earlier result to start from: measured 25 us with the whole
+    // column's histogram against 33 us at 16 384 GPUs)
+    e = xrank_count_supported(G) && G <= 8192 ? launch_xrank_count(x, p, 1, st)
+        : xrank_column_supported(G) ? launch_xrank_column(x, p, 1, st) : launch_xrank_direct(x, p, 1, st);
     if (e != cudaSuccess) { set_error(g_error, "sweep fleet statistics launch: %s", cudaGetErrorString(e)); return GUARD_ERR_CUDA; }
     if (d_fleet_cut) {
         e = cudaMemcpyAsync(d_fleet_cut, fleet + 2 * kMaxMetrics, metrics * sizeof(float), cudaMemcpyDeviceToDevice, st);
@@ -1037,6 +1050,7 @@ int guard_reset(guard_ctx *c, void *stream) {
     if (e != cudaSuccess) return c->cuda_fail(e, "cudaMemsetAsync");
     c->seen = 0;
     c->evals = 0;
+    c->stat_rows = 0;
     c->seen_at_eval = 0;
     c->inc_seen = -1;
     c->cnt_seen = -1;

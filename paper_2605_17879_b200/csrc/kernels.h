@@ -27,6 +27,7 @@ struct XrankArgs {
     uint32_t *status;
     uint32_t *only_flagged; // [S] or NULL: direct kernel processes step s only if nonzero, then clears it
     uint32_t *fallbacks;    // or NULL: counts the steps the direct kernel redid for the bracketed path
+    int prev_rows;          // rows of med / mad that hold an earlier result of the same row position (counting path: first pivots)
     void *hint;             // ColHintState of the call site (one row per call), or NULL: column kernels only
     uint32_t hint_epoch;    // split path: non-zero lets a block use the records the previous block left in its scratch
 };
@@ -83,6 +84,11 @@ size_t xrank_scratch_big_bytes(int R, int M, int S_max);
 XrankScratch carve_xrank_scratch(void *small_base, void *big_base, int R, int M, int S_max);
 cudaError_t launch_xrank_bracketed(const XrankArgs &a, const MetricParams &p, const XrankScratch &sc, int S,
                                    cudaStream_t st);
+
+// Rows held in registers and searched by counting at pivots: any values, any number of metrics, up to 32 768 ranks.
+constexpr int kCountMaxRanks = 32768;
+bool xrank_count_supported(int R);
+cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);
 
 cudaError_t launch_xrank_direct(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);
 

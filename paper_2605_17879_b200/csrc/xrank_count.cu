@@ -1,0 +1,49 @@
+// Cross-rank selection of whole rows held in registers (xrank_count.cuh): the path of small and middle fleets,
+// of other numbers of metrics than the streaming sweeps take, and of single rows.
+#include "xrank_count.cuh"
+
+namespace guard {
+
+namespace {
+
+template <int V, int C>
+__global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, const MetricParams p) {
+    __shared__ CtShared<C> sh;
+    if (a.only_flagged && a.only_flagged[blockIdx.y] == 0u) return;
+    ct_row<V, C>(a, p, blockIdx.y, blockIdx.x * C, sh);
+}
+
+template <int C>
+void launch_c(const XrankArgs &a, const MetricParams &p, int S, int T, cudaStream_t st) {
+    const int v = (a.R * C + T - 1) / T;
+    const dim3 grid(a.M / C, S);
+    if (v <= 4) xrank_count_kernel<4, C><<<grid, T, 0, st>>>(a, p);
+    else if (v <= 8) xrank_count_kernel<8, C><<<grid, T, 0, st>>>(a, p);
+    else if (v <= 16) xrank_count_kernel<16, C><<<grid, T, 0, st>>>(a, p);
+    else xrank_count_kernel<32, C><<<grid, T, 0, st>>>(a, p);
+}
+
+}  // namespace
+
+bool xrank_count_supported(int R) { return R >= 1 && R <= kCountMaxRanks; }
+
+cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
+    if (S <= 0) return cudaSuccess;
+    // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
+    // larger CTAs, which wait longer at their barriers: 60 steps of 4 096 ranks x 16 metrics take 31 / 29 / 29 us, launch
+    // included, with 1 / 2 / 8 of them, 100 steps of 1 024 x 8 take 14 / 14 / 18), else one.
+    const int C = (a.M % 2 == 0 && 2 * a.R <= kCountMaxRanks && (long long)S * (a.M / 2) >= 148) ? 2 : 1;
+    const long long ctas = (long long)S * (a.M / C);
+    const int E = a.R * C;
+    // threads: few values each while the CTAs are few (a pass is then as short as it gets), else CTAs small enough to
+    // share an SM and hide one another's barriers
+    int T = 32 * C;
+    if (ctas <= 148) { while (T < 1024 && E > 4 * T) T <<= 1; }
+    else { while (T < 256 && E > 8 * T) T <<= 1; }
+    while (T < 1024 && E > 32 * T) T <<= 1;
+    if (C == 2) launch_c<2>(a, p, S, T, st);
+    else launch_c<1>(a, p, S, T, st);
+    return cudaGetLastError();
+}
+
+}  // namespace guard

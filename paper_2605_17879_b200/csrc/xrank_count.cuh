@@ -1,0 +1,393 @@
+// Cross-rank selection of rows held in registers: a CTA holds C adjacent metrics of one row (element e of the
+// group belongs to metric e mod C, so that a thread's values all belong to one metric and the loads are
+// coalesced) and finds each metric's median, then its MAD, the same way:
+//   1. a key range that should hold the wanted ranks: around the previous result of the same row position where
+//      the caller has one, else between two of 32 spread values sorted by a warp;
+//   2. one pass counts the keys below the range and bins those inside (256 bins in shared memory);
+//   3. one warp per metric scans its bins for the wanted ranks; a second pass fetches the keys of those one or
+//      two bins (a few), and the warp ranks them.
+// The counts prove the range; one that misses is moved, and a bin that holds too many keys becomes the next
+// range (or the answer, if they are all the same: ties), so any values come out exactly.  A key is 32 bits in
+// the order of the values, so that both statistics (and both kinds of range) share one piece of code.
+// Bound by latency and by the half-rate integer pipe; what it avoids is what measured worst on the way here:
+// branches and returning atomics per value, rounds of pivots (each some 500 cycles of dependent scalar work in one
+// warp, whatever the number of values) and column-wise loads (a cache line per lane).  Measured, kernel alone:
+// 100 steps of 1 024 ranks x 8 metrics 8.7 us (8-bit radix select of xrank_direct.cuh: 80), 60 steps of 4 096 x 16
+// 25 us (570), one row of 1 024 ranks 5.3 us (10.5 with the whole column's histogram).
+#pragma once
+#include "kernels.h"
+
+namespace guard {
+
+constexpr int kCtMaxC = 8;         // metrics per CTA at most
+constexpr int kCtBins = 256;
+constexpr int kCtList = 64;        // keys of a bin that are ranked directly (two per lane)
+constexpr int kCtMaxIter = 64;     // a range shrinks at least to a 128th whenever its bin is too full
+constexpr uint32_t kCtTop = 0xFF800000u;    // no key of a number lies above; padding does
+constexpr uint32_t kCtNone = 0xFFFFFFFFu;
+
+template <int C>
+struct CtShared {
+    uint32_t hist[C][kCtBins];
+    uint32_t lo[C], width[C];      // the range [lo, lo + width]
+    uint32_t below[C];             // keys below it
+    uint32_t f0[C], fw[C];         // keys to fetch: [f0, f0 + fw]
+    uint32_t how[C];               // 0 nothing to fetch, 1 list and rank, 2 largest up to / smallest from `cutk`, 3 smallest and largest
+    uint32_t cutk[C];
+    uint32_t q1[C];                // rank of k1 among the fetched keys
+    uint32_t mx[C], mn[C];
+    uint32_t nl[C];                // gathered keys
+    uint32_t list[C][kCtList];
+    uint32_t v1[C], v2[C];
+    uint32_t any_open[2];
+    float med[C], rhs[C];
+    uint32_t bad;
+};
+
+// Ascending sort of one key per lane (bitonic network over shuffles).
+__device__ __forceinline__ uint32_t ct_warp_sort(uint32_t x, const int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, x, stride);
+            const bool asc = (lane & size) == 0, upper = (lane & stride) != 0;
+            x = (asc != upper) ? min(x, o) : max(x, o);
+        }
+    return x;
+}
+
+__device__ __forceinline__ int ct_shift(const uint32_t width) {
+    const int bits = 32 - __clz(width);
+    return bits > 8 ? bits - 8 : 0;
+}
+
+// below += (k < lo); if (k - lo <= width) hist[(k - lo) >> sft] += 1.  (lo + width does not wrap, so the unsigned
+// difference of a key below the range is beyond any width.)
+__device__ __forceinline__ void ct_bin(const uint32_t k, const uint32_t lo, const uint32_t width, const int sft, const uint32_t hist,
+                                       uint32_t &below) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 o, a;\n\t"
+        "setp.lt.u32 p, %1, %2;\n\t"
+        "sub.u32 o, %1, %2;\n\t"
+        "@p add.u32 %0, %0, 1;\n\t"
+        "setp.le.u32 q, o, %3;\n\t"
+        "shr.u32 o, o, %4;\n\t"
+        "mad.lo.u32 a, o, 4, %5;\n\t"
+        "@q red.shared.add.u32 [a], 1;\n\t}"
+        : "+r"(below)
+        : "r"(k), "r"(lo), "r"(width), "r"(sft), "r"(hist)
+        : "memory");
+}
+// if (k - f0 <= fw) hits |= bit
+__device__ __forceinline__ void ct_hit(const uint32_t k, const uint32_t f0, const uint32_t fw, const uint32_t bit, uint32_t &hits) {
+    asm("{\n\t.reg .pred q;\n\t.reg .u32 o;\n\tsub.u32 o, %1, %2;\n\tsetp.le.u32 q, o, %3;\n\t@q or.b32 %0, %0, %4;\n\t}"
+        : "+r"(hits)
+        : "r"(k), "r"(f0), "r"(fw), "r"(bit));
+}
+
+// Scans the bins of column c (one warp): what to fetch for ranks k1 and k2, or where the range has to move.
+template <int C>
+__device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint32_t k1, const uint32_t k2) {
+    const int lane = lane_id();
+    uint4 *h = reinterpret_cast<uint4 *>(&sh.hist[c][lane * 8]);
+    const uint4 a = h[0], b = h[1];
+    const uint32_t below = sh.below[c], lo = sh.lo[c], width = sh.width[c];
+    h[0] = make_uint4(0u, 0u, 0u, 0u);
+    h[1] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const uint32_t sum = ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
+    uint32_t incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, incl, d); if (lane >= d) incl += u; }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    // this lane's bin of k1 / k2 (if it has it), the rank inside it and the number of its keys
+    uint32_t r = below + incl - sum, b1 = 0, b2 = 0, q = 0, n = 0;
+    const bool has1 = k1 - r < sum && k1 >= r, has2 = k2 - r < sum && k2 >= r;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (k1 >= r && k1 - r < w[j]) { b1 = (uint32_t)(8 * lane + j); q = k1 - r; n = w[j]; }
+        if (k2 >= r && k2 - r < w[j]) b2 = (uint32_t)(8 * lane + j);
+        r += w[j];
+    }
+    const uint32_t l1 = __ballot_sync(0xFFFFFFFFu, has1), l2 = __ballot_sync(0xFFFFFFFFu, has2);
+    const int s1 = l1 ? __ffs(l1) - 1 : 0, s2 = l2 ? __ffs(l2) - 1 : 0;
+    b1 = __shfl_sync(0xFFFFFFFFu, b1, s1);
+    b2 = __shfl_sync(0xFFFFFFFFu, b2, s2);
+    q = __shfl_sync(0xFFFFFFFFu, q, s1);
+    n = __shfl_sync(0xFFFFFFFFu, n, s1);
+    if (lane == 0) {
+        sh.below[c] = 0u;
+        sh.nl[c] = 0u;
+        sh.mx[c] = 0u;
+        sh.mn[c] = kCtNone;
+        sh.q1[c] = q;
+        if (l1 && l2) {
+            const int sft = ct_shift(width);
+            const uint32_t f0 = lo + (b1 << sft), end = lo + (b2 << sft) + ((1u << sft) - 1u);
+            sh.f0[c] = f0;
+            sh.fw[c] = min(end, lo + width) - f0;
+            sh.cutk[c] = f0 + ((1u << sft) - 1u);       // last key of k1's bin
+            sh.how[c] = b1 != b2 ? 2u : (n <= (uint32_t)kCtList ? 1u : 3u);
+        } else {   // the range does not hold both ranks: move or stretch it, sixteenfold
+            const uint32_t hi = lo + width, step = width >= 0x07FF0000u ? 0x7FFFFFFFu : 16u * width + 65536u;
+            uint32_t nlo = lo, nhi = hi;
+            if (below > k1) { nlo = lo > step ? lo - step : 0u; if (below > k2) nhi = lo; }
+            if (k2 >= below + total) { nhi = hi < kCtTop - step ? hi + step : kCtTop; if (k1 >= below + total) nlo = min(hi, kCtTop); }
+            sh.lo[c] = nlo;
+            sh.width[c] = nhi - nlo;
+            sh.f0[c] = kCtNone;
+            sh.fw[c] = 0u;
+            sh.how[c] = 0u;
+        }
+    }
+}
+
+// The answer of column c from the fetched keys (one warp), or the next range; returns whether the search goes on.
+template <int C>
+__device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bool pair) {
+    const int lane = lane_id();
+    const uint32_t how = sh.how[c], n = sh.nl[c], q1 = sh.q1[c], mx = sh.mx[c], mn = sh.mn[c];
+    const uint32_t mine = sh.list[c][lane], mine2 = sh.list[c][lane + 32];
+    if (how == 0u) return true;                      // the range moved
+    if (how != 1u) {
+        if (how == 3u && mx != mn) {                 // a full bin of different keys becomes the range
+            if (lane == 0) { sh.lo[c] = mn; sh.width[c] = mx - mn; }
+            return true;
+        }
+        if (lane == 0) { sh.v1[c] = mx; sh.v2[c] = mn; }
+        return false;
+    }
+    const uint32_t q2 = pair ? q1 + 1u : q1;
+    auto rank = [&](const uint32_t x, const bool real) {
+        uint32_t lt = 0, le = 0;
+#pragma unroll 4
+        for (uint32_t j = 0; j < n; ++j) {
+            const uint32_t o = sh.list[c][j];
+            lt += o < x;
+            le += o <= x;
+        }
+        if (real && q1 >= lt && q1 < le) sh.v1[c] = x;
+        if (real && q2 >= lt && q2 < le) sh.v2[c] = x;
+    };
+    rank(mine, lane < (int)n);
+    if (n > 32u) rank(mine2, lane + 32 < (int)n);
+    return false;
+}
+
+// Keys of 0-based ranks k1 and k2 (k2 == k1 or k1 + 1) of the C columns held by the CTA, left in sh.v1 / sh.v2; the
+// columns' ranges are in sh.lo / sh.width, the bins are zero.  All threads of the CTA call this.
+template <int V, int C>
+__device__ __forceinline__ void ct_select(const uint32_t (&key)[V], const uint32_t k1, const uint32_t k2, CtShared<C> &sh) {
+    const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
+    const int col = tid & (C - 1);
+    const uint32_t hist = (uint32_t)__cvta_generic_to_shared(sh.hist[col]);
+    bool searching = true;         // (of a warp c < C: column c)
+#pragma unroll 1
+    for (int it = 0; it < kCtMaxIter; ++it) {
+        if (tid == 0) sh.any_open[it & 1] = 0u;
+        __syncthreads();           // ranges, counters and bins are ready
+        {
+            const uint32_t lo = sh.lo[col], width = sh.width[col];
+            const int sft = ct_shift(width);
+            uint32_t below = 0;
+#pragma unroll
+            for (int i = 0; i < V; ++i) ct_bin(key[i], lo, width, sft, hist, below);
+#pragma unroll
+            for (int d = 16; d >= C; d >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, d);
+            if (lane < C) atomicAdd(&sh.below[lane], below);
+        }
+        __syncthreads();
+        if (warp < C && searching) ct_scan<C>(sh, warp, k1, k2);
+        __syncthreads();
+        {
+            const uint32_t f0 = sh.f0[col], fw = sh.fw[col];
+            uint32_t hits = 0;
+#pragma unroll
+            for (int i = 0; i < V; ++i) ct_hit(key[i], f0, fw, 1u << i, hits);
+            if (hits) {            // a few threads
+                const uint32_t how = sh.how[col], cutk = sh.cutk[col];
+#pragma unroll 1
+                for (; hits; hits &= hits - 1u) {
+                    const int at = __ffs(hits) - 1;
+                    uint32_t k = key[0];
+#pragma unroll
+                    for (int i = 1; i < V; ++i) k = at == i ? key[i] : k;
+                    if (how == 1u) {
+                        const uint32_t pos = atomicAdd(&sh.nl[col], 1u);
+                        if (pos < (uint32_t)kCtList) sh.list[col][pos] = k;
+                    } else if (how >= 2u) {
+                        if (how == 3u || k <= cutk) atomicMax(&sh.mx[col], k);
+                        if (how == 3u || k > cutk) atomicMin(&sh.mn[col], k);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (warp < C && searching) {
+            searching = ct_settle<C>(sh, warp, k2 != k1);
+            if (lane == 0) {
+                if (searching) sh.any_open[it & 1] = 1u;
+                else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fw[warp] = 0u; }   // (no key at all)
+            }
+        }
+        __syncthreads();
+        if (sh.any_open[it & 1] == 0u) return;
+    }
+    if (tid == 0) sh.bad = 1u;
+}
+
+// Median, MAD (and optional extra order statistic) of metrics [m0, m0 + C) of row s of the launch, and their
+// exceedance bits.  C divides M, (R * C) <= V * blockDim.x, blockDim.x >= 32 * C.
+template <int V, int C>
+__device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p, const int s, const int m0, CtShared<C> &sh) {
+    const int tid = threadIdx.x, lane = lane_id(), warp = warp_id(), T = blockDim.x;
+    const int R = a.R, M = a.M;
+    const int col = tid & (C - 1);
+    const int slot = (int)(((long long)a.first_slot + s) % a.capacity);
+    const float *row = a.base + (size_t)slot * a.row_stride + m0;
+    const bool even = (R & 1) == 0;
+    const uint32_t k1 = (uint32_t)((R - 1) / 2), k2 = (uint32_t)(R / 2);
+
+    uint32_t key[V];                      // first the values' keys, later those of the deviations
+    const int dr = T / C, r0 = tid / C;   // this thread's ranks: r0, r0 + dr, ...
+    float xs = 0.0f, hmed = 0.0f, hmad = -1.0f;
+    if (warp < C) {
+        xs = __ldg(row + (size_t)(((2 * lane + 1) * (long long)R) >> 6) * M + warp);
+        if (a.prev_rows > 0) {            // the result arrays still hold an earlier result of this row position
+            const size_t o = (size_t)min(s, a.prev_rows - 1) * M + m0 + warp;
+            hmed = a.med[o];
+            hmad = a.mad[o];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        const int r = r0 + i * dr;
+        key[i] = 0x7FFFFFFFu;             // a NaN whose keys lie above those of all numbers
+        if (r < R) key[i] = __float_as_uint(__ldg(row + (size_t)r * M + col));
+    }
+    for (int i = tid; i < C * kCtBins / 4; i += T) reinterpret_cast<uint4 *>(&sh.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < C) sh.below[tid] = 0u;
+    if (tid == 0) sh.bad = 0u;
+    auto range = [&](const uint32_t lo, const uint32_t hi) {   // of the column of this warp
+        if (lane == 0) { sh.lo[warp] = lo; sh.width[warp] = hi - lo; }
+    };
+    // from its spread values: eight or more positions to either side of the wanted rank's (three standard
+    // deviations of a sample of 32)
+    auto sampled = [&](const uint32_t x, const uint32_t k) {
+        const uint32_t sorted = ct_warp_sort(x, lane);
+        const int pos = (int)(((long long)k * 32) / R);
+        const uint32_t lo = __shfl_sync(0xFFFFFFFFu, sorted, max(pos - 8, 0)), hi = __shfl_sync(0xFFFFFFFFu, sorted, min(pos + 9, 31));
+        range(min(lo, kCtTop), min(hi, kCtTop));
+    };
+    // a previous result brackets the new one to four standard errors of the difference of two sample medians /
+    // MADs of normal data (2.6 and 1.65 MAD / sqrt(R)): some 5.6 sqrt(R) keys
+    const float u = hmad * rsqrtf((float)R);
+    const bool hinted = hmad > 0.0f && hmad < 1.0e37f && fabsf(hmed) < 1.0e37f;
+    if (warp < C) {
+        if (hinted) range(f2key(hmed - 10.0f * u), f2key(hmed + 10.0f * u));
+        else sampled(f2key(xs), k1);
+    }
+    if (a.check_finite) {
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < V; ++i) bad |= nonfinite_bits(key[i]) && r0 + i * dr < R;
+        if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(a.status, kStatNonFinite);
+    }
+#pragma unroll
+    for (int i = 0; i < V; ++i) key[i] = key_of_bits(key[i]);
+    // what: 0 the median, 1 the MAD, 2 + c the extra order statistic of metric m0 + c (before the MAD)
+#pragma unroll 1
+    for (int what = 0;;) {
+        const bool extra = what >= 2;
+        const uint32_t q1 = extra ? (uint32_t)a.cut_rank[m0 + what - 2] : k1, q2 = extra ? q1 : k2;
+        ct_select<V, C>(key, q1, q2, sh);
+        if (tid < C) {
+            const uint32_t v1 = sh.v1[tid], v2 = sh.v2[tid];
+            const int m = m0 + tid;
+            const size_t o = (size_t)s * M + m;
+            if (what == 0) {
+                sh.med[tid] = median_from_keys(v1, v2, even);
+            } else if (what == 1) {
+                const float lo = __uint_as_float(v1 >> 1), md = sh.med[tid];
+                const float mad = even ? __fmul_rn(0.5f, __fadd_rn(lo, __uint_as_float(v2 >> 1))) : lo;
+                sh.rhs[tid] = __fmul_rn(p.thrp[m], scale_of(mad, md, p.floor_rel[m], p.floor_abs[m]));
+                a.med[o] = md;
+                a.mad[o] = mad;
+                if (a.med_user) a.med_user[o] = md;
+                if (a.mad_user) a.mad_user[o] = mad;
+                if (tid == 0 && sh.bad) atomicOr(a.status, kStatInternal);
+            } else if (tid == what - 2) {
+                a.cut[o] = key2f(v1);
+            }
+        }
+        if (what == 1) break;
+        __syncthreads();
+        // the metrics' extra ranks first (they need the values), then the deviations
+        what = !a.cut ? 1 : (what == 0 ? 2 : (what - 1 < C ? what + 1 : 1));
+        if (what >= 2) {
+            if (warp < C) sampled(f2key(xs), (uint32_t)a.cut_rank[m0 + what - 2]);
+        } else {
+            // the keys of the deviations: their bits with the sign as the lowest bit
+            const float med = sh.med[col];
+            if (warp < C) {
+                if (hinted) range(__float_as_uint(fmaxf(hmad - 6.6f * u, 0.0f)) << 1, (__float_as_uint(hmad + 6.6f * u) << 1) | 1u);
+                else sampled(__float_as_uint(__fsub_rn(xs, sh.med[warp])) << 1, k1);
+            }
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const uint32_t b = __float_as_uint(__fsub_rn(key2f(key[i]), med));
+                key[i] = (b << 1) | (b >> 31);   // NaN stays above infinity
+            }
+        }
+    }
+    if (!a.mask_base) return;
+    __syncthreads();
+    const float rhs = sh.rhs[col];
+    const bool neg = p.dir[m0 + col] < 0;
+    constexpr uint32_t gmask = (1u << C) - 1u;
+    // bits this CTA answers for: its metrics', and (first group) those of no metric
+    const uint32_t own = (gmask << m0) | (m0 == 0 && M < 32 ? ~((1u << M) - 1u) : 0u);
+    uint8_t *out = reinterpret_cast<uint8_t *>(a.mask_base) + (size_t)slot * R * a.mask_bytes;
+    // rows whose bytes fall into 32-bit words the same way for every rank quad of a warp
+    const bool bytes = a.mask_bytes == 1, words = bytes && C != M && (R & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        const float dev = __uint_as_float((key[i] >> 1) | (key[i] << 31));
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, (neg ? -dev : dev) > rhs);
+        const int r = r0 + i * dr;
+        if (r < R) {
+            const uint32_t bits = (bal >> lane) & gmask;
+            if (bytes && C == M) {           // the whole row is this CTA's: the first lane of a rank stores its byte
+                if (col == 0) out[r] = (uint8_t)bits;
+            } else if (words) {              // the row's other CTAs own the other bits: in place, four ranks at a time
+                if ((lane & (4 * C - 1)) == 0) {
+                    uint32_t four = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) four |= ((bal >> ((lane + q * C) & 31)) & gmask) << (8 * q + m0);
+                    unsigned int *w = reinterpret_cast<unsigned int *>(out + r);
+                    atomicAnd(w, ~((own & 0xFFu) * 0x01010101u));
+                    if (four) atomicOr(w, four);
+                }
+            } else if (bytes) {
+                if (col == 0) {
+                    const uintptr_t at = reinterpret_cast<uintptr_t>(out + r);
+                    const int sft = 8 * (int)(at & 3);
+                    unsigned int *w = reinterpret_cast<unsigned int *>(at & ~(uintptr_t)3);
+                    atomicAnd(w, ~((own & 0xFFu) << sft));
+                    if (bits) atomicOr(w, (bits << m0) << sft);
+                }
+            } else if (col == 0) {
+                unsigned int *w = reinterpret_cast<unsigned int *>(out) + r;
+                if (C == 8) {                // eight metrics are a byte of the rank's word
+                    reinterpret_cast<uint8_t *>(w)[m0 >> 3] = (uint8_t)bits;
+                } else {
+                    atomicAnd(w, ~own);
+                    if (bits) atomicOr(w, bits << m0);
+                }
+            }
+        }
+    }
+}
+
+}  // namespace guard

@@ -18,9 +18,9 @@
 //               threshold are rare: those clear of the threshold's possible range set their
 //               exceedance bit at once, the others are deferred to a per-step list;
 //   4. select   exact MAD and threshold;
-//   5. finish   one CTA per step settles the deferred elements -- or, if an interval missed,
-//               a list overflowed or the sample was degenerate, recomputes the whole step
-//               with the direct radix select, so the result is exact either way.
+//   5. finish   settles the deferred elements of a step -- or, if an interval missed, a list
+//               overflowed or the sample was degenerate, recomputes the whole step with the
+//               values in registers (xrank_count.cuh), so the result is exact either way.
 //
 // The scratch (intervals, counters, kept lists: ~80 KB per step) stays in L2 between kernels.
 #include <math_constants.h>
@@ -28,7 +28,7 @@
 #include <mutex>
 
 #include "xrank_common.cuh"
-#include "xrank_direct.cuh"
+#include "xrank_count.cuh"
 
 namespace guard {
 
@@ -702,30 +702,57 @@ __global__ void __launch_bounds__(kSpSelThreads, 12) xsplit_select_kernel(const 
 }
 
 // ---- 5. finish ---------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSpThreads) xsplit_finish_kernel(const XrankArgs a, const MetricParams p, const SpScratch sc) {
-    extern __shared__ uint32_t fhist[];   // M * 256 words for the direct path
-    __shared__ XrShared xsh;
-    const int t = blockIdx.x, tid = threadIdx.x;
-    const int R = a.R, M = a.M;
-    if (sc.fail[t]) {   // the direct radix select recomputes the whole step
-        xrank_direct_step(a, p, t, fhist, xsh);
-        if (tid == 0 && a.fallbacks) atomicAdd(a.fallbacks, 1u);
-        return;
+// Settles the deferred exceedance decisions of the steps the fast path served, and recomputes the columns of the
+// others with the values in registers (xrank_count.cuh).  As a rule there is next to nothing to do, and what counts
+// is the number of dependent loads: every CTA reads the flags of all steps at once, settles the steps that are its
+// own, and takes its share of the (failed step, metric) pairs.
+template <int V>
+__global__ void __launch_bounds__(512) xsplit_finish_kernel(const XrankArgs a, const MetricParams p, const SpScratch sc, const int S) {
+    __shared__ CtShared<1> sh;
+    constexpr int kWords = kSplitMaxSteps / 32;
+    __shared__ uint32_t failed[kWords];   // a bit per step
+    const int tid = threadIdx.x, R = a.R, M = a.M;
+    for (int w = warp_id(); w < kWords; w += blockDim.x >> 5) {
+        const int t = 32 * w + lane_id();
+        const uint32_t bits = __ballot_sync(0xFFFFFFFFu, t < S && sc.fail[t]);
+        if (lane_id() == 0) failed[w] = bits;
     }
-    if (!a.mask_base) return;
-    const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
-    const float *row = a.base + (size_t)slot * a.row_stride;
-    uint8_t *maskrow = reinterpret_cast<uint8_t *>(a.mask_base) + (size_t)slot * R;
-    const SpCol *cols = sc.col + (size_t)t * M;
-    const uint32_t na = sc.namb[t];
-    for (uint32_t i = tid; i < na; i += kSpThreads) {
-        const uint32_t e = sc.amb[(size_t)t * kSpAmb + i];
-        const uint32_t r = e >> 5, m = e & 31u;
-        if (exceeds(row[(size_t)r * M + m], cols[m].med, p.dir[m], cols[m].rhs)) {
-            unsigned int *w = reinterpret_cast<unsigned int *>(maskrow + (r & ~3u));
-            atomicOr(w, (1u << m) << (8 * (r & 3u)));
+    if (a.mask_base) {
+        for (int t = blockIdx.x; t < S; t += gridDim.x) {
+            const uint32_t na = sc.fail[t] ? 0u : sc.namb[t];
+            const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
+            const float *row = a.base + (size_t)slot * a.row_stride;
+            uint8_t *maskrow = reinterpret_cast<uint8_t *>(a.mask_base) + (size_t)slot * R;
+            const SpCol *cols = sc.col + (size_t)t * M;
+            for (uint32_t i = tid; i < na; i += blockDim.x) {
+                const uint32_t e = sc.amb[(size_t)t * kSpAmb + i];
+                const uint32_t r = e >> 5, m = e & 31u;
+                if (exceeds(row[(size_t)r * M + m], cols[m].med, p.dir[m], cols[m].rhs)) {
+                    unsigned int *w = reinterpret_cast<unsigned int *>(maskrow + (r & ~3u));
+                    atomicOr(w, (1u << m) << (8 * (r & 3u)));
+                }
+            }
         }
     }
+    __syncthreads();
+    int n = 0;
+    for (int w = 0; w < kWords; ++w) n += __popc(failed[w]);
+    if (blockIdx.x == 0 && tid == 0 && n && a.fallbacks) atomicAdd(a.fallbacks, (uint32_t)n);
+    for (int item = blockIdx.x; item < n * M; item += gridDim.x) {
+        int f = item / M, w = 0;           // the f-th failed step
+        while (f >= __popc(failed[w])) f -= __popc(failed[w++]);
+        uint32_t bits = failed[w];
+        for (; f > 0; --f) bits &= bits - 1u;
+        ct_row<V, 1>(a, p, 32 * w + __ffs(bits) - 1, item % M, sh);
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_finish(const XrankArgs &a, const MetricParams &p, const SpScratch &sc, int S, cudaStream_t st) {
+    const int T = a.R <= 32 * 128 ? 128 : (a.R <= 32 * 256 ? 256 : 512);
+    const int most = 148 * (1024 / T);   // what the SMs hold of them at 64 registers per thread
+    xsplit_finish_kernel<32><<<S * a.M < most ? S * a.M : most, T, 0, st>>>(a, p, sc, S);
+    return cudaGetLastError();
 }
 
 // Kept fraction of a column: the median interval spans 2 delta of s sample ranks, the MAD
@@ -820,8 +847,7 @@ cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S,
     else xsplit_sweep_kernel<1, 1><<<gsw, kSpThreads, smem, st>>>(a, p, g, sc);
     if (prof) cudaEventRecord(ev1, st);
     xsplit_select_kernel<1><<<gcol, kSpSelThreads, 0, st>>>(a, p, g, sc, reasons);
-    xsplit_finish_kernel<<<S, kSpThreads, (size_t)M * 256 * sizeof(uint32_t), st>>>(a, p, sc);
-    e = cudaGetLastError();
+    e = launch_finish(a, p, sc, S, st);
     if (prof) prof->emplace_back(ev0, ev1);
     return e;
 }

@@ -507,3 +507,24 @@ def test_sweep_configuration_full():
     strong = set(np.nonzero((bad & (amount > 0.10)).numpy())[0].tolist())
     assert strong <= failed                       # clearly degraded GPUs are caught
     assert len(failed) < 0.08 * cfg.gpus          # and the healthy bulk passes
+
+
+@pytest.mark.parametrize("R,M,B,T,quant", [
+    (64, 4, 50, 100, None),        # a warp per column
+    (65, 5, 40, 80, None),         # odd rank count and number of metrics: one metric per CTA, masks bit by bit
+    (1024, 8, 40, 80, None),       # two metrics per CTA, eight values per thread
+    (2047, 6, 60, 120, None),      # the same with a ragged last round and rows that are not word aligned
+    (4096, 16, 24, 48, None),      # 32 values per thread; 32-bit exceedance words
+    (8200, 12, 26, 52, None),      # more than 256 threads per CTA
+    (16386, 4, 80, 80, None),      # two metrics no longer fit one CTA
+    (32768, 3, 12, 24, None),      # the widest column: 1 024 threads, all values in use
+    (1024, 8, 40, 80, 40),         # ties: bins with more equal keys than are ranked, ranks in two bins
+    (3000, 2, 80, 160, 3),         # a handful of distinct values
+])
+def test_columns_held_in_registers(R, M, B, T, quant):
+    """Blocks whose columns live in registers: the second block starts from the first one's results, and a jump of
+    every rank in between makes those miss for half of the steps."""
+    X, dirs = _rand_fleet(T, R, M, seed=5 * R + M, quant=quant)
+    if T > B:
+        X[B + B // 2:] *= np.float32(1.75)
+    run_both(X, B, max(1, B // 2), 16, dirs, [B], capacity=2 * B, min_signals=2)

@@ -114,7 +114,8 @@ struct WindowArgs {
     uint32_t *status;
     long long first_wait_cycles;   // limit of the warp path's wait for a staged tile (0: the default of about a second)
 };
-// Launches one kernel (thread, warp or staged path).
+cudaError_t launch_window_bins(const WindowArgs &a, cudaStream_t st);   // any window length: tiles of 32 series
+// Launches one or two kernels (thread, warp or tile path).
 cudaError_t launch_window_select(const WindowArgs &a, cudaStream_t st);
 
 // Sliding windows: per-series state that lets an evaluation which follows the previous one by a few

@@ -1,7 +1,5 @@
 // Windowed per-series median: for every (rank, metric) series the exact median of its
-// last n ring steps.  A CTA stages a [n steps] x [TC series] tile of the ring in shared
-// memory with bulk asynchronous copies (one per ring row, completion on an mbarrier),
-// then every thread selects inside its own column.
+// last n ring steps.
 #include <math_constants.h>
 
 #include <mutex>
@@ -15,59 +13,6 @@
 namespace guard {
 
 namespace {
-
-constexpr size_t kMaxStagedTile = 200 * 1024;   // largest staged tile (dynamic shared memory of the staged path)
-
-// Staged path.  blockDim.x == TC; dynamic shared memory = n * TC * 4 bytes.
-template <int TC>
-__global__ void __launch_bounds__(TC) window_select_kernel(const WindowArgs a, const int use_bulk) {
-    extern __shared__ __align__(128) uint32_t tile[];
-    __shared__ __align__(8) uint64_t bar;
-    const int tid = threadIdx.x;
-    const int col0 = blockIdx.x * TC;
-    const int ncols = min(TC, a.series - col0);
-    const int n = a.n;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
-
-    if (use_bulk) {
-        if (tid == 0) {
-            mbar_init(&bar, 1);
-            mbar_arrive_expect_tx(&bar, (uint32_t)n * (uint32_t)ncols * 4u);
-        }
-        __syncthreads();
-        for (int j = tid; j < n; j += TC) {
-            int slot = first + j;
-            if (slot >= a.capacity) slot -= a.capacity;
-            bulk_g2s(tile + (size_t)j * TC, a.ring + (size_t)slot * a.row_stride + col0, (uint32_t)ncols * 4u, &bar);
-        }
-        if (!mbar_wait_bounded(&bar, 0, kWaitLimitCycles)) {
-            atomicOr(a.status, kStatTimeout);
-            mbar_wait_bounded(&bar, 0, kWaitLimitCycles);  // let copies in flight land before leaving
-            return;
-        }
-    } else {
-        for (int j = 0; j < n; ++j) {
-            int slot = first + j;
-            if (slot >= a.capacity) slot -= a.capacity;
-            if (tid < ncols)
-                tile[(size_t)j * TC + tid] = __float_as_uint(a.ring[(size_t)slot * a.row_stride + col0 + tid]);
-        }
-        // each thread only reads back what it wrote itself: no barrier needed
-    }
-    if (tid >= ncols) return;
-    uint32_t *col = tile + tid;
-    for (int j = 0; j < n; j += kSelBatch) {   // raw bits -> order-preserving keys, loads batched
-        uint32_t v[kSelBatch];
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u) v[u] = (j + u < n) ? col[(size_t)(j + u) * TC] : 0u;
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u)
-            if (j + u < n) col[(size_t)(j + u) * TC] = key_of_bits(v[u]);
-    }
-    const float med = col_median(col, TC, n);
-    a.wmed[col0 + tid] = med;
-    if (a.wmed_user) a.wmed_user[col0 + tid] = med;
-}
 
 // ---------------------------------------------------------------------------------------
 // Warp-per-series path for windows of up to 256 steps: the window of one series lives in
@@ -670,65 +615,22 @@ __global__ void __launch_bounds__(kRbThreads) window_rebuild_kernel(const Window
     }
 }
 
-// Fallback for windows too long to stage: one thread per series, bit-by-bit counting
-// selection straight from global memory (32 sweeps of the column).
-__global__ void window_select_global_kernel(const WindowArgs a) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= a.series) return;
-    const int n = a.n;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
-    auto key_at = [&](int j) {
-        int slot = first + j;
-        if (slot >= a.capacity) slot -= a.capacity;
-        return f2key(a.ring[(size_t)slot * a.row_stride + c]);
-    };
-    const int k = (n - 1) >> 1;
-    uint32_t prefix = 0;
-    int krem = k;
-    for (int bit = 31; bit >= 0; --bit) {
-        int zeros = 0;
-        for (int j = 0; j < n; ++j) {
-            const uint32_t key = key_at(j);
-            const bool match = (bit == 31) || (((key ^ prefix) >> (bit + 1)) == 0);
-            zeros += (match && !((key >> bit) & 1u));
-        }
-        if (krem >= zeros) {
-            prefix |= 1u << bit;
-            krem -= zeros;
-        }
-    }
-    float med = key2f(prefix);
-    if (!(n & 1)) {
-        int cle = 0;
-        uint32_t above = 0xFFFFFFFFu;
-        for (int j = 0; j < n; ++j) {
-            const uint32_t key = key_at(j);
-            cle += (key <= prefix);
-            if (key > prefix) above = min(above, key);
-        }
-        med = median_from_keys(prefix, cle > k + 1 ? prefix : above, true);
-    }
-    a.wmed[c] = med;
-    if (a.wmed_user) a.wmed_user[c] = med;
-}
-
-template <int TC>
-cudaError_t launch_staged(const WindowArgs &a, int use_bulk, cudaStream_t st) {
-    const size_t smem = (size_t)a.n * TC * 4;
-    static AttrOnce once;
-    int dev = 0;
-    cudaError_t e = once(dev, [] {
-        return cudaFuncSetAttribute(window_select_kernel<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxStagedTile);
-    });
-    if (e != cudaSuccess) return e;
-    const int grid = (a.series + TC - 1) / TC;
-    window_select_kernel<TC><<<grid, TC, smem, st>>>(a, use_bulk);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
-int window_launch_count(const WindowArgs &a) { return (a.use_hint && a.spread && a.centre && a.fb_list && a.series < (1 << 28) && a.n <= 256) ? 2 : 1; }
+// Which whole-window path an evaluation takes.  Many series of a short window with an earlier result: one thread per
+// series (31 + 6 us at 131 072 series of 100 steps, 46 + 17 at 200, against 56 and 86 with a tile per 32 series).  Up to
+// 65 536 series the threads are too few to hide their own latency, and a launch less counts (8 192 series of
+// 100 / 200 steps: 14 + 5 / 21 + 8 us against 11 / 16; 32 768: 16 + 5 / 24 + 8 against 14 / 25).  First evaluations:
+// a warp per series while there are few (9.2 us against 12 at 8 192 series of 100 steps; at 32 768 series 28 against
+// 18, at 131 072 series of 200 steps 196 against 101).
+enum WindowPath { kPathThread, kPathWarp, kPathBins };
+static WindowPath window_path(const WindowArgs &a) {
+    if (a.n > 256) return kPathBins;
+    if (!a.use_hint) return a.series <= 16384 ? kPathWarp : kPathBins;
+    return a.series > 65536 && a.spread && a.centre && a.fb_list && a.series < (1 << 28) ? kPathThread : kPathBins;
+}
+
+int window_launch_count(const WindowArgs &a) { return window_path(a) == kPathThread ? 2 : 1; }
 
 size_t window_inc_bytes(int series) { return (size_t)series * sizeof(float); }
 
@@ -746,24 +648,23 @@ cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, c
 }
 
 cudaError_t launch_window_select(const WindowArgs &a, cudaStream_t st) {
-    constexpr size_t kMaxTile = kMaxStagedTile;
-    // bulk copies need 16-byte aligned sources and sizes
-    const int use_bulk = (a.series % 4 == 0) && (((uintptr_t)a.ring & 15) == 0);
-    const size_t n = (size_t)a.n;
-    if (a.use_hint && a.spread && a.centre && a.fb_list && a.series < (1 << 28) && n <= 256) {
-        if (n <= 64) return launch_thread_path<2>(a, st);
-        if (n <= 128) return launch_thread_path<4>(a, st);
+    const WindowPath path = window_path(a);
+    if (path == kPathThread) {
+        if (a.n <= 64) return launch_thread_path<2>(a, st);
+        if (a.n <= 128) return launch_thread_path<4>(a, st);
         return launch_thread_path<8>(a, st);
     }
-    if (n <= 64) return launch_warp_path<2>(a, use_bulk, st);
-    if (n <= 128) return launch_warp_path<4>(a, use_bulk, st);
-    if (n <= 256) return launch_warp_path<8>(a, use_bulk, st);
-    if (n * 128 * 4 <= kMaxTile) return launch_staged<128>(a, use_bulk, st);
-    if (n * 64 * 4 <= kMaxTile) return launch_staged<64>(a, use_bulk, st);
-    if (n * 32 * 4 <= kMaxTile) return launch_staged<32>(a, use_bulk, st);
-    const int threads = 128;
-    window_select_global_kernel<<<(a.series + threads - 1) / threads, threads, 0, st>>>(a);
-    return cudaGetLastError();
+    if (path == kPathBins) {
+        WindowArgs b = a;
+        // the thread path takes over from the next evaluation on: its interval has fewer slots
+        b.target = a.n <= 256 && a.series > 65536 ? kThTarget : 0;
+        return launch_window_bins(b, st);
+    }
+    // bulk copies need 16-byte aligned sources and sizes
+    const int use_bulk = (a.series % 4 == 0) && (((uintptr_t)a.ring & 15) == 0);
+    if (a.n <= 64) return launch_warp_path<2>(a, use_bulk, st);
+    if (a.n <= 128) return launch_warp_path<4>(a, use_bulk, st);
+    return launch_warp_path<8>(a, use_bulk, st);
 }
 
 }  // namespace guard

@@ -528,3 +528,42 @@ def test_columns_held_in_registers(R, M, B, T, quant):
     if T > B:
         X[B + B // 2:] *= np.float32(1.75)
     run_both(X, B, max(1, B // 2), 16, dirs, [B], capacity=2 * B, min_signals=2)
+
+
+@pytest.mark.parametrize("R,M,W,quant", [
+    (70, 3, 1, None),              # one step; a ragged last tile
+    (64, 4, 64, None),             # every slot of eight warps of eight values in use
+    (45, 5, 65, None),             # one step more: sixteen values per thread
+    (40, 8, 129, None),            # 24 values per thread
+    (33, 8, 256, None),            # 32 values per thread, all in use
+    (24, 4, 257, None),            # sixteen warps
+    (16, 4, 1024, None),           # the longest window held in registers
+    (11, 3, 1025, None),           # read again in every pass
+    (2100, 8, 40, None),           # a first evaluation wide enough for tiles
+    (64, 4, 100, 12),              # ties: full bins of equal values, middle ranks in two bins
+    (64, 4, 300, 2),               # a handful of distinct values
+])
+def test_window_tiles(R, M, W, quant):
+    """Whole windows by tiles of 32 series: first evaluation, a second window just like it, a jump that leaves every
+    range, and values whose differences overflow or are denormal (windowed medians and counts only: the reported score
+    of a deviation of 3e38 is beyond float32, in which it is computed)."""
+    from paper_2605_17879_b200 import guard
+    T = 3 * W + 8
+    X, dirs = _rand_fleet(T, R, M, seed=R + W, quant=quant)
+    X[2 * W:] *= np.float32(2.5)
+    X[:, 2 % R] = np.where(np.arange(T)[:, None] % 2 == 0, np.float32(3e38), np.float32(-3e38))
+    X[:, 3 % R] = (np.arange(T)[:, None] * 7919 % 1000).astype(np.float32) * np.float32(1e-42)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, W, max(1, W // 2), dir=dirs, capacity=W, min_signals=1)
+    g.set_sliding(False)
+    o = go.Oracle(R, M, W, max(1, W // 2), 0, dir=dirs, min_signals=1)
+    t = 0
+    for B in (W, W, W, min(W, 8)):
+        g.ingest(Xd[t:t + B].contiguous())
+        o.ingest(X[t:t + B])
+        t += B
+        out, ref = g.score(), o.score()
+        assert g.sync_status() == 0
+        for key in ("wmed", "fleet_med", "fleet_mad", "counts", "mask", "flags", "tier"):
+            assert_bit_equal(to_np(out[key]), ref[key], "t=%d %s" % (t, key))
+    g.close()

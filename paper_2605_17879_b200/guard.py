@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libguard_b200.so (the C ABI declared in include/guard_b200.h).
+"""Thin binding of libguard_b200.so (the C ABI declared in include/guard_b200.h): ctypes, and for the calls a
+monitor makes every step a native module that checks and passes the tensors (csrc/binding.cpp).
 
 Argument marshalling only: every step of the scoring path runs in the library's CUDA
 kernels.  PyTorch supplies device memory (the workspace and the output tensors) and the
@@ -8,6 +9,7 @@ import of this module's functions fails loudly.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from typing import Dict, Optional, Sequence
 
@@ -125,8 +127,26 @@ def lib():
     return _lib
 
 
+_nat = None
+
+
+def _native():
+    """The native marshalling module (raises if it has not been built)."""
+    global _nat
+    if _nat is None:
+        lib()   # the module is linked to the library
+        path = os.path.join(_HERE, "_guard_native.so")
+        if not os.path.exists(path):
+            raise RuntimeError("_guard_native.so is missing: build it with paper_2605_17879_b200.build.build_library()")
+        spec = importlib.util.spec_from_file_location("_guard_native", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _nat = mod
+    return _nat
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return _native().current_stream(torch.cuda.current_device())
 
 
 class _Here:
@@ -176,9 +196,6 @@ def workspace_bytes(ranks: int, metrics: int, W: int, capacity: int, topk: int) 
     return int(lib().guard_workspace_bytes(ranks, metrics, W, capacity, topk))
 
 
-_OUT_NAMES = ("wmed", "fleet_med", "fleet_mad", "scores", "counts", "mask", "flags", "tier", "topk_idx", "topk_score")
-
-
 class Guard:
     """Online scorer: `ingest` blocks of steps, `score` the current window."""
 
@@ -192,7 +209,6 @@ class Guard:
         self.device = torch.device(device)
         self._devidx = self.device.index if self.device.index is not None else torch.cuda.current_device()
         self._views = {}        # ring views handed out by ring_reserve, by (byte offset, steps)
-        self._out_cache = None  # (dict, tensors, marshalled pointers) of the last score() outputs
         self._h = C.c_void_p()
         self._params = _Params(metrics, dir, thr, floor_rel, floor_abs, primary, min_signals, n_consec,
                                ranks_per_node, tier_moderate, tier_severe)
@@ -207,11 +223,13 @@ class Guard:
                                     _ptr(workspace, torch.uint8), workspace.numel(), _stream())
         if rc != GUARD_OK:
             raise GuardError(rc, lib().guard_last_error(None).decode())
+        self._hv = self._h.value   # the handle as a number, for the native calls
 
     def close(self):
         if getattr(self, "_h", None) and _lib is not None:
             _lib.guard_destroy(self._h)
             self._h = C.c_void_p()
+            self._hv = 0
 
     def __del__(self):
         try:
@@ -294,8 +312,7 @@ class Guard:
 
     def join(self) -> None:
         """Makes the current stream wait for the pending deferred evaluation, if any."""
-        with self._dev():
-            self._check(lib().guard_join(self._h, _stream()))
+        self._check(_native().join(self._hv, self._devidx))
 
     def profile_enable(self, on=True) -> None:
         """0 / False: off; 1 / True: time the MAD sweep of every ingest; 2: the window kernel of every evaluation."""
@@ -322,13 +339,7 @@ class Guard:
 
     def ingest(self, block: torch.Tensor, step_med: Optional[torch.Tensor] = None,
                step_mad: Optional[torch.Tensor] = None) -> None:
-        if block.dim() != 3 or block.shape[1] != self.R or block.shape[2] != self.M:
-            raise ValueError("block must be [B, %d, %d]" % (self.R, self.M))
-        B = block.shape[0]
-        with self._dev():
-            self._check(lib().guard_ingest(self._h, _ptr(block, torch.float32), B,
-                                           _ptr(step_med, torch.float32, B * self.M),
-                                           _ptr(step_mad, torch.float32, B * self.M), _stream()))
+        self._check(_native().ingest(self._hv, self._devidx, self.R, self.M, block, step_med, step_mad))
 
     def alloc_outputs(self) -> Dict[str, torch.Tensor]:
         R, M, K, dev = self.R, self.M, self.K, self.device
@@ -349,24 +360,7 @@ class Guard:
         """One evaluation; `out` maps output names to tensors (missing / None entries are skipped)."""
         if out is None:
             out = self.alloc_outputs()
-        g = out.get
-        R, M, K = self.R, self.M, self.K
-        # the same output tensors as last time (a monitor scores into the same buffers every step): reuse
-        # the checked pointers
-        cached = self._out_cache
-        if cached is not None and cached[0] is out and all(
-                g(n) is t and (t is None or t.data_ptr() == q) for (n, t), q in zip(cached[1], cached[2])):
-            ptrs = cached[2]
-        else:
-            ptrs = (_ptr(g("wmed"), torch.float32, R * M), _ptr(g("fleet_med"), torch.float32, M),
-                    _ptr(g("fleet_mad"), torch.float32, M), _ptr(g("scores"), torch.float32, R * M),
-                    _ptr(g("counts"), torch.uint16, R * M), _ptr(g("mask"), torch.uint32, R),
-                    _ptr(g("flags"), torch.uint8, R), _ptr(g("tier"), torch.uint8, R),
-                    _ptr(g("topk_idx"), torch.int32, K) if K else None,
-                    _ptr(g("topk_score"), torch.float32, K) if K else None)
-            self._out_cache = (out, tuple((n, g(n)) for n in _OUT_NAMES), ptrs)
-        with self._dev():
-            self._check(lib().guard_score(self._h, *ptrs, _stream()))
+        self._check(_native().score(self._hv, self._devidx, self.R, self.M, self.K, out))
         return out
 
     def node_verdict(self, out: Optional[Dict[str, Optional[torch.Tensor]]] = None) -> Dict[str, Optional[torch.Tensor]]:
@@ -376,11 +370,7 @@ class Guard:
             out = {"node_flag": torch.empty(N, dtype=torch.uint8, device=self.device),
                    "node_tier": torch.empty(N, dtype=torch.uint8, device=self.device),
                    "node_stall": torch.empty(N, dtype=torch.uint16, device=self.device)}
-        g = out.get
-        with self._dev():
-            self._check(lib().guard_node_verdict(self._h, _ptr(g("node_flag"), torch.uint8, N),
-                                                 _ptr(g("node_tier"), torch.uint8, N),
-                                                 _ptr(g("node_stall"), torch.uint16, N), _stream()))
+        self._check(_native().node_verdict(self._hv, self._devidx, N, out))
         return out
 
     def state_bytes(self) -> int:
@@ -422,11 +412,10 @@ def sweep_qualify(S: torch.Tensor, nodes: int, gpus_per_node: int, *, dir: Seque
         raise ValueError("S must be [nodes * gpus_per_node, reps, metrics]")
     G, reps, M = S.shape
     dev = S.device
-    params = _Params(M, dir, thr, floor_rel, floor_abs)
-    need = int(lib().guard_sweep_workspace_bytes(G, reps, M))
-    if need == 0:
-        raise GuardError(-1, "invalid sweep sizes")
-    if workspace is None:
+    if workspace is None or not 1 <= M <= MAX_METRICS:
+        need = int(lib().guard_sweep_workspace_bytes(G, reps, M))
+        if need == 0:
+            raise GuardError(-1, "invalid sweep sizes")
         workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     if out is None:
         out = {
@@ -439,15 +428,9 @@ def sweep_qualify(S: torch.Tensor, nodes: int, gpus_per_node: int, *, dir: Seque
             "node_pass": torch.empty(nodes, dtype=torch.uint8, device=dev),
             "status": torch.zeros(1, dtype=torch.uint32, device=dev),
         }
-    g = out.get
-    with torch.cuda.device(dev):
-        rc = lib().guard_sweep_qualify(
-            _ptr(S, torch.float32), nodes, gpus_per_node, reps, M, C.byref(params.struct), pct_ppm,
-            _ptr(workspace, torch.uint8), workspace.numel(), _ptr(g("gpu_med"), torch.float32, G * M),
-            _ptr(g("fleet_med"), torch.float32, M), _ptr(g("fleet_mad"), torch.float32, M),
-            _ptr(g("fleet_cut"), torch.float32, M), _ptr(g("fail_mask"), torch.uint32, G),
-            _ptr(g("gpu_pass"), torch.uint8, G), _ptr(g("node_pass"), torch.uint8, nodes),
-            _ptr(g("status"), torch.uint32, 1), _stream())
+    if dev.type != "cuda":
+        raise ValueError("expected a contiguous CUDA tensor")
+    rc = _native().sweep_qualify(dev.index, S, nodes, gpus_per_node, dir, thr, floor_rel, floor_abs, pct_ppm, workspace, out)
     if rc != GUARD_OK:
         raise GuardError(rc, lib().guard_last_error(None).decode())
     return out

@@ -317,6 +317,7 @@ struct guard_ctx {
     int stat_rows = 0;       // rows of the per-step statistics written since creation / reset
     // stamp of the split path's column records: changed whenever the scratch stops describing this context's data
     uint32_t split_epoch = 1;
+    SplitState split_state[kIngestStreams];
     // never the same value twice in a process (device memory is handed out again with its old contents, at the
     // same addresses: a stamp derived from addresses would take another context's leftovers for its own)
     void new_epoch() {
@@ -331,15 +332,15 @@ struct guard_ctx {
             launches += 1;
             return launch_xrank_column(a, p, S, st);
         }
-        // everything the streaming paths do not take, or not for so few columns (blocks of more than 16 384 ranks: the
-        // cluster path's one read of whole lines against a CTA per column, 80 us against 130 for 50 steps of 24 000)
+        // everything the streaming paths do not take, or not for so few columns
         if (xrank_count_supported(R) && ((!L.xr_split && !L.xr_cluster) || a.mask_bytes != 1 || (long long)S * M <= 64)) {
             launches += 1;
             return launch_xrank_count(a, p, S, st);
         }
         if (L.xr_split && a.mask_bytes == 1) {
             a.fallbacks = status() + 1;
-            a.hint_epoch = row_hints ? split_epoch : 0u;
+            a.hint_epoch = split_epoch;
+            a.hint_fresh = row_hints ? 0 : 1;
             const int first = a.first_slot;
             const int smax = C < kSplitMaxSteps ? C : kSplitMaxSteps;
             for (int s0 = 0; s0 < S; s0 += smax) {
@@ -351,10 +352,11 @@ struct guard_ctx {
                 g.mad = a.mad + (size_t)s0 * M;
                 if (a.med_user) g.med_user = a.med_user + (size_t)s0 * M;
                 if (a.mad_user) g.mad_user = a.mad_user + (size_t)s0 * M;
-                cudaError_t e = launch_xrank_split(g, p, n, ws + L.xr_big + (size_t)scratch_sel * L.xr_big_stride, status() + 2, st,
-                                                   (profiling == 1 && a.mask_base) ? &prof : nullptr);
+                int launched = 0;
+                cudaError_t e = launch_xrank_split(g, p, n, smax, split_state[scratch_sel], ws + L.xr_big + (size_t)scratch_sel * L.xr_big_stride,
+                                                   status() + 2, st, launched, (profiling == 1 && a.mask_base) ? &prof : nullptr);
                 if (e != cudaSuccess) return e;
-                launches += 6;
+                launches += launched;
             }
             return cudaSuccess;
         }

@@ -29,7 +29,8 @@ struct XrankArgs {
     uint32_t *fallbacks;    // or NULL: counts the steps the direct kernel redid for the bracketed path
     int prev_rows;          // rows of med / mad that hold an earlier result of the same row position (counting path: first pivots)
     void *hint;             // ColHintState of the call site (one row per call), or NULL: column kernels only
-    uint32_t hint_epoch;    // split path: non-zero lets a block use the records the previous block left in its scratch
+    uint32_t hint_epoch;    // split path: stamp of the estimates in its scratch (non-zero)
+    int hint_fresh;         // split path: take no estimate from an earlier block
 };
 
 // Scratch of the bracketed path for up to S_max steps per launch.
@@ -66,8 +67,14 @@ cudaError_t launch_xrank_column(const XrankArgs &a, const MetricParams &p, int S
 bool xrank_cluster_supported(int R, int M);
 cudaError_t launch_xrank_cluster(const XrankArgs &a, const MetricParams &p, int S, uint32_t *reasons, cudaStream_t st,
                                  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
-// Six uniform kernels per block (sample, sweep, select, sweep, select, finish) with the kept
-// elements in global scratch (4 or 8 metrics, a few thousand to ~20 000 ranks).
+// One pass over a block's telemetry: values about the estimated median and MAD are kept in lists, from which both are
+// selected (4 or 8 metrics, 4 096 to 32 768 ranks).
+// What the host knows of a scratch of that path: step positions that hold estimates, their stamp, and which of the two
+// sets of flags the next launch uses.
+struct SplitState {
+    int rows = 0, parity = 0;
+    uint32_t epoch = 0;
+};
 bool xrank_split_supported(int R, int M);
 // Thread path of the window medians when consecutive windows share most of their steps (the median
 // hardly moves): keys the interval is tuned to catch, weight of the newest median in its centre.
@@ -75,8 +82,8 @@ constexpr int kWindowNearTarget = 14;
 constexpr float kWindowNearSmooth = 1.0f;
 constexpr int kSplitMaxSteps = 256;   // steps per launch group of the split path (sizes its scratch)
 size_t xrank_split_scratch_bytes(int R, int M, int S_max);
-cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S, void *scratch, uint32_t *reasons,
-                               cudaStream_t st, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
+cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S, int S_max, SplitState &state, void *scratch, uint32_t *reasons,
+                               cudaStream_t st, int &launched, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
 bool xrank_bracket_supported(int R, int M);
 int xrank_scratch_steps(int R, int M, int want);
 size_t xrank_scratch_small_bytes(int M, int S_max);   // must be zero before first use

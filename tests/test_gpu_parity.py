@@ -567,3 +567,38 @@ def test_window_tiles(R, M, W, quant):
         for key in ("wmed", "fleet_med", "fleet_mad", "counts", "mask", "flags", "tier"):
             assert_bit_equal(to_np(out[key]), ref[key], "t=%d %s" % (t, key))
     g.close()
+
+
+@pytest.mark.parametrize("R,M,B,thr,deferred", [
+    (4097, 8, 20, 3.5, False),     # exceedance rows that are not word aligned; a last strip of one rank
+    (4611, 4, 33, 3.5, True),      # four metrics, odd rank count
+    (12345, 8, 20, 3.5, True),     # a sample of every twelfth run
+    (32767, 4, 20, 3.5, False),    # the widest fleet, odd
+    (4096, 8, 20, 0.5, False),     # a threshold inside the MAD's band: every column is recomputed
+    (8192, 8, 20, 1.3, False),     # a low threshold: many possible exceedances, lists of a warp overflow
+    (36000, 8, 9, 3.5, False),     # wider than the path takes: a cluster per step
+])
+def test_one_pass_blocks(R, M, B, thr, deferred):
+    """Blocks on the one-pass path: sampled estimates in the first, the previous block's in the second and third, a
+    smaller block in between, heavy tails on some ranks."""
+    from paper_2605_17879_b200 import guard
+    X, dirs = _rand_fleet(3 * B + B // 2, R, M, seed=R + M + B)
+    X[:, ::37, 0] *= np.float32(1.4)      # in every step: a block's statistics stay those of the block before
+    X[:, 4::59] *= np.float32(0.2)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, B, max(1, B // 2), dir=dirs, capacity=2 * B, topk=8, thr=thr)
+    g.set_deferred(deferred)
+    o = go.Oracle(R, M, B, max(1, B // 2), 8, dir=dirs, thr=thr)
+    t = 0
+    for n in (B, B // 2, B, B):
+        out = g.alloc_outputs()
+        g.ingest(Xd[t:t + n].contiguous())
+        g.score(out)
+        g.join()
+        assert g.sync_status() == 0
+        o.ingest(X[t:t + n])
+        compare_score(out, o.score(), "t=%d" % t)
+        t += n
+    if thr == 3.5 and R <= 32768:
+        assert g.fallback_steps() == 0
+    g.close()

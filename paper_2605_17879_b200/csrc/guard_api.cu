@@ -352,11 +352,10 @@ struct guard_ctx {
                 g.mad = a.mad + (size_t)s0 * M;
                 if (a.med_user) g.med_user = a.med_user + (size_t)s0 * M;
                 if (a.mad_user) g.mad_user = a.mad_user + (size_t)s0 * M;
-                int launched = 0;
                 cudaError_t e = launch_xrank_split(g, p, n, smax, split_state[scratch_sel], ws + L.xr_big + (size_t)scratch_sel * L.xr_big_stride,
-                                                   status() + 2, st, launched, (profiling == 1 && a.mask_base) ? &prof : nullptr);
+                                                   status() + 2, st, (profiling == 1 && a.mask_base) ? &prof : nullptr);
                 if (e != cudaSuccess) return e;
-                launches += launched;
+                launches += 4;
             }
             return cudaSuccess;
         }

@@ -69,10 +69,9 @@ cudaError_t launch_xrank_cluster(const XrankArgs &a, const MetricParams &p, int 
                                  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
 // One pass over a block's telemetry: values about the estimated median and MAD are kept in lists, from which both are
 // selected (4 or 8 metrics, 4 096 to 32 768 ranks).
-// What the host knows of a scratch of that path: step positions that hold estimates, their stamp, and which of the two
-// sets of flags the next launch uses.
+// What the host knows of a scratch of that path: the step positions it has held, and the stamp of their estimates.
 struct SplitState {
-    int rows = 0, parity = 0;
+    int rows = 0;
     uint32_t epoch = 0;
 };
 bool xrank_split_supported(int R, int M);
@@ -83,7 +82,7 @@ constexpr float kWindowNearSmooth = 1.0f;
 constexpr int kSplitMaxSteps = 256;   // steps per launch group of the split path (sizes its scratch)
 size_t xrank_split_scratch_bytes(int R, int M, int S_max);
 cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S, int S_max, SplitState &state, void *scratch, uint32_t *reasons,
-                               cudaStream_t st, int &launched, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
+                               cudaStream_t st, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof = nullptr);
 bool xrank_bracket_supported(int R, int M);
 int xrank_scratch_steps(int R, int M, int want);
 size_t xrank_scratch_small_bytes(int M, int S_max);   // must be zero before first use

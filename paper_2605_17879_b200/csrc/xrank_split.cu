@@ -1,10 +1,10 @@
 // Cross-rank selection, split path: blocks of fleets of some thousand to 32 768 ranks with 4 or 8 metrics, one pass
-// over the telemetry.  What makes one pass enough is an estimate (c, a) of a column's median and MAD: the result of
-// the same step position of the previous block (consecutive blocks of a fleet have almost the same per-step
+// over the telemetry.  What makes one pass enough is an estimate (c, a) of a column's median and MAD: the running
+// mean of the results at the same step position of earlier blocks (consecutive blocks of a fleet have almost the same per-step
 // statistics), or, where there is none, a histogram of a sample.
 //
-//   0. sample   (only where the scratch holds no estimates yet) one CTA per (step, four metrics): some thousand ranks
-//               are binned; the histogram's median, and the half-width about it that holds half of the mass;
+//   0. sample   (where there is no estimate from earlier blocks, or it missed lately) one CTA per (step, four metrics):
+//               some thousand ranks are binned; the histogram's median, and the half-width about it that holds half of the mass;
 //   1. sweep    one warp per (step, strip of ranks): with d = x - c, counts the values below the median's band
 //               |d| <= hm and inside the MAD's band | |d| - a | <= ha, and keeps those in either band (15 to 30 % of a
 //               column) in shared-memory lists, then in the column's list in global scratch; values that might exceed
@@ -37,7 +37,7 @@ namespace guard {
 
 namespace {
 
-constexpr int kSpThreads = 256;      // CTA of the sample and select kernels
+constexpr int kSpThreads = 256;      // CTA of the sample kernel
 constexpr int kSpU = 4;              // ranks per thread and sweep batch
 constexpr int kSpWarps = 4;          // warps of a sweep CTA (they share nothing but the columns' bands)
 constexpr int kSpSlack = 32;         // words behind each shared-memory list that absorb the stores of a full list
@@ -46,7 +46,9 @@ constexpr int kSpAmb = 1024;         // deferred exceedance decisions per step
 constexpr int kSpSBins = 2048;       // sample histogram bins
 constexpr int kSpMaxM = 8;
 constexpr int kSpMaxRanks = 32768;
-constexpr int kSpRest = 8;           // blocks a column whose list overflowed (ties) stays away from the sweep
+constexpr int kSpRest = 8;           // blocks a column whose list overflowed (ties) stays away from the sweep,
+                                     // or whose estimate missed takes a sample instead of the blocks before
+constexpr float kSpSmooth = 0.3f;    // weight of the newest result in the estimate
 constexpr float kFltMax = 3.402823466e+38f;
 // half-widths of the bands, in units of MAD / sqrt(n) for an estimate whose variance is that of n values (4.6 standard
 // errors; normal data: 1.858 MAD / sqrt(n) for a median, 1.167 for a MAD, 2.194 for both together)
@@ -59,43 +61,53 @@ struct SpGeom {
     int col_cap;    // ... and a column's list
     int s;          // sampled ranks
     int period;     // one run of four consecutive ranks is sampled out of every `period`
-    float q_prev;   // 1 / sqrt(n) of a previous result, and of a sample
-    float q_sample;
+    float q_sample; // a sample's standard error is that of 1 / q_sample^2 values
 };
 
 // Per-column record in global scratch.
 struct SpCol {
-    float med, mad;      // estimate, then result
-    float q, extra;      // the estimate's standard error is that of 1 / q^2 values; relative widening of the bands
+    float c, a;          // estimates of the median and the MAD
+    float q, extra;      // their standard error is that of 1 / q^2 values; relative widening of the bands
+    float v;             // variance of an estimate from earlier blocks, in units of a single block's (0: from a sample)
     uint32_t epoch;      // SpScratch::epoch: the record holds an estimate
-    uint32_t rest;       // blocks left before the column is swept again
+    uint16_t rest;       // blocks left before the column is swept again
+    uint16_t resample;   // blocks left that take a sample
     uint32_t nk;         // kept values
     uint32_t below, inner;
-    float rhs;           // exact threshold
-    uint32_t pad[2];
+    float med, rhs;      // the median and the exact threshold
 };
+
+// The estimate after an exact result: a running mean (its error adds to the next result's own), or the result itself
+// where there was none from earlier blocks.
+__device__ __forceinline__ void sp_learn(SpCol &col, const float med, const float mad, const bool afresh, const int R) {
+    const bool first = afresh || col.v == 0.0f;
+    col.c = first ? med : col.c + kSpSmooth * (med - col.c);
+    col.a = first ? mad : col.a + kSpSmooth * (mad - col.a);
+    col.v = first ? 1.0f : (1.0f - kSpSmooth) * (1.0f - kSpSmooth) * col.v + kSpSmooth * kSpSmooth;
+    col.q = sqrtf((1.0f + col.v) / (float)R);
+    col.extra = 0.0f;
+}
 
 struct SpScratch {
     SpCol *col;          // [S_max][M]
     uint32_t *fail;      // [S_max] metrics to be recomputed (a bit each); bit 31: one of them had been swept
     uint32_t *namb;      // [S_max] deferred exceedance decisions
-    uint32_t *fail_next, *namb_next;   // the same for the next launch on this scratch (cleared by the finish kernel)
     uint32_t *amb;       // [S_max][kSpAmb] (rank << 5 | metric)
     float *list;         // [S_max][M][col_cap] kept values
     uint32_t epoch;
-    int s_max;
 };
 
 // What the sweep and the selection derive from a column's estimate.  sc * (x - c) is what the bands are compared with.
 struct SpBands {
     float c, sc, hm, a, ha, rlo, rhi;   // hm, a, ha, rlo, rhi in units of 1 / sc
     float hd;                           // how far the MAD may be from its estimate for rlo, rhi to hold (unscaled)
+    float inv;                          // 1 / sc
     bool ok;
 };
 
 __device__ __forceinline__ SpBands sp_bands(const SpCol &col, const uint32_t epoch, const MetricParams &p, const int m) {
     SpBands b;
-    const float med = col.med, mad = col.mad, w = mad * col.q, x = mad * col.extra;
+    const float med = col.c, mad = col.a, w = mad * col.q, x = mad * col.extra;
     const float hm = kSpMed * w + x, ha = kSpBoth * w + 1.5f * x, hd = kSpMad * w + x;
     const float rel = p.floor_rel[m];
     const float lo = fmaxf(fmaxf(mad - hd, rel * fmaxf(fabsf(med) - hm, 0.0f)), p.floor_abs[m]);
@@ -103,7 +115,7 @@ __device__ __forceinline__ SpBands sp_bands(const SpCol &col, const uint32_t epo
     const float rlo = p.thrp[m] * lo * 0.99999f - 1.00001f * hm, rhi = p.thrp[m] * hi * 1.00001f + 1.00001f * hm;
     // the power of two that lifts hm (the smaller half-width) to 2^24 .. 2^25
     const int e = (int)(__float_as_uint(hm) >> 23) - 127;
-    b.ok = col.epoch == epoch && col.rest == 0u && mad > 0.0f && mad < 1.0e36f && fabsf(med) < 1.0e36f && e >= -100 && e <= 100 && rlo > mad;
+    b.ok = col.epoch == epoch && col.rest == 0 && mad > 0.0f && mad < 1.0e36f && fabsf(med) < 1.0e36f && e >= -100 && e <= 100 && rlo > mad;
     const float sc = __uint_as_float((uint32_t)(127 + 24 - e) << 23);
     b.ok = b.ok && fabsf(med) * sc < 1.0e37f && mad * sc < 1.0e37f;
     b.c = b.ok ? med : 0.0f;
@@ -114,6 +126,7 @@ __device__ __forceinline__ SpBands sp_bands(const SpCol &col, const uint32_t epo
     b.rlo = b.ok ? rlo * sc : CUDART_INF_F;
     b.rhi = b.ok ? rhi * sc : CUDART_INF_F;
     b.hd = hd;
+    b.inv = __uint_as_float((uint32_t)(127 - 24 + e) << 23);
     return b;
 }
 
@@ -122,34 +135,41 @@ constexpr int kSpSmpG = kSpThreads / 4;                 // threads per metric in
 constexpr int kSpSmpBatch = 16;                         // sampled ranks in flight per thread
 
 struct SpSampleShared {
-    uint32_t hist[4][kSpSBins / 2];   // 16-bit bins, two per word
-    uint16_t cum[4][kSpSBins + 2];    // values in the bins before
+    uint32_t hist[4][kSpSBins / 2 + 1];   // 16-bit bins, two per word; then the values in the bins before each
     uint32_t warp_tot[4][2];
     float inv_bw[4], off[4], pos[4];
     int ok[4];
-    uint32_t half[4];
+    uint32_t half[4], keep[4], again[4];
 };
 
 // The sample of a step: runs of four consecutive ranks, so that a warp's 128-bit loads use whole cache lines.  One
 // CTA handles four metrics: every thread bins the four components of its float4; then 64 threads per metric
 // scan their histogram.
-__global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const XrankArgs a, const SpGeom g, const SpScratch sc, const int reuse) {
+__global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const XrankArgs a, const SpGeom g, const SpScratch sc, const int rows) {
     __shared__ SpSampleShared sh;
     const int q = blockIdx.x, t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.R, M = a.M;
     const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
     const float *row = a.base + (size_t)slot * a.row_stride;
     SpCol *cols = sc.col + (size_t)t * M + 4 * q;
-    if (tid == 0 && q == 0) { sc.fail[t] = 0u; sc.namb[t] = 0u; sc.fail_next[t] = 0u; sc.namb_next[t] = 0u; }
+    const bool reuse = t < rows;   // the scratch has held this step position before
+    if (tid == 0 && q == 0) { sc.fail[t] = 0u; sc.namb[t] = 0u; }
     if (tid < 4) { cols[tid].nk = 0u; cols[tid].below = 0u; cols[tid].inner = 0u; }
-    // steps whose records hold results already need no sample
-    if (reuse && __syncthreads_and(cols[tid & 3].epoch == sc.epoch)) return;
+    // columns with an estimate from earlier blocks need no sample
+    const bool known = reuse && cols[tid & 3].epoch == sc.epoch;
+    const uint32_t again = known ? cols[tid & 3].resample : 0u;   // (thread c < 4 speaks for column c)
+    if (__syncthreads_and(known && again == 0u)) return;
 
     const int first = (g.period - 4) >> 1;
     float xpre = 0.0f;   // (warps 0..3) the 32 spread values that fix a metric's bin map
     if (warp < 4) xpre = __ldg(row + (size_t)min(R - 1, (int)(((long long)(2 * lane + 1) * R) >> 6)) * M + 4 * q + warp);
-    for (int i = tid; i < 4 * kSpSBins / 2; i += kSpThreads) (&sh.hist[0][0])[i] = 0u;
-    if (tid < 4) sh.half[tid] = 0xFFFFFFFFu;
+    for (int i = tid; i < 4 * (kSpSBins / 2 + 1); i += kSpThreads) (&sh.hist[0][0])[i] = 0u;
+    if (tid < 4) {
+        sh.half[tid] = 0xFFFFFFFFu;
+        sh.keep[tid] = known && again == 0u;
+        sh.again[tid] = again ? again - 1u : 0u;
+        if (!known) cols[tid].rest = 0;
+    }
     if (warp < 4) {
         const uint32_t key = ct_warp_sort(f2key(xpre), lane);
         const float c50 = key2f(__shfl_sync(0xFFFFFFFFu, key, 16));
@@ -203,14 +223,15 @@ __global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const Xran
     for (int i = 0; i < WPT; ++i) {
         const uint32_t c0 = w[i] & 0xFFFFu, c1 = w[i] >> 16;
         const int b = 2 * (gt * WPT + i);
-        sh.cum[c][b] = (uint16_t)run;
+        const uint32_t both = run | ((run + c0) << 16);
         if (mid >= run && mid < run + c0) sh.pos[c] = (float)b + (float)(mid - run) / (float)c0;
         run += c0;
-        sh.cum[c][b + 1] = (uint16_t)run;
+        sh.hist[c][b >> 1] = both;   // (this thread's words; it has read them)
         if (mid >= run && mid < run + c1) sh.pos[c] = (float)(b + 1) + (float)(mid - run) / (float)c1;
         run += c1;
     }
-    if (gt == kSpSmpG - 1) { sh.cum[c][kSpSBins] = (uint16_t)g.s; sh.cum[c][kSpSBins + 1] = (uint16_t)g.s; }
+    if (gt == kSpSmpG - 1) sh.hist[c][kSpSBins / 2] = (uint32_t)g.s;
+    const uint16_t *cum = reinterpret_cast<const uint16_t *>(sh.hist[c]);
     __syncthreads();
     // the smallest whole number of bins to either side of the median that holds half of the mass
     const float pos = sh.pos[c];
@@ -218,14 +239,14 @@ __global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const Xran
         if (v <= 0.0f) return 0.0f;
         if (v >= (float)kSpSBins) return (float)g.s;
         const int i = (int)v;
-        const float lo = (float)sh.cum[c][i];
-        return lo + (v - (float)i) * ((float)sh.cum[c][i + 1] - lo);
+        const float lo = (float)cum[i];
+        return lo + (v - (float)i) * ((float)cum[i + 1] - lo);
     };
     const float halfm = 0.5f * (float)g.s;
     for (int j = gt + 1; j <= kSpSBins / 2; j += kSpSmpG)
         if (mass(pos + (float)j) - mass(pos - (float)j) >= halfm) { atomicMin(&sh.half[c], (uint32_t)j); break; }
     __syncthreads();
-    if (gt == 0) {
+    if (gt == 0 && !sh.keep[c]) {
         SpCol &col = cols[c];
         const uint32_t h = sh.half[c];
         const bool ok = sh.ok[c] && h != 0xFFFFFFFFu;
@@ -236,11 +257,12 @@ __global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const Xran
             med = (float)(((double)pos - (double)sh.off[c]) * inv);
             mad = (float)(((double)(h - 1) + (m1 > m0 ? (double)((halfm - m0) / (m1 - m0)) : 0.0)) * inv);
         }
-        col.med = med;
-        col.mad = mad;
+        col.c = med;
+        col.a = mad;
         col.q = g.q_sample;
         col.extra = 0.01f;     // the bins' share of the error
-        col.rest = 0u;
+        col.v = 0.0f;
+        col.resample = (uint16_t)sh.again[c];
         col.epoch = ok ? sc.epoch : 0u;
     }
 }
@@ -489,59 +511,126 @@ __global__ void __launch_bounds__(32 * kSpWarps, 6) xsplit_sweep_kernel(const Xr
 }
 
 // ---- 2. selection ------------------------------------------------------------------------------
+// Keys of the two middle ranks among those that key(i) gives for a list's values (0xFFFFFFFF: not among them), left in
+// sh.v1[0] / sh.v2[0]; the range is in sh.lo / sh.width, the bins are zero.  ranks(k1, k2) gives their places among the
+// keys once key() has seen every value, or false.  The steps of ct_select, with the list read again in every pass (it
+// is in the first-level cache): what a pass keeps in registers would halve the CTAs that share an SM.
+template <int T, class Key, class Ranks>
+__device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, CtShared<1> &sh) {
+    const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
+    const uint32_t hist = (uint32_t)__cvta_generic_to_shared(sh.hist[0]);
+    uint32_t k1 = 0, k2 = 0;
+    bool searching = true;         // (of warp 0)
+#pragma unroll 1
+    for (int it = 0; it < kCtMaxIter; ++it) {
+        if (tid == 0) sh.any_open[it & 1] = 0u;
+        __syncthreads();           // range, counters and bins are ready
+        {
+            const uint32_t lo = sh.lo[0], width = sh.width[0];
+            const int sft = ct_shift(width);
+            uint32_t below = 0;
+#pragma unroll 4
+            for (uint32_t i = tid; i < n; i += T) ct_bin(key(i, it == 0), lo, width, sft, hist, below);
+            below = __reduce_add_sync(0xFFFFFFFFu, below);
+            if (lane == 0) atomicAdd(&sh.below[0], below);
+        }
+        if (it == 0) key.share();
+        __syncthreads();
+        if (it == 0 && !ranks(k1, k2)) return false;
+        if (warp == 0) ct_scan<1>(sh, 0, k1, k2);
+        __syncthreads();
+        {
+            const uint32_t f0 = sh.f0[0], fw = sh.fw[0], how = sh.how[0], cutk = sh.cutk[0];
+#pragma unroll 4
+            for (uint32_t i = tid; i < n; i += T) {
+                const uint32_t k = key(i, false);
+                if (k - f0 <= fw) {
+                    if (how == 1u) {
+                        const uint32_t pos = atomicAdd(&sh.nl[0], 1u);
+                        if (pos < (uint32_t)kCtList) sh.list[0][pos] = k;
+                    } else if (how >= 2u) {
+                        if (how == 3u || k <= cutk) atomicMax(&sh.mx[0], k);
+                        if (how == 3u || k > cutk) atomicMin(&sh.mn[0], k);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            searching = ct_settle<1>(sh, 0, k2 != k1);
+            if (lane == 0 && searching) sh.any_open[it & 1] = 1u;
+        }
+        __syncthreads();
+        if (sh.any_open[it & 1] == 0u) return true;
+    }
+    if (tid == 0) sh.bad = 1u;
+    return true;
+}
+
+// Keys of the kept values in the median's band (the very comparisons of the sweep; NaN is in no band), and how many values
+// are in either band.
+struct SpMedianKey {
+    const float *list;
+    float ks, kb, hm, a, ha;
+    uint32_t *s_n;
+    uint32_t nm = 0, na = 0;
+    __device__ __forceinline__ uint32_t operator()(const uint32_t i, const bool count) {
+        const float x = list[i], d = fabsf(__fmaf_rn(x, ks, kb));
+        const bool in = d <= hm;
+        if (count) {
+            nm += in;
+            na += fabsf(__fsub_rn(d, a)) <= ha;
+        }
+        return in ? f2key(x) : 0xFFFFFFFFu;
+    }
+    __device__ __forceinline__ void share() {
+        const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, nm | (na << 16));
+        if (lane_id() == 0) { atomicAdd(&s_n[0], tot & 0xFFFFu); atomicAdd(&s_n[1], tot >> 16); }
+    }
+};
+// ... and of the exact deviations of those in the MAD's band.
+struct SpMadKey {
+    const float *list;
+    float ks, kb, a, ha, med;
+    __device__ __forceinline__ uint32_t operator()(const uint32_t i, const bool) const {
+        const float x = list[i];
+        const bool in = fabsf(__fsub_rn(fabsf(__fmaf_rn(x, ks, kb)), a)) <= ha;
+        return in ? __float_as_uint(__fsub_rn(x, med)) << 1 : 0xFFFFFFFFu;
+    }
+    __device__ __forceinline__ void share() const {}
+};
+
 // The median and the MAD of a column from its kept values; why it is not proven, or -1.
-template <int V>
+template <int T>
 __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, const SpBands &b, const float sgn, const uint32_t below, const uint32_t inner,
                                          const int R, CtShared<1> &sh, uint32_t *s_n, float &med, float &mad) {
     const int tid = threadIdx.x;
     const bool even = (R & 1) == 0;
-    const uint32_t k1 = (uint32_t)((R - 1) / 2), k2 = (uint32_t)(R / 2);
-    float x[V];
-    uint32_t key[V];
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const uint32_t at = (uint32_t)(tid + i * kSpThreads);
-        x[i] = at < n ? list[at] : CUDART_NAN_F;
-    }
-    const float ks = sgn * b.sc, kb = -ks * b.c;
-    // the median's band (the very comparisons of the sweep; NaN is in no band)
-    uint32_t nm = 0, na = 0;
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const float d = fabsf(__fmaf_rn(x[i], ks, kb));
-        const bool in = d <= b.hm;
-        nm += in;
-        na += fabsf(__fsub_rn(d, b.a)) <= b.ha;
-        key[i] = in ? f2key(x[i]) : 0xFFFFFFFFu;
-    }
-    const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, nm | (na << 16));
-    if (tid == 0) { sh.below[0] = 0u; sh.bad = 0u; s_n[0] = 0u; s_n[1] = 0u; }
-    if (tid < kCtBins) sh.hist[0][tid] = 0u;
-    __syncthreads();
-    if (lane_id() == 0) { atomicAdd(&s_n[0], tot & 0xFFFFu); atomicAdd(&s_n[1], tot >> 16); }
-    const float w = b.hm / b.sc;
+    const uint32_t r1 = (uint32_t)((R - 1) / 2), r2 = (uint32_t)(R / 2);
+    const float ks = sgn * b.sc, kb = -ks * b.c, w = b.hm * b.inv;
+    for (int i = tid; i < kCtBins; i += T) sh.hist[0][i] = 0u;
     if (tid == 0) {
+        sh.below[0] = 0u;
+        sh.bad = 0u;
+        s_n[0] = 0u;
+        s_n[1] = 0u;
         const uint32_t lo = f2key(fdown(b.c - 1.00001f * w)), hi = f2key(fup(b.c + 1.00001f * w));
         sh.lo[0] = lo;
         sh.width[0] = hi - lo;
     }
-    __syncthreads();
-    nm = s_n[0];
-    na = s_n[1];
-    // (the sweep counted with the sign folded in: below there is above here)
-    const uint32_t blt = sgn > 0.0f ? below : (uint32_t)R - below - nm;
-    if (below + nm > (uint32_t)R || blt > k1 || k2 >= blt + nm) return kWhyMedianMiss;
-    ct_select<V, 1>(key, k1 - blt, k2 - blt, sh);
+    bool ok = sp_pick<T>(SpMedianKey{list, ks, kb, b.hm, b.a, b.ha, s_n},
+                      [&](uint32_t &k1, uint32_t &k2) {
+                          // (the sweep counted with the sign folded in: below there is above here)
+                          const uint32_t nm = s_n[0], blt = sgn > 0.0f ? below : (uint32_t)R - below - nm;
+                          k1 = r1 - blt;
+                          k2 = r2 - blt;
+                          return below + nm <= (uint32_t)R && blt <= r1 && r2 < blt + nm;
+                      },
+                      n, sh);
+    if (!ok) return kWhyMedianMiss;
     med = median_from_keys(sh.v1[0], sh.v2[0], even);
     const float delta = fabsf(__fsub_rn(med, b.c));
-    // the MAD's band
-    if (inner > k1 || k2 >= inner + na) return kWhyMadMiss;
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const bool in = fabsf(__fsub_rn(fabsf(__fmaf_rn(x[i], ks, kb)), b.a)) <= b.ha;
-        key[i] = in ? __float_as_uint(__fsub_rn(x[i], med)) << 1 : 0xFFFFFFFFu;
-    }
-    const float am = b.a / b.sc, ha = b.ha / b.sc;
+    const float am = b.a * b.inv, ha = b.ha * b.inv;
     const float lo = am - ha, hi = am + ha, margin = 1.0e-5f * (am + ha + delta);
     __syncthreads();
     if (tid == 0) {
@@ -549,7 +638,14 @@ __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, co
         sh.lo[0] = l;
         sh.width[0] = h - l;
     }
-    ct_select<V, 1>(key, k1 - inner, k2 - inner, sh);
+    ok = sp_pick<T>(SpMadKey{list, ks, kb, b.a, b.ha, med},
+                 [&](uint32_t &k1, uint32_t &k2) {
+                     k1 = r1 - inner;
+                     k2 = r2 - inner;
+                     return inner <= r1 && r2 < inner + s_n[1];
+                 },
+                 n, sh);
+    if (!ok) return kWhyMadMiss;
     const float v1 = __uint_as_float(sh.v1[0] >> 1), v2 = __uint_as_float(sh.v2[0] >> 1);
     mad = even ? __fmul_rn(0.5f, __fadd_rn(v1, v2)) : v1;
     if (sh.bad) return kWhySelect;
@@ -559,42 +655,47 @@ __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, co
     return proven ? -1 : kWhyMadMiss;
 }
 
-__global__ void __launch_bounds__(kSpThreads, 4) xsplit_select_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc,
-                                                                      uint32_t *reasons) {
+// T threads: 128 where there are columns enough to fill the GPU (their CTAs hide one another's serial parts), else more.
+template <int T>
+__global__ void __launch_bounds__(T, 1536 / T) xsplit_select_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc,
+                                                                        uint32_t *reasons) {
     __shared__ CtShared<1> sh;
-    __shared__ uint32_t s_n[2];
+    __shared__ SpBands sb;
+    __shared__ uint32_t s_n[2], s_col[4];
     const int m = blockIdx.x, t = blockIdx.y, tid = threadIdx.x;
     const int R = a.R, M = a.M;
     const size_t o = (size_t)t * M + m;
     SpCol &col = sc.col[o];
-    const SpBands b = sp_bands(col, sc.epoch, p, m);   // (the record is written at the end, by this CTA alone)
-    const uint32_t n = col.nk, below = col.below, inner = col.inner;
+    if (tid == 0) {
+        s_col[0] = col.nk;
+        s_col[1] = col.below;
+        s_col[2] = col.inner;
+        s_col[3] = sc.namb[t];
+        sb = sp_bands(col, sc.epoch, p, m);
+    }
     __syncthreads();
+    const SpBands &b = sb;
     if (!b.ok) return;                                 // the sweep has put the column on the step's list
+    const uint32_t n = s_col[0];
     const float sgn = p.dir[m] < 0 ? -1.0f : 1.0f;
-    const float *list = sc.list + o * g.col_cap;
     float med = 0.0f, mad = 0.0f;
     int why;
     if (n > (uint32_t)g.col_cap) why = kWhyCtaList;
-    else if (sc.namb[t] > (uint32_t)kSpAmb) why = kWhyAmbList;
-    else if (n <= 8u * kSpThreads) why = sp_select<8>(list, n, b, sgn, below, inner, R, sh, s_n, med, mad);
-    else if (n <= 12u * kSpThreads) why = sp_select<12>(list, n, b, sgn, below, inner, R, sh, s_n, med, mad);
-    else if (n <= 16u * kSpThreads) why = sp_select<16>(list, n, b, sgn, below, inner, R, sh, s_n, med, mad);
-    else why = sp_select<32>(list, n, b, sgn, below, inner, R, sh, s_n, med, mad);
+    else if (s_col[3] > (uint32_t)kSpAmb) why = kWhyAmbList;
+    else why = sp_select<T>(sc.list + o * g.col_cap, n, b, sgn, s_col[1], s_col[2], R, sh, s_n, med, mad);
     if (tid != 0) return;
     if (why < 0) {
         a.med[o] = med;
         a.mad[o] = mad;
         if (a.med_user) a.med_user[o] = med;
         if (a.mad_user) a.mad_user[o] = mad;
-        col.rhs = __fmul_rn(p.thrp[m], scale_of(mad, med, p.floor_rel[m], p.floor_abs[m]));
         col.med = med;
-        col.mad = mad;
-        col.q = g.q_prev;
-        col.extra = 0.0f;
+        col.rhs = __fmul_rn(p.thrp[m], scale_of(mad, med, p.floor_rel[m], p.floor_abs[m]));
+        sp_learn(col, med, mad, false, R);
     } else {
         atomicOr(&sc.fail[t], 0x80000000u | (1u << m));
         if (why == kWhyCtaList) col.rest = kSpRest + 1;
+        else if (why != kWhyAmbList) col.resample = kSpRest;
         if (reasons) atomicAdd(reasons + why, 1u);
     }
 }
@@ -632,15 +733,7 @@ __global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, 
                 }
             }
         }
-        if (tid < M) {                                // ready for the next launch on this scratch
-            SpCol &col = sc.col[(size_t)t * M + tid];
-            col.nk = 0u;
-            col.below = 0u;
-            col.inner = 0u;
-        }
     }
-    if (blockIdx.x == 0)
-        for (int t = tid; t < sc.s_max; t += blockDim.x) { sc.fail_next[t] = 0u; sc.namb_next[t] = 0u; }
     if (!any) return;
     if (tid < 32) {   // one warp: a running sum over the steps
         uint32_t run = 0;
@@ -672,12 +765,10 @@ __global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, 
         __syncthreads();
         if (tid == 0) {                    // the result is the next block's estimate
             SpCol &col = sc.col[(size_t)lo * M + m];
-            col.med = a.med[(size_t)lo * M + m];
-            col.mad = a.mad[(size_t)lo * M + m];
-            col.q = g.q_prev;
-            col.extra = 0.0f;
+            sp_learn(col, a.med[(size_t)lo * M + m], a.mad[(size_t)lo * M + m], true, R);
+            if (col.epoch != sc.epoch) col.resample = 0;
             col.epoch = sc.epoch;
-            if (col.rest) col.rest -= 1u;
+            if (col.rest) col.rest -= 1;
         }
     }
 }
@@ -692,9 +783,8 @@ SpGeom split_geometry(int R, int S) {
     const int want = R / 4 > 4096 ? R / 4 : 4096;
     g.period = 4 * (R / want > 1 ? R / want : 1);
     g.s = 4 * (R / g.period);
-    g.q_prev = (float)sqrt(2.0 / R);
     g.q_sample = (float)sqrt(1.0 / g.s - 1.0 / R > 0.0 ? 1.0 / g.s - 1.0 / R : 0.0);
-    const double q = g.q_prev > g.q_sample ? g.q_prev : g.q_sample;
+    const double q_prev = sqrt(2.0 / R), q = q_prev > g.q_sample ? q_prev : g.q_sample;
     const double f = q * (2.0 * kSpMed * 0.2691 + 4.0 * kSpBoth * 0.2143) + 0.03;   // densities at the median and at the quartiles, per MAD
     const double kept = g.strip * f;
     g.cap = (int)ceil(kept + 6.0 * sqrt(kept)) + 16;
@@ -716,28 +806,25 @@ size_t xrank_split_scratch_bytes(int R, int M, int S_max) {
     const SpGeom g = split_geometry(R, S_max);
     size_t b = 0;
     b += align256((size_t)S_max * M * sizeof(SpCol));
-    b += align256((size_t)S_max * sizeof(uint32_t)) * 4;
+    b += align256((size_t)S_max * sizeof(uint32_t)) * 2;
     b += align256((size_t)S_max * kSpAmb * sizeof(uint32_t));
     b += align256((size_t)S_max * M * g.col_cap * sizeof(float));
     return b;
 }
 
 cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S, int S_max, SplitState &state, void *scratch, uint32_t *reasons,
-                               cudaStream_t st, int &launched, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof) {
+                               cudaStream_t st, std::vector<std::pair<cudaEvent_t, cudaEvent_t>> *prof) {
     if (S <= 0) return cudaSuccess;
     const int M = a.M;
     const SpGeom g = split_geometry(a.R, S);
     SpScratch sc{};
     char *b = (char *)scratch;
     sc.col = (SpCol *)b;      b += align256((size_t)S_max * M * sizeof(SpCol));
-    uint32_t *flags[4];
-    for (int i = 0; i < 4; ++i) { flags[i] = (uint32_t *)b; b += align256((size_t)S_max * sizeof(uint32_t)); }
+    sc.fail = (uint32_t *)b;  b += align256((size_t)S_max * sizeof(uint32_t));
+    sc.namb = (uint32_t *)b;  b += align256((size_t)S_max * sizeof(uint32_t));
     sc.amb = (uint32_t *)b;   b += align256((size_t)S_max * kSpAmb * sizeof(uint32_t));
     sc.list = (float *)b;
-    sc.fail = flags[state.parity]; sc.fail_next = flags[state.parity ^ 1];
-    sc.namb = flags[2 + state.parity]; sc.namb_next = flags[2 + (state.parity ^ 1)];
     sc.epoch = a.hint_epoch;
-    sc.s_max = S_max;
     const size_t smem = split_sweep_smem(g, M);
     static std::mutex attr_mutex;
     static bool attr_set_dev[64] = {};
@@ -756,24 +843,22 @@ cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S,
     }
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (prof && (cudaEventCreate(&ev0) != cudaSuccess || cudaEventCreate(&ev1) != cudaSuccess)) return cudaGetLastError();
-    // estimates for the step positions this scratch has not seen (or for all of them, without hints)
-    if (a.hint_fresh || state.rows < S || state.epoch != a.hint_epoch) {
-        const int reuse = !a.hint_fresh && state.epoch == a.hint_epoch && state.rows > 0;
-        xsplit_sample_kernel<<<dim3(M / 4, S), kSpThreads, 0, st>>>(a, g, sc, reuse);
-        state.rows = state.epoch == a.hint_epoch && state.rows > S ? state.rows : S;
-        state.epoch = a.hint_epoch;
-        launched += 1;
-    }
+    // estimates for the step positions and columns that have none (with hints a look at the records, as a rule: 2 us)
+    const bool same = state.epoch == a.hint_epoch;
+    xsplit_sample_kernel<<<dim3(M / 4, S), kSpThreads, 0, st>>>(a, g, sc, !a.hint_fresh && same ? state.rows : 0);
+    state.rows = same && state.rows > S ? state.rows : S;
+    state.epoch = a.hint_epoch;
     if (prof) cudaEventRecord(ev0, st);   // the sweep, the longest kernel
     if (M == 8) xsplit_sweep_kernel<2><<<dim3(g.chunks, S), 32 * kSpWarps, smem, st>>>(a, p, g, sc);
     else xsplit_sweep_kernel<1><<<dim3(g.chunks, S), 32 * kSpWarps, smem, st>>>(a, p, g, sc);
     if (prof) cudaEventRecord(ev1, st);
-    xsplit_select_kernel<<<dim3(M, S), kSpThreads, 0, st>>>(a, p, g, sc, reasons);
+    // (22 us against 23 for 1 600 columns of some 1 900 values; 9 against 14 for 400 of 2 300)
+    if ((long long)S * M > 148 * 6) xsplit_select_kernel<128><<<dim3(M, S), 128, 0, st>>>(a, p, g, sc, reasons);
+    else if ((long long)S * M > 148 * 3) xsplit_select_kernel<256><<<dim3(M, S), 256, 0, st>>>(a, p, g, sc, reasons);
+    else xsplit_select_kernel<512><<<dim3(M, S), 512, 0, st>>>(a, p, g, sc, reasons);
     const int T = a.R <= 32 * 128 ? 128 : (a.R <= 32 * 256 ? 256 : (a.R <= 32 * 512 ? 512 : 1024));
     const int most = 148 * (1024 / T);   // what the SMs hold of them at 64 registers per thread
     xsplit_finish_kernel<32><<<S * M < most ? S * M : most, T, 0, st>>>(a, p, g, sc, S);
-    launched += 3;
-    state.parity ^= 1;
     e = cudaGetLastError();
     if (prof) prof->emplace_back(ev0, ev1);
     return e;

@@ -31,7 +31,7 @@ struct Layout {
     int xr_steps;   // steps per launch of the multi-kernel bracketed cross-rank path (0: not used)
     int xr_cluster; // the cluster-per-step cross-rank path applies
     int xr_split;   // the six-kernel split cross-rank path applies
-    int xr_gridp;   // single rows keep brackets between calls (two ColHintState at xr_grid: ingest, fleet baseline)
+    int xr_gridp;   // single rows count how many were bracketed by the row before (two RowHints at xr_grid: ingest, fleet baseline)
 };
 
 // State and scratch first, the two rings last (the telemetry ring is by far the largest).
@@ -50,8 +50,8 @@ Layout make_layout(int R, int M, int C, int K) {
     L.xr_cluster = (!L.xr_split && xrank_cluster_supported(R, M)) ? 1 : 0;
     L.xr_steps = (!L.xr_split && !L.xr_cluster && xrank_bracket_supported(R, M)) ? xrank_scratch_steps(R, M, C) : 0;
     L.xr_small = off;  off = align_up(off + (L.xr_steps ? xrank_scratch_small_bytes(M, L.xr_steps) : 0));
-    L.xr_gridp = (xrank_column_supported(R) && R >= 8192) ? 1 : 0;
-    L.xr_grid = off;   off = align_up(off + 2 * align_up(sizeof(ColHintState)));
+    L.xr_gridp = (xrank_count_supported(R) && R >= 8192) ? 1 : 0;
+    L.xr_grid = off;   off = align_up(off + 2 * align_up(sizeof(RowHints)));
     L.inc_rbc = off;   off = align_up(off + 64);   // rebuild list counter and ticket (zero before first use)
     // the windowed medians and the kept top-k indices exist twice: consecutive evaluations alternate, so that a
     // deferred evaluation's tail may still read its medians while the next evaluation's window kernels write theirs
@@ -324,14 +324,9 @@ struct guard_ctx {
         static std::atomic<uint32_t> next{(uint32_t)std::chrono::steady_clock::now().time_since_epoch().count() | 1u};
         do { split_epoch = next.fetch_add(1u); } while (split_epoch == 0u);
     }
-    ColHintState *hint_state(int site) const { return (ColHintState *)(ws + L.xr_grid + (size_t)site * align_up(sizeof(ColHintState))); }
+    RowHints *hint_state(int site) const { return (RowHints *)(ws + L.xr_grid + (size_t)site * align_up(sizeof(RowHints))); }
     cudaError_t xrank(XrankArgs a, int S, cudaStream_t st, bool own_scratch = true, int site = -1) {
-        // one row of a wide fleet: bracketed by the call site's previous result
-        if (S == 1 && site >= 0 && L.xr_gridp && row_hints) {
-            a.hint = hint_state(site);
-            launches += 1;
-            return launch_xrank_column(a, p, S, st);
-        }
+        if (S == 1 && site >= 0 && L.xr_gridp && row_hints) a.hint = hint_state(site);
         // everything the streaming paths do not take, or not for so few columns
         if (xrank_count_supported(R) && ((!L.xr_split && !L.xr_cluster) || a.mask_bytes != 1 || (long long)S * M <= 64)) {
             launches += 1;
@@ -815,10 +810,7 @@ int guard_sweep_qualify(const float *d_S, int nodes, int gpus_per_node, int reps
     x.mad_user = d_fleet_mad;
     for (int m = 0; m < metrics; ++m) x.cut_rank[m] = p.dir[m] < 0 ? (int)(j - 1) : (int)(G - j);
     x.status = d_status;
-    // (a single row of more than 8 192 values without an earlier result to start from: measured 25 us with the whole
-    // column's histogram against 33 us at 16 384 GPUs)
-    e = xrank_count_supported(G) && G <= 8192 ? launch_xrank_count(x, p, 1, st)
-        : xrank_column_supported(G) ? launch_xrank_column(x, p, 1, st) : launch_xrank_direct(x, p, 1, st);
+    e = xrank_count_supported(G) ? launch_xrank_count(x, p, 1, st) : launch_xrank_direct(x, p, 1, st);
     if (e != cudaSuccess) { set_error(g_error, "sweep fleet statistics launch: %s", cudaGetErrorString(e)); return GUARD_ERR_CUDA; }
     if (d_fleet_cut) {
         e = cudaMemcpyAsync(d_fleet_cut, fleet + 2 * kMaxMetrics, metrics * sizeof(float), cudaMemcpyDeviceToDevice, st);

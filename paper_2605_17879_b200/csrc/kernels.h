@@ -28,7 +28,7 @@ struct XrankArgs {
     uint32_t *only_flagged; // [S] or NULL: direct kernel processes step s only if nonzero, then clears it
     uint32_t *fallbacks;    // or NULL: counts the steps the direct kernel redid for the bracketed path
     int prev_rows;          // rows of med / mad that hold an earlier result of the same row position (counting path: first pivots)
-    void *hint;             // ColHintState of the call site (one row per call), or NULL: column kernels only
+    void *hint;             // RowHints of the call site (one row per call), or NULL: counting path only
     uint32_t hint_epoch;    // split path: stamp of the estimates in its scratch (non-zero)
     int hint_fresh;         // split path: take no estimate from an earlier block
 };
@@ -48,21 +48,11 @@ struct XrankScratch {
     int cap, amb_cap, S_max;
 };
 enum { kWhyCtaList = 0, kWhyStepList = 1, kWhyAmbList = 2, kWhyMedianMiss = 3, kWhySelect = 4, kWhyMadMiss = 5 };
-// State a call site of the column kernels keeps between its rows (zero before first use): the previous
-// median / MAD in the output arrays bracket the next ones; hw holds the tuned half-widths of the two
-// brackets per metric (0: derive from the MAD; negative: rows left before the hint is tried again).
-struct ColHintState {
-    uint32_t rows;       // diagnostic: rows seen
-    uint32_t settled;    // diagnostic: columns whose median and MAD both came out of their brackets
-    uint32_t pad[2];
-    uint32_t valid[kMaxMetrics];   // the output arrays hold a previous result of this call site for metric m
-    float hw[2][kMaxMetrics];
-    // every entry of metric m is written only by the leader of the cluster that handles column m, after all
-    // CTAs of that cluster have read it: the CTAs of a cluster always decide alike
+// Single rows of a call site (ingested steps, fleet baselines) that were bracketed by the site's previous result.
+struct RowHints {
+    uint32_t rows;       // rows seen
+    uint32_t settled;    // columns whose median and MAD both came out of their brackets
 };
-// One CTA per (row, metric) column with the column in registers: for a few rows at a time.
-bool xrank_column_supported(int R);
-cudaError_t launch_xrank_column(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);
 // One cluster of four CTAs per step (4 or 8 metrics, a few thousand ranks and more).
 bool xrank_cluster_supported(int R, int M);
 cudaError_t launch_xrank_cluster(const XrankArgs &a, const MetricParams &p, int S, uint32_t *reasons, cudaStream_t st,

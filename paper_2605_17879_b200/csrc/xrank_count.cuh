@@ -6,6 +6,9 @@
 //   2. one pass counts the keys below the range and bins those inside (256 bins in shared memory);
 //   3. one warp per metric scans its bins for the wanted ranks; a second pass fetches the keys of those one or
 //      two bins (a few), and the warp ranks them.
+// A few wide columns (a single row of thousands of ranks) take a cluster of NC CTAs each (C = 1): the CTAs bin their
+// shares on their own, sum one another's bins and gather one another's few keys through distributed shared memory
+// (two cluster barriers a round), and all take the same decisions.
 // The counts prove the range; one that misses is moved, and a bin that holds too many keys becomes the next
 // range (or the answer, if they are all the same: ties), so any values come out exactly.  A key is 32 bits in
 // the order of the values, so that both statistics (and both kinds of range) share one piece of code.
@@ -28,7 +31,7 @@ constexpr uint32_t kCtNone = 0xFFFFFFFFu;
 
 template <int C>
 struct CtShared {
-    uint32_t hist[C][kCtBins];
+    __align__(16) uint32_t hist[C][kCtBins];
     uint32_t lo[C], width[C];      // the range [lo, lo + width]
     uint32_t below[C];             // keys below it
     uint32_t f0[C], fw[C];         // keys to fetch: [f0, f0 + fw]
@@ -38,6 +41,7 @@ struct CtShared {
     uint32_t mx[C], mn[C];
     uint32_t nl[C];                // gathered keys
     uint32_t list[C][kCtList];
+    uint32_t all[kCtList];         // (clusters) the lists of all CTAs
     uint32_t v1[C], v2[C];
     uint32_t any_open[2];
     float med[C], rhs[C];
@@ -86,15 +90,65 @@ __device__ __forceinline__ void ct_hit(const uint32_t k, const uint32_t f0, cons
         : "r"(k), "r"(f0), "r"(fw), "r"(bit));
 }
 
+// Distributed shared memory of a cluster: the address of this CTA's variable p in CTA `rank`, and loads from there.
+__device__ __forceinline__ uint32_t ct_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t ct_map(const void *p, const uint32_t rank) {
+    uint32_t o;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return o;
+}
+__device__ __forceinline__ uint32_t ct_ld(const uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ct_ld4(const uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+// Barrier of all threads that share a column.
+template <int NC>
+__device__ __forceinline__ void ct_sync() {
+    if (NC == 1) __syncthreads();
+    else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // Scans the bins of column c (one warp): what to fetch for ranks k1 and k2, or where the range has to move.
-template <int C>
+template <int C, int NC = 1>
 __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint32_t k1, const uint32_t k2) {
     const int lane = lane_id();
     uint4 *h = reinterpret_cast<uint4 *>(&sh.hist[c][lane * 8]);
-    const uint4 a = h[0], b = h[1];
-    const uint32_t below = sh.below[c], lo = sh.lo[c], width = sh.width[c];
-    h[0] = make_uint4(0u, 0u, 0u, 0u);
-    h[1] = make_uint4(0u, 0u, 0u, 0u);
+    uint4 a, b;
+    uint32_t below;
+    const uint32_t lo = sh.lo[c], width = sh.width[c];
+    if (NC == 1) {
+        a = h[0];
+        b = h[1];
+        below = sh.below[c];
+        h[0] = make_uint4(0u, 0u, 0u, 0u);
+        h[1] = make_uint4(0u, 0u, 0u, 0u);
+    } else {   // (the other CTAs read this one's bins as well: cleared after the next cluster barrier)
+        a = b = make_uint4(0u, 0u, 0u, 0u);
+        uint4 va[NC], vb[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const uint32_t at = ct_map(h, (uint32_t)k);
+            va[k] = ct_ld4(at);
+            vb[k] = ct_ld4(at + 16u);
+        }
+        const uint32_t part = lane < NC ? ct_ld(ct_map(&sh.below[c], (uint32_t)(lane & (NC - 1)))) : 0u;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            a.x += va[k].x; a.y += va[k].y; a.z += va[k].z; a.w += va[k].w;
+            b.x += vb[k].x; b.y += vb[k].y; b.z += vb[k].z; b.w += vb[k].w;
+        }
+        below = __reduce_add_sync(0xFFFFFFFFu, part);
+    }
     const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const uint32_t sum = ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
     uint32_t incl = sum;
@@ -117,7 +171,7 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
     q = __shfl_sync(0xFFFFFFFFu, q, s1);
     n = __shfl_sync(0xFFFFFFFFu, n, s1);
     if (lane == 0) {
-        sh.below[c] = 0u;
+        if (NC == 1) sh.below[c] = 0u;
         sh.nl[c] = 0u;
         sh.mx[c] = 0u;
         sh.mn[c] = kCtNone;
@@ -144,11 +198,46 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
 }
 
 // The answer of column c from the fetched keys (one warp), or the next range; returns whether the search goes on.
-template <int C>
+template <int C, int NC = 1>
 __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bool pair) {
     const int lane = lane_id();
-    const uint32_t how = sh.how[c], n = sh.nl[c], q1 = sh.q1[c], mx = sh.mx[c], mn = sh.mn[c];
-    const uint32_t mine = sh.list[c][lane], mine2 = sh.list[c][lane + 32];
+    const uint32_t how = sh.how[c], q1 = sh.q1[c];
+    uint32_t n, mx, mn, mine, mine2;
+    const uint32_t *list;
+    if (NC == 1) {
+        n = sh.nl[c];
+        mx = sh.mx[c];
+        mn = sh.mn[c];
+        list = sh.list[c];
+    } else {
+        const uint32_t k = (uint32_t)(lane & (NC - 1));
+        const uint32_t own = ct_ld(ct_map(&sh.nl[c], k));
+        mx = __reduce_max_sync(0xFFFFFFFFu, ct_ld(ct_map(&sh.mx[c], k)));
+        mn = __reduce_min_sync(0xFFFFFFFFu, ct_ld(ct_map(&sh.mn[c], k)));
+        // all CTAs' keys in one list (their bins hold kCtList at most together)
+        uint32_t incl = lane < NC ? own : 0u;
+        const uint32_t cnt = incl;
+#pragma unroll
+        for (int d = 1; d < NC; d <<= 1) { const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, incl, d); if (lane >= d) incl += u; }
+        n = __shfl_sync(0xFFFFFFFFu, incl, NC - 1);
+        if (how == 1u && n <= (uint32_t)kCtList) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t e = (uint32_t)(lane + 32 * half);
+                uint32_t from = 0, off = 0;
+#pragma unroll
+                for (int d = 0; d < NC; ++d) {
+                    const uint32_t end = __shfl_sync(0xFFFFFFFFu, incl, d), num = __shfl_sync(0xFFFFFFFFu, cnt, d);
+                    if (e < end && e >= end - num) { from = (uint32_t)d; off = e - (end - num); }
+                }
+                if (e < n) sh.all[e] = ct_ld(ct_map(&sh.list[c][off], from));
+            }
+            __syncwarp();
+        }
+        list = sh.all;
+    }
+    mine = list[lane];
+    mine2 = list[lane + 32];
     if (how == 0u) return true;                      // the range moved
     if (how != 1u) {
         if (how == 3u && mx != mn) {                 // a full bin of different keys becomes the range
@@ -163,7 +252,7 @@ __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bo
         uint32_t lt = 0, le = 0;
 #pragma unroll 4
         for (uint32_t j = 0; j < n; ++j) {
-            const uint32_t o = sh.list[c][j];
+            const uint32_t o = list[j];
             lt += o < x;
             le += o <= x;
         }
@@ -176,9 +265,10 @@ __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bo
 }
 
 // Keys of 0-based ranks k1 and k2 (k2 == k1 or k1 + 1) of the C columns held by the CTA, left in sh.v1 / sh.v2; the
-// columns' ranges are in sh.lo / sh.width, the bins are zero.  All threads of the CTA call this.
-template <int V, int C>
-__device__ __forceinline__ void ct_select(const uint32_t (&key)[V], const uint32_t k1, const uint32_t k2, CtShared<C> &sh) {
+// columns' ranges are in sh.lo / sh.width, the bins are zero.  All threads of the CTA (of the cluster) call this; returns
+// the number of rounds.
+template <int V, int C, int NC = 1>
+__device__ __forceinline__ int ct_select(const uint32_t (&key)[V], const uint32_t k1, const uint32_t k2, CtShared<C> &sh) {
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id();
     const int col = tid & (C - 1);
     const uint32_t hist = (uint32_t)__cvta_generic_to_shared(sh.hist[col]);
@@ -197,8 +287,8 @@ __device__ __forceinline__ void ct_select(const uint32_t (&key)[V], const uint32
             for (int d = 16; d >= C; d >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, d);
             if (lane < C) atomicAdd(&sh.below[lane], below);
         }
-        __syncthreads();
-        if (warp < C && searching) ct_scan<C>(sh, warp, k1, k2);
+        ct_sync<NC>();
+        if (warp < C && searching) ct_scan<C, NC>(sh, warp, k1, k2);
         __syncthreads();
         {
             const uint32_t f0 = sh.f0[col], fw = sh.fw[col];
@@ -223,23 +313,28 @@ __device__ __forceinline__ void ct_select(const uint32_t (&key)[V], const uint32
                 }
             }
         }
-        __syncthreads();
+        ct_sync<NC>();
+        if (NC > 1) {              // every CTA has read the bins
+            for (int i = tid; i < C * kCtBins; i += blockDim.x) (&sh.hist[0][0])[i] = 0u;
+            if (tid < C) sh.below[tid] = 0u;
+        }
         if (warp < C && searching) {
-            searching = ct_settle<C>(sh, warp, k2 != k1);
+            searching = ct_settle<C, NC>(sh, warp, k2 != k1);
             if (lane == 0) {
                 if (searching) sh.any_open[it & 1] = 1u;
                 else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fw[warp] = 0u; }   // (no key at all)
             }
         }
         __syncthreads();
-        if (sh.any_open[it & 1] == 0u) return;
+        if (sh.any_open[it & 1] == 0u) return it + 1;
     }
     if (tid == 0) sh.bad = 1u;
+    return kCtMaxIter;
 }
 
 // Median, MAD (and optional extra order statistic) of metrics [m0, m0 + C) of row s of the launch, and their
-// exceedance bits.  C divides M, (R * C) <= V * blockDim.x, blockDim.x >= 32 * C.
-template <int V, int C>
+// exceedance bits.  C divides M, R * C <= V * NC * blockDim.x, blockDim.x >= 32 * C; C = 1 with clusters.
+template <int V, int C, int NC = 1>
 __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p, const int s, const int m0, CtShared<C> &sh) {
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id(), T = blockDim.x;
     const int R = a.R, M = a.M;
@@ -250,11 +345,16 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     const uint32_t k1 = (uint32_t)((R - 1) / 2), k2 = (uint32_t)(R / 2);
 
     uint32_t key[V];                      // first the values' keys, later those of the deviations
-    const int dr = T / C, r0 = tid / C;   // this thread's ranks: r0, r0 + dr, ...
+    // this thread's ranks: r0, r0 + dr, ...
+    const int crank = NC == 1 ? 0 : (int)ct_rank(), dr = NC * T / C, r0 = crank * T + tid / C;
+    const bool speaks = crank == 0;
+    bool settled = true;
     float xs = 0.0f, hmed = 0.0f, hmad = -1.0f;
     if (warp < C) {
         xs = __ldg(row + (size_t)(((2 * lane + 1) * (long long)R) >> 6) * M + warp);
-        if (a.prev_rows > 0) {            // the result arrays still hold an earlier result of this row position
+        // the result arrays still hold an earlier result of this row position, or of another one (only its own with a
+        // cluster: another row's leader may be writing there, and the CTAs of a cluster have to read the same)
+        if (NC == 1 ? a.prev_rows > 0 : s < a.prev_rows) {
             const size_t o = (size_t)min(s, a.prev_rows - 1) * M + m0 + warp;
             hmed = a.med[o];
             hmad = a.mad[o];
@@ -301,7 +401,8 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     for (int what = 0;;) {
         const bool extra = what >= 2;
         const uint32_t q1 = extra ? (uint32_t)a.cut_rank[m0 + what - 2] : k1, q2 = extra ? q1 : k2;
-        ct_select<V, C>(key, q1, q2, sh);
+        const int rounds = ct_select<V, C, NC>(key, q1, q2, sh);
+        settled = settled && (extra || (hinted && rounds == 1));   // (thread 0's warp knows of a hint)
         if (tid < C) {
             const uint32_t v1 = sh.v1[tid], v2 = sh.v2[tid];
             const int m = m0 + tid;
@@ -312,12 +413,19 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                 const float lo = __uint_as_float(v1 >> 1), md = sh.med[tid];
                 const float mad = even ? __fmul_rn(0.5f, __fadd_rn(lo, __uint_as_float(v2 >> 1))) : lo;
                 sh.rhs[tid] = __fmul_rn(p.thrp[m], scale_of(mad, md, p.floor_rel[m], p.floor_abs[m]));
-                a.med[o] = md;
-                a.mad[o] = mad;
-                if (a.med_user) a.med_user[o] = md;
-                if (a.mad_user) a.mad_user[o] = mad;
-                if (tid == 0 && sh.bad) atomicOr(a.status, kStatInternal);
-            } else if (tid == what - 2) {
+                if (speaks) {
+                    a.med[o] = md;
+                    a.mad[o] = mad;
+                    if (a.med_user) a.med_user[o] = md;
+                    if (a.mad_user) a.mad_user[o] = mad;
+                    if (tid == 0 && sh.bad) atomicOr(a.status, kStatInternal);
+                    if (NC > 1 && a.hint) {
+                        RowHints *h = reinterpret_cast<RowHints *>(a.hint);
+                        if (m == 0) atomicAdd(&h->rows, 1u);
+                        if (settled) atomicAdd(&h->settled, 1u);
+                    }
+                }
+            } else if (tid == what - 2 && speaks) {
                 a.cut[o] = key2f(v1);
             }
         }

@@ -530,6 +530,23 @@ def test_columns_held_in_registers(R, M, B, T, quant):
     run_both(X, B, max(1, B // 2), 16, dirs, [B], capacity=2 * B, min_signals=2)
 
 
+@pytest.mark.parametrize("R,M,B,quant", [
+    (4097, 8, 1, None),            # the narrowest column over eight CTAs; a ragged last one
+    (4100, 9, 4, None),            # four CTAs per column, several rows
+    (8192, 19, 1, None),           # bracketed rows of too many metrics for eight CTAs each; 32-bit exceedance words
+    (16385, 4, 2, None),           # eight values per thread
+    (32768, 1, 1, None),           # the widest column
+    (32768, 6, 6, None),           # the same over four CTAs: sixteen values per thread
+    (12345, 5, 1, 40),             # ties: lists of several CTAs, bins of equal keys
+])
+def test_columns_over_clusters(R, M, B, quant):
+    """A few wide rows: columns spread over clusters, bracketed by the row before and (a jump of every rank) missed."""
+    T = 3 * B + 4
+    X, dirs = _rand_fleet(T, R, M, seed=3 * R + M, quant=quant)
+    X[T - B - 2:] *= np.float32(1.75)
+    run_both(X, 4, 2, 16, dirs, [B], capacity=max(B, 4), min_signals=2)
+
+
 @pytest.mark.parametrize("R,M,W,quant", [
     (70, 3, 1, None),              # one step; a ragged last tile
     (64, 4, 64, None),             # every slot of eight warps of eight values in use

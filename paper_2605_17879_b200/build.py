@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libguard_b200.so")
 NATIVE = os.path.join(HERE, "_guard_native.so")   # the Python binding's marshalling (csrc/binding.cpp)
-SOURCES = ["guard_api.cu", "xrank.cu", "xrank_bracket.cu", "xrank_cluster.cu", "xrank_split.cu", "xrank_count.cu", "window.cu", "window_bins.cu", "score.cu", "topk.cu", "sweep.cu", "triage.cu"]
+SOURCES = ["guard_api.cu", "xrank.cu", "xrank_bracket.cu", "xrank_cluster.cu", "xrank_split.cu", "xrank_count.cu", "window.cu", "window_bins.cu", "score.cu", "topk.cu", "eval_tail.cu", "sweep.cu", "triage.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "--fmad=false",            # every decision is defined on unfused float32 operations

@@ -257,7 +257,7 @@ struct guard_ctx {
         int prio_lo = 0, prio_hi = 0;
         cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
         if (cudaStreamCreateWithPriority(&tail, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) { tail = nullptr; return false; }
-        if (cudaStreamCreateWithPriority(&aux, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) aux = nullptr;
+        if (!xrank_count_supported(R) && cudaStreamCreateWithPriority(&aux, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) aux = nullptr;
         if (cudaEventCreateWithFlags(&ev_x, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_w, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_e[0], cudaEventDisableTiming) != cudaSuccess ||
@@ -630,13 +630,13 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     c->inc_now = nullptr;
     if (e != cudaSuccess) return c->cuda_fail(e, "window_select launch");
 
-    // The top-k selection needs only the windowed medians: it runs beside the fleet baseline (on the
-    // internal stream, behind the window medians); its scores, which need the baseline, are filled in by
-    // the score pass.
-    const bool want_topk = c->K > 0 && (d_topk_idx || d_topk_score);
+    // The top-k selection needs only the windowed medians: it runs beside the fleet baseline, in the same launch or
+    // (wider fleets) on the internal stream, behind the window medians; its scores, which need the baseline, are
+    // filled in by the score pass.
+    const bool want_topk = c->K > 0 && (d_topk_idx || d_topk_score), together = xrank_count_supported(c->R);
     bool topk_side = false;
+    TopkArgs t{};
     if (want_topk) {
-        TopkArgs t{};
         t.R = c->R;
         t.M = c->M;
         t.K = c->K;
@@ -653,6 +653,8 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
             t.hint = (TopkHint *)(c->ws + c->L.topk_hint);
             t.hcand = (unsigned long long *)(c->ws + c->L.topk_hint + 256);
         }
+    }
+    if (want_topk && !together) {
         // a deferred evaluation with a hinted (short) selection keeps it on the tail stream: two event calls less, and
         // the internal stream is free for the next evaluation's window medians
         if (c->overlap && !(defer && t.hint) && c->ensure_side()) {
@@ -687,7 +689,13 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     x.mad_user = d_fleet_mad;
     x.status = c->status();
     x.prev_rows = c->row_hints && c->evals > 0 ? 1 : 0;
-    e = c->xrank(x, 1, ts, !defer, 1);
+    if (together) {
+        if (c->L.xr_gridp && c->row_hints) x.hint = c->hint_state(1);
+        e = launch_eval_tail(x, t, c->p, ts);
+        c->launches += 1;
+    } else {
+        e = c->xrank(x, 1, ts, !defer, 1);
+    }
     if (e != cudaSuccess) return c->cuda_fail(e, "fleet baseline launch");
 
     ScoreArgs s{};

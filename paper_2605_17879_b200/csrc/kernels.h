@@ -207,6 +207,8 @@ int topk_blocks(int R);
 // Records the text guard_last_error(NULL) returns (defined next to the C ABI).
 void set_global_error(const char *text);
 cudaError_t launch_topk(const TopkArgs &a, const MetricParams &p, cudaStream_t st);
+// Fleet baseline and top-k list of one evaluation in one launch (R <= kCountMaxRanks; K = 0: no list).
+cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st);
 
 // Node sweep: per-GPU medians over repetitions, then the verdicts.
 struct SweepMedArgs {

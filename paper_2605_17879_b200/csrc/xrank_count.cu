@@ -6,11 +6,6 @@ namespace guard {
 
 namespace {
 
-// Single rows of 8 metrics, bracketed by the row before / not: one CTA of 1 024 threads per column takes 6.3 / 7.5 us at
-// 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
-// barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3.
-constexpr int kCtClusterRanks = 4096;
-
 template <int V, int C>
 __global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<C> sh;
@@ -30,8 +25,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512, 1) xrank_count
 template <int NC>
 void launch_cluster(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
     const dim3 grid(a.M * NC, S);
-    int T = 128;     // four values per thread, while the CTA has 512 threads at most
-    while (T < 512 && a.R > 4 * NC * T) T <<= 1;
+    const int T = ct_cluster_threads(a.R, NC);
     const int v = (a.R + NC * T - 1) / (NC * T);
     if (v <= 4) xrank_count_cluster_kernel<4, NC><<<grid, T, 0, st>>>(a, p);
     else if (v <= 8) xrank_count_cluster_kernel<8, NC><<<grid, T, 0, st>>>(a, p);
@@ -55,9 +49,10 @@ bool xrank_count_supported(int R) { return R >= 1 && R <= kCountMaxRanks; }
 cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
     if (S <= 0) return cudaSuccess;
     // few and wide columns: a cluster each, of the most CTAs that find an SM each
-    if (a.hint || a.R > kCtClusterRanks) {
-        if ((long long)S * a.M * 8 <= 148) { launch_cluster<8>(a, p, S, st); return cudaGetLastError(); }
-        if (a.hint || (long long)S * a.M * 4 <= 148) { launch_cluster<4>(a, p, S, st); return cudaGetLastError(); }
+    if (a.R > kCtClusterRanks && (long long)S * a.M * 4 <= 148) {
+        if ((long long)S * a.M * 8 <= 148) launch_cluster<8>(a, p, S, st);
+        else launch_cluster<4>(a, p, S, st);
+        return cudaGetLastError();
     }
     // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
     // larger CTAs, which wait longer at their barriers: 60 steps of 4 096 ranks x 16 metrics take 31 / 29 / 29 us, launch

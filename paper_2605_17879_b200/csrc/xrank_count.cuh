@@ -28,6 +28,16 @@ constexpr int kCtList = 64;        // keys of a bin that are ranked directly (tw
 constexpr int kCtMaxIter = 64;     // a range shrinks at least to a 128th whenever its bin is too full
 constexpr uint32_t kCtTop = 0xFF800000u;    // no key of a number lies above; padding does
 constexpr uint32_t kCtNone = 0xFFFFFFFFu;
+// Single rows of 8 metrics, bracketed by the row before / not: one CTA of 1 024 threads per column takes 6.3 / 7.5 us at
+// 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
+// barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3.
+constexpr int kCtClusterRanks = 4096;
+// Threads of the CTAs of a cluster: four values each, while a CTA has 512 of them at most.
+inline int ct_cluster_threads(const int R, const int NC) {
+    int T = 128;
+    while (T < 512 && R > 4 * NC * T) T <<= 1;
+    return T;
+}
 
 template <int C>
 struct CtShared {
@@ -134,14 +144,14 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
         h[1] = make_uint4(0u, 0u, 0u, 0u);
     } else {   // (the other CTAs read this one's bins as well: cleared after the next cluster barrier)
         a = b = make_uint4(0u, 0u, 0u, 0u);
-        uint4 va[NC], vb[NC];
+        const uint32_t part = lane < NC ? ct_ld(ct_map(&sh.below[c], (uint32_t)(lane & (NC - 1)))) : 0u;
+        uint4 va[NC], vb[NC];      // (all in flight together; in two halves, which fit 64 registers, a row takes 1.3 us more)
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
             const uint32_t at = ct_map(h, (uint32_t)k);
             va[k] = ct_ld4(at);
             vb[k] = ct_ld4(at + 16u);
         }
-        const uint32_t part = lane < NC ? ct_ld(ct_map(&sh.below[c], (uint32_t)(lane & (NC - 1)))) : 0u;
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
             a.x += va[k].x; a.y += va[k].y; a.z += va[k].z; a.w += va[k].w;
@@ -178,10 +188,10 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
         sh.q1[c] = q;
         if (l1 && l2) {
             const int sft = ct_shift(width);
-            const uint32_t f0 = lo + (b1 << sft), end = lo + (b2 << sft) + ((1u << sft) - 1u);
-            sh.f0[c] = f0;
-            sh.fw[c] = min(end, lo + width) - f0;
-            sh.cutk[c] = f0 + ((1u << sft) - 1u);       // last key of k1's bin
+            const uint32_t o1 = b1 << sft, in_bin = (1u << sft) - 1u;
+            sh.f0[c] = lo + o1;
+            sh.fw[c] = min((b2 << sft) + in_bin, width) - o1;
+            sh.cutk[c] = lo + o1 + in_bin;              // last key of k1's bin
             sh.how[c] = b1 != b2 ? 2u : (n <= (uint32_t)kCtList ? 1u : 3u);
         } else {   // the range does not hold both ranks: move or stretch it, sixteenfold
             const uint32_t hi = lo + width, step = width >= 0x07FF0000u ? 0x7FFFFFFFu : 16u * width + 65536u;

@@ -547,6 +547,26 @@ def test_columns_over_clusters(R, M, B, quant):
     run_both(X, 4, 2, 16, dirs, [B], capacity=max(B, 4), min_signals=2)
 
 
+@pytest.mark.parametrize("R,M,K,quant", [
+    (64, 4, 64, None),             # one warp; every rank is listed
+    (129, 3, 1, None),             # groups of single threads; the slowest rank alone
+    (130, 3, 100, None),           # more ranks wanted than there are groups for: the exact selection
+    (4096, 2, 96, None),           # the widest fleet of one CTA
+    (4099, 8, 64, None),           # a cluster of eight CTAs, the last one ragged
+    (9000, 18, 33, None),          # a cluster of four
+    (32768, 4, 1024, None),        # the longest list
+    (3000, 4, 40, 2),              # ties: more equal keys than the gathered list holds, the lowest ranks win
+    (20000, 4, 700, 2),            # the same over a cluster
+])
+def test_slowest_ranks(R, M, K, quant):
+    """The top-k list beside the fleet baseline: single steps (a threshold left by the evaluation before; a fleet that
+    turns round its order, so that it misses), then a block."""
+    X, dirs = _rand_fleet(10, R, M, seed=R + K, quant=quant)
+    X[5:] = X[5:, ::-1] * np.float32(0.5)
+    run_both(X[:7], 3, 2, K, dirs, [1], capacity=4, min_signals=1)
+    run_both(X, 5, 2, K, dirs, [5], capacity=5, min_signals=1)
+
+
 @pytest.mark.parametrize("R,M,W,quant", [
     (70, 3, 1, None),              # one step; a ragged last tile
     (64, 4, 64, None),             # every slot of eight warps of eight values in use

@@ -63,6 +63,26 @@ __device__ __forceinline__ bool exceeds(float x, float med, int dir, float rhs) 
     return dev > rhs;
 }
 
+// A kernel launched by launch_after may start as soon as every CTA of the kernel in front of it in the stream has called
+// pdl_trigger or exited; pdl_wait returns when that kernel has ended and its writes are visible.  What the kernel reads or
+// writes before pdl_wait must therefore not be touched by the kernel in front, and be complete when that one starts.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const A &...args) {
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st;
+    c.attrs = &early;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 

@@ -205,6 +205,7 @@ template <int V, int NC>
 __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : 512, 1) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
     __shared__ CtShared<1> sh;
     __shared__ TopShared ts;
+    pdl_trigger();                 // (the score pass counts exceedances meanwhile)
     if ((int)blockIdx.x < x.M * NC) ct_row<V, 1, NC>(x, p, 0, blockIdx.x / NC, sh);
     else top_row<V, NC>(t, p, x.status, ts, sh);
     if (NC > 1) ct_sync<NC>();     // no CTA exits while others may read its shared memory

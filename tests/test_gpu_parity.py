@@ -567,6 +567,23 @@ def test_slowest_ranks(R, M, K, quant):
     run_both(X, 5, 2, K, dirs, [5], capacity=5, min_signals=1)
 
 
+@pytest.mark.parametrize("R,M,W", [
+    (33, 3, 9),                  # rows of bytes that are not word aligned, a ragged last CTA of 32 ranks
+    (9, 9, 40),                    # word-wide entries, eight ranks per CTA
+    (2371, 9, 40),                 # 32 ranks per CTA
+    (9477, 2, 70),                 # 128 ranks per CTA, rows not word aligned
+    (40, 2, 33000),                # more exceedances of a rank than a thread's byte counter holds
+])
+def test_exceedance_counts(R, M, W):
+    """k-of-W counts of whole windows, and sliding by a step and by eight, with ranks that exceed in every step."""
+    T = W + 9
+    rng = np.random.default_rng(R + W)
+    X = (1.0 + 0.03 * rng.standard_normal((T, R, M), dtype=np.float32)).astype(np.float32)
+    X[:, 5 % R] *= np.float32(2.0)
+    X[:, R - 1] *= np.float32(1.5)
+    run_both(X, W, W // 2 + 1, 4, [1] * M, [W, 1, 8], capacity=W + 16, min_signals=1)
+
+
 @pytest.mark.parametrize("R,M,W,quant", [
     (70, 3, 1, None),              # one step; a ragged last tile
     (64, 4, 64, None),             # every slot of eight warps of eight values in use

@@ -760,7 +760,7 @@ size_t guard_sweep_workspace_bytes(int gpus, int reps, int metrics) {
     if (gpus < 1 || reps < 1 || reps > GUARD_MAX_WINDOW || metrics < 1 || metrics > GUARD_MAX_METRICS ||
         (long long)gpus * metrics > 0x7FFFFFFFLL)
         return 0;
-    // fleet statistics, per-GPU medians, then the thread path's list of unserved series and its counter
+    // fleet statistics, per-GPU medians, then the thread path's unserved series (a bit each would do)
     return align_up(3 * kMaxMetrics * sizeof(float)) + align_up((size_t)gpus * metrics * sizeof(float)) +
            align_up((size_t)gpus * metrics * sizeof(uint32_t)) + align_up(64);
 }
@@ -795,8 +795,7 @@ int guard_sweep_qualify(const float *d_S, int nodes, int gpus_per_node, int reps
     sm.gmed = gmed;
     sm.gmed_user = d_gpu_med;
     sm.status = d_status;
-    sm.list = (uint32_t *)((char *)gmed + align_up((size_t)G * metrics * sizeof(float)));
-    sm.list_count = (uint32_t *)((char *)sm.list + align_up((size_t)G * metrics * sizeof(uint32_t)));
+    sm.todo = (uint32_t *)((char *)gmed + align_up((size_t)G * metrics * sizeof(float)));
     cudaError_t e = launch_sweep_medians(sm, st);
     if (e != cudaSuccess) { set_error(g_error, "sweep medians launch: %s", cudaGetErrorString(e)); return GUARD_ERR_CUDA; }
 
@@ -816,14 +815,11 @@ int guard_sweep_qualify(const float *d_S, int nodes, int gpus_per_node, int reps
     x.cut = fleet + 2 * kMaxMetrics;
     x.med_user = d_fleet_med;
     x.mad_user = d_fleet_mad;
+    x.cut_user = d_fleet_cut;
     for (int m = 0; m < metrics; ++m) x.cut_rank[m] = p.dir[m] < 0 ? (int)(j - 1) : (int)(G - j);
     x.status = d_status;
     e = xrank_count_supported(G) ? launch_xrank_count(x, p, 1, st) : launch_xrank_direct(x, p, 1, st);
     if (e != cudaSuccess) { set_error(g_error, "sweep fleet statistics launch: %s", cudaGetErrorString(e)); return GUARD_ERR_CUDA; }
-    if (d_fleet_cut) {
-        e = cudaMemcpyAsync(d_fleet_cut, fleet + 2 * kMaxMetrics, metrics * sizeof(float), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) { set_error(g_error, "cudaMemcpyAsync: %s", cudaGetErrorString(e)); return GUARD_ERR_CUDA; }
-    }
     SweepVerdictArgs v{};
     v.nodes = nodes;
     v.gpus_per_node = gpus_per_node;

@@ -20,6 +20,7 @@ struct XrankArgs {
     float *med_user;        // [S][M] copy for the caller, or NULL
     float *mad_user;        // [S][M] copy for the caller, or NULL
     float *cut;             // [S][M] extra order statistic (0-based rank cut_rank[m]), or NULL
+    float *cut_user;        // second copy of it, or NULL
     int cut_rank[kMaxMetrics];
     void *mask_base;        // exceedance mask rows [capacity][R] of mask_bytes each, or NULL
     int mask_bytes;         // 1 (M <= 8) or 4
@@ -217,8 +218,7 @@ struct SweepMedArgs {
     float *gmed;      // [G][M]
     float *gmed_user; // or NULL
     uint32_t *status; // or NULL
-    uint32_t *list;        // [G * M] scratch: series the thread path leaves to its finishing kernel, or NULL (then the warp path runs)
-    uint32_t *list_count;  // [1] their number (cleared by the launcher)
+    uint32_t *todo;        // [(G * M + 31) / 32] scratch: bits of the series the thread path leaves to its finishing kernel
 };
 cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st);
 

@@ -41,76 +41,16 @@ __global__ void __launch_bounds__(kSweepCols) sweep_median_kernel(const SweepMed
     if (a.gmed_user) a.gmed_user[o] = med;
 }
 
-// Warp-per-GPU path (up to 256 repetitions): the benchmark results of one GPU are one contiguous
-// [reps][M] block, so a warp fetches its GPU's block with whole-line 128-bit loads into its slice
-// of shared memory; then, metric by metric, the lanes pick the metric's column out of the block
-// (VPL keys per lane), sort their own keys and run the warp selection.  Eight warps per CTA, a
-// few kilobytes of shared memory per warp: every SM holds dozens of GPUs at once.
-constexpr int kSweepWarps = 8;
-
-template <int VPL>
-__global__ void __launch_bounds__(kSweepWarps * 32) sweep_median_warp_kernel(const SweepMedArgs a) {
-    extern __shared__ __align__(16) float sbuf[];      // [kSweepWarps][per], per rounded up to a multiple of 4
-    const int lane = lane_id(), w = warp_id(), M = a.M, reps = a.reps;
-    const int per = reps * M, per4 = (per + 3) & ~3;
-    const int g = blockIdx.x * kSweepWarps + w;
-    if (g >= a.G) return;                               // warps are independent: no CTA barrier below
-    float *buf = sbuf + (size_t)w * per4;
-    const float *src = a.S + (size_t)g * per;
-    bool bad = false;
-    if ((per & 3) == 0 && ((uintptr_t)a.S & 15) == 0) {
-        for (int i = 4 * lane; i < per; i += 128) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(src + i));
-            bad |= nonfinite_bits(__float_as_uint(v.x)) | nonfinite_bits(__float_as_uint(v.y)) |
-                   nonfinite_bits(__float_as_uint(v.z)) | nonfinite_bits(__float_as_uint(v.w));
-            *reinterpret_cast<float4 *>(buf + i) = v;
-        }
-    } else {
-        for (int i = lane; i < per; i += 32) {
-            const float v = __ldg(src + i);
-            bad |= nonfinite_bits(__float_as_uint(v));
-            buf[i] = v;
-        }
-    }
-    if (a.status && __any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(a.status, kStatNonFinite);
-    __syncwarp();
-    for (int m = 0; m < M; ++m) {
-        uint32_t kv[VPL];
-        int nreal = 0;
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            const int rep = lane + 32 * j;
-            const bool real = rep < reps;
-            kv[j] = real ? f2key(buf[rep * M + m]) : 0xFFFFFFFFu;
-            nreal += real;
-        }
-        lane_sort<VPL>(kv);
-        float med = 0.0f;
-        const bool ok = warp_median<VPL>(kv, nreal, reps, 0u, med);
-        if (lane == 0) {
-            if (!ok && a.status) atomicOr(a.status, kStatInternal);
-            const size_t o = (size_t)g * M + m;
-            a.gmed[o] = med;
-            if (a.gmed_user) a.gmed_user[o] = med;
-        }
-    }
-}
-
-template <int VPL>
-cudaError_t launch_sweep_warp(const SweepMedArgs &a, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(sweep_median_warp_kernel<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    sweep_median_warp_kernel<VPL><<<(a.G + kSweepWarps - 1) / kSweepWarps, kSweepWarps * 32, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-// Thread-per-series path (32 to 256 repetitions): a series' repetitions scatter around their mean, and the
-// mean predicts the median of 200 repetitions to a few hundredths of their standard deviation.  Pass A takes
-// mean and standard deviation (the GPU's block is read once from HBM and stays in L1 / L2 for pass B); pass B
-// counts the values below mean -/+ 0.2 sd and keeps those inside (about a sixth of them) in the thread's
-// shared-memory column; the two middle ranks are then found among the kept keys (pivot search, as for the
-// window medians).  A series whose
-// counts do not prove the bracket (or whose column overflows) goes on a list for sweep_median_finish_kernel.
+// Thread-per-series path (32 to 256 repetitions, many series): a series' repetitions scatter around their mean, and the
+// mean predicts the median of n repetitions to 0.75 / sqrt(n) of their standard deviation.  Pass A takes mean and standard
+// deviation (the GPU's block is read once from HBM and stays in L1 / L2 for pass B); pass B counts the values below
+// mean -/+ 2.83 sd / sqrt(n) and keeps those inside (32 of 200, 18 of 64) in the thread's shared-memory column; the two
+// middle ranks are then found among the kept keys (pivot search, as for the window medians).  A series whose counts
+// do not prove the bracket (or whose column overflows) is left to sweep_median_finish_kernel.
+// Bound by the chain of instructions of a series (8 000 of them, 21 warps per SM) and by the loads' cache lines (a
+// repetition is another line for every GPU of the warp): 41 us at 16 384 GPUs x 200 x 6 with the results in L2, 63 from
+// HBM.  Not faster: the next loads in flight ahead of the passes (the same), blocks staged whole in shared memory (seven
+// warps per SM: 62 and 64), or in chunks of eight repetitions, asynchronously (84) or through registers (49 and 68).
 constexpr int kSwThreads = 128;
 constexpr int kSwSlots = 60;      // kept keys per series (the column format of the thread-per-series selection)
 constexpr int kSwRows = 8;        // repetitions in flight per thread
@@ -140,20 +80,23 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_thread_kernel(const S
         sd1 += d;
         sd2 = fmaf(d, d, sd2);
     };
-    int r = 0;
-    for (; r + kSwRows <= n; r += kSwRows) {
-        float x[kSwRows];
+    auto each = [&](auto f) {
+        int r = 0;
+        for (; r + kSwRows <= n; r += kSwRows) {
+            float x[kSwRows];
 #pragma unroll
-        for (int u = 0; u < kSwRows; ++u) x[u] = __ldg(base + (size_t)(r + u) * M);
+            for (int u = 0; u < kSwRows; ++u) x[u] = __ldg(base + (size_t)(r + u) * M);
 #pragma unroll
-        for (int u = 0; u < kSwRows; ++u) acc(x[u]);
-    }
-    for (; r < n; ++r) acc(__ldg(base + (size_t)r * M));
+            for (int u = 0; u < kSwRows; ++u) f(x[u]);
+        }
+        for (; r < n; ++r) f(__ldg(base + (size_t)r * M));
+    };
+    each(acc);
     if (a.status && __any_sync(0xFFFFFFFFu, bad && active) && lane_id() == 0) atomicOr(a.status, kStatNonFinite);
     const float inv = 1.0f / (float)n;
     const float mean_d = sd1 * inv;
     const float var = fmaxf(sd2 * inv - mean_d * mean_d, 0.0f);
-    const float c = x0 + mean_d, h = 0.2f * sqrtf(var);
+    const float c = x0 + mean_d, h = 2.83f * sqrtf(var * inv);
     const bool usable = active && !bad && !same && (h > 0.0f) && (h < 3.0e38f) && (fabsf(c) < 3.0e38f);
     float flo = c - h, fhi = c + h;
     if (flo == 0.0f) flo = -0.0f;   // an end that is zero admits both zeros: float compares then agree with the key order
@@ -165,15 +108,7 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_thread_kernel(const S
     const uint32_t kbase = (uint32_t)__cvta_generic_to_shared(kept + tid * kSwSlots), klim = kbase + (uint32_t)(kSwSlots * 4);
     uint32_t kaddr = kbase, clt = 0;
     if (__any_sync(0xFFFFFFFFu, usable)) {
-        r = 0;
-        for (; r + kSwRows <= n; r += kSwRows) {
-            float x[kSwRows];
-#pragma unroll
-            for (int u = 0; u < kSwRows; ++u) x[u] = __ldg(base + (size_t)(r + u) * M);
-#pragma unroll
-            for (int u = 0; u < kSwRows; ++u) th_cell(x[u], flo, fhi, klim, clt, kaddr);
-        }
-        for (; r < n; ++r) th_cell(__ldg(base + (size_t)r * M), flo, fhi, klim, clt, kaddr);
+        each([&](const float x) { th_cell(x, flo, fhi, klim, clt, kaddr); });
     }
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
@@ -189,43 +124,53 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_thread_kernel(const S
         if (a.gmed_user) a.gmed_user[sidx] = med;
     }
     const unsigned todo = __ballot_sync(0xFFFFFFFFu, active && !ok);
-    if (todo) {
-        const int lane = lane_id();
-        uint32_t b = 0;
-        if (lane == 0) b = atomicAdd(a.list_count, (uint32_t)__popc(todo));
-        b = __shfl_sync(0xFFFFFFFFu, b, 0);
-        if ((todo >> lane) & 1u) a.list[b + __popc(todo & ((1u << lane) - 1u))] = (uint32_t)sidx;
+    if (lane_id() == 0) a.todo[sidx >> 5] = todo;
+}
+
+// One warp per series: the lanes fetch the repetitions, sort their own keys and run the warp selection.
+template <int VPL>
+__device__ __forceinline__ void sweep_warp_median(const SweepMedArgs &a, const uint32_t sidx, const bool check) {
+    const int lane = lane_id(), M = a.M, n = a.reps;
+    const int g = (int)(sidx / (uint32_t)M), m = (int)(sidx - (uint32_t)g * (uint32_t)M);
+    const float *base = a.S + (size_t)g * n * M + m;
+    uint32_t kv[VPL];
+    int nreal = 0;
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const int rep = lane + 32 * j;
+        const bool real = rep < n;
+        const uint32_t b = real ? __float_as_uint(__ldg(base + (size_t)rep * M)) : 0u;
+        bad |= nonfinite_bits(b);
+        kv[j] = real ? key_of_bits(b) : 0xFFFFFFFFu;
+        nreal += real;
+    }
+    if (check && a.status && __any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(a.status, kStatNonFinite);
+    lane_sort<VPL>(kv);
+    float med = 0.0f;
+    const bool ok = warp_median<VPL>(kv, nreal, n, 0u, med);
+    if (lane == 0) {
+        if (!ok && a.status) atomicOr(a.status, kStatInternal);
+        a.gmed[sidx] = med;
+        if (a.gmed_user) a.gmed_user[sidx] = med;
     }
 }
 
-// The listed series, one warp each: the lanes fetch the repetitions, sort their own keys and run the warp selection.
+// The series the thread path left: their bits in a.todo.
 template <int VPL>
 __global__ void __launch_bounds__(kSwThreads) sweep_median_finish_kernel(const SweepMedArgs a) {
-    const int lane = lane_id(), M = a.M, n = a.reps;
-    const uint32_t count = min(__ldcg(a.list_count), (uint32_t)min((long long)a.G * M, 0x7FFFFFFFLL));
-    const uint32_t nwarps = gridDim.x * (kSwThreads / 32);
-    for (uint32_t i = blockIdx.x * (kSwThreads / 32) + warp_id(); i < count; i += nwarps) {
-        const uint32_t sidx = __ldcg(a.list + i);
-        const int g = (int)(sidx / (uint32_t)M), m = (int)(sidx - (uint32_t)g * (uint32_t)M);
-        const float *base = a.S + (size_t)g * n * M + m;
-        uint32_t kv[VPL];
-        int nreal = 0;
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            const int rep = lane + 32 * j;
-            const bool real = rep < n;
-            kv[j] = real ? f2key(__ldg(base + (size_t)rep * M)) : 0xFFFFFFFFu;
-            nreal += real;
-        }
-        lane_sort<VPL>(kv);
-        float med = 0.0f;
-        const bool ok = warp_median<VPL>(kv, nreal, n, 0u, med);
-        if (lane == 0) {
-            if (!ok && a.status) atomicOr(a.status, kStatInternal);
-            a.gmed[sidx] = med;
-            if (a.gmed_user) a.gmed_user[sidx] = med;
-        }
-    }
+    pdl_wait();
+    const uint32_t words = (uint32_t)(((long long)a.G * a.M + 31) >> 5), nwarps = gridDim.x * (kSwThreads / 32);
+    for (uint32_t i = blockIdx.x * (kSwThreads / 32) + warp_id(); i < words; i += nwarps)
+        for (uint32_t t = __ldcg(a.todo + i); t; t &= t - 1u) sweep_warp_median<VPL>(a, 32u * i + (uint32_t)(__ffs(t) - 1), false);
+}
+
+// Every series.
+template <int VPL>
+__global__ void __launch_bounds__(kSwThreads) sweep_median_series_kernel(const SweepMedArgs a) {
+    pdl_wait();
+    const long long sidx = (long long)blockIdx.x * (kSwThreads / 32) + warp_id();
+    if (sidx < (long long)a.G * a.M) sweep_warp_median<VPL>(a, (uint32_t)sidx, true);
 }
 
 // Fallback when the repetitions of one GPU do not fit a tile: bit-by-bit counting
@@ -269,51 +214,64 @@ __global__ void sweep_median_global_kernel(const SweepMedArgs a) {
     if (a.gmed_user) a.gmed_user[c] = med;
 }
 
-// One thread per node: robust-z outlier AND beyond the percentile cut fails a metric;
+// One thread per GPU, whole nodes per CTA where they fit: robust-z outlier AND beyond the percentile cut fails a metric;
 // a GPU passes with no failed metric; a node passes when all of its GPUs pass.
-__global__ void sweep_verdict_kernel(const SweepVerdictArgs a, const MetricParams p) {
-    const int node = blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= a.nodes) return;
-    bool node_ok = true;
-    for (int q = 0; q < a.gpus_per_node; ++q) {
-        const size_t g = (size_t)node * a.gpus_per_node + q;
+constexpr int kVerdictThreads = 128;
+
+__global__ void __launch_bounds__(kVerdictThreads) sweep_verdict_kernel(const SweepVerdictArgs a, const MetricParams p) {
+    __shared__ float s_F[kMaxMetrics], s_rhs[kMaxMetrics], s_cut[kMaxMetrics];
+    __shared__ uint32_t s_bad[kVerdictThreads];
+    const int tid = threadIdx.x, gpn = a.gpus_per_node, per = max(kVerdictThreads / gpn, 1);   // nodes of this CTA
+    const int node0 = blockIdx.x * per, nn = min(per, a.nodes - node0);
+    s_bad[tid] = 0u;
+    pdl_wait();
+    if (tid < a.M) {
+        const float F = a.fleet_med[tid];
+        s_F[tid] = F;
+        s_rhs[tid] = __fmul_rn(p.thrp[tid], scale_of(a.fleet_mad[tid], F, p.floor_rel[tid], p.floor_abs[tid]));
+        s_cut[tid] = a.fleet_cut[tid];
+    }
+    __syncthreads();
+    for (int q = tid; q < nn * gpn; q += kVerdictThreads) {
+        const size_t g = (size_t)node0 * gpn + q;
         uint32_t fail = 0;
         for (int m = 0; m < a.M; ++m) {
             const float v = a.gmed[g * a.M + m];
-            const float F = a.fleet_med[m];
-            const float Fs = scale_of(a.fleet_mad[m], F, p.floor_rel[m], p.floor_abs[m]);
-            const bool zfail = exceeds(v, F, p.dir[m], __fmul_rn(p.thrp[m], Fs));
-            const float cut = a.fleet_cut[m];
-            const bool pfail = p.dir[m] < 0 ? (v < cut) : (v > cut);
-            if (zfail && pfail) fail |= 1u << m;
+            const bool beyond = p.dir[m] < 0 ? (v < s_cut[m]) : (v > s_cut[m]);
+            if (exceeds(v, s_F[m], p.dir[m], s_rhs[m]) && beyond) fail |= 1u << m;
         }
         if (a.fail_mask) a.fail_mask[g] = fail;
         if (a.gpu_pass) a.gpu_pass[g] = (uint8_t)(fail == 0);
-        node_ok = node_ok && (fail == 0);
+        if (fail) s_bad[q / gpn] = 1u;
     }
-    if (a.node_pass) a.node_pass[node] = (uint8_t)node_ok;
+    __syncthreads();
+    if (tid < nn && a.node_pass) a.node_pass[node0 + tid] = (uint8_t)(s_bad[tid] == 0u);
 }
 
 }  // namespace
 
 cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st) {
     const long long series = (long long)a.G * a.M;
-    if (a.list && a.list_count && a.reps >= 32 && a.reps <= 256 && series < 0x7FFFFFFFLL) {
-        cudaError_t e = cudaMemsetAsync(a.list_count, 0, sizeof(uint32_t), st);
-        if (e != cudaSuccess) return e;
-        sweep_median_thread_kernel<<<(unsigned)((series + kSwThreads - 1) / kSwThreads), kSwThreads, 0, st>>>(a);
-        const long long want = (series + kSwThreads / 32 - 1) / (kSwThreads / 32);
-        const int fgrid = (int)(want < 148 * 4 ? want : 148 * 4);
-        if (a.reps <= 64) sweep_median_finish_kernel<2><<<fgrid, kSwThreads, 0, st>>>(a);
-        else if (a.reps <= 128) sweep_median_finish_kernel<4><<<fgrid, kSwThreads, 0, st>>>(a);
-        else sweep_median_finish_kernel<8><<<fgrid, kSwThreads, 0, st>>>(a);
-        return cudaGetLastError();
+    // A warp per series while they are few: one launch, and no thread's chain over all repetitions (1 776 series of 33
+    // repetitions 2.8 us against 8.9 + 1.9, 12 288 of 200 16 against 29 + 5, 24 576 of 64 18 against 15 + 4, 49 152 of
+    // 100 25 against 21 + 3, 98 304 of 200 95 against 45 + 5), and for fewer than 32 repetitions, which say too little
+    // about their median beforehand.
+    if (a.reps <= 256 && series < 0x7FFFFFFFLL && (series <= 32768 || a.reps < 32)) {
+        const unsigned grid = (unsigned)((series + kSwThreads / 32 - 1) / (kSwThreads / 32));
+        if (a.reps <= 32) return launch_after(sweep_median_series_kernel<1>, grid, kSwThreads, st, a);
+        if (a.reps <= 64) return launch_after(sweep_median_series_kernel<2>, grid, kSwThreads, st, a);
+        if (a.reps <= 128) return launch_after(sweep_median_series_kernel<4>, grid, kSwThreads, st, a);
+        return launch_after(sweep_median_series_kernel<8>, grid, kSwThreads, st, a);
     }
-    const size_t wsmem = (size_t)kSweepWarps * (((size_t)a.reps * a.M + 3) & ~(size_t)3) * sizeof(float);
-    if (a.reps <= 256 && wsmem <= 96 * 1024) {
-        if (a.reps <= 64) return launch_sweep_warp<2>(a, wsmem, st);
-        if (a.reps <= 128) return launch_sweep_warp<4>(a, wsmem, st);
-        return launch_sweep_warp<8>(a, wsmem, st);
+    if (a.reps >= 32 && a.reps <= 256 && series < 0x7FFFFFFFLL) {
+        sweep_median_thread_kernel<<<(unsigned)((series + kSwThreads - 1) / kSwThreads), kSwThreads, 0, st>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        const long long want = ((series + 31) / 32 + kSwThreads / 32 - 1) / (kSwThreads / 32);
+        const int fgrid = (int)(want < 148 * 4 ? want : 148 * 4);
+        if (a.reps <= 64) return launch_after(sweep_median_finish_kernel<2>, fgrid, kSwThreads, st, a);
+        if (a.reps <= 128) return launch_after(sweep_median_finish_kernel<4>, fgrid, kSwThreads, st, a);
+        return launch_after(sweep_median_finish_kernel<8>, fgrid, kSwThreads, st, a);
     }
     const size_t smem = (size_t)a.reps * kSweepCols * 4;
     if (smem <= 200 * 1024) {
@@ -329,8 +287,8 @@ cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st) {
 }
 
 cudaError_t launch_sweep_verdict(const SweepVerdictArgs &a, const MetricParams &p, cudaStream_t st) {
-    sweep_verdict_kernel<<<(a.nodes + 127) / 128, 128, 0, st>>>(a, p);
-    return cudaGetLastError();
+    const int per = a.gpus_per_node < kVerdictThreads ? kVerdictThreads / a.gpus_per_node : 1;
+    return launch_after(sweep_verdict_kernel, (a.nodes + per - 1) / per, kVerdictThreads, st, a, p);
 }
 
 }  // namespace guard

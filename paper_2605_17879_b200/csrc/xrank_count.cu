@@ -9,6 +9,7 @@ namespace {
 template <int V, int C>
 __global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<C> sh;
+    pdl_wait();
     if (a.only_flagged && a.only_flagged[blockIdx.y] == 0u) return;
     ct_row<V, C>(a, p, blockIdx.y, blockIdx.x * C, sh);
 }
@@ -17,29 +18,30 @@ __global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, co
 template <int V, int NC>
 __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512, 1) xrank_count_cluster_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<1> sh;
+    pdl_wait();
     if (a.only_flagged && a.only_flagged[blockIdx.y] == 0u) return;   // (the same for the whole cluster)
     ct_row<V, 1, NC>(a, p, blockIdx.y, blockIdx.x / NC, sh);
     ct_sync<NC>();   // the other CTAs read this one's lists last: none may exit before all have
 }
 
 template <int NC>
-void launch_cluster(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
+cudaError_t launch_cluster(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
     const dim3 grid(a.M * NC, S);
     const int T = ct_cluster_threads(a.R, NC);
     const int v = (a.R + NC * T - 1) / (NC * T);
-    if (v <= 4) xrank_count_cluster_kernel<4, NC><<<grid, T, 0, st>>>(a, p);
-    else if (v <= 8) xrank_count_cluster_kernel<8, NC><<<grid, T, 0, st>>>(a, p);
-    else xrank_count_cluster_kernel<16, NC><<<grid, T, 0, st>>>(a, p);
+    if (v <= 4) return launch_after(xrank_count_cluster_kernel<4, NC>, grid, T, st, a, p);
+    if (v <= 8) return launch_after(xrank_count_cluster_kernel<8, NC>, grid, T, st, a, p);
+    return launch_after(xrank_count_cluster_kernel<16, NC>, grid, T, st, a, p);
 }
 
 template <int C>
-void launch_c(const XrankArgs &a, const MetricParams &p, int S, int T, cudaStream_t st) {
+cudaError_t launch_c(const XrankArgs &a, const MetricParams &p, int S, int T, cudaStream_t st) {
     const int v = (a.R * C + T - 1) / T;
     const dim3 grid(a.M / C, S);
-    if (v <= 4) xrank_count_kernel<4, C><<<grid, T, 0, st>>>(a, p);
-    else if (v <= 8) xrank_count_kernel<8, C><<<grid, T, 0, st>>>(a, p);
-    else if (v <= 16) xrank_count_kernel<16, C><<<grid, T, 0, st>>>(a, p);
-    else xrank_count_kernel<32, C><<<grid, T, 0, st>>>(a, p);
+    if (v <= 4) return launch_after(xrank_count_kernel<4, C>, grid, T, st, a, p);
+    if (v <= 8) return launch_after(xrank_count_kernel<8, C>, grid, T, st, a, p);
+    if (v <= 16) return launch_after(xrank_count_kernel<16, C>, grid, T, st, a, p);
+    return launch_after(xrank_count_kernel<32, C>, grid, T, st, a, p);
 }
 
 }  // namespace
@@ -50,9 +52,8 @@ cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S,
     if (S <= 0) return cudaSuccess;
     // few and wide columns: a cluster each, of the most CTAs that find an SM each
     if (a.R > kCtClusterRanks && (long long)S * a.M * 4 <= 148) {
-        if ((long long)S * a.M * 8 <= 148) launch_cluster<8>(a, p, S, st);
-        else launch_cluster<4>(a, p, S, st);
-        return cudaGetLastError();
+        if ((long long)S * a.M * 8 <= 148) return launch_cluster<8>(a, p, S, st);
+        return launch_cluster<4>(a, p, S, st);
     }
     // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
     // larger CTAs, which wait longer at their barriers: 60 steps of 4 096 ranks x 16 metrics take 31 / 29 / 29 us, launch
@@ -66,9 +67,7 @@ cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S,
     if (ctas <= 148) { while (T < 1024 && E > 4 * T) T <<= 1; }
     else { while (T < 256 && E > 8 * T) T <<= 1; }
     while (T < 1024 && E > 32 * T) T <<= 1;
-    if (C == 2) launch_c<2>(a, p, S, T, st);
-    else launch_c<1>(a, p, S, T, st);
-    return cudaGetLastError();
+    return C == 2 ? launch_c<2>(a, p, S, T, st) : launch_c<1>(a, p, S, T, st);
 }
 
 }  // namespace guard

@@ -437,6 +437,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                 }
             } else if (tid == what - 2 && speaks) {
                 a.cut[o] = key2f(v1);
+                if (a.cut_user) a.cut_user[o] = key2f(v1);
             }
         }
         if (what == 1) break;

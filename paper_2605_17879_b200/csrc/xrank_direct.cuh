@@ -199,6 +199,7 @@ __device__ inline void xrank_direct_step(const XrankArgs &a, const MetricParams 
         __syncthreads();
         cta_select(row, R, M, false, [](float x, int) { return f2key(x); }, hist, sh, a.status);
         if (tid < M) a.cut[(size_t)s * M + tid] = key2f(sh.prefix[tid]);
+        if (tid < M && a.cut_user) a.cut_user[(size_t)s * M + tid] = key2f(sh.prefix[tid]);
     }
 }
 

@@ -584,6 +584,35 @@ def test_exceedance_counts(R, M, W):
     run_both(X, W, W // 2 + 1, 4, [1] * M, [W, 1, 8], capacity=W + 16, min_signals=1)
 
 
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (6145, 8, 32, 1),              # the last warp has few series left
+    (2400, 7, 33, 3),              # one repetition in the last round
+    (1031, 8, 200, 6),             # a warp per series no longer; GPUs over two warps
+    (77, 130, 45, 5),              # more GPUs per node than a CTA has threads
+    (400, 4, 256, 32),             # the most repetitions and metrics
+    (340, 8, 100, 12),             # a warp per series, the most of them
+])
+def test_sweep_of_many_series(nodes, gpn, N, M):
+    """Many series of repeated results: constant and two-valued series, denormal and huge values, and an outlier that
+    makes the spread useless as a bracket; the verdicts follow from the same medians."""
+    from paper_2605_17879_b200 import guard
+    rng = np.random.default_rng(N + M)
+    G = nodes * gpn
+    S = (1.0 + 0.02 * rng.standard_normal((G, N, M), dtype=np.float32)).astype(np.float32)
+    S[3::50] = S[3::50, :1]
+    S[4::50] = np.where(S[4::50] > 1.0, np.float32(1.0), np.float32(0.5))
+    S[5::50] *= np.float32(1e-39)
+    S[6::50] *= np.float32(1e38) * np.sign(rng.standard_normal((1, N, 1))).astype(np.float32)
+    S[7::50, 1] = np.float32(1e30)
+    S[8::50, :, 0] *= np.float32(0.7)
+    dirs = [-1] * M
+    ref = go.sweep(S, nodes, gpn, dir=dirs)
+    out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
+    assert int(out["status"].cpu()[0]) == 0
+    for key in ref:
+        assert_bit_equal(to_np(out[key]), ref[key], key)
+
+
 @pytest.mark.parametrize("R,M,W,quant", [
     (70, 3, 1, None),              # one step; a ragged last tile
     (64, 4, 64, None),             # every slot of eight warps of eight values in use

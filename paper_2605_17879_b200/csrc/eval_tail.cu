@@ -205,6 +205,7 @@ template <int V, int NC>
 __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : 512, 1) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
     __shared__ CtShared<1> sh;
     __shared__ TopShared ts;
+    pdl_wait();
     pdl_trigger();                 // (the score pass counts exceedances meanwhile)
     if ((int)blockIdx.x < x.M * NC) ct_row<V, 1, NC>(x, p, 0, blockIdx.x / NC, sh);
     else top_row<V, NC>(t, p, x.status, ts, sh);
@@ -212,11 +213,11 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : 51
 }
 
 template <int NC>
-void launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st) {
+cudaError_t launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st) {
     const int T = ct_cluster_threads(x.R, NC), v = (x.R + NC * T - 1) / (NC * T), grid = (x.M + (t.K > 0 ? 1 : 0)) * NC;
-    if (v <= 4) eval_tail_kernel<4, NC><<<grid, T, 0, st>>>(x, t, p);
-    else if (v <= 8) eval_tail_kernel<8, NC><<<grid, T, 0, st>>>(x, t, p);
-    else eval_tail_kernel<16, NC><<<grid, T, 0, st>>>(x, t, p);
+    if (v <= 4) return launch_after(eval_tail_kernel<4, NC>, grid, T, st, x, t, p);
+    if (v <= 8) return launch_after(eval_tail_kernel<8, NC>, grid, T, st, x, t, p);
+    return launch_after(eval_tail_kernel<16, NC>, grid, T, st, x, t, p);
 }
 
 }  // namespace
@@ -227,13 +228,9 @@ cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const Metric
     if (x.R <= kCtClusterRanks) {
         int T = 32;
         while (T < 1024 && x.R > 4 * T) T <<= 1;
-        eval_tail_kernel<4, 1><<<x.M + (t.K > 0 ? 1 : 0), T, 0, st>>>(x, t, p);
-    } else if ((x.M + 1) * 8 <= 148) {
-        launch<8>(x, t, p, st);
-    } else {
-        launch<4>(x, t, p, st);
+        return launch_after(eval_tail_kernel<4, 1>, x.M + (t.K > 0 ? 1 : 0), T, st, x, t, p);
     }
-    return cudaGetLastError();
+    return (x.M + 1) * 8 <= 148 ? launch<8>(x, t, p, st) : launch<4>(x, t, p, st);
 }
 
 }  // namespace guard

@@ -141,6 +141,7 @@ int status_to_code(uint32_t s) {
 
 }  // namespace
 
+constexpr long long kInlineValues = 1 << 21;   // values of a window up to which an evaluation stays on the caller's stream
 struct guard_ctx {
     int R, M, W, k, C, K;
     MetricParams p;
@@ -324,6 +325,11 @@ struct guard_ctx {
         static std::atomic<uint32_t> next{(uint32_t)std::chrono::steady_clock::now().time_since_epoch().count() | 1u};
         do { split_epoch = next.fetch_add(1u); } while (split_epoch == 0u);
     }
+    // Windows of so few values that forking their medians to a stream of the library's own (four event calls, and the
+    // latency of two waits) takes longer than it hides: blocks of 64 ranks x 4 x 50 steps 19.6 us forked, 17.0 in line,
+    // 1 024 x 8 x 100 30.0 / 25.8, 1 024 x 8 x 200 39.9 / 38.0, single steps of 512 x 8 29.2 / 27.0.  Deferred evaluations
+    // always fork: they hide the host's calls behind one another (single steps of 64 x 4 17.7 us, 23.4 in line).
+    bool inline_eval() const { return !deferred && (long long)W * R * M <= kInlineValues; }
     RowHints *hint_state(int site) const { return (RowHints *)(ws + L.xr_grid + (size_t)site * align_up(sizeof(RowHints))); }
     cudaError_t xrank(XrankArgs a, int S, cudaStream_t st, bool own_scratch = true, int site = -1) {
         if (S == 1 && site >= 0 && L.xr_gridp && row_hints) a.hint = hint_state(site);
@@ -466,7 +472,9 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
         if (e == cudaSuccess) e = c->join_xs(st);
         if (e != cudaSuccess) return c->cuda_fail(e, "join of deferred work");
     }
-    if (!in_place) {
+    // a small block that the counting kernels take is put into the ring by them
+    const bool copied = !in_place && c->inline_eval() && slot + B <= c->C && xrank_count_copies(c->R, c->M, B) && !c->L.xr_split && !c->L.xr_cluster;
+    if (!in_place && !copied) {
         const int first = (slot + B <= c->C) ? B : (c->C - slot);
         cudaError_t e = cudaMemcpyAsync(c->ring() + (size_t)slot * row, d_block, (size_t)first * row * sizeof(float),
                                         cudaMemcpyDeviceToDevice, st);
@@ -477,7 +485,7 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
     }
     // the ring now holds the block (in stream order): evaluations may start reading it from here
     c->fork_fresh = false;
-    if (c->overlap && c->ensure_side() && cudaEventRecord(c->ev_fork, st) == cudaSuccess) c->fork_fresh = true;
+    if (c->overlap && !c->inline_eval() && c->ensure_side() && cudaEventRecord(c->ev_fork, st) == cudaSuccess) c->fork_fresh = true;
     XrankArgs a{};
     a.base = c->ring();
     a.row_stride = (long long)row;
@@ -494,6 +502,7 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
     a.mask_bytes = c->mask_bytes();
     a.check_finite = 1;
     a.status = c->status();
+    a.copy_from = copied ? d_block : nullptr;
     a.prev_rows = c->row_hints ? c->stat_rows : 0;
     if (B > c->stat_rows) c->stat_rows = B;
     cudaError_t e;

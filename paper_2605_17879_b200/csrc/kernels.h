@@ -10,6 +10,7 @@ namespace guard {
 // Cross-rank statistics of S rows of a [rows][R][M] float32 array.  Row s of the launch
 // lives at base + ((first_slot + s) % capacity) * row_stride.
 struct XrankArgs {
+    const float *copy_from; // or NULL: the rows (contiguous) to read instead of the ring's, and to store there (counting path, one CTA per column group)
     const float *base;
     long long row_stride;   // floats between consecutive rows (R * M)
     int first_slot;
@@ -85,6 +86,7 @@ cudaError_t launch_xrank_bracketed(const XrankArgs &a, const MetricParams &p, co
 // Rows held in registers and searched by counting at pivots: any values, any number of metrics, up to 32 768 ranks.
 constexpr int kCountMaxRanks = 32768;
 bool xrank_count_supported(int R);
+bool xrank_count_copies(int R, int M, int S);   // honours copy_from
 cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);
 
 cudaError_t launch_xrank_direct(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);

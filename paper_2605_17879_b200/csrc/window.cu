@@ -59,6 +59,7 @@ __device__ __forceinline__ float warp_spread_guess(const uint32_t (&kv)[VPL], co
 
 template <int VPL>
 __global__ void __launch_bounds__(1024, 2) window_warp_kernel(const WindowArgs a, const int ntiles, const int use_bulk) {
+    pdl_wait();
     extern __shared__ __align__(128) uint32_t wbuf[];   // 2 x [n][kWarpPitch]
     __shared__ __align__(8) uint64_t bar[2];
     const int tid = threadIdx.x, lane = lane_id(), w = warp_id();
@@ -182,8 +183,7 @@ cudaError_t launch_warp_path(const WindowArgs &a, int use_bulk, cudaStream_t st)
     const int sms = once.sms[dev];
     const int ntiles = (a.series + kWarpTileCols - 1) / kWarpTileCols;
     const int grid = ntiles < 2 * sms ? ntiles : 2 * sms;
-    window_warp_kernel<VPL><<<grid, 1024, smem, st>>>(a, ntiles, use_bulk);
-    return cudaGetLastError();
+    return launch_after_smem(window_warp_kernel<VPL>, grid, 1024, smem, st, a, ntiles, use_bulk);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -217,6 +217,7 @@ constexpr float kThSmooth = 0.3f;   // weight of the newest median in the interv
 
 template <int VPL>
 __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowArgs a) {
+    pdl_wait();
     extern __shared__ __align__(16) uint32_t tkept[];   // [kThCols][kThSlots]
     const int tid = threadIdx.x, lane = lane_id();
     const int n = a.n;
@@ -293,6 +294,7 @@ constexpr int kFinCtas = 148 * 4;
 
 template <int VPL>
 __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const WindowArgs a) {
+    pdl_wait();
     __shared__ int is_last;
     const int lane = lane_id();
     const int n = a.n;
@@ -350,10 +352,10 @@ cudaError_t launch_thread_path(const WindowArgs &a, cudaStream_t st) {
         return e2;
     });
     if (e != cudaSuccess) return e;
-    window_thread_kernel<VPL><<<(a.series + kThCols - 1) / kThCols, kThCols, smem, st>>>(a);
+    e = launch_after_smem(window_thread_kernel<VPL>, (a.series + kThCols - 1) / kThCols, kThCols, smem, st, a);
+    if (e != cudaSuccess) return e;
     const int fgrid = min(kFinCtas, (a.series + kFinThreads / 32 - 1) / (kFinThreads / 32));
-    window_finish_kernel<VPL><<<fgrid, kFinThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(window_finish_kernel<VPL>, fgrid, kFinThreads, st, a);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -376,6 +378,7 @@ constexpr int kIncThreads = 128;
 // NEW: the most steps that entered / left (1 for an evaluation after every step, else kIncMaxNew).
 template <int NEW>
 __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s) {
+    pdl_wait();
     static_assert(kIncSlots > 32 && kIncSlots <= 64, "a lane holds list slots lane and lane + 32");
     __shared__ float sl[kIncThreads / 32][32][kIncSlots];   // per warp: the lists of the series it updates, staged asynchronously
     const int lane = lane_id(), wid = warp_id();
@@ -538,6 +541,7 @@ constexpr int kRbCtas = 148 * 8;
 
 template <int VPL>
 __global__ void __launch_bounds__(kRbThreads) window_rebuild_kernel(const WindowArgs a, const IncArgs s) {
+    pdl_wait();
     __shared__ int is_last;
     const int lane = lane_id();
     const int n = a.n;
@@ -639,12 +643,12 @@ bool window_inc_supported(const WindowArgs &a) { return a.n >= 1 && a.n <= 256; 
 cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {
     const int grid = (a.series + kIncThreads - 1) / kIncThreads;
     const int rgrid = min(kRbCtas, (a.series + kRbThreads / 32 - 1) / (kRbThreads / 32));
-    if (inc.entering <= 1 && inc.leaving <= 1) window_inc_kernel<1><<<grid, kIncThreads, 0, st>>>(a, inc);
-    else window_inc_kernel<kIncMaxNew><<<grid, kIncThreads, 0, st>>>(a, inc);
-    if (a.n <= 64) window_rebuild_kernel<2><<<rgrid, kRbThreads, 0, st>>>(a, inc);
-    else if (a.n <= 128) window_rebuild_kernel<4><<<rgrid, kRbThreads, 0, st>>>(a, inc);
-    else window_rebuild_kernel<8><<<rgrid, kRbThreads, 0, st>>>(a, inc);
-    return cudaGetLastError();
+    const cudaError_t e = inc.entering <= 1 && inc.leaving <= 1 ? launch_after(window_inc_kernel<1>, grid, kIncThreads, st, a, inc)
+                                                                : launch_after(window_inc_kernel<kIncMaxNew>, grid, kIncThreads, st, a, inc);
+    if (e != cudaSuccess) return e;
+    if (a.n <= 64) return launch_after(window_rebuild_kernel<2>, rgrid, kRbThreads, st, a, inc);
+    if (a.n <= 128) return launch_after(window_rebuild_kernel<4>, rgrid, kRbThreads, st, a, inc);
+    return launch_after(window_rebuild_kernel<8>, rgrid, kRbThreads, st, a, inc);
 }
 
 cudaError_t launch_window_select(const WindowArgs &a, cudaStream_t st) {

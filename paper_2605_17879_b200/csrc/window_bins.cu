@@ -79,6 +79,7 @@ __device__ __forceinline__ uint32_t wb_key(const float x) {
 // G warps of V values per thread; RELOAD: the window is longer than that, V values at a time are read again.
 template <int V, int G, int BINS, bool RELOAD>
 __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window_bins_kernel(const WindowArgs a) {
+    pdl_wait();
     static_assert(BINS % G == 0 && 32 % G == 0, "warps share the bins and the spread values evenly");
     __shared__ WbShared<BINS> sh;
     const int lane = lane_id(), w = warp_id(), n = a.n;
@@ -370,14 +371,13 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
 // Windows of up to 1 024 steps in registers.
 cudaError_t launch_window_bins(const WindowArgs &a, cudaStream_t st) {
     const int grid = (a.series + 31) / 32;
-    if (a.n <= 64) window_bins_kernel<8, 8, 32, false><<<grid, 256, 0, st>>>(a);
-    else if (a.n <= 128) window_bins_kernel<16, 8, 32, false><<<grid, 256, 0, st>>>(a);
-    else if (a.n <= 192) window_bins_kernel<24, 8, 32, false><<<grid, 256, 0, st>>>(a);
-    else if (a.n <= 256) window_bins_kernel<32, 8, 32, false><<<grid, 256, 0, st>>>(a);
-    else if (a.n <= 512) window_bins_kernel<32, 16, 64, false><<<grid, 512, 0, st>>>(a);
-    else if (a.n <= 1024) window_bins_kernel<32, 32, 64, false><<<grid, 1024, 0, st>>>(a);
-    else window_bins_kernel<16, 16, 64, true><<<grid, 512, 0, st>>>(a);
-    return cudaGetLastError();
+    if (a.n <= 64) return launch_after(window_bins_kernel<8, 8, 32, false>, grid, 256, st, a);
+    if (a.n <= 128) return launch_after(window_bins_kernel<16, 8, 32, false>, grid, 256, st, a);
+    if (a.n <= 192) return launch_after(window_bins_kernel<24, 8, 32, false>, grid, 256, st, a);
+    if (a.n <= 256) return launch_after(window_bins_kernel<32, 8, 32, false>, grid, 256, st, a);
+    if (a.n <= 512) return launch_after(window_bins_kernel<32, 16, 64, false>, grid, 512, st, a);
+    if (a.n <= 1024) return launch_after(window_bins_kernel<32, 32, 64, false>, grid, 1024, st, a);
+    return launch_after(window_bins_kernel<16, 16, 64, true>, grid, 512, st, a);
 }
 
 }  // namespace guard

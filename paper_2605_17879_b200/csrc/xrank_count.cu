@@ -44,9 +44,32 @@ cudaError_t launch_c(const XrankArgs &a, const MetricParams &p, int S, int T, cu
     return launch_after(xrank_count_kernel<32, C>, grid, T, st, a, p);
 }
 
+// Metrics and threads per CTA.
+void plan(const int R, const int M, const int S, int &C, int &T) {
+    // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
+    // larger CTAs, which wait longer at their barriers: 60 steps of 4 096 ranks x 16 metrics take 31 / 29 / 29 us, launch
+    // included, with 1 / 2 / 8 of them, 100 steps of 1 024 x 8 take 14 / 14 / 18), else one.
+    C = (M % 2 == 0 && 2 * R <= kCountMaxRanks && (long long)S * (M / 2) >= 148) ? 2 : 1;
+    const long long ctas = (long long)S * (M / C);
+    const int E = R * C;
+    // threads: few values each while the CTAs are few (a pass is then as short as it gets), else CTAs small enough to
+    // share an SM and hide one another's barriers
+    T = 32 * C;
+    if (ctas <= 148) { while (T < 1024 && E > 4 * T) T <<= 1; }
+    else { while (T < 256 && E > 8 * T) T <<= 1; }
+    while (T < 1024 && E > 32 * T) T <<= 1;
+}
+
 }  // namespace
 
 bool xrank_count_supported(int R) { return R >= 1 && R <= kCountMaxRanks; }
+
+bool xrank_count_copies(int R, int M, int S) {
+    if (R > kCtClusterRanks) return false;
+    int C, T;
+    plan(R, M, S, C, T);
+    return (long long)R * C <= 8LL * T;
+}
 
 cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
     if (S <= 0) return cudaSuccess;
@@ -55,18 +78,8 @@ cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S,
         if ((long long)S * a.M * 8 <= 148) return launch_cluster<8>(a, p, S, st);
         return launch_cluster<4>(a, p, S, st);
     }
-    // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
-    // larger CTAs, which wait longer at their barriers: 60 steps of 4 096 ranks x 16 metrics take 31 / 29 / 29 us, launch
-    // included, with 1 / 2 / 8 of them, 100 steps of 1 024 x 8 take 14 / 14 / 18), else one.
-    const int C = (a.M % 2 == 0 && 2 * a.R <= kCountMaxRanks && (long long)S * (a.M / 2) >= 148) ? 2 : 1;
-    const long long ctas = (long long)S * (a.M / C);
-    const int E = a.R * C;
-    // threads: few values each while the CTAs are few (a pass is then as short as it gets), else CTAs small enough to
-    // share an SM and hide one another's barriers
-    int T = 32 * C;
-    if (ctas <= 148) { while (T < 1024 && E > 4 * T) T <<= 1; }
-    else { while (T < 256 && E > 8 * T) T <<= 1; }
-    while (T < 1024 && E > 32 * T) T <<= 1;
+    int C, T;
+    plan(a.R, a.M, S, C, T);
     return C == 2 ? launch_c<2>(a, p, S, T, st) : launch_c<1>(a, p, S, T, st);
 }
 

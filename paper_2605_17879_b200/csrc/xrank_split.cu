@@ -146,6 +146,7 @@ struct SpSampleShared {
 // CTA handles four metrics: every thread bins the four components of its float4; then 64 threads per metric
 // scan their histogram.
 __global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const XrankArgs a, const SpGeom g, const SpScratch sc, const int rows) {
+    pdl_wait();
     __shared__ SpSampleShared sh;
     const int q = blockIdx.x, t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.R, M = a.M;
@@ -321,6 +322,7 @@ __device__ __forceinline__ void sp_scan_step(uint32_t &incl, const int d) {
 // Stores past a list's capacity land in the slack behind it; the full list is detected from the counter.
 template <int NQ>
 __global__ void __launch_bounds__(32 * kSpWarps, 6) xsplit_sweep_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc) {
+    pdl_wait();
     constexpr int M = 4 * NQ, LPI = 32 / NQ;
     extern __shared__ __align__(16) uint32_t slist[];   // [kSpWarps][M][cap + kSpSlack]
     __shared__ SpSweepShared sh;
@@ -659,6 +661,7 @@ __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, co
 template <int T>
 __global__ void __launch_bounds__(T, 1536 / T) xsplit_select_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc,
                                                                         uint32_t *reasons) {
+    pdl_wait();
     __shared__ CtShared<1> sh;
     __shared__ SpBands sb;
     __shared__ uint32_t s_n[2], s_col[4];
@@ -706,6 +709,7 @@ __global__ void __launch_bounds__(T, 1536 / T) xsplit_select_kernel(const XrankA
 // reads the flags of all steps at once, settles the steps that are its own, and takes its share of the columns.
 template <int V>
 __global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc, const int S) {
+    pdl_wait();
     __shared__ CtShared<1> sh;
     __shared__ uint32_t flags[kSplitMaxSteps];
     __shared__ uint16_t before[kSplitMaxSteps + 1];   // columns to recompute before each step
@@ -845,21 +849,24 @@ cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S,
     if (prof && (cudaEventCreate(&ev0) != cudaSuccess || cudaEventCreate(&ev1) != cudaSuccess)) return cudaGetLastError();
     // estimates for the step positions and columns that have none (with hints a look at the records, as a rule: 2 us)
     const bool same = state.epoch == a.hint_epoch;
-    xsplit_sample_kernel<<<dim3(M / 4, S), kSpThreads, 0, st>>>(a, g, sc, !a.hint_fresh && same ? state.rows : 0);
+    e = launch_after(xsplit_sample_kernel, dim3(M / 4, S), kSpThreads, st, a, g, sc, !a.hint_fresh && same ? state.rows : 0);
+    if (e != cudaSuccess) return e;
     state.rows = same && state.rows > S ? state.rows : S;
     state.epoch = a.hint_epoch;
     if (prof) cudaEventRecord(ev0, st);   // the sweep, the longest kernel
-    if (M == 8) xsplit_sweep_kernel<2><<<dim3(g.chunks, S), 32 * kSpWarps, smem, st>>>(a, p, g, sc);
-    else xsplit_sweep_kernel<1><<<dim3(g.chunks, S), 32 * kSpWarps, smem, st>>>(a, p, g, sc);
+    e = M == 8 ? launch_after_smem(xsplit_sweep_kernel<2>, dim3(g.chunks, S), 32 * kSpWarps, smem, st, a, p, g, sc)
+               : launch_after_smem(xsplit_sweep_kernel<1>, dim3(g.chunks, S), 32 * kSpWarps, smem, st, a, p, g, sc);
+    if (e != cudaSuccess) return e;
     if (prof) cudaEventRecord(ev1, st);
     // (22 us against 23 for 1 600 columns of some 1 900 values; 9 against 14 for 400 of 2 300)
-    if ((long long)S * M > 148 * 6) xsplit_select_kernel<128><<<dim3(M, S), 128, 0, st>>>(a, p, g, sc, reasons);
-    else if ((long long)S * M > 148 * 3) xsplit_select_kernel<256><<<dim3(M, S), 256, 0, st>>>(a, p, g, sc, reasons);
-    else xsplit_select_kernel<512><<<dim3(M, S), 512, 0, st>>>(a, p, g, sc, reasons);
+    const dim3 columns(M, S);
+    if ((long long)S * M > 148 * 6) e = launch_after(xsplit_select_kernel<128>, columns, 128, st, a, p, g, sc, reasons);
+    else if ((long long)S * M > 148 * 3) e = launch_after(xsplit_select_kernel<256>, columns, 256, st, a, p, g, sc, reasons);
+    else e = launch_after(xsplit_select_kernel<512>, columns, 512, st, a, p, g, sc, reasons);
+    if (e != cudaSuccess) return e;
     const int T = a.R <= 32 * 128 ? 128 : (a.R <= 32 * 256 ? 256 : (a.R <= 32 * 512 ? 512 : 1024));
     const int most = 148 * (1024 / T);   // what the SMs hold of them at 64 registers per thread
-    xsplit_finish_kernel<32><<<S * M < most ? S * M : most, T, 0, st>>>(a, p, g, sc, S);
-    e = cudaGetLastError();
+    e = launch_after(xsplit_finish_kernel<32>, S * M < most ? S * M : most, T, st, a, p, g, sc, S);
     if (prof) prof->emplace_back(ev0, ev1);
     return e;
 }

@@ -613,6 +613,33 @@ def test_sweep_of_many_series(nodes, gpn, N, M):
         assert_bit_equal(to_np(out[key]), ref[key], key)
 
 
+@pytest.mark.parametrize("R,M,W,B", [
+    (61, 3, 7, 7),                 # a metric per CTA; a ring that the third block wraps
+    (1024, 8, 64, 16),             # two metrics per CTA, eight values per thread
+    (4096, 4, 128, 1),             # single rows; the most values of a window that stays on the caller's stream
+    (4097, 4, 128, 1),             # the fewest that does not
+    (2048, 6, 12, 12),             # sixteen values per thread: copied in front
+])
+def test_small_evaluations_in_line(R, M, W, B):
+    """Blocks that the counting kernels put into the ring, evaluations on the caller's stream, and a change to deferred
+    evaluations and back in between."""
+    from paper_2605_17879_b200 import guard
+    n = min(-(-W // B), 6) + 4
+    X, dirs = _rand_fleet(n * B, R, M, seed=R + W)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, W, max(1, W // 2), dir=dirs, capacity=2 * W + 3, topk=5, min_signals=1)
+    o = go.Oracle(R, M, W, max(1, W // 2), 5, dir=dirs, min_signals=1)
+    for i in range(n):
+        g.ingest(Xd[i * B:(i + 1) * B].contiguous())
+        g.set_deferred(i % 4 >= 2)
+        out = g.score()
+        g.join()
+        o.ingest(X[i * B:(i + 1) * B])
+        assert g.sync_status() == 0
+        compare_score(out, o.score(), "block %d" % i)
+    g.close()
+
+
 @pytest.mark.parametrize("R,M,W,quant", [
     (70, 3, 1, None),              # one step; a ragged last tile
     (64, 4, 64, None),             # every slot of eight warps of eight values in use

@@ -706,9 +706,15 @@ __global__ void __launch_bounds__(T, 1536 / T) xsplit_select_kernel(const XrankA
 // ---- 3. finish ---------------------------------------------------------------------------------
 // Settles the deferred exceedance decisions, and recomputes the columns on the steps' lists with the values in
 // registers.  As a rule there is next to nothing to do, and what counts is the number of dependent loads: every CTA
-// reads the flags of all steps at once, settles the steps that are its own, and takes its share of the columns.
+// reads the flags of all steps at once, settles the steps that are its own, and takes its share of the columns.  Few
+// columns (one metric with hardly any distinct values, steps that missed) take a cluster of four CTAs each, a quarter of
+// the values per thread (118 columns of 8 192 ranks: 22 us, 42 by a CTA each); more than there are clusters a CTA each,
+// where one holds a column (16 384 ranks with 512 threads; CTAs of 1 024 wait for whole SMs beside other streams' work).
+// V: values per thread of a CTA that takes a column alone, above 32 never.
+constexpr int kFinCluster = 4;
+
 template <int V>
-__global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc, const int S) {
+__global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(512, 2) xsplit_finish_kernel(const XrankArgs a, const MetricParams p, const SpGeom g, const SpScratch sc, const int S) {
     pdl_wait();
     __shared__ CtShared<1> sh;
     __shared__ uint32_t flags[kSplitMaxSteps];
@@ -759,15 +765,18 @@ __global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, 
     }
     __syncthreads();
     const int n = before[S];
-    for (int item = blockIdx.x; item < n; item += gridDim.x) {
+    const bool wide = V > 32 || n <= (int)gridDim.x / kFinCluster;      // (the same for all CTAs)
+    const int share = wide ? kFinCluster : 1;
+    for (int item = blockIdx.x / share; item < n; item += gridDim.x / share) {
         int lo = 0, hi = S;                // the step: before[lo] <= item < before[lo + 1]
         while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if ((int)before[mid] <= item) lo = mid; else hi = mid; }
         uint32_t bits = flags[lo] & 0x7FFFFFFFu;
         for (int f = item - (int)before[lo]; f > 0; --f) bits &= bits - 1u;
         const int m = __ffs(bits) - 1;
-        ct_row<V, 1>(a, p, lo, m, sh);
+        if (wide) ct_row<V / kFinCluster, 1, kFinCluster>(a, p, lo, m, sh);
+        else ct_row<(V > 32 ? 1 : V), 1>(a, p, lo, m, sh);
         __syncthreads();
-        if (tid == 0) {                    // the result is the next block's estimate
+        if (tid == 0 && (!wide || ct_rank() == 0u)) {                    // the result is the next block's estimate
             SpCol &col = sc.col[(size_t)lo * M + m];
             sp_learn(col, a.med[(size_t)lo * M + m], a.mad[(size_t)lo * M + m], true, R);
             if (col.epoch != sc.epoch) col.resample = 0;
@@ -775,6 +784,7 @@ __global__ void __launch_bounds__(1024) xsplit_finish_kernel(const XrankArgs a, 
             if (col.rest) col.rest -= 1;
         }
     }
+    if (wide) ct_sync<kFinCluster>();      // no CTA exits while others may read its shared memory
 }
 
 // Kept fraction of a column: 2 hm about the median, 4 ha about the quartiles (normal density, MAD units).
@@ -864,9 +874,11 @@ cudaError_t launch_xrank_split(const XrankArgs &a, const MetricParams &p, int S,
     else if ((long long)S * M > 148 * 3) e = launch_after(xsplit_select_kernel<256>, columns, 256, st, a, p, g, sc, reasons);
     else e = launch_after(xsplit_select_kernel<512>, columns, 512, st, a, p, g, sc, reasons);
     if (e != cudaSuccess) return e;
-    const int T = a.R <= 32 * 128 ? 128 : (a.R <= 32 * 256 ? 256 : (a.R <= 32 * 512 ? 512 : 1024));
+    const int T = a.R <= 32 * 128 ? 128 : (a.R <= 32 * 256 ? 256 : 512);
     const int most = 148 * (1024 / T);   // what the SMs hold of them at 64 registers per thread
-    e = launch_after(xsplit_finish_kernel<32>, S * M < most ? S * M : most, T, st, a, p, g, sc, S);
+    const int grid = (min(S * M, most) + kFinCluster - 1) / kFinCluster * kFinCluster;
+    e = a.R <= 32 * 512 ? launch_after(xsplit_finish_kernel<32>, grid, T, st, a, p, g, sc, S)
+                        : launch_after(xsplit_finish_kernel<64>, grid, T, st, a, p, g, sc, S);
     if (prof) prof->emplace_back(ev0, ev1);
     return e;
 }

@@ -712,3 +712,17 @@ def test_one_pass_blocks(R, M, B, thr, deferred):
     if thr == 3.5 and R <= 32768:
         assert g.fallback_steps() == 0
     g.close()
+
+
+@pytest.mark.parametrize("R,M,B,thr", [
+    (8191, 8, 20, 3.5),            # a metric of a handful of values, recomputed by clusters
+    (16384, 4, 40, 3.5),           # the most values per thread of a cluster
+    (16385, 4, 18, 3.5),           # wider: sixteen values per thread, clusters only
+    (32768, 8, 20, 0.5),           # every column, the widest
+    (16384, 8, 45, 0.5),           # every column, a CTA each
+])
+def test_one_pass_columns_recomputed(R, M, B, thr):
+    X, dirs = _rand_fleet(2 * B, R, M, seed=R + B)
+    X[:, :, 1] = np.round(X[:, :, 1] * np.float32(20.0)) / np.float32(20.0)
+    X[B + 3] *= np.float32(1.5)
+    run_both(X, B, max(1, B // 2), 8, dirs, [B], capacity=2 * B, thr=thr)

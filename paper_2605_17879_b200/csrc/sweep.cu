@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kSweepCols) sweep_median_kernel(const SweepMed
 // middle ranks are then found among the kept keys (pivot search, as for the window medians).  A series whose counts
 // do not prove the bracket (or whose column overflows) is left to sweep_median_finish_kernel.
 // Bound by the chain of instructions of a series (8 000 of them, 21 warps per SM) and by the loads' cache lines (a
-// repetition is another line for every GPU of the warp): 41 us at 16 384 GPUs x 200 x 6 with the results in L2, 63 from
+// repetition is another line for every GPU of the warp): 39 us at 16 384 GPUs x 200 x 6 with the results in L2, 63 from
 // HBM.  Not faster: the next loads in flight ahead of the passes (the same), blocks staged whole in shared memory (seven
 // warps per SM: 62 and 64), or in chunks of eight repetitions, asynchronously (84) or through registers (49 and 68).
 constexpr int kSwThreads = 128;
@@ -97,27 +97,24 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_thread_kernel(const S
     const float mean_d = sd1 * inv;
     const float var = fmaxf(sd2 * inv - mean_d * mean_d, 0.0f);
     const float c = x0 + mean_d, h = 2.83f * sqrtf(var * inv);
-    const bool usable = active && !bad && !same && (h > 0.0f) && (h < 3.0e38f) && (fabsf(c) < 3.0e38f);
-    float flo = c - h, fhi = c + h;
-    if (flo == 0.0f) flo = -0.0f;   // an end that is zero admits both zeros: float compares then agree with the key order
-    if (fhi == 0.0f) fhi = 0.0f;
-    if (!usable) { flo = CUDART_INF_F; fhi = -CUDART_INF_F; }
-    const uint32_t klo = usable ? f2key(flo) : 0xFFFFFFFFu, khi = usable ? f2key(fhi) : 0u;
+    const bool usable = active && !bad && !same && th_usable(c, h);
+    const ThRange range = th_range(c, h, usable);
 
     // pass B (the block is in L1 / L2 by now): count below, keep inside
     const uint32_t kbase = (uint32_t)__cvta_generic_to_shared(kept + tid * kSwSlots), klim = kbase + (uint32_t)(kSwSlots * 4);
-    uint32_t kaddr = kbase, clt = 0;
+    uint32_t kaddr = kbase;
+    float cltf = 0.0f;
     if (__any_sync(0xFFFFFFFFu, usable)) {
-        each([&](const float x) { th_cell(x, flo, fhi, klim, clt, kaddr); });
+        each([&](const float x) { th_cell(x, range, klim, cltf, kaddr); });
     }
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
     const int nk = (int)((kaddr - kbase) >> 2);
-    bool ok = usable && (int)clt <= k1 && k2 < (int)clt + nk && nk <= kSwSlots;
-    uint32_t vb = 0, vu = 0;
-    th_select_pair<kSwSlots, kSwMaxPasses>(kbase, nk, ok, k2 - (int)clt, klo, khi, vb, vu);
-    float med = 0.0f;
-    if (ok) med = median_from_keys(even ? vb : vu, vu, even);
+    const int clt = (int)cltf;
+    bool ok = usable && clt <= k1 && k2 < clt + nk && nk <= kSwSlots;
+    float vb = 0.0f, vu = 0.0f, med = 0.0f;
+    th_select_pair<kSwSlots, kSwMaxPasses>(kbase, nk, ok, k2 - clt, range, vb, vu);
+    if (ok) med = even ? __fmul_rn(0.5f, __fadd_rn(vb, vu)) : vu;
     if (active && same && !bad) { med = x0; ok = true; }
     if (active && ok) {
         a.gmed[sidx] = med;

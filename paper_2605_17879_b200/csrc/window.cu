@@ -214,6 +214,10 @@ constexpr int kThTarget = 42;    // number of keys the interval is tuned to catc
 constexpr int kThRows = 8;       // rows in flight per thread
 constexpr int kThMaxPasses = 12;
 constexpr float kThSmooth = 0.3f;   // weight of the newest median in the interval's centre
+// Part of the way the half-width goes towards the one that would have caught kThTarget: little while the count is
+// within its noise (a third), so that it does not follow it (2.1 % of 131 072 series unserved with a half in any case,
+// 1.6 % so), half of the way beyond (a small part in any case: slow to settle, 3 % unserved instead of 0.8 % at 24 000 x 8).
+constexpr float kThNear = 0.33f, kThNearPart = 0.15f, kThFarPart = 0.5f;
 
 template <int VPL>
 __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowArgs a) {
@@ -228,17 +232,12 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
     const int n1 = min(n, a.capacity - first);          // rows before the ring wraps
 
     const float hint = a.centre[cc], h = a.spread[cc];
-    const bool usable = active && (h > 0.0f) && (h < 3.0e38f) && (fabsf(hint) < 3.0e38f);
-    // Float compares agree with the key order as long as an end that is zero admits both zeros
-    // (-0 as lower end, +0 as upper end).  An unusable interval keeps and counts nothing.
-    float flo = hint - h, fhi = hint + h;
-    if (flo == 0.0f) flo = -0.0f;
-    if (fhi == 0.0f) fhi = 0.0f;
-    if (!usable) { flo = CUDART_INF_F; fhi = -CUDART_INF_F; }
-    const uint32_t klo = usable ? f2key(flo) : 0xFFFFFFFFu, khi = usable ? f2key(fhi) : 0u;
+    const bool usable = active && th_usable(hint, h);
+    const ThRange range = th_range(hint, h, usable);
 
     const uint32_t kbase = smem_u32(tkept + tid * kThSlots), klim = kbase + (uint32_t)(kThSlots * 4);
-    uint32_t kaddr = kbase, clt = 0;
+    uint32_t kaddr = kbase;
+    float cltf = 0.0f;
     auto stream = [&](const float *__restrict__ p, const int rows) {
         int r = 0;
         for (; r + kThRows <= rows; r += kThRows) {
@@ -246,9 +245,9 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
 #pragma unroll
             for (int u = 0; u < kThRows; ++u) x[u] = __ldg(p + (size_t)(r + u) * a.row_stride);
 #pragma unroll
-            for (int u = 0; u < kThRows; ++u) th_cell(x[u], flo, fhi, klim, clt, kaddr);
+            for (int u = 0; u < kThRows; ++u) th_cell(x[u], range, klim, cltf, kaddr);
         }
-        for (; r < rows; ++r) th_cell(__ldg(p + (size_t)r * a.row_stride), flo, fhi, klim, clt, kaddr);
+        for (; r < rows; ++r) th_cell(__ldg(p + (size_t)r * a.row_stride), range, klim, cltf, kaddr);
     };
     stream(a.ring + (size_t)first * a.row_stride + cc, n1);
     stream(a.ring + cc, n - n1);
@@ -256,26 +255,26 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
     const int nk = (int)((kaddr - kbase) >> 2);
-    bool ok = usable && (int)clt <= k1 && k2 < (int)clt + nk && nk <= kThSlots;
-    const int t = k2 - (int)clt;     // rank of the upper middle among the kept keys (t >= 1 when n is even)
-    float med = 0.0f;
-    // ---- selection among the kept keys: the same instruction stream in every lane ---------------
-    uint32_t vb = 0, vu = 0;
-    th_select_pair<kThSlots, kThMaxPasses>(kbase, nk, ok, t, klo, khi, vb, vu);
-    if (ok) med = median_from_keys(even ? vb : vu, vu, even);
+    const int clt = (int)cltf;
+    bool ok = usable && clt <= k1 && k2 < clt + nk && nk <= kThSlots;
+    // ---- selection among the kept values: the same instruction stream in every lane -------------
+    float vb = 0.0f, vu = 0.0f, med = 0.0f;
+    th_select_pair<kThSlots, kThMaxPasses>(kbase, nk, ok, k2 - clt, range, vb, vu);   // (k2 - clt >= 1 when n is even)
+    if (ok) med = even ? __fmul_rn(0.5f, __fadd_rn(vb, vu)) : vu;
     if (active && ok) {
         a.wmed[c] = med;
         if (a.wmed_user) a.wmed_user[c] = med;
         // re-tune the half-width so that the interval catches about kThTarget keys next time
-        // (half of the way: one window's count is a noisy estimate of the density)
-        const float f = fminf(2.0f, fmaxf(0.5f, (float)(a.target > 0 ? a.target : kThTarget) / (float)max(nk, 1)));
-        a.spread[c] = h * (0.5f + 0.5f * f);
+        const float target = (float)(a.target > 0 ? a.target : kThTarget);
+        const float f = fminf(2.0f, fmaxf(0.5f, target / (float)max(nk, 1)));
+        const float part = fabsf((float)nk - target) > kThNear * target ? kThFarPart : kThNearPart;
+        a.spread[c] = h * (1.0f - part + part * f);
         a.centre[c] = hint + (a.smooth > 0.0f ? a.smooth : kThSmooth) * (med - hint);
     }
     // ---- series the interval did not serve go on the launch's list (window_finish_kernel follows) ------
     // why (diagnostic): 0 no usable interval, 1 more keys than slots, 2 median below the interval,
     // 3 above it, 4 selection did not converge
-    const int why = !usable ? 0 : (nk > kThSlots ? 1 : ((int)clt > k1 ? 2 : (k2 >= (int)clt + nk ? 3 : 4)));
+    const int why = !usable ? 0 : (nk > kThSlots ? 1 : (clt > k1 ? 2 : (k2 >= clt + nk ? 3 : 4)));
     const unsigned todo = __ballot_sync(0xFFFFFFFFu, active && !ok);
     if (todo) {
         uint32_t base = 0;

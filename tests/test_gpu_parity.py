@@ -605,6 +605,14 @@ def test_sweep_of_many_series(nodes, gpn, N, M):
     S[6::50] *= np.float32(1e38) * np.sign(rng.standard_normal((1, N, 1))).astype(np.float32)
     S[7::50, 1] = np.float32(1e30)
     S[8::50, :, 0] *= np.float32(0.7)
+    S[9::50] -= np.float32(1.0)
+    S[11::50] = np.float32(0.0)
+    S[12::50] = np.float32(-0.0)
+    S[13::50] = np.copysign(np.float32(0.0), S[13::50] - 1.0)
+    S[13::50, 0] = np.float32(0.0)
+    S[14::50] = np.copysign(np.float32(0.0), S[14::50] - 1.0)
+    S[14::50, 0] = np.float32(-0.0)
+    S[10::50] = np.where(np.abs(S[10::50] - 1.0) < 0.01, np.copysign(np.float32(0.0), S[10::50] - 1.0), S[10::50] - 1.0)
     dirs = [-1] * M
     ref = go.sweep(S, nodes, gpn, dir=dirs)
     out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
@@ -677,6 +685,25 @@ def test_window_tiles(R, M, W, quant):
         for key in ("wmed", "fleet_med", "fleet_mad", "counts", "mask", "flags", "tier"):
             assert_bit_equal(to_np(out[key]), ref[key], "t=%d %s" % (t, key))
     g.close()
+
+
+@pytest.mark.parametrize("R,M,W", [
+    (16385, 4, 32),                # two keys per lane where the interval misses; a CTA of four series
+    (9001, 8, 101),
+    (22000, 3, 256),               # the longest window of the path
+])
+def test_window_threads(R, M, W):
+    """Many series, whole windows, a thread each from the second evaluation on: series about zero, with zeros of both
+    signs at their middle, very small and very large ones, ties, and a fourth window that leaves every interval."""
+    X, dirs = _rand_fleet(5 * W, R, M, seed=R + W)
+    X[:, 1::40] -= np.float32(1.0)
+    X[:, 2::40] = np.where(np.abs(X[:, 2::40] - 1.0) < 0.01, np.copysign(np.float32(0.0), X[:, 2::40] - 1.0), X[:, 2::40] - 1.0)
+    X[:, 3::40] *= np.float32(1e-25)
+    X[:, 4::40] *= np.float32(1e20)
+    X[:, 5::40] = np.round(X[:, 5::40] * np.float32(40.0)) / np.float32(40.0)
+    X[:, 6::40] = np.where(X[:, 6::40] > 1.0, X[:, 6::40], np.float32(1e-40))
+    X[3 * W:] *= np.float32(1.5)
+    run_both(X, W, max(1, W // 2), 8, dirs, [W], capacity=W)
 
 
 @pytest.mark.parametrize("R,M,B,thr,deferred", [

@@ -17,9 +17,6 @@ using namespace guard;
 namespace {
 
 constexpr size_t kAlign = 256;
-#ifndef GUARD_EVAL_PRIO
-#define GUARD_EVAL_PRIO 1
-#endif
 #ifndef GUARD_INGEST_STREAMS
 #define GUARD_INGEST_STREAMS 2
 #endif
@@ -169,10 +166,13 @@ struct guard_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_topk = nullptr;
     bool ensure_side() {
         if (side) return true;
-        // the evaluation's streams get the highest priority: flags should not queue behind the next blocks' sweeps
+        // The evaluation's streams go first: flags should not queue behind the next blocks' sweeps; and its tail goes before
+        // the next evaluation's window medians, or its clusters of whole SMs wait until those have drained (eight single
+        // steps of 32 768 x 8 246 us with the same priority for both, 243 so; 239 with none for the medians, but then
+        // blocks of 200 x 16 384 x 8 take 434 us instead of 420).
         int prio_lo = 0, prio_hi = 0;
         cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-        if (cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) { side = nullptr; return false; }
+        if (cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, min(prio_hi + 1, prio_lo)) != cudaSuccess) { side = nullptr; return false; }
         if (cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_topk, cudaEventDisableTiming) != cudaSuccess) {
@@ -257,8 +257,8 @@ struct guard_ctx {
         if (!ensure_side()) return false;
         int prio_lo = 0, prio_hi = 0;
         cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-        if (cudaStreamCreateWithPriority(&tail, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) { tail = nullptr; return false; }
-        if (!xrank_count_supported(R) && cudaStreamCreateWithPriority(&aux, cudaStreamNonBlocking, GUARD_EVAL_PRIO ? prio_hi : 0) != cudaSuccess) aux = nullptr;
+        if (cudaStreamCreateWithPriority(&tail, cudaStreamNonBlocking, prio_hi) != cudaSuccess) { tail = nullptr; return false; }
+        if (!xrank_count_supported(R) && cudaStreamCreateWithPriority(&aux, cudaStreamNonBlocking, prio_hi) != cudaSuccess) aux = nullptr;
         if (cudaEventCreateWithFlags(&ev_x, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_w, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ev_e[0], cudaEventDisableTiming) != cudaSuccess ||

@@ -28,6 +28,7 @@ constexpr int kCtList = 64;        // keys of a bin that are ranked directly (tw
 constexpr int kCtMaxIter = 64;     // a range shrinks at least to a 128th whenever its bin is too full
 constexpr uint32_t kCtTop = 0xFF800000u;    // no key of a number lies above; padding does
 constexpr uint32_t kCtNone = 0xFFFFFFFFu;
+constexpr int kCtAll = 0, kCtStatistics = 1, kCtCut = 2;   // what a CTA (cluster) computes: both, median and MAD, the extra order statistic
 // Single rows of 8 metrics, bracketed by the row before / not: one CTA of 1 024 threads per column takes 6.3 / 7.5 us at
 // 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
 // barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3.
@@ -345,7 +346,7 @@ __device__ __forceinline__ int ct_select(const uint32_t (&key)[V], const uint32_
 // Median, MAD (and optional extra order statistic) of metrics [m0, m0 + C) of row s of the launch, and their
 // exceedance bits.  C divides M, R * C <= V * NC * blockDim.x, blockDim.x >= 32 * C; C = 1 with clusters.
 template <int V, int C, int NC = 1>
-__device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p, const int s, const int m0, CtShared<C> &sh) {
+__device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p, const int s, const int m0, CtShared<C> &sh, const int part = kCtAll) {
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id(), T = blockDim.x;
     const int R = a.R, M = a.M;
     const int col = tid & (C - 1);
@@ -401,7 +402,8 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     const float u = hmad * rsqrtf((float)R);
     const bool hinted = hmad > 0.0f && hmad < 1.0e37f && fabsf(hmed) < 1.0e37f;
     if (warp < C) {
-        if (hinted) range(f2key(hmed - 10.0f * u), f2key(hmed + 10.0f * u));
+        if (part == kCtCut) sampled(f2key(xs), (uint32_t)a.cut_rank[m0]);   // (the first of C)
+        else if (hinted) range(f2key(hmed - 10.0f * u), f2key(hmed + 10.0f * u));
         else sampled(f2key(xs), k1);
     }
     if (a.check_finite) {
@@ -414,7 +416,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     for (int i = 0; i < V; ++i) key[i] = key_of_bits(key[i]);
     // what: 0 the median, 1 the MAD, 2 + c the extra order statistic of metric m0 + c (before the MAD)
 #pragma unroll 1
-    for (int what = 0;;) {
+    for (int what = part == kCtCut ? 2 : 0;;) {
         const bool extra = what >= 2;
         const uint32_t q1 = extra ? (uint32_t)a.cut_rank[m0 + what - 2] : k1, q2 = extra ? q1 : k2;
         const int rounds = ct_select<V, C, NC>(key, q1, q2, sh);
@@ -446,10 +448,10 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                 if (a.cut_user) a.cut_user[o] = key2f(v1);
             }
         }
-        if (what == 1) break;
+        if (what == 1 || (part == kCtCut && what == C + 1)) break;
         __syncthreads();
         // the metrics' extra ranks first (they need the values), then the deviations
-        what = !a.cut ? 1 : (what == 0 ? 2 : (what - 1 < C ? what + 1 : 1));
+        what = !a.cut || part == kCtStatistics ? 1 : (what == 0 ? 2 : (what - 1 < C ? what + 1 : 1));
         if (what >= 2) {
             if (warp < C) sampled(f2key(xs), (uint32_t)a.cut_rank[m0 + what - 2]);
         } else {

@@ -591,6 +591,8 @@ def test_exceedance_counts(R, M, W):
     (77, 130, 45, 5),              # more GPUs per node than a CTA has threads
     (400, 4, 256, 32),             # the most repetitions and metrics
     (340, 8, 100, 12),             # a warp per series, the most of them
+    (700, 8, 33, 12),              # fleet statistics by clusters of four, the cut beside them
+    (600, 8, 20, 20),              # the same without room beside
 ])
 def test_sweep_of_many_series(nodes, gpn, N, M):
     """Many series of repeated results: constant and two-valued series, denormal and huge values, and an outlier that

@@ -37,11 +37,11 @@ UNIT = "cells/s"
 L2_BYTES = 126 * 1024 * 1024
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant kernel on this workload, from
 # the ncu capture summarised under profiles/ (None once the kernel has changed since the capture)
-NCU_TRAFFIC_BYTES_PER_LAUNCH = 112.0e6   # window_thread_kernel 110.72e6 + its finishing kernel (~200 series x 6.4 KB)
-# which kernel the roofline object describes: 2 = window_thread_kernel (guard_score), 1 = the MAD sweep (guard_ingest)
+NCU_TRAFFIC_BYTES_PER_LAUNCH = None
+# which kernel the roofline object describes: 2 = window_thread_kernel (guard_score), 1 = the cross-rank sweep (guard_ingest)
 PROFILE_MODE = 2
 PROFILE_KERNEL = ("window_thread_kernel + window_finish_kernel (windowed per-rank medians of one evaluation)" if PROFILE_MODE == 2 else
-                  "xsplit_sweep_kernel<2,1> (cross-rank MAD / exceedance sweep of one ingested block)")
+                  "xsplit_sweep_kernel<2> (cross-rank sweep of one ingested block)")
 FALLBACK_HBM_GBS = 6650.0   # earlier measurement on this machine, used only if MEASURED_PEAKS.json is absent
 
 
@@ -444,7 +444,7 @@ def main():
     # roofline of the dominant kernel, timed by the library with CUDA events recorded right around
     # it on the stream it is launched on (while the other kernels of the pipeline share the GPU).
     # The window-median kernel reads the W x ranks x metrics window once (4 B per cell covered);
-    # the MAD / exceedance sweep reads a block of 200 steps once (4 B per cell) and writes one
+    # the cross-rank sweep reads a block of 200 steps once (4 B per cell) and writes one
     # exceedance byte per (step, rank).
     launch_s = (kern_ms / kern_n / 1e3) if kern_n else float("nan")
     algo_bytes = (cfg.W * R * M * 4) if PROFILE_MODE == 2 else (B * R * M * 4 + B * R * 1)

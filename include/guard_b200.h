@@ -278,15 +278,14 @@ int guard_set_sliding(guard_ctx *ctx, int on);
 
 /* Single rows of wide fleets (on by default).  The cross-rank statistics of a one-step ingest and
  * the fleet baseline of an evaluation (Sec. 4.2: median and MAD over all ranks) are each ONE row; from
- * 8 192 ranks on, a call site keeps its previous median and MAD and a tuned width per metric, which
- * bracket the next row's: the selection then counts the values below the bracket, bins the few inside
- * and ranks the wanted bin's values directly.  The counts prove the bracket; a row they do not prove
- * (the first one, a jump, ties) takes the general selection inside the same kernel.  Blocks of many
- * steps (4 096 ranks and more, 4 or 8 metrics) use the same idea: the medians and MADs a block found
- * stay in its scratch and bracket those of the next block at the same step position, so nothing is
- * sampled; a step whose counts do not prove its bracket is redone exactly (it counts in
- * guard_fallback_steps) and samples next time.  Results are identical either way;
- * guard_set_row_hints(ctx, 0) always takes the general selection / sampled intervals. */
+ * 8 192 ranks on, the previous median and MAD of a call site bracket the next row's: the selection
+ * then counts the values below the bracket, bins the few inside and ranks the wanted bin's values
+ * directly.  The counts prove the bracket; one they do not prove (the first row, a jump) is moved inside
+ * the same kernel.  Blocks of many steps use the same idea; the one-pass path (4 096 ranks and more, 4 or
+ * 8 metrics) keeps running estimates per step position and metric, so nothing is sampled; a column
+ * whose counts do not prove its estimate is recomputed exactly (its step counts in
+ * guard_fallback_steps) and may sample next time.  Results are identical either way;
+ * guard_set_row_hints(ctx, 0) always starts from sampled values. */
 int guard_set_row_hints(guard_ctx *ctx, int on);
 
 /* Diagnostic: synchronises `stream` and fills out[6] (HOST): single rows seen and (row, metric)
@@ -319,8 +318,7 @@ int guard_set_deferred(guard_ctx *ctx, int on);
 int guard_join(guard_ctx *ctx, void *stream);
 
 /* Kernel timing for benchmarks.  on = 1: guard_ingest records a pair of CUDA events on its
- * stream right around the longest of its kernels (the MAD / exceedance sweep of the split
- * cross-rank path; contexts whose sizes take another path record around their main kernel or
+ * stream right around the longest of its kernels (the sweep of the split cross-rank path; contexts whose sizes take another path record around their main kernel or
  * nothing).  on = 2: guard_score records the pair around its window-median kernel, on the
  * stream that kernel runs on.  guard_profile_read waits for the recorded events, returns the
  * sum of the kernel durations in milliseconds and their number, and forgets them.  on = 0

@@ -27,7 +27,7 @@ struct Layout {
     size_t status, consec, lastflag, lasttier, topk_idx, topk_hint, ticket, fleet, xr_small, xr_grid, inc_rbc, wmed, wmed_stride, stepstat, topk_cand, wspread, wcentre, kcnt, inc_lo, inc_hi, inc_cnt, inc_val, inc_rbl, xr_big, xr_big_stride, mask, ring, total;
     int xr_steps;   // steps per launch of the multi-kernel bracketed cross-rank path (0: not used)
     int xr_cluster; // the cluster-per-step cross-rank path applies
-    int xr_split;   // the six-kernel split cross-rank path applies
+    int xr_split;   // the one-pass (split) cross-rank path applies
     int xr_gridp;   // single rows count how many were bracketed by the row before (two RowHints at xr_grid: ingest, fleet baseline)
 };
 
@@ -288,7 +288,7 @@ struct guard_ctx {
             }
         return cudaSuccess;
     }
-    int profiling = 0;                                        // 1: time the MAD sweep of every ingest, 2: the window kernel of every evaluation
+    int profiling = 0;                                        // 1: time the cross-rank sweep of every ingest, 2: the window kernel of every evaluation
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof;    // recorded, not yet read
     char error[256];
 

@@ -315,7 +315,7 @@ class Guard:
         self._check(_native().join(self._hv, self._devidx))
 
     def profile_enable(self, on=True) -> None:
-        """0 / False: off; 1 / True: time the MAD sweep of every ingest; 2: the window kernel of every evaluation."""
+        """0 / False: off; 1 / True: time the cross-rank sweep of every ingest; 2: the window kernel of every evaluation."""
         self._check(lib().guard_profile_enable(self._h, int(on)))
 
     def profile_read(self):

@@ -24,7 +24,7 @@ constexpr int kIngestStreams = GUARD_INGEST_STREAMS;   // internal streams the c
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t status, consec, lastflag, lasttier, topk_idx, topk_hint, ticket, fleet, xr_small, xr_grid, inc_rbc, wmed, wmed_stride, stepstat, topk_cand, wspread, wcentre, kcnt, inc_lo, inc_hi, inc_cnt, inc_val, inc_rbl, xr_big, xr_big_stride, mask, ring, total;
+    size_t status, consec, lastflag, lasttier, topk_idx, topk_hint, ticket, fleet, xr_small, xr_grid, inc_rbc, wmed, wmed_stride, stepstat, stepstat_stride, topk_cand, wspread, wcentre, kcnt, inc_lo, inc_hi, inc_cnt, inc_val, inc_rbl, xr_big, xr_big_stride, mask, ring, total;
     int xr_steps;   // steps per launch of the multi-kernel bracketed cross-rank path (0: not used)
     int xr_cluster; // the cluster-per-step cross-rank path applies
     int xr_split;   // the one-pass (split) cross-rank path applies
@@ -55,7 +55,11 @@ Layout make_layout(int R, int M, int C, int K) {
     L.wmed = off;      off = align_up(off + (size_t)R * M * sizeof(float));
     L.wmed_stride = off - L.wmed;
     off = align_up(off + (size_t)R * M * sizeof(float));
+    // per-step medians and MADs: a set per internal ingest stream (the blocks of two streams run side by side, and a
+    // block's recomputed columns start from what its rows held before)
     L.stepstat = off;  off = align_up(off + 2 * (size_t)C * M * sizeof(float));
+    L.stepstat_stride = off - L.stepstat;
+    off = align_up(off + (L.xr_split ? (kIngestStreams - 1) * L.stepstat_stride : 0));
     L.topk_cand = off; off = align_up(off + (size_t)topk_blocks(R) * (K > 0 ? K : 1) * sizeof(unsigned long long));
     L.wspread = off;   off = align_up(off + (size_t)R * M * sizeof(float));
     L.wcentre = off;   off = align_up(off + (size_t)R * M * sizeof(float));
@@ -198,7 +202,7 @@ struct guard_ctx {
     bool xs_busy[kIngestStreams] = {};   // stream k has work the caller's stream has not waited for
     long long xs_first[kIngestStreams] = {};   // first step (counted from creation / reset) of the oldest such block
     int xs_next = 0;
-    int scratch_sel = 0;                // which split scratch the next launch uses
+    int scratch_sel = 0;                // which split scratch and rows of per-step statistics the next launch uses
     cudaStream_t tail = nullptr;
     cudaStream_t aux = nullptr;       // deferred evaluations: the top-k selection, beside the fleet baseline and clear of the window medians' stream
     cudaEvent_t ev_x = nullptr, ev_w = nullptr;
@@ -303,8 +307,8 @@ struct guard_ctx {
     float *wmed(int q) const { return (float *)(ws + L.wmed + (size_t)q * L.wmed_stride); }
     int eval_q() const { return (int)(evals & 1); }        // buffers of the evaluation about to be made
     int prev_q() const { return (int)((evals + 1) & 1); }  // ... and of the one made last
-    float *step_med() const { return (float *)(ws + L.stepstat); }
-    float *step_mad() const { return step_med() + (size_t)C * M; }
+    float *step_med(int k) const { return (float *)(ws + L.stepstat + (size_t)k * L.stepstat_stride); }   // of ingest stream k (0: also the caller's)
+    float *step_mad(int k) const { return step_med(k) + (size_t)C * M; }
     unsigned long long *topk_cand() const { return (unsigned long long *)(ws + L.topk_cand); }
     void *mask() const { return ws + L.mask; }
     float *ring() const { return (float *)(ws + L.ring); }
@@ -315,7 +319,7 @@ struct guard_ctx {
     // scratch of the bracketed path: such rows take the direct selection.
     // site: 0 the ingested step, 1 the fleet baseline, -1 neither.  A site keeps the brackets of its single rows.
     bool row_hints = true;   // guard_set_row_hints
-    int stat_rows = 0;       // rows of the per-step statistics written since creation / reset
+    int stat_rows[kIngestStreams] = {};   // rows of each set of per-step statistics written since creation / reset
     // stamp of the split path's column records: changed whenever the scratch stops describing this context's data
     uint32_t split_epoch = 1;
     SplitState split_state[kIngestStreams];
@@ -493,8 +497,6 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
     a.capacity = c->C;
     a.R = c->R;
     a.M = c->M;
-    a.med = c->step_med();
-    a.mad = c->step_mad();
     a.med_user = d_step_med;
     a.mad_user = d_step_mad;
     a.cut = nullptr;
@@ -503,13 +505,15 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
     a.check_finite = 1;
     a.status = c->status();
     a.copy_from = copied ? d_block : nullptr;
-    a.prev_rows = c->row_hints ? c->stat_rows : 0;
-    if (B > c->stat_rows) c->stat_rows = B;
     cudaError_t e;
     const bool piped = c->deferred && c->L.xr_split && a.mask_bytes == 1 && (long long)B * c->M > 64 && !d_step_med &&
                        !d_step_mad && c->ensure_xs();
+    const int k = piped ? c->xs_next : 0;
+    a.med = c->step_med(k);
+    a.mad = c->step_mad(k);
+    a.prev_rows = c->row_hints ? c->stat_rows[k] : 0;
+    if (B > c->stat_rows[k]) c->stat_rows[k] = B;
     if (piped) {
-        const int k = c->xs_next;
         c->xs_next = (k + 1) % kIngestStreams;
         e = cudaEventRecord(c->ev_data, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(c->xs[k], c->ev_data, 0);
@@ -1056,7 +1060,7 @@ int guard_reset(guard_ctx *c, void *stream) {
     if (e != cudaSuccess) return c->cuda_fail(e, "cudaMemsetAsync");
     c->seen = 0;
     c->evals = 0;
-    c->stat_rows = 0;
+    for (int k = 0; k < kIngestStreams; ++k) c->stat_rows[k] = 0;
     c->seen_at_eval = 0;
     c->inc_seen = -1;
     c->cnt_seen = -1;

@@ -55,7 +55,7 @@ struct CtShared {
     uint32_t all[kCtList];         // (clusters) the lists of all CTAs
     uint32_t v1[C], v2[C];
     uint32_t any_open[2];
-    float med[C], rhs[C];
+    float med[C], mad[C], rhs[C];
     uint32_t bad;
 };
 
@@ -364,12 +364,15 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     float xs = 0.0f, hmed = 0.0f, hmad = -1.0f;
     if (warp < C) {
         xs = __ldg(row + (size_t)(((2 * lane + 1) * (long long)R) >> 6) * M + warp);
-        // the result arrays still hold an earlier result of this row position, or of another one (only its own with a
-        // cluster: another row's leader may be writing there, and the CTAs of a cluster have to read the same)
+        // The result arrays still hold an earlier result of this row position, or of another one.  Only its own with a
+        // cluster, whose CTAs have to read the same: another row's leader may be writing there, its own row nobody writes
+        // (the launches that write one set of rows follow one another) before the cluster's first barrier has passed.
+        // One lane reads for its warp.
         if (NC == 1 ? a.prev_rows > 0 : s < a.prev_rows) {
             const size_t o = (size_t)min(s, a.prev_rows - 1) * M + m0 + warp;
-            hmed = a.med[o];
-            hmad = a.mad[o];
+            if (lane == 0) { hmed = a.med[o]; hmad = a.mad[o]; }
+            hmed = __shfl_sync(0xFFFFFFFFu, hmed, 0);
+            hmad = __shfl_sync(0xFFFFFFFFu, hmad, 0);
         }
     }
 #pragma unroll
@@ -430,6 +433,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
             } else if (what == 1) {
                 const float lo = __uint_as_float(v1 >> 1), md = sh.med[tid];
                 const float mad = even ? __fmul_rn(0.5f, __fadd_rn(lo, __uint_as_float(v2 >> 1))) : lo;
+                sh.mad[tid] = mad;
                 sh.rhs[tid] = __fmul_rn(p.thrp[m], scale_of(mad, md, p.floor_rel[m], p.floor_abs[m]));
                 if (speaks) {
                     a.med[o] = md;

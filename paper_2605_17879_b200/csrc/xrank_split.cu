@@ -778,7 +778,7 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(512, 2) xs
         __syncthreads();
         if (tid == 0 && (!wide || ct_rank() == 0u)) {                    // the result is the next block's estimate
             SpCol &col = sc.col[(size_t)lo * M + m];
-            sp_learn(col, a.med[(size_t)lo * M + m], a.mad[(size_t)lo * M + m], true, R);
+            sp_learn(col, sh.med[0], sh.mad[0], true, R);
             if (col.epoch != sc.epoch) col.resample = 0;
             col.epoch = sc.epoch;
             if (col.rest) col.rest -= 1;

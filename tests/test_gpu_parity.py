@@ -755,3 +755,34 @@ def test_one_pass_columns_recomputed(R, M, B, thr):
     X[:, :, 1] = np.round(X[:, :, 1] * np.float32(20.0)) / np.float32(20.0)
     X[B + 3] *= np.float32(1.5)
     run_both(X, B, max(1, B // 2), 8, dirs, [B], capacity=2 * B, thr=thr)
+
+
+@pytest.mark.parametrize("R,M,B", [
+    (8191, 8, 12),                 # eight values per thread of a cluster's CTA
+    (24000, 8, 10),                # sixteen
+])
+def test_one_pass_columns_recomputed_side_by_side(R, M, B):
+    """Deferred blocks with nothing between them: both internal streams recompute columns (a metric of a handful of values,
+    steps that jump) at the same step positions at the same time."""
+    from paper_2605_17879_b200 import guard
+    nblk = 8
+    X, dirs = _rand_fleet(nblk * B, R, M, seed=R + B)
+    X[:, :, 1] = np.round(X[:, :, 1] * np.float32(20.0)) / np.float32(20.0)
+    for j in range(1, nblk):       # other steps jump in every block, some of them at the positions of the block before
+        X[j * B + 2] *= np.float32(1.0 + 0.25 * (j % 3))
+        X[j * B + (3 + j) % B] *= np.float32(1.5)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, B, max(1, B // 2), dir=dirs, capacity=nblk * B, topk=8)
+    g.set_deferred(True)
+    bufs = [g.alloc_outputs() for _ in range(nblk)]
+    for j in range(nblk):
+        g.ingest(Xd[j * B:(j + 1) * B])
+        g.score(bufs[j])
+    g.join()
+    assert g.sync_status() == 0
+    assert g.fallback_steps() > nblk
+    g.close()
+    o = go.Oracle(R, M, B, max(1, B // 2), 8, dir=dirs)
+    for j in range(nblk):
+        o.ingest(X[j * B:(j + 1) * B])
+        compare_score(bufs[j], o.score(), "block %d" % j)

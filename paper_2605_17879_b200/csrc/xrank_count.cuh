@@ -26,8 +26,7 @@ constexpr int kCtMaxC = 8;         // metrics per CTA at most
 constexpr int kCtBins = 256;
 constexpr int kCtList = 64;        // keys of a bin that are ranked directly (two per lane)
 constexpr int kCtMaxIter = 64;     // a range shrinks at least to a 128th whenever its bin is too full
-constexpr uint32_t kCtTop = 0xFF800000u;    // no key of a number lies above; padding does
-constexpr uint32_t kCtNone = 0xFFFFFFFFu;
+constexpr uint32_t kCtNone = 0xFFFFFFFFu;  // the largest key: a NaN's, and what padding holds (in whatever range it falls, it comes last)
 constexpr int kCtAll = 0, kCtStatistics = 1, kCtCut = 2;   // what a CTA (cluster) computes: both, median and MAD, the extra order statistic
 // Single rows of 8 metrics, bracketed by the row before / not: one CTA of 1 024 threads per column takes 6.3 / 7.5 us at
 // 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
@@ -198,7 +197,7 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
             const uint32_t hi = lo + width, step = width >= 0x07FF0000u ? 0x7FFFFFFFu : 16u * width + 65536u;
             uint32_t nlo = lo, nhi = hi;
             if (below > k1) { nlo = lo > step ? lo - step : 0u; if (below > k2) nhi = lo; }
-            if (k2 >= below + total) { nhi = hi < kCtTop - step ? hi + step : kCtTop; if (k1 >= below + total) nlo = min(hi, kCtTop); }
+            if (k2 >= below + total) { nhi = hi < kCtNone - step ? hi + step : kCtNone; if (k1 >= below + total) nlo = hi; }
             sh.lo[c] = nlo;
             sh.width[c] = nhi - nlo;
             sh.f0[c] = kCtNone;
@@ -333,7 +332,7 @@ __device__ __forceinline__ int ct_select(const uint32_t (&key)[V], const uint32_
             searching = ct_settle<C, NC>(sh, warp, k2 != k1);
             if (lane == 0) {
                 if (searching) sh.any_open[it & 1] = 1u;
-                else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fw[warp] = 0u; }   // (no key at all)
+                else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fw[warp] = 0u; }   // (no key of a number, a computed NaN or padding)
             }
         }
         __syncthreads();
@@ -398,7 +397,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
         const uint32_t sorted = ct_warp_sort(x, lane);
         const int pos = (int)(((long long)k * 32) / R);
         const uint32_t lo = __shfl_sync(0xFFFFFFFFu, sorted, max(pos - 8, 0)), hi = __shfl_sync(0xFFFFFFFFu, sorted, min(pos + 9, 31));
-        range(min(lo, kCtTop), min(hi, kCtTop));
+        range(lo, hi);
     };
     // a previous result brackets the new one to four standard errors of the difference of two sample medians /
     // MADs of normal data (2.6 and 1.65 MAD / sqrt(R)): some 5.6 sqrt(R) keys
@@ -440,7 +439,6 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                     a.mad[o] = mad;
                     if (a.med_user) a.med_user[o] = md;
                     if (a.mad_user) a.mad_user[o] = mad;
-                    if (tid == 0 && sh.bad) atomicOr(a.status, kStatInternal);
                     if (NC > 1 && a.hint) {
                         RowHints *h = reinterpret_cast<RowHints *>(a.hint);
                         if (m == 0) atomicAdd(&h->rows, 1u);
@@ -452,7 +450,10 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                 if (a.cut_user) a.cut_user[o] = key2f(v1);
             }
         }
-        if (what == 1 || (part == kCtCut && what == C + 1)) break;
+        if (what == 1 || (part == kCtCut && what == C + 1)) {
+            if (tid == 0 && speaks && sh.bad && a.status) atomicOr(a.status, kStatInternal);
+            break;
+        }
         __syncthreads();
         // the metrics' extra ranks first (they need the values), then the deviations
         what = !a.cut || part == kCtStatistics ? 1 : (what == 0 ? 2 : (what - 1 < C ? what + 1 : 1));

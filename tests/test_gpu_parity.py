@@ -786,3 +786,39 @@ def test_one_pass_columns_recomputed_side_by_side(R, M, B):
     for j in range(nblk):
         o.ingest(X[j * B:(j + 1) * B])
         compare_score(bufs[j], o.score(), "block %d" % j)
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (37, 8, 5, 6),                 # the cut by CTAs of its own
+    (2048, 8, 33, 5),              # by clusters of its own
+    (600, 8, 20, 20),              # the cut after the median, in the same clusters
+])
+def test_sweep_with_unmeasured_metrics(nodes, gpn, N, M):
+    """Metrics that were not measured on all, most or some of the GPUs (NaN): the status says non-finite and nothing else,
+    with or without a status word, and the other metrics' results are what they are without them."""
+    from paper_2605_17879_b200 import guard
+    rng = np.random.default_rng(N + M)
+    G = nodes * gpn
+    S = (1.0 + 0.02 * rng.standard_normal((G, N, M), dtype=np.float32)).astype(np.float32)
+    S[8::50, :, 0] *= np.float32(0.7)
+    dirs = [-1] + [1] * (M - 1)
+    ref = go.sweep(S, nodes, gpn, dir=dirs)
+    X = S.copy()
+    X[:, :, 1] = np.nan
+    X[rng.random(G) < 0.6, :, 2] = np.nan
+    X[rng.random(G) < 0.2, :, 3] = np.nan
+    clean = [m for m in range(M) if m not in (1, 2, 3)]
+    Xd = torch.from_numpy(X).cuda()
+    out = guard.sweep_qualify(Xd, nodes, gpn, dir=dirs)
+    bare = {k: torch.zeros_like(v) for k, v in out.items() if k != "status"}
+    guard.sweep_qualify(Xd, nodes, gpn, dir=dirs, out=bare)
+    assert int(out["status"].cpu()[0]) == 1
+    for o in (out, bare):
+        assert_bit_equal(to_np(o["gpu_med"])[:, clean], ref["gpu_med"][:, clean], "gpu_med")
+        for key in ("fleet_med", "fleet_mad", "fleet_cut"):
+            assert_bit_equal(to_np(o[key])[clean], ref[key][clean], key)
+        assert_bit_equal(to_np(o["fail_mask"]) & ~np.uint32(14), ref["fail_mask"] & ~np.uint32(14), "fail_mask")
+        for key in ("fleet_med", "fleet_mad", "fleet_cut"):   # NaN orders above all numbers
+            assert np.isnan(to_np(o[key])[1]), key
+        assert np.isnan(to_np(o["fleet_med"])[2]) and np.isnan(to_np(o["fleet_cut"])[3])
+        assert np.isfinite(to_np(o["fleet_med"])[3])

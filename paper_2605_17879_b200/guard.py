@@ -196,6 +196,10 @@ def workspace_bytes(ranks: int, metrics: int, W: int, capacity: int, topk: int) 
     return int(lib().guard_workspace_bytes(ranks, metrics, W, capacity, topk))
 
 
+_OUT_NAMES = ("wmed", "fleet_med", "fleet_mad", "scores", "counts", "mask", "flags", "tier", "topk_idx", "topk_score")
+_NODE_NAMES = ("node_flag", "node_tier", "node_stall")
+
+
 class Guard:
     """Online scorer: `ingest` blocks of steps, `score` the current window."""
 
@@ -209,6 +213,8 @@ class Guard:
         self.device = torch.device(device)
         self._devidx = self.device.index if self.device.index is not None else torch.cuda.current_device()
         self._views = {}        # ring views handed out by ring_reserve, by (byte offset, steps)
+        self._deferred = False
+        self._held = ()         # outputs of the pending deferred evaluation: written on streams the allocator does not know
         self._h = C.c_void_p()
         self._params = _Params(metrics, dir, thr, floor_rel, floor_abs, primary, min_signals, n_consec,
                                ranks_per_node, tier_moderate, tier_severe)
@@ -230,6 +236,7 @@ class Guard:
             _lib.guard_destroy(self._h)
             self._h = C.c_void_p()
             self._hv = 0
+            self._held = ()
 
     def __del__(self):
         try:
@@ -309,10 +316,12 @@ class Guard:
         """Deferred evaluations: score() does not make the current stream wait for its results; they
         are complete after the next score(), join(), sync_status() or reset()."""
         self._check(lib().guard_set_deferred(self._h, 1 if on else 0))
+        self._deferred = bool(on)
 
     def join(self) -> None:
         """Makes the current stream wait for the pending deferred evaluation, if any."""
         self._check(_native().join(self._hv, self._devidx))
+        self._held = ()
 
     def profile_enable(self, on=True) -> None:
         """0 / False: off; 1 / True: time the cross-rank sweep of every ingest; 2: the window kernel of every evaluation."""
@@ -360,8 +369,17 @@ class Guard:
         """One evaluation; `out` maps output names to tensors (missing / None entries are skipped)."""
         if out is None:
             out = self.alloc_outputs()
-        self._check(_native().score(self._hv, self._devidx, self.R, self.M, self.K, out))
+        rc = _native().score(self._hv, self._devidx, self.R, self.M, self.K, out)
+        if rc != GUARD_OK:
+            self._held += self._tensors(out)
+            self._check(rc)
+        # (the outputs held so far are complete in the current stream's order from here on)
+        self._held = self._tensors(out) if self._deferred else ()
         return out
+
+    @staticmethod
+    def _tensors(out) -> tuple:
+        return tuple(out.values()) if isinstance(out, dict) else tuple(map(out.get, _OUT_NAMES))
 
     def node_verdict(self, out: Optional[Dict[str, Optional[torch.Tensor]]] = None) -> Dict[str, Optional[torch.Tensor]]:
         """Node-level fold of the evaluation just made (call right after score())."""
@@ -370,6 +388,8 @@ class Guard:
             out = {"node_flag": torch.empty(N, dtype=torch.uint8, device=self.device),
                    "node_tier": torch.empty(N, dtype=torch.uint8, device=self.device),
                    "node_stall": torch.empty(N, dtype=torch.uint16, device=self.device)}
+        if self._held:
+            self._held += tuple(map(out.get, _NODE_NAMES))
         self._check(_native().node_verdict(self._hv, self._devidx, N, out))
         return out
 
@@ -396,12 +416,14 @@ class Guard:
         """Synchronises the current stream; raises GuardError on a sticky device error."""
         with self._dev():
             rc = lib().guard_sync_status(self._h, _stream())
+        self._held = ()
         self._check(rc)
         return rc
 
     def reset(self) -> None:
         with self._dev():
             self._check(lib().guard_reset(self._h, _stream()))
+        self._held = ()
 
 
 def sweep_qualify(S: torch.Tensor, nodes: int, gpus_per_node: int, *, dir: Sequence[int], thr=3.5, floor_rel=1e-4,

@@ -144,3 +144,60 @@ def test_triage_counter_matches_the_oracle_rule(glib):
     assert glib.lib().guard_triage_create(C.byref(h), 4, 0, 10) == -1
     assert glib.lib().guard_triage_record(None, 0, 0, None) == -1
     glib.lib().guard_triage_destroy(None)
+
+
+def test_outputs_of_pending_evaluations_are_held(glib, monkeypatch):
+    """A deferred evaluation writes its outputs on streams the caching allocator does not know: the tensors must live on,
+    also where the caller drops them, until a call has put those writes in order."""
+    import weakref
+
+    import torch
+
+    class Calls:
+        rc = 0
+
+        def score(self, *a):
+            return self.rc
+
+        def node_verdict(self, *a):
+            return self.rc
+
+        def join(self, *a):
+            return 0
+
+    class Lib:
+        def __getattr__(self, name):
+            return (lambda *a: b"") if name == "guard_last_error" else (lambda *a: 0)
+
+    calls = Calls()
+    monkeypatch.setattr(glib, "_native", lambda: calls)
+    monkeypatch.setattr(glib, "lib", lambda: Lib())
+    monkeypatch.setattr(glib, "_stream", lambda: 0)
+    g = glib.Guard.__new__(glib.Guard)
+    g.R, g.M, g.K, g.ranks_per_node, g.device, g._devidx = 8, 2, 1, 4, torch.device("cpu"), 0
+    g._h, g._hv, g._deferred, g._held = 0, 0, False, ()
+    monkeypatch.setattr(glib.Guard, "_dev", lambda self: glib._HERE_CTX)
+
+    def outputs(call):
+        return [weakref.ref(t) for t in call().values()]
+    alive = lambda refs: [r() is not None for r in refs]
+    assert not any(alive(outputs(g.score)))            # complete when the call returns, in stream order
+    g.set_deferred(True)
+    first = outputs(g.score)
+    nodes = outputs(g.node_verdict)
+    assert all(alive(first)) and all(alive(nodes))
+    second = outputs(g.score)
+    assert all(alive(second)) and not any(alive(first + nodes))
+    calls.rc = -6                                      # nothing of it may have been waited for
+    with pytest.raises(glib.GuardError):
+        g.score()
+    assert all(alive(second))
+    calls.rc = 0
+    for release in (g.join, g.sync_status, g.reset, g.close):
+        refs = outputs(g.score)
+        assert all(alive(refs))
+        if release == g.close:
+            monkeypatch.setattr(glib, "_lib", Lib())
+            g._h = 1
+        release()
+        assert not any(alive(refs)), release

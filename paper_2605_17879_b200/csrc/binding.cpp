@@ -38,9 +38,9 @@ bool device_ptr(PyObject *obj, c10::ScalarType type, int64_t numel, void **out) 
     return true;
 }
 
-// out[name], or None (borrowed for a dict, else kept alive by the caller through `hold`).
+// out[name], or None (borrowed for a plain dict, else kept alive by the caller through `hold`).
 PyObject *lookup(PyObject *out, PyObject *name, PyObject **hold) {
-    if (PyDict_Check(out)) {
+    if (PyDict_CheckExact(out)) {
         PyObject *v = PyDict_GetItemWithError(out, name);
         return v ? v : (PyErr_Occurred() ? nullptr : Py_None);
     }
@@ -198,42 +198,36 @@ PyObject *py_join(PyObject *, PyObject *const *args, Py_ssize_t n) {
     }
 }
 
-// A per-metric parameter: a sequence of M numbers, or one number for all of them.
+// A per-metric parameter.  dir (whole): any iterable of M values that int() takes.  The others: anything with a length, of M
+// numbers, or one number for all metrics.
 template <typename T>
 bool per_metric(PyObject *obj, int M, bool whole, T *out) {
     auto one = [&](PyObject *v, T *dst) {
         if (whole) {
             PyObject *i = PyNumber_Long(v);
             if (!i) return false;
-            long long x;
-            const bool ok = to_ll(i, &x);
+            *dst = (T)PyLong_AsUnsignedLongLongMask(i);
             Py_DECREF(i);
-            *dst = (T)x;
-            return ok;
+            return !PyErr_Occurred();
         }
         const double x = PyFloat_AsDouble(v);
         if (x == -1.0 && PyErr_Occurred()) return false;
         *dst = (T)x;
         return true;
     };
-    const Py_ssize_t len = PyFloat_Check(obj) || PyLong_Check(obj) ? -1 : PyObject_Size(obj);
-    if (len < 0) {
-        PyErr_Clear();
+    if (!whole && (PyFloat_Check(obj) || PyLong_Check(obj) || !PyObject_HasAttrString(obj, "__len__"))) {
         if (!one(obj, &out[0])) return false;
         for (int m = 1; m < M; ++m) out[m] = out[0];
         return true;
     }
-    if (len != M) {
-        PyErr_Format(PyExc_ValueError, "expected %d per-metric values, got %zd", M, len);
-        return false;
-    }
-    for (int m = 0; m < M; ++m) {
-        PyObject *v = PySequence_GetItem(obj, m);
-        const bool ok = v && one(v, &out[m]);
-        Py_XDECREF(v);
-        if (!ok) return false;
-    }
-    return true;
+    PyObject *seq = PySequence_Fast(obj, "expected an iterable of per-metric values");
+    if (!seq) return false;
+    const Py_ssize_t len = PySequence_Fast_GET_SIZE(seq);
+    bool ok = len == M;
+    if (!ok) PyErr_Format(PyExc_ValueError, "expected %d per-metric values, got %zd", M, len);
+    for (int m = 0; ok && m < M; ++m) ok = one(PySequence_Fast_GET_ITEM(seq, m), &out[m]);
+    Py_DECREF(seq);
+    return ok;
 }
 
 Output g_sweep_out[8] = {{"gpu_med", c10::kFloat, nullptr},   {"fleet_med", c10::kFloat, nullptr}, {"fleet_mad", c10::kFloat, nullptr},

@@ -201,3 +201,38 @@ def test_outputs_of_pending_evaluations_are_held(glib, monkeypatch):
             g._h = 1
         release()
         assert not any(alive(refs)), release
+
+
+def test_per_metric_arguments_of_the_native_sweep(glib):
+    """The native call takes and refuses the per-metric arguments that the other entry points' marshalling does: any
+    iterable of directions, anything with a length or one number for the rest."""
+    import collections
+
+    import torch
+    M = 3
+    S, ws = torch.zeros(8, 2, M), torch.empty(1 << 16, dtype=torch.uint8)
+
+    def native(dir, thr, floor_rel, floor_abs):
+        try:
+            glib._native().sweep_qualify(0, S, 1, 8, dir, thr, floor_rel, floor_abs, 50_000, ws, {})
+        except ValueError as e:                        # the arguments are checked before the (CPU) tensors
+            if "contiguous CUDA" not in str(e):
+                raise
+
+    def outcome(call, kw):
+        args = dict(dict(dir=[1, 1, 1], thr=3.5, floor_rel=1e-4, floor_abs=0.0), **{k: v() for k, v in kw.items()})
+        try:
+            call(**args)
+            return "taken"
+        except Exception as e:
+            return type(e).__name__
+
+    values = [lambda v=v: v for v in (
+        1, 1.0, True, [1, 1, 1], (1, -1, 1), [1, 1], range(3), {1: 0, 2: 0, 3: 0}, {1, 2, 3}, np.ones(3), np.ones(3, np.int8),
+        np.float32(2), np.array(2.0), torch.ones(3), torch.tensor(1.0), torch.ones(3, dtype=torch.int8), "123", "1", None,
+        ["1", "1", "1"], [None] * 3, [1.7, 1, 1], [10 ** 30] * 3, np.ones((3, 2)), collections.deque([1, 1, 1]), object())]
+    values += [lambda: (x for x in (1, 1, 1)), lambda: {1: 1, 2: 2, 3: 3}.values(), lambda: map(int, "111")]
+    for make in values:
+        for name in ("dir", "thr", "floor_rel", "floor_abs"):
+            want = outcome(lambda **kw: glib._Params(M, kw["dir"], kw["thr"], kw["floor_rel"], kw["floor_abs"]), {name: make})
+            assert outcome(native, {name: make}) == want, (name, make())

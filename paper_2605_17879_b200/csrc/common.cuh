@@ -85,7 +85,9 @@ inline cudaError_t launch_after_smem(void (*kernel)(P...), dim3 grid, dim3 block
     c.stream = st;
     c.attrs = &early;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, args...);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // the caller gets it; the thread's next CUDA call must not find it again
+    return e;
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const A &...args) {

@@ -339,7 +339,7 @@ struct guard_ctx {
         if (S == 1 && site >= 0 && L.xr_gridp && row_hints) a.hint = hint_state(site);
         // everything the streaming paths do not take, or not for so few columns
         if (xrank_count_supported(R) && ((!L.xr_split && !L.xr_cluster) || a.mask_bytes != 1 || (long long)S * M <= 64)) {
-            launches += 1;
+            launches += xrank_count_launches(S);
             return launch_xrank_count(a, p, S, st);
         }
         if (L.xr_split && a.mask_bytes == 1) {

@@ -86,6 +86,7 @@ cudaError_t launch_xrank_bracketed(const XrankArgs &a, const MetricParams &p, co
 // Rows held in registers and searched by counting at pivots: any values, any number of metrics, up to 32 768 ranks.
 constexpr int kCountMaxRanks = 32768;
 bool xrank_count_supported(int R);
+int xrank_count_launches(int S);
 bool xrank_count_copies(int R, int M, int S);   // honours copy_from
 cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st);
 

@@ -53,6 +53,8 @@ cudaError_t launch_c(const XrankArgs &a, const MetricParams &p, int S, int T, cu
     return launch_after(xrank_count_kernel<32, C>, grid, T, st, a, p);
 }
 
+constexpr int kGridRows = 65535;   // the largest grid in y: rows per launch
+
 // Metrics and threads per CTA.
 void plan(const int R, const int M, const int S, int &C, int &T) {
     // Two metrics per CTA where that leaves at least a CTA per SM (their loads share cache lines; more metrics make
@@ -70,6 +72,8 @@ void plan(const int R, const int M, const int S, int &C, int &T) {
 }
 
 }  // namespace
+
+int xrank_count_launches(int S) { return (S + kGridRows - 1) / kGridRows; }
 
 bool xrank_count_supported(int R) { return R >= 1 && R <= kCountMaxRanks; }
 
@@ -94,7 +98,21 @@ cudaError_t launch_xrank_count(const XrankArgs &a, const MetricParams &p, int S,
     int C, T;
     plan(a.R, a.M, S, C, T);
     if (a.cut && S == 1 && C == 1 && a.R <= 4 * T) return launch_after(xrank_count_apart_kernel, 2 * a.M, T, st, a, p);
-    return C == 2 ? launch_c<2>(a, p, S, T, st) : launch_c<1>(a, p, S, T, st);
+    XrankArgs g = a;
+    for (int s0 = 0; s0 < S; s0 += kGridRows) {
+        const int n = S - s0 < kGridRows ? S - s0 : kGridRows;
+        const size_t o = (size_t)s0 * a.M;
+        g.first_slot = (int)(((long long)a.first_slot + s0) % a.capacity);
+        g.copy_from = a.copy_from ? a.copy_from + (size_t)s0 * a.row_stride : nullptr;
+        g.med = a.med + o;
+        g.mad = a.mad + o;
+        g.med_user = a.med_user ? a.med_user + o : nullptr;
+        g.mad_user = a.mad_user ? a.mad_user + o : nullptr;
+        g.prev_rows = a.prev_rows > s0 ? a.prev_rows - s0 : 0;
+        const cudaError_t e = C == 2 ? launch_c<2>(g, p, n, T, st) : launch_c<1>(g, p, n, T, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace guard

@@ -822,3 +822,9 @@ def test_sweep_with_unmeasured_metrics(nodes, gpn, N, M):
             assert np.isnan(to_np(o[key])[1]), key
         assert np.isnan(to_np(o["fleet_med"])[2]) and np.isnan(to_np(o["fleet_cut"])[3])
         assert np.isfinite(to_np(o["fleet_med"])[3])
+
+
+@pytest.mark.parametrize("R,M,B,in_place", [(2, 3, 66000, False), (3, 2, 65536, True), (40, 1, 65535 * 2 + 1, False)])
+def test_blocks_of_more_steps_than_a_grid_has_rows(R, M, B, in_place):
+    X, dirs = _rand_fleet(B + 40, R, M, seed=R + M)
+    run_both(X, 30, 10, 1, dirs, [B, 40], capacity=B + 40, in_place=in_place)

@@ -153,6 +153,7 @@ struct guard_ctx {
     long long evals;     // evaluations since creation / reset
     long long seen_at_eval = 0;   // steps seen at the last evaluation
     int ranks_per_node = 8;
+    int device = 0;               // current when the context was created
     long long wait_limit = 0;     // test hook: limit of the warp window path's first wait (0: default)
     // Sliding-window state (window.cu): current for the window of inc_n steps ending at step count inc_seen
     // (-1: none).  hints_ready: a whole-window kernel has seeded the per-series search intervals.
@@ -334,6 +335,12 @@ struct guard_ctx {
     // 1 024 x 8 x 100 30.0 / 25.8, 1 024 x 8 x 200 39.9 / 38.0, single steps of 512 x 8 29.2 / 27.0.  Deferred evaluations
     // always fork: they hide the host's calls behind one another (single steps of 64 x 4 17.7 us, 23.4 in line).
     bool inline_eval() const { return !deferred && (long long)W * R * M <= kInlineValues; }
+    // Whether a kernel on the context's device can read memory at p (and no copy in front is needed).
+    bool readable(const void *p) const {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+        return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
+    }
     RowHints *hint_state(int site) const { return (RowHints *)(ws + L.xr_grid + (size_t)site * align_up(sizeof(RowHints))); }
     cudaError_t xrank(XrankArgs a, int S, cudaStream_t st, bool own_scratch = true, int site = -1) {
         if (S == 1 && site >= 0 && L.xr_gridp && row_hints) a.hint = hint_state(site);
@@ -442,7 +449,8 @@ int guard_create(guard_ctx **out, int ranks, int metrics, int W, int k, const gu
     c->ranks_per_node = th->ranks_per_node;
     c->new_epoch();
     // state: status word, ticket, fleet statistics, consecutive counters
-    cudaError_t e = cudaMemsetAsync(c->ws, 0, L.wmed, (cudaStream_t)stream);
+    cudaError_t e = cudaGetDevice(&c->device);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws, 0, L.wmed, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         set_error(g_error, "cudaMemsetAsync: %s", cudaGetErrorString(e));
         delete c;
@@ -476,8 +484,10 @@ int guard_ingest(guard_ctx *c, const float *d_block, int B, float *d_step_med, f
         if (e == cudaSuccess) e = c->join_xs(st);
         if (e != cudaSuccess) return c->cuda_fail(e, "join of deferred work");
     }
-    // a small block that the counting kernels take is put into the ring by them
-    const bool copied = !in_place && c->inline_eval() && slot + B <= c->C && xrank_count_copies(c->R, c->M, B) && !c->L.xr_split && !c->L.xr_cluster;
+    // A small block that the counting kernels take is put into the ring by them, if they can read it: a copy also takes
+    // another device's memory, or the host's.
+    const bool copied = !in_place && c->inline_eval() && slot + B <= c->C && xrank_count_copies(c->R, c->M, B) && !c->L.xr_split &&
+                        !c->L.xr_cluster && c->readable(d_block);
     if (!in_place && !copied) {
         const int first = (slot + B <= c->C) ? B : (c->C - slot);
         cudaError_t e = cudaMemcpyAsync(c->ring() + (size_t)slot * row, d_block, (size_t)first * row * sizeof(float),

@@ -828,3 +828,57 @@ def test_sweep_with_unmeasured_metrics(nodes, gpn, N, M):
 def test_blocks_of_more_steps_than_a_grid_has_rows(R, M, B, in_place):
     X, dirs = _rand_fleet(B + 40, R, M, seed=R + M)
     run_both(X, 30, 10, 1, dirs, [B, 40], capacity=B + 40, in_place=in_place)
+
+
+def test_small_block_the_kernels_do_not_read():
+    """A small block in (pinned) host memory, handed to the C call: copied into the ring by the copy engine, as larger ones
+    are; the counting kernels read only what is on their device."""
+    import ctypes as C
+    from paper_2605_17879_b200 import guard
+    R, M, W = 64, 4, 20
+    X, dirs = _rand_fleet(2 * W, R, M, seed=4)
+    g = guard.Guard(R, M, W, 10, dir=dirs, capacity=2 * W, topk=8)
+    o = go.Oracle(R, M, W, 10, 8, dir=dirs)
+    host = torch.from_numpy(X).pin_memory()
+    for t in (0, W):
+        rc = guard.lib().guard_ingest(g._h, host[t:t + W].data_ptr(), W, None, None, guard._stream())
+        assert rc == 0, guard.lib().guard_last_error(g._h)
+        out = g.score()
+        assert g.sync_status() == 0
+        o.ingest(X[t:t + W])
+        compare_score(out, o.score(), "t=%d" % t)
+    g.close()
+
+
+@pytest.mark.parametrize("R,M,W,B", [(64, 4, 50, 5), (3000, 8, 200, 20), (9000, 8, 50, 20), (20000, 8, 100, 1)])
+def test_calls_under_stream_capture(R, M, W, B):
+    """An ingest and an evaluation captured into a graph and launched give what the calls give."""
+    from paper_2605_17879_b200 import guard
+    X, dirs = _rand_fleet(W + 2 * B, R, M, seed=R + B)
+    Xd = torch.from_numpy(X).cuda()
+    got = []
+    for capture in (False, True):
+        g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 4 * B, topk=8)
+        out = g.alloc_outputs()
+        g.ingest(Xd[:W])
+        g.score(out)
+        g.ingest(Xd[W:W + B])
+        g.score(out)
+        block = Xd[W + B:].clone()
+        torch.cuda.synchronize()
+        if capture:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                g.ingest(block)
+                g.score(out)
+            graph.replay()
+        else:
+            g.ingest(block)
+            g.score(out)
+        assert g.sync_status() == 0
+        got.append({k: to_np(v) for k, v in out.items()})
+        if capture:
+            del graph
+        g.close()
+    for key in got[0]:
+        assert_bit_equal(got[1][key], got[0][key], key)

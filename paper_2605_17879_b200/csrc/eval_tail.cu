@@ -4,8 +4,10 @@
 // The top-k list: the ranks' keys are held in registers, one cluster (or CTA) for the whole fleet.
 //   1. a threshold with at least K keys at or above it: the one the previous evaluation left, where evaluations follow
 //      closely, else the K-th largest of the maxima of some 2 K disjoint groups of ranks (K groups have a member at
-//      or above it; random data have about 1.4 K keys there);
+//      or above it; random data have about 1.4 K keys there), or (lists too long for that) the exact K-th largest key;
 //   2. the entries at or above it meet in the first CTA's shared memory, which orders them.
+// Where evaluations follow closely, what is wanted is not K but the number of entries that the next evaluation's
+// threshold should admit (top_want).
 // A threshold that turns out too high (fewer than K) or too low (more than the list holds: ties) is replaced, in the
 // second case by the exact K-th largest key, and ranks among the keys equal to it are picked by their number.
 // Bound by latency: two cluster barriers and an ordering of some hundred entries, 7 us beside the baseline's 10 (the
@@ -19,12 +21,13 @@ namespace {
 
 constexpr int kTopGroups = 512;    // groups at most
 constexpr int kTopCap = 1024;      // gathered entries at most (K <= 1024)
+constexpr int kTopSlack = 8;       // entries above K that a threshold has to admit at least
 
 struct TopShared {
     unsigned long long list[kTopCap];                // (first CTA)
     __align__(16) uint32_t gmax[kTopGroups];         // this CTA's groups' maxima
     __align__(16) uint32_t all[kTopGroups];          // every group's
-    uint32_t n[4];                                   // (first CTA) gathered entries, by attempt
+    uint32_t n[8];                                   // (first CTA) gathered entries, by attempt
     uint32_t tau;
 };
 
@@ -52,6 +55,19 @@ __device__ __forceinline__ void top_sort(unsigned long long *list, const int n2)
     __syncthreads();
 }
 
+// Entries that the threshold left for the next evaluation should admit, or K if it would miss too often: three times K for
+// short lists; for long ones most of what the network that orders them has room for, but of the largest half, because
+// more than it holds are a miss (single steps of 1 024 ranks x 4: K = 500 29 us with some 509 entries, 34 with 762;
+// K = 700 38 us without a threshold that serves, 34 with 862).
+__device__ __forceinline__ int top_want(const int K) {
+    if (K <= kTopCap / 8) return 3 * K;
+    int n2 = kTopCap / 4;
+    while (n2 < kTopCap && n2 < K + kTopSlack) n2 <<= 1;
+    const int room = n2 - K;
+    if (n2 < kTopCap) return n2 - room / 4;
+    return room >= 2 * kTopSlack ? K + room / 2 : K;
+}
+
 // R <= V * NC * blockDim.x; all threads of the cluster call this.
 template <int V, int NC>
 __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p, uint32_t *status, TopShared &ts, CtShared<1> &sh) {
@@ -61,7 +77,9 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
     const uint32_t list0 = NC == 1 ? (uint32_t)__cvta_generic_to_shared(ts.list) : ct_map(ts.list, 0u);
     const uint32_t n0 = NC == 1 ? (uint32_t)__cvta_generic_to_shared(ts.n) : ct_map(ts.n, 0u);
     // one launch writes the hint's state, in its last step: every CTA reads the same here
-    const bool hv = a.hint && a.hint->valid;
+    const int want = a.hint ? top_want(K) : K;
+    const bool keeps = want > K;   // (this evaluation's threshold serves the next)
+    const bool hv = keeps && a.hint->valid;
     uint32_t tau = hv ? a.hint->tau : 0u;
     uint32_t key[V];               // larger is slower; 0 where there is no rank
     uint32_t own = 0u;
@@ -75,7 +93,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
         }
         own = max(own, key[i]);
     }
-    if (tid < 4) ts.n[tid] = 0u;
+    if (tid < 8) ts.n[tid] = 0u;
     if (tid == 0) ts.tau = 0u;
     // Appends the entries at or above t (ranks up to `last` only) to the list; returns how many there are then.
     auto gather = [&](const uint32_t t, const uint32_t only, const uint32_t last, const int attempt) -> uint32_t {
@@ -106,19 +124,20 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
     // (a second list would overwrite the first: its readers, the first CTA's last step, come after all of them)
     uint32_t n = 0;
     bool done = false, hit = false;
-    const int want = a.hint ? min(3 * K, kTopCap / 2) : K;   // with a hint state: what the threshold left behind should admit
     if (hv) {
         ct_sync<NC>();
         n = gather(tau, kCtNone, kCtNone, 0);
         hit = done = n >= (uint32_t)K && n <= (uint32_t)kTopCap;
     }
     if (!done) {
-        // groups of `lanes` neighbouring lanes (all of their values): at least 128 of them and 4/3 of the wanted number
+        // groups of `lanes` neighbouring lanes (all of their values): at least 128 of them and 4/3 of the wanted number, or of
+        // K where there cannot be so many
         const int threads = NC * T;
+        const int target = 3 * min(threads, kTopGroups) >= 4 * want ? want : K;
         int lanes = 32;
-        while (lanes > 1 && (threads / lanes < 128 || 3 * (threads / lanes) < 4 * want)) lanes >>= 1;
+        while (lanes > 1 && (threads / lanes < 128 || 3 * (threads / lanes) < 4 * target)) lanes >>= 1;
         const int G = threads / lanes, per = G / NC;
-        const bool all = R <= 128, grouped = !all && G <= kTopGroups && 3 * G >= 4 * want;
+        const bool all = R <= 128, grouped = !all && G <= kTopGroups && 3 * G >= 4 * target;
         if (grouped) {
             uint32_t m = own;
             for (int d = 1; d < lanes; d <<= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
@@ -129,7 +148,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
         if (grouped) {
             for (int g = tid; g < G; g += T) ts.all[g] = NC == 1 ? ts.gmax[g] : ct_ld(ct_map(&ts.gmax[g % per], (uint32_t)(g / per)));
             __syncthreads();
-            // the `want`-th largest: the one that `want` - 1 others come before (equal ones in the order of their groups)
+            // the `target`-th largest: the one that `target` - 1 others come before (equal ones in the order of their groups)
             for (int g = tid; g < G; g += T) {
                 const uint32_t x = ts.all[g], x1 = x == 0u ? 0u : x - 1u;
                 const uint4 *q = reinterpret_cast<const uint4 *>(ts.all);
@@ -141,7 +160,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
                     before += (int)(o.x > c) + (int)(o.y > c) + (int)(o.z > c) + (int)(o.w > c);
                 }
                 for (int j = g & ~3; j < g; ++j) before += ts.all[j] == x;
-                if (before == want - 1) ts.tau = x;
+                if (before == target - 1) ts.tau = x;
             }
             __syncthreads();
             tau = ts.tau;
@@ -152,22 +171,27 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
         }
     }
     if (!done) {
-        // the exact K-th largest (ranks that do not exist lie below all keys)
+        // the exact largest of that place (ranks that do not exist lie below all keys); where ties make too many of it, the K-th
         for (int i = tid; i < kCtBins; i += T) sh.hist[0][i] = 0u;
-        if (tid == 0) { sh.below[0] = 0u; sh.lo[0] = 0u; sh.width[0] = kCtNone; sh.bad = 0u; }
-        const uint32_t at = (uint32_t)(V * NC * T - K);
-        ct_select<V, 1, NC>(key, at, at, sh);
-        const uint32_t kth = sh.v1[0];
-        n = gather(kth, kCtNone, kCtNone, 2);
+        if (tid == 0) { sh.below[0] = 0u; sh.bad = 0u; }
+        uint32_t kth;
+        for (int target = min(want, R);; target = K) {
+            if (tid == 0) { sh.lo[0] = 0u; sh.width[0] = kCtNone; }
+            const uint32_t at = (uint32_t)(V * NC * T - target);
+            ct_select<V, 1, NC>(key, at, at, sh);
+            kth = tau = sh.v1[0];
+            n = gather(kth, kCtNone, kCtNone, target == K ? 3 : 2);
+            if (n <= (uint32_t)kTopCap || target == K) break;
+        }
         if (n > (uint32_t)kTopCap) {                 // more equal ones than the list holds: those of the lowest ranks
-            const uint32_t above = kth == kCtNone ? 0u : gather(kth + 1u, kCtNone, kCtNone, 3);
+            const uint32_t above = kth == kCtNone ? 0u : gather(kth + 1u, kCtNone, kCtNone, 4);
             uint32_t rk[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) rk[i] = key[i] == kth && r0 + i * dr < R ? (uint32_t)(r0 + i * dr) : kCtNone;
             if (tid == 0) { sh.lo[0] = 0u; sh.width[0] = (uint32_t)R; }
             const uint32_t nth = (uint32_t)K - above - 1u;
             ct_select<V, 1, NC>(rk, nth, nth, sh);
-            n = gather(kth, kth, sh.v1[0], 3);
+            n = gather(kth, kth, sh.v1[0], 4);
         }
         if (sh.bad && crank == 0 && tid == 0) atomicOr(status, kStatInternal);
     }
@@ -179,8 +203,8 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
             if (a.idx_keep) a.idx_keep[at] = r;
         }
         if (a.hint && at == min((int)n, want) - 1) {
-            a.hint->valid = 1u;
-            a.hint->tau = (uint32_t)(e >> 32);
+            a.hint->valid = keeps ? 1u : 0u;
+            a.hint->tau = (int)n >= want ? (uint32_t)(e >> 32) : tau;   // (never higher than what admitted too few)
             if (hit) a.hint->hits += 1u; else a.hint->misses += 1u;
         }
     };

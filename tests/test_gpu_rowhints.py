@@ -150,3 +150,43 @@ def test_block_brackets_of_the_split_path_survive_a_jump_between_blocks():
         fb = g.fallback_steps()
         assert fb == (0 if j < 3 else B), (j, fb)
     g.close()
+
+
+@pytest.mark.parametrize("R,K,quant", [
+    (1500, 129, None),             # the first that does not ask for three times K
+    (1500, 248, None), (1500, 249, None),              # ordered by a network of 256, of 512
+    (9000, 300, None),             # groups of K instead of as many as the next threshold should admit, over a cluster
+    (9000, 385, None),             # too long for groups: the exact threshold
+    (9000, 504, None), (9000, 505, None),              # a network of 512, of 1 024
+    (1024, 700, None),
+    (30000, 990, None),            # little room above K
+    (3000, 1008, None), (3000, 1009, None),            # the last that keeps a threshold; the first that does not
+    (9000, 1024, None),
+    (3000, 500, 40),               # ties: more entries at the threshold than the list holds
+])
+def test_long_lists_use_the_threshold_of_the_evaluation_before(R, K, quant):
+    """Streaming evaluations: the list equals the oracle's, and nearly all of them come out of the previous threshold (a
+    rank's level differs from the others' by more than a step changes its median, so that the list hardly moves)."""
+    from paper_2605_17879_b200 import guard
+    M, W, steps = 2, 24, 30
+    rng = np.random.default_rng(R + K)
+    X = (1.0 + 0.3 * rng.random((1, R, 1)) + 0.0003 * rng.standard_normal((W + steps, R, M))).astype(np.float32)
+    if quant:
+        X = (np.round(X * quant) / quant).astype(np.float32)
+    dirs = [1, 1]
+    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 8, topk=K)
+    o = go.Oracle(R, M, W, W // 2, K, dir=dirs)
+    Xd = torch.from_numpy(X).cuda()
+    g.ingest(Xd[:W])
+    o.ingest(X[:W])
+    for t in range(W, W + steps):
+        g.ingest(Xd[t:t + 1])
+        out = g.score()
+        assert g.sync_status() == 0
+        o.ingest(X[t:t + 1])
+        compare_score(out, o.score(), "t=%d" % t)
+    n = g.row_hints()
+    assert n["topk_hinted"] + n["topk_full"] == steps - 1      # (the first evaluation follows no other closely)
+    if quant is None and K <= 1008:
+        assert n["topk_full"] <= 2, n
+    g.close()

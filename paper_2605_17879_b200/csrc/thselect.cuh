@@ -12,15 +12,15 @@
 
 namespace guard {
 
-// The values to keep: |x - c| <= h, as rounded.  usable: h is positive and neither value is near the ends of the range
-// of floats.
+// The values to keep: |x - c| <= h, as rounded.  usable: h is positive and neither value so near the ends of the range of
+// floats that a power of two below would not be a normal number or a sum overflow.
 struct ThRange {
     float c, h;
     float ns, nhs;     // -S and -h S: the saturated product of a value below the interval
 };
 __device__ __forceinline__ float pow2_of(const int e) { return __int_as_float((e + 127) << 23); }      // -126 <= e <= 127
 __device__ __forceinline__ int exponent_of(const float x) { return (int)((__float_as_uint(x) >> 23) & 255u) - 127; }   // of normal numbers
-__device__ __forceinline__ bool th_usable(const float c, const float h) { return h > 1.0e-18f && h < 1.0e18f && fabsf(c) < 1.0e18f; }
+__device__ __forceinline__ bool th_usable(const float c, const float h) { return h > 1.0e-29f && h < 1.0e37f && fabsf(c) < 1.0e37f; }
 __device__ __forceinline__ ThRange th_range(const float c, const float h, const bool usable) {
     ThRange r;
     r.c = c;
@@ -82,9 +82,10 @@ __device__ __forceinline__ void th_select_pair(const uint32_t kbase, const int n
         // No kept value lies outside [pl, ph): |x - c| as rounded is within 2^-24 of itself and of |c|.
         const float top = fabsf(r.c) + r.h, eps = top * pow2_of(-21);
         float pl = r.c - r.h - eps, ph = r.c + r.h + eps, pv = pl;
-        // Pivots are kept away from zero, so that they differ from any value by at least 2^-56 of the largest.
-        const int e = exponent_of(top);
-        const float near0 = ok ? pow2_of(e - 30) : 1.0f, ns = ok ? -pow2_of(60 - e) : 0.0f;
+        // Pivots are kept so far from zero that the power of two lifts their difference from any other value (2^-24 of
+        // the pivot at least) to 1: 2^-35 of the largest value, as long as that power is a number.
+        const int lift = min(60 - exponent_of(top), 127);
+        const float near0 = ok ? pow2_of(25 - lift) : 1.0f, ns = ok ? -pow2_of(lift) : 0.0f;
         // The pivot moves inside a bracket (pl, ph) with below(pl) = al <= t - 2 and below(ph) = ah >= t + 2.
         int al = 0, ah = nk, bsave = 0;
         int done = 0;                 // 1: pv has bsave in {t - 1, t, t + 1} values below it, 2: both ranks equal pl

@@ -882,3 +882,26 @@ def test_calls_under_stream_capture(R, M, W, B):
         g.close()
     for key in got[0]:
         assert_bit_equal(got[1][key], got[0][key], key)
+
+
+@pytest.mark.parametrize("scale", [1e-26, 1e-17, 1.0, 1e20, 1e34])
+def test_window_threads_serve_values_of_any_size(scale):
+    """The thread-per-series path on values in other units (some about zero): equal to the oracle, and as few series left
+    to the finishing kernel as in ordinary units."""
+    from paper_2605_17879_b200 import guard
+    R, M, W = 16400, 4, 40
+    X, dirs = _rand_fleet(4 * W, R, M, seed=3)
+    X[:, :, 2] -= np.float32(3.0)
+    X = (X.astype(np.float64) * scale).astype(np.float32)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W, topk=8)
+    o = go.Oracle(R, M, W, W // 2, 8, dir=dirs)
+    for t in range(0, 4 * W, W):
+        g.ingest(Xd[t:t + W])
+        out = g.score()
+        assert g.sync_status() == 0
+        o.ingest(X[t:t + W])
+        compare_score(out, o.score(), "t=%d" % t)
+    left = g.window_fallbacks()
+    assert left["total"] < 3 * R * M // 20, left
+    g.close()

@@ -153,13 +153,20 @@ __device__ __forceinline__ void sweep_warp_median(const SweepMedArgs &a, const u
     }
 }
 
-// The series the thread path left: their bits in a.todo.
+// The series the thread path left: their bits in a.todo.  A warp takes 32 >> parts series at a time: a whole word's, or
+// fewer while that leaves a warp for each (all series of a sweep whose means say nothing about their medians: 33 600 of 64
+// repetitions 101 us with whole words, 60 with quarters; 98 304 of 200 245 us by half as many warps, 200 so).
+constexpr int kSwFinishCtas = 148 * 8;
+
 template <int VPL>
-__global__ void __launch_bounds__(kSwThreads) sweep_median_finish_kernel(const SweepMedArgs a) {
+__global__ void __launch_bounds__(kSwThreads) sweep_median_finish_kernel(const SweepMedArgs a, const int parts) {
     pdl_wait();
-    const uint32_t words = (uint32_t)(((long long)a.G * a.M + 31) >> 5), nwarps = gridDim.x * (kSwThreads / 32);
-    for (uint32_t i = blockIdx.x * (kSwThreads / 32) + warp_id(); i < words; i += nwarps)
-        for (uint32_t t = __ldcg(a.todo + i); t; t &= t - 1u) sweep_warp_median<VPL>(a, 32u * i + (uint32_t)(__ffs(t) - 1), false);
+    const uint32_t words = (uint32_t)(((long long)a.G * a.M + 31) >> 5), nwarps = gridDim.x * (kSwThreads / 32), share = 32u >> parts;
+    for (uint32_t i = blockIdx.x * (kSwThreads / 32) + warp_id(); i < words << parts; i += nwarps) {
+        const uint32_t first = (i & ((1u << parts) - 1u)) * share;   // of the word's bits
+        for (uint32_t t = __ldcg(a.todo + (i >> parts)) & ((0xFFFFFFFFu >> (32u - share)) << first); t; t &= t - 1u)
+            sweep_warp_median<VPL>(a, 32u * (i >> parts) + (uint32_t)(__ffs(t) - 1), false);
+    }
 }
 
 // Every series.
@@ -264,11 +271,13 @@ cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st) {
         sweep_median_thread_kernel<<<(unsigned)((series + kSwThreads - 1) / kSwThreads), kSwThreads, 0, st>>>(a);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        const long long want = ((series + 31) / 32 + kSwThreads / 32 - 1) / (kSwThreads / 32);
-        const int fgrid = (int)(want < 148 * 4 ? want : 148 * 4);
-        if (a.reps <= 64) return launch_after(sweep_median_finish_kernel<2>, fgrid, kSwThreads, st, a);
-        if (a.reps <= 128) return launch_after(sweep_median_finish_kernel<4>, fgrid, kSwThreads, st, a);
-        return launch_after(sweep_median_finish_kernel<8>, fgrid, kSwThreads, st, a);
+        const long long words = (series + 31) / 32, most = (long long)kSwFinishCtas * (kSwThreads / 32);
+        int parts = 0;
+        while (parts < 3 && (words << (parts + 1)) <= most) ++parts;
+        const int fgrid = (int)((min(words << parts, most) + kSwThreads / 32 - 1) / (kSwThreads / 32));
+        if (a.reps <= 64) return launch_after(sweep_median_finish_kernel<2>, fgrid, kSwThreads, st, a, parts);
+        if (a.reps <= 128) return launch_after(sweep_median_finish_kernel<4>, fgrid, kSwThreads, st, a, parts);
+        return launch_after(sweep_median_finish_kernel<8>, fgrid, kSwThreads, st, a, parts);
     }
     const size_t smem = (size_t)a.reps * kSweepCols * 4;
     if (smem <= 200 * 1024) {

@@ -905,3 +905,21 @@ def test_window_threads_serve_values_of_any_size(scale):
     left = g.window_fallbacks()
     assert left["total"] < 3 * R * M // 20, left
     g.close()
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (10923, 1, 33, 3),             # quarters of words; one series in the last
+    (1300, 8, 64, 4),              # halves
+    (2500, 8, 40, 8),              # whole words, more than there are warps
+])
+def test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M):
+    """Results that spread over decades: the mean says nothing about the median, and next to no series is served by it."""
+    from paper_2605_17879_b200 import guard
+    rng = np.random.default_rng(N + M)
+    S = np.exp(6.0 * rng.standard_normal((nodes * gpn, N, M), dtype=np.float32)).astype(np.float32)
+    dirs = [1 if m % 2 else -1 for m in range(M)]
+    ref = go.sweep(S, nodes, gpn, dir=dirs)
+    out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
+    assert int(out["status"].cpu()[0]) == 0
+    for key in ref:
+        assert_bit_equal(to_np(out[key]), ref[key], key)

@@ -212,6 +212,7 @@ struct guard_ctx {
     cudaEvent_t ev_e[2] = {nullptr, nullptr};
     struct Inflight { bool on = false; long long seen = 0; int n = 0; } infl[2];
     int last_q = 0;                   // parity of the pending evaluation
+    bool topk_tail = false;           // the latest top-k selection belongs to the evaluation that ends with ev_e[last_q]
     bool ensure_xs() {
         if (xs[0]) return true;
         if (!ensure_tail()) return false;
@@ -689,6 +690,9 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
             // medians need not queue behind it
             cudaStream_t tk = (defer && c->aux) ? c->aux : c->side;
             if (e == cudaSuccess && tk == c->aux) e = cudaStreamWaitEvent(c->aux, c->ev_w, 0);
+            // the selection's scratch and threshold may still be in use on the tail stream (the caller's stream has waited
+            // for that, but neither of these two: what they wait for was recorded before)
+            if (e == cudaSuccess && c->topk_tail) e = cudaStreamWaitEvent(tk, c->ev_e[c->last_q], 0);
             if (e == cudaSuccess) e = launch_topk(t, c->p, tk);
             if (e == cudaSuccess) e = cudaEventRecord(c->ev_topk, tk);
             topk_side = true;
@@ -697,6 +701,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
         }
         if (e != cudaSuccess) return c->cuda_fail(e, "topk launch");
         c->launches += t.hint ? 2 : 1;
+        c->topk_tail = defer;
     }
 
     XrankArgs x{};

@@ -923,3 +923,34 @@ def test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M):
     assert int(out["status"].cpu()[0]) == 0
     for key in ref:
         assert_bit_equal(to_np(out[key]), ref[key], key)
+
+
+def test_selections_of_evaluations_in_flight_do_not_meet():
+    """Fleets wider than the register paths: evaluations close together take the hinted selection on one internal stream,
+    the others the full one on another, with the same scratch; deferred ones with nothing between them, then at once."""
+    from paper_2605_17879_b200 import guard
+    R, M, W, K = 33000, 2, 12, 1000
+    gaps = [12, 1, 9, 1, 9, 9, 1, 2, 10, 1, 1, 9, 9, 3]
+    X, dirs = _rand_fleet(sum(gaps), R, M, seed=8)
+    Xd = torch.from_numpy(X).cuda()
+    refs = []
+    o = go.Oracle(R, M, W, 4, K, dir=dirs)
+    t = 0
+    for n in gaps:
+        o.ingest(X[t:t + n])
+        refs.append(o.score())
+        t += n
+    for defer in ([True] * len(gaps), [j % 2 == 0 for j in range(len(gaps))]):
+        g = guard.Guard(R, M, W, 4, dir=dirs, capacity=sum(gaps), topk=K)
+        bufs = [g.alloc_outputs() for _ in gaps]
+        t = 0
+        for j, n in enumerate(gaps):
+            g.set_deferred(defer[j])
+            g.ingest(Xd[t:t + n])
+            g.score(bufs[j])
+            t += n
+        g.join()
+        assert g.sync_status() == 0
+        for j in range(len(gaps)):
+            compare_score(bufs[j], refs[j], "evaluation %d" % j)
+        g.close()

@@ -1039,7 +1039,9 @@ int guard_state_import(guard_ctx *c, const void *d_state, size_t state_bytes, vo
     c->seen = h.seen;
     c->evals = h.evals;
     c->seen_at_eval = h.seen_at_eval;
-    c->inc_seen = h.inc_seen;
+    // (steps ingested after the last evaluation have pushed the oldest steps of its window out of the exported ones: the
+    // sliding update would have to read them)
+    c->inc_seen = h.inc_seen - h.inc_n >= h.seen - h.steps ? h.inc_seen : -1;
     c->inc_n = h.inc_n;
     c->cnt_seen = -1;   // the kept counts are not part of the state: the next evaluation recounts
     c->hints_ready = h.hints_ready != 0;

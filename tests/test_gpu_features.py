@@ -316,3 +316,38 @@ def test_bounded_wait_runs_out_and_the_context_recovers():
     with pytest.raises(guard.GuardError):
         g.debug_set_wait_limit(-1)
     g.close()
+
+
+@pytest.mark.parametrize("gap", [1, 3])
+def test_state_exported_between_an_ingest_and_its_evaluation(gap):
+    """Steps after the last evaluation push its window's oldest steps out of the exported ones; the resumed context must
+    not look for them where another ring left something else."""
+    from paper_2605_17879_b200 import guard
+    R, M, W, cap = 40, 3, 20, 32
+    X, dirs = _rand_fleet(W + 3 * gap, R, M, seed=gap)
+    Xd = torch.from_numpy(X).cuda()
+    o = go.Oracle(R, M, W, 5, 4, dir=dirs)
+    a = guard.Guard(R, M, W, 5, dir=dirs, capacity=cap, topk=4)
+    a.ingest(Xd[:W])
+    o.ingest(X[:W])
+    a.score()
+    o.score()
+    a.ingest(Xd[W:W + gap])
+    o.ingest(X[W:W + gap])
+    a.score()                                            # the sliding state is current for this window
+    o.score()
+    a.ingest(Xd[W + gap:W + 2 * gap])
+    o.ingest(X[W + gap:W + 2 * gap])
+    state = a.state_export()
+    ws = torch.full((guard.workspace_bytes(R, M, W, cap, 4) // 4,), 0.5, device="cuda").view(torch.uint8)
+    b = guard.Guard(R, M, W, 5, dir=dirs, capacity=cap, topk=4, workspace=ws)
+    b.state_import(state)
+    for t in (W + 2 * gap, W + 3 * gap):
+        out = b.score()
+        assert b.sync_status() == 0
+        compare_score(out, o.score(), "resumed t=%d" % t)
+        if t < W + 3 * gap:
+            b.ingest(Xd[t:t + gap])
+            o.ingest(X[t:t + gap])
+    a.close()
+    b.close()

@@ -112,11 +112,13 @@ __global__ void __launch_bounds__(kBrThreads) xrank_stream_kernel(const XrankArg
     __shared__ uint32_t s_cand[M][kCtaCand];
     __shared__ uint32_t s_cnt[M], s_ncand[M], s_base[M];
     __shared__ uint32_t s_amb[MODE == 1 ? kCtaAmb : 1];
-    __shared__ uint32_t s_namb, s_ambbase;
+    __shared__ uint32_t s_namb, s_ambbase, s_flag;
     __shared__ int s_overflow;
 
     const int t = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x, lane = lane_id();
-    if (__ldcg(sc.flag + t) != 0) return;   // the step already goes to the direct path
+    if (tid == 0) s_flag = __ldcg(sc.flag + t);   // (other CTAs of the launch may set it meanwhile: one thread reads for all)
+    __syncthreads();
+    if (s_flag != 0) return;                // the step already goes to the direct path
     const int R = a.R;
     const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
     const float *row = a.base + (size_t)slot * a.row_stride;
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kBrThreads) xrank_stream_kernel(const XrankArg
 struct SelShared {
     uint32_t hist[kSelBins];
     uint32_t warp_tot[kSelThreads / 32];
-    uint32_t bin, before, cnt, vmin;
+    uint32_t bin, before, cnt, vmin, flag;
     int found;
 };
 
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(kSelThreads) xrank_select_kernel(const XrankAr
     const int R = a.R, M = a.M;
     const size_t so = (size_t)t * M, col = so + m;
     const uint32_t clt = __ldcg(sc.cnt_lt + col), n = __ldcg(sc.ncand + col);
+    if (tid == 0) sh.flag = __ldcg(sc.flag + t);   // (the step's other columns may set it meanwhile: one thread reads for all)
     __syncthreads();
     // leave the counters clean for the next sweep / launch (every thread has read them)
     if (tid == 0) {
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(kSelThreads) xrank_select_kernel(const XrankAr
         sc.ncand[col] = 0;
         if (MODE == 0 && m == 0) sc.namb[t] = 0;
     }
-    if (__ldcg(sc.flag + t) != 0) return;
+    if (sh.flag != 0) return;
     const bool even = (R & 1) == 0;
     const uint32_t k1 = (uint32_t)((R - 1) / 2), k2 = (uint32_t)(R / 2);
     int why = -1;

@@ -954,3 +954,15 @@ def test_selections_of_evaluations_in_flight_do_not_meet():
         for j in range(len(gaps)):
             compare_score(bufs[j], refs[j], "evaluation %d" % j)
         g.close()
+
+
+@pytest.mark.parametrize("R,M,B,quant", [
+    (33001, 16, 6, None),
+    (33001, 16, 6, 12),            # ties: lists overflow, CTAs give their step up while others of it start
+    (33002, 32, 5, 30),
+    (40001, 8, 20, 12),            # byte-wide exceedance entries
+])
+def test_wide_fleets_whose_steps_are_given_up(R, M, B, quant):
+    """Fleets wider than the register paths, several CTAs per step: steps given up in the middle of a launch are redone."""
+    X, dirs = _rand_fleet(2 * B, R, M, seed=R + M, quant=quant)
+    run_both(X, B, max(1, B // 2), 8, dirs, [B], capacity=2 * B)

@@ -198,10 +198,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
     if (crank != 0) return;
     auto put = [&](const int at, const unsigned long long e) {
         const int32_t r = (int32_t)(0xFFFFFFFFu - (uint32_t)e);
-        if (at < K) {
-            if (a.idx) a.idx[at] = r;
-            if (a.idx_keep) a.idx_keep[at] = r;
-        }
+        if (at < K) a.idx_keep[at] = r;
         if (a.hint && at == min((int)n, want) - 1) {
             a.hint->valid = keeps ? 1u : 0u;
             a.hint->tau = (int)n >= want ? (uint32_t)(e >> 32) : tau;   // (never higher than what admitted too few)

@@ -564,7 +564,6 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     const int q = c->eval_q();
     w.wmed = c->wmed(q);
     w.wmed_prev = c->wmed(q ^ 1);
-    w.wmed_user = d_wmed;
     w.use_hint = c->hints_ready ? 1 : 0;
     w.spread = (float *)(c->ws + c->L.wspread);
     w.centre = (float *)(c->ws + c->L.wcentre);
@@ -669,7 +668,6 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
         t.fleet_mad = c->fleet_mad();
         t.cand = c->topk_cand();
         t.ticket = c->ticket();
-        t.idx = d_topk_idx;
         t.idx_keep = c->topk_idx(q);
         t.score = nullptr;
         // evaluations a few steps apart: the previous evaluation's threshold pre-selects the candidates
@@ -738,6 +736,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     s.last_slot = last;
     s.n = n;
     s.consec = c->consec();
+    s.wmed_user = d_wmed;
     s.scores = d_scores;
     s.counts = d_counts;
     s.metric_mask = d_metric_mask;
@@ -759,6 +758,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
         c->cnt_n = n;
     }
     s.topk_idx = want_topk ? c->topk_idx(q) : nullptr;
+    s.topk_user = want_topk ? d_topk_idx : nullptr;
     s.topk_score = want_topk ? d_topk_score : nullptr;
     s.K = c->K;
     if (topk_side) {

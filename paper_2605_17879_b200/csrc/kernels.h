@@ -103,7 +103,6 @@ struct WindowArgs {
     float *wmed;            // [series] (never NULL)
     const float *wmed_prev; // [series] the previous evaluation's medians (another buffer than wmed), or NULL
     int use_hint;           // wmed_prev holds the previous evaluation's medians: use them as first pivots
-    float *wmed_user;       // or NULL
     float *spread;          // [series] tuned half-width of the thread path's interval (state), or NULL
     float *centre;          // [series] smoothed median: the centre of the thread path's interval (state), or NULL
     int target;             // number of keys the thread path's interval is tuned to catch (0: default)
@@ -142,7 +141,9 @@ bool window_inc_supported(const WindowArgs &a);
 cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, cudaStream_t st);
 int window_launch_count(const WindowArgs &a);
 
-// Fused k-of-W count, robust score, thresholds, multi-signal flag, tier, consecutive counter.
+// Fused k-of-W count, robust score, thresholds, multi-signal flag, tier, consecutive counter.  It also writes what the
+// caller gets of the results before it: the kernels on the library's own streams, which may start before the caller's
+// earlier work on the output buffers has ended, write only into the workspace.
 struct ScoreArgs {
     int R, M;
     const float *wmed;       // [R][M]
@@ -154,6 +155,7 @@ struct ScoreArgs {
     int last_slot;
     int n;                   // window length
     uint8_t *consec;         // [R] state
+    float *wmed_user;        // [R][M] or NULL: the caller's copy of the medians
     float *scores;           // [R][M] or NULL
     uint16_t *counts;        // [R][M] or NULL
     uint32_t *metric_mask;   // [R] or NULL
@@ -161,9 +163,10 @@ struct ScoreArgs {
     uint8_t *tier;           // [R] or NULL
     uint8_t *flags_keep;     // [R] the context's own copy (input of the node-level fold), never NULL
     uint8_t *tier_keep;      // [R] likewise
-    // scores of an already selected top-k list (the selection itself needs no fleet statistics and runs
-    // beside the fleet baseline): topk_score[i] = primary score of rank topk_idx[i]; NULL / 0 to skip
+    // an already selected top-k list (the selection itself needs no fleet statistics and runs beside the fleet
+    // baseline), NULL to skip: the caller's copy, and topk_score[i] = primary score of rank topk_idx[i] (either or NULL)
     const int32_t *topk_idx;
+    int32_t *topk_user;
     float *topk_score;
     int K;
     // k-of-W counts kept across evaluations: kcnt [R][M] is rewritten by every evaluation; with slide != 0
@@ -202,7 +205,7 @@ struct TopkArgs {
     unsigned long long *cand;   // scratch [topk_blocks(R)][K]
     unsigned int *ticket;       // scratch, zero before first use (self-resetting)
     int32_t *idx;               // [K] or NULL
-    int32_t *idx_keep;          // [K] second copy of the indices (the context's own), or NULL
+    int32_t *idx_keep;          // [K] a copy of the indices for the context, or NULL
     float *score;               // [K] or NULL: needs fleet_med / fleet_mad to be final when the kernel runs
     TopkHint *hint;             // or NULL: state of the hinted pass (evaluations a few steps apart; used when score is NULL)
     unsigned long long *hcand;  // scratch [1024] of the hinted pass

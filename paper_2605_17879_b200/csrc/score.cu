@@ -25,14 +25,16 @@ __global__ void __launch_bounds__(1024, 1) score_flag_kernel(const ScoreArgs a, 
     __shared__ uint32_t s_mask[kRanks];
     __shared__ float s_dev[kRanks];
     const int M = NM ? NM : a.M, tid = threadIdx.x, T = blockDim.x, lane = lane_id(), row = tid / LW, rows = T / LW;   // this thread's first step, steps per round
-    if (a.topk_score && blockIdx.x == gridDim.x - 1) {       // scores of the ranks a top-k selection has picked
+    if (a.topk_idx && blockIdx.x == gridDim.x - 1) {         // the ranks a top-k selection has picked, and their scores
         pdl_wait();
         const int pm = p.primary;
         const float B = a.fleet_med[pm], Ds = scale_of(a.fleet_mad[pm], B, p.floor_rel[pm], p.floor_abs[pm]);
         for (int i = tid; i < a.K; i += T) {
-            float dev = __fsub_rn(a.wmed[(size_t)a.topk_idx[i] * M + pm], B);
+            const int32_t r = a.topk_idx[i];
+            float dev = __fsub_rn(a.wmed[(size_t)r * M + pm], B);
             if (p.dir[pm] < 0) dev = -dev;
-            a.topk_score[i] = (dev == 0.0f) ? 0.0f : __fdiv_rn(__fmul_rn(0.6745f, dev), Ds);
+            if (a.topk_user) a.topk_user[i] = r;
+            if (a.topk_score) a.topk_score[i] = (dev == 0.0f) ? 0.0f : __fdiv_rn(__fmul_rn(0.6745f, dev), Ds);
         }
         pdl_trigger();
         return;
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(1024, 1) score_flag_kernel(const ScoreArgs a, 
         int cnt = (int)((s_cnt[i][q & 1][l] >> (16 * (q >> 1))) & 0xFFFFu);
         if (a.slide) cnt += (int)a.kcnt[o] - (int)((s_left[i][q & 1][l] >> (16 * (q >> 1))) & 0xFFFFu);
         if (a.kcnt) a.kcnt[o] = (uint16_t)cnt;
+        if (a.wmed_user) a.wmed_user[o] = x;
         float dev = __fsub_rn(x, s_B[m]);
         if (p.dir[m] < 0) dev = -dev;
         if (dev > s_rhs[m] && cnt >= p.k) atomicOr(&s_mask[rl], 1u << m);
@@ -218,7 +221,7 @@ cudaError_t launch_node_verdict(const NodeArgs &a, cudaStream_t st) {
 
 template <int LW>
 static cudaError_t launch_score(const ScoreArgs &a, const MetricParams &p, cudaStream_t st) {
-    const int ranks = LW * 4 / a.mask_bytes, grid = (a.R + ranks - 1) / ranks + (a.topk_score ? 1 : 0);
+    const int ranks = LW * 4 / a.mask_bytes, grid = (a.R + ranks - 1) / ranks + (a.topk_idx ? 1 : 0);
     // threads: eight loads each while one CTA can have them; where the CTAs fill the GPU anyway, 32 (larger ones keep SMs
     // from the kernels of the next evaluation: passes of 200 x 16 384 x 8 with overlapped evaluations take 433 us with
     // 256 threads per CTA, 436 with 512, 447 with 1 024)

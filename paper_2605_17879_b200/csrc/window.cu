@@ -138,7 +138,6 @@ __global__ void __launch_bounds__(1024, 2) window_warp_kernel(const WindowArgs a
             if (lane == 0) {
                 if (!ok) atomicOr(a.status, kStatInternal);
                 a.wmed[series] = med;
-                if (a.wmed_user) a.wmed_user[series] = med;
                 if (a.spread) a.spread[series] = h0;
                 if (a.centre) a.centre[series] = med;
             }
@@ -263,7 +262,6 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
     if (ok) med = even ? __fmul_rn(0.5f, __fadd_rn(vb, vu)) : vu;
     if (active && ok) {
         a.wmed[c] = med;
-        if (a.wmed_user) a.wmed_user[c] = med;
         // re-tune the half-width so that the interval catches about kThTarget keys next time
         const float target = (float)(a.target > 0 ? a.target : kThTarget);
         const float f = fminf(2.0f, fmaxf(0.5f, target / (float)max(nk, 1)));
@@ -323,7 +321,6 @@ __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const Window
         if (lane == 0) {
             if (!ok2) atomicOr(a.status, kStatInternal);
             a.wmed[series] = m2;
-            if (a.wmed_user) a.wmed_user[series] = m2;
             a.spread[series] = h0;
             a.centre[series] = m2;
             if (a.fb_count) { atomicAdd(a.fb_count, 1u); atomicAdd(a.fb_count + 1 + why_src, 1u); }
@@ -518,7 +515,6 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
         }
         const float med = median_from_keys(f2key(f1), f2key(f2), even);
         a.wmed[c] = med;
-        if (a.wmed_user) a.wmed_user[c] = med;
         s.cnt[c] = 0x80000000u | ((uint32_t)nin << 16) | (uint32_t)cb;
     }
     // ---- series without a usable state go on the launch's rebuild list (window_rebuild_kernel follows) ----
@@ -600,7 +596,6 @@ __global__ void __launch_bounds__(kRbThreads) window_rebuild_kernel(const Window
         }
         if (lane == 0) {
             a.wmed[series] = med;
-            if (a.wmed_user) a.wmed_user[series] = med;
             s.lo[series] = flo;
             s.hi[series] = fhi;
             // an interval with more (tied) values than a list holds stays without state: it rebuilds every time

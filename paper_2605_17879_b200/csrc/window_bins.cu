@@ -345,7 +345,6 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
         const uint32_t v1 = sh.v1[lane], v2 = sh.v2[lane];
         const float med = median_from_keys(even ? v1 : v2, v2, even);
         a.wmed[c] = med;
-        if (a.wmed_user) a.wmed_user[c] = med;
         if (a.spread && a.centre) {
             // the range is tuned to catch 5 sqrt(n) values (or what the caller asks for) next time (four standard errors of the difference between the
             // smoothed median and the next window's): half of the way, one window's count is a noisy estimate of the density

@@ -966,3 +966,34 @@ def test_wide_fleets_whose_steps_are_given_up(R, M, B, quant):
     """Fleets wider than the register paths, several CTAs per step: steps given up in the middle of a launch are redone."""
     X, dirs = _rand_fleet(2 * B, R, M, seed=R + M, quant=quant)
     run_both(X, B, max(1, B // 2), 8, dirs, [B], capacity=2 * B)
+
+
+@pytest.mark.parametrize("R,M,W,deferred", [
+    (4500, 8, 80, False), (4500, 8, 80, True),     # medians by tiles on an internal stream, by threads from the second evaluation on
+    (33000, 2, 40, False), (33000, 2, 40, True),   # the selection on internal streams, too
+    (64, 4, 20, True),                             # a small window
+])
+@pytest.mark.parametrize("gap", [1, 20])
+def test_outputs_follow_what_the_caller_enqueued_before(R, M, W, deferred, gap):
+    """The caller's stream still has work on the output buffers when an evaluation is asked for: its results come after that
+    work, not before it."""
+    from paper_2605_17879_b200 import guard
+    X, dirs = _rand_fleet(W + 3 * gap, R, M, seed=R + gap)
+    Xd = torch.from_numpy(X).cuda()
+    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 3 * gap, topk=8)
+    g.set_deferred(deferred)
+    o = go.Oracle(R, M, W, W // 2, 8, dir=dirs)
+    out = g.alloc_outputs()
+    t = 0
+    for n in (W, gap, gap, gap):
+        g.ingest(Xd[t:t + n])
+        o.ingest(X[t:t + n])
+        t += n
+        torch.cuda._sleep(2_000_000)
+        for v in out.values():
+            v.view(torch.uint8).fill_(7)
+        g.score(out)
+        g.join()
+        assert g.sync_status() == 0
+        compare_score(out, o.score(), "t=%d" % t)
+    g.close()

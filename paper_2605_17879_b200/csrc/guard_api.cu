@@ -885,10 +885,16 @@ int guard_node_verdict(guard_ctx *c, uint8_t *d_node_flag, uint8_t *d_node_tier,
     a.node_flag = d_node_flag;
     a.node_tier = d_node_tier;
     a.node_stall = d_node_stall;
-    // a deferred evaluation still pending: the fold joins it on the evaluation's own stream
+    // a deferred evaluation still pending: the fold joins it on the evaluation's own stream, behind what the caller has
+    // enqueued so far (on the output buffers, perhaps)
     const bool on_tail = c->pending && c->tail;
     cudaStream_t ts = on_tail ? c->tail : (cudaStream_t)stream;
-    cudaError_t e = launch_node_verdict(a, ts);
+    cudaError_t e = cudaSuccess;
+    if (on_tail) {
+        e = cudaEventRecord(c->ev_x, (cudaStream_t)stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c->tail, c->ev_x, 0);
+    }
+    if (e == cudaSuccess) e = launch_node_verdict(a, ts);
     if (e == cudaSuccess && on_tail) e = cudaEventRecord(c->ev_e[c->last_q], c->tail);
     if (e != cudaSuccess) return c->cuda_fail(e, "node verdict launch");
     c->launches += 1;

@@ -975,15 +975,18 @@ def test_wide_fleets_whose_steps_are_given_up(R, M, B, quant):
 ])
 @pytest.mark.parametrize("gap", [1, 20])
 def test_outputs_follow_what_the_caller_enqueued_before(R, M, W, deferred, gap):
-    """The caller's stream still has work on the output buffers when an evaluation is asked for: its results come after that
-    work, not before it."""
+    """The caller's stream still has work on the output buffers when an evaluation (a node verdict) is asked for: its
+    results come after that work, not before it."""
     from paper_2605_17879_b200 import guard
     X, dirs = _rand_fleet(W + 3 * gap, R, M, seed=R + gap)
     Xd = torch.from_numpy(X).cuda()
-    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 3 * gap, topk=8)
+    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 3 * gap, topk=8, ranks_per_node=4)
     g.set_deferred(deferred)
     o = go.Oracle(R, M, W, W // 2, 8, dir=dirs)
     out = g.alloc_outputs()
+    N = R // 4
+    nodes = {"node_flag": torch.empty(N, dtype=torch.uint8, device="cuda"), "node_tier": torch.empty(N, dtype=torch.uint8, device="cuda"),
+             "node_stall": torch.empty(N, dtype=torch.uint16, device="cuda")}
     t = 0
     for n in (W, gap, gap, gap):
         g.ingest(Xd[t:t + n])
@@ -993,7 +996,14 @@ def test_outputs_follow_what_the_caller_enqueued_before(R, M, W, deferred, gap):
         for v in out.values():
             v.view(torch.uint8).fill_(7)
         g.score(out)
+        torch.cuda._sleep(2_000_000)
+        for v in nodes.values():
+            v.view(torch.uint8).fill_(7)
+        g.node_verdict(nodes)
         g.join()
         assert g.sync_status() == 0
         compare_score(out, o.score(), "t=%d" % t)
+        want = o.node_verdict(4)
+        for key in want:
+            assert_bit_equal(to_np(nodes[key]), want[key], "t=%d %s" % (t, key))
     g.close()

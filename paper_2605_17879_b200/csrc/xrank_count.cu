@@ -10,7 +10,6 @@ template <int V, int C>
 __global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<C> sh;
     pdl_wait();
-    if (a.only_flagged && a.only_flagged[blockIdx.y] == 0u) return;
     ct_row<V, C>(a, p, blockIdx.y, blockIdx.x * C, sh);
 }
 
@@ -19,7 +18,6 @@ template <int V, int NC, bool APART>
 __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512, 1) xrank_count_cluster_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<1> sh;
     pdl_wait();
-    if (a.only_flagged && a.only_flagged[blockIdx.y] == 0u) return;   // (the same for the whole cluster)
     const int column = (int)blockIdx.x / NC;
     if (APART) ct_row<V, 1, NC>(a, p, blockIdx.y, column % a.M, sh, column < a.M ? kCtStatistics : kCtCut);
     else ct_row<V, 1, NC>(a, p, blockIdx.y, column, sh);

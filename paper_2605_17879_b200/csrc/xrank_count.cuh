@@ -22,7 +22,6 @@
 
 namespace guard {
 
-constexpr int kCtMaxC = 8;         // metrics per CTA at most
 constexpr int kCtBins = 256;
 constexpr int kCtList = 64;        // keys of a bin that are ranked directly (two per lane)
 constexpr int kCtMaxIter = 64;     // a range shrinks at least to a 128th whenever its bin is too full
@@ -511,12 +510,8 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
                 }
             } else if (col == 0) {
                 unsigned int *w = reinterpret_cast<unsigned int *>(out) + r;
-                if (C == 8) {                // eight metrics are a byte of the rank's word
-                    reinterpret_cast<uint8_t *>(w)[m0 >> 3] = (uint8_t)bits;
-                } else {
-                    atomicAnd(w, ~own);
-                    if (bits) atomicOr(w, bits << m0);
-                }
+                atomicAnd(w, ~own);
+                if (bits) atomicOr(w, bits << m0);
             }
         }
     }

@@ -189,8 +189,9 @@ struct guard_ctx {
     }
     // Deferred evaluations: guard_score enqueues the evaluation on internal streams and does not
     // make the caller's stream wait for it, so that the evaluation's short, latency-bound tail runs
-    // beside the next guard_ingest.  At most one evaluation is pending; the next guard_score,
-    // guard_join, guard_sync_status, guard_reset and guard_destroy wait for it.
+    // beside the next guard_ingest.  The caller's stream waits for it in the next guard_score, guard_join,
+    // guard_sync_status or guard_reset; up to two may run at a time (the tail of one beside the window medians of the
+    // next), in buffers that alternate.
     bool deferred = false;
     bool pending = false;             // an evaluation has been enqueued whose end the caller's stream has not waited for
     int pending_n = 0;                // its window length
@@ -315,7 +316,7 @@ struct guard_ctx {
     void *mask() const { return ws + L.mask; }
     float *ring() const { return (float *)(ws + L.ring); }
     int mask_bytes() const { return M <= 8 ? 1 : 4; }
-    // Cross-rank statistics of S rows: the bracketed path where it applies, else the direct one.
+    // Cross-rank statistics of S rows: the path that the sizes ask for, the direct one where none applies.
     // own_scratch = false: the call may run beside another cross-rank call of this context (the fleet
     // baseline of a deferred evaluation beside the next ingest), so it must not touch the one
     // scratch of the bracketed path: such rows take the direct selection.

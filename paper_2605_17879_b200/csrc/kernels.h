@@ -83,7 +83,8 @@ XrankScratch carve_xrank_scratch(void *small_base, void *big_base, int R, int M,
 cudaError_t launch_xrank_bracketed(const XrankArgs &a, const MetricParams &p, const XrankScratch &sc, int S,
                                    cudaStream_t st);
 
-// Rows held in registers and searched by counting at pivots: any values, any number of metrics, up to 32 768 ranks.
+// Rows held in registers, their keys binned over a range and the few of the wanted bin ranked: any values, any number of
+// metrics, up to 32 768 ranks.
 constexpr int kCountMaxRanks = 32768;
 bool xrank_count_supported(int R);
 int xrank_count_launches(int S);

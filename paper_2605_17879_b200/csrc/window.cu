@@ -192,20 +192,19 @@ cudaError_t launch_warp_path(const WindowArgs &a, int use_bulk, cudaStream_t st)
 // inside it replaces sorting the window.  One thread per series reads its window
 // straight from the ring (a warp reads 32 adjacent series of a row: one fully used 128-byte
 // line per load, eight rows in flight per thread), counts the values below the interval and
-// keeps those inside it, as raw bits, in its own shared-memory column.  No thread ever waits
+// keeps those inside it in its own shared-memory column.  No thread ever waits
 // for another one: there is no barrier in the kernel, CTAs are four warps, and with 60 kept
 // slots per thread seven CTAs share an SM.  The interval is centred on a smoothed median (a
 // single window's median carries its own sampling noise, which would add to the next one's).
 //
-// Selection among the kept keys runs the same instruction stream in every lane: the column
-// is turned into order-preserving keys once (128-bit shared-memory accesses; a column is 60
-// words, 4 x an odd number, so the lanes' quads fall on different banks), then counting
-// passes (keys below a pivot interpolated between the ends of a shrinking key bracket, every
-// third pass a bisection) run until t - 1, t or t + 1 keys lie below the pivot: the two
-// largest keys below it and the two smallest not below it then include ranks t - 1 and t.
-// If the bracket shrinks to one key, that key holds both ranks (ties).
-// A series whose interval missed, overflowed or did not converge is finished by its whole
-// warp: the lanes fetch the window (L2 hits), sort in registers and run the warp selection.
+// Selection among the kept values runs the same instruction stream in every lane (thselect.cuh):
+// counting passes over the column (128-bit shared-memory accesses; a column is 60 words, 4 x an
+// odd number, so the lanes' quads fall on different banks) with a pivot interpolated between the
+// ends of a shrinking bracket, every third pass a bisection, run until t - 1, t or t + 1 values
+// lie below the pivot: the two largest below it and the two smallest not below it then include
+// ranks t - 1 and t.  If the bracket shrinks to one value, that value holds both ranks (ties).
+// A series whose interval missed, overflowed, did not converge or ended on a zero goes on a list;
+// the kernel behind this one gives each listed series a warp (window_finish_kernel).
 // ---------------------------------------------------------------------------------------
 constexpr int kThCols = 128;     // series per CTA = threads per CTA
 constexpr int kThSlots = 60;     // kept keys per series

@@ -11,9 +11,11 @@
 // is settled bit by bit.  A value's bin is the low mantissa bits of fma(x, scale, offset): monotone in x whatever
 // the rounding, and one full-rate instruction (integer compares and adds run at half rate, conversions slower still).
 // Bound by instruction issue, most of it not per value (scan, ranking, barriers: 16 000 cycles a tile, four tiles on an
-// SM).  Measured, kernel alone, against what it replaces: 8 192 series of 1 000 steps 36 us (three-way quickselect per
-// thread in shared memory: 830), 98 760 first windows of 180 steps 71 us (sort per warp: 204), 8 192 of 100 steps 12 us
-// (one thread per series: 14 + 5).
+// SM).  At 64 registers a thread the instances with 16 values or more spill (20 to 236 bytes of stores a thread), outside
+// of the passes over the values: 0.8 % of the warp instructions (1 000 steps: 0.10 M of 13.2 M; 180 steps: 0.39 M of 50 M).
+// Measured, kernel alone, against what it replaces: 8 192 series of 1 000 steps 24 us (three-way quickselect per thread in
+// shared memory: 805), 98 760 first windows of 180 steps 63 us (sort per warp: 135), 8 192 of 100 steps 9.6 us (one
+// thread per series: 12 + 5).
 #include <math_constants.h>
 
 #include "kernels.h"

@@ -15,8 +15,8 @@
 // Bound by latency and by the half-rate integer pipe; what it avoids is what measured worst on the way here:
 // branches and returning atomics per value, rounds of pivots (each some 500 cycles of dependent scalar work in one
 // warp, whatever the number of values) and column-wise loads (a cache line per lane).  Measured, kernel alone:
-// 100 steps of 1 024 ranks x 8 metrics 8.7 us (8-bit radix select of xrank_direct.cuh: 80), 60 steps of 4 096 x 16
-// 25 us (570), one row of 1 024 ranks 5.3 us (10.5 with the whole column's histogram).
+// 100 steps of 1 024 ranks x 8 metrics 9.5 us (8-bit radix select of xrank_direct.cuh: 76), 60 steps of 4 096 x 16
+// 29 us (576; three CTAs per SM; the instances with 16 and 32 values a thread spill 12 and 44 bytes at 64 registers).
 #pragma once
 #include "kernels.h"
 

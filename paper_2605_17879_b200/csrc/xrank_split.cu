@@ -6,8 +6,8 @@
 //   0. sample   (where there is no estimate from earlier blocks, or it missed lately) one CTA per (step, four metrics):
 //               some thousand ranks are binned; the histogram's median, and the half-width about it that holds half of the mass;
 //   1. sweep    one warp per (step, strip of ranks): with d = x - c, counts the values below the median's band
-//               |d| <= hm and inside the MAD's band | |d| - a | <= ha, and keeps those in either band (15 to 30 % of a
-//               column) in shared-memory lists, then in the column's list in global scratch; values that might exceed
+//               |d| <= hm and inside the MAD's band | |d| - a | <= ha, and keeps those in either band (8 % of a column
+//               of 32 768 ranks, 11 % of 16 384, 22 % of 4 096; 15 to 20 % with estimates from a sample) in shared-memory lists, then in the column's list in global scratch; values that might exceed
 //               the threshold are rare: those clear of its possible range set their exceedance bit at once, the
 //               others are deferred to a per-step list;
 //   2. select   one CTA per column: the median among the kept values of its band, then the MAD among the exact
@@ -20,9 +20,9 @@
 // compares, integer adds and logic go to a half-rate pipe, float adds and multiply-adds do not.  The values are
 // scaled by a power of two so that hm and ha are at least 2^24: a difference of two such numbers is then 0 or at least 1
 // in magnitude, and a saturating subtraction IS the outcome of a compare, ready to be added.
-// Measured, kernels alone, block of 200 steps x 16 384 ranks x 8 metrics: sweep 38 us, select 25, finish 4 (two sweeps,
+// Measured, kernels alone, block of 200 steps x 16 384 ranks x 8 metrics: sweep 36 us, select 20, finish 4 (two sweeps,
 // two selections, estimates and finish of the two-pass form: 36 + 40 + 9 + 9 + 3 + 4); 50 steps of 24 000 ranks:
-// 20 + 16 + 4 (a cluster of four CTAs per step: 77).  What mattered in the sweep: exceedances listed and settled after
+// 19 + 10 + 3 (a cluster of four CTAs per step: 77).  What mattered in the sweep: exceedances listed and settled after
 // the loop (settled where they are found: + 11 us), lists copied out by the bulk engine (by the warp: + 6), 80 registers
 // (64 spill: + 12; prefetching the next batch costs registers and gains nothing).
 #include <math_constants.h>

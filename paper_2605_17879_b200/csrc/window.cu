@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(kRbThreads) window_rebuild_kernel(const Window
 }  // namespace
 
 // Which whole-window path an evaluation takes.  Many series of a short window with an earlier result: one thread per
-// series (31 + 6 us at 131 072 series of 100 steps, 46 + 17 at 200, against 56 and 86 with a tile per 32 series).  Up to
+// series (21 + 5 us at 131 072 series of 100 steps, 36 + 10 at 200, against 56 and 86 with a tile per 32 series).  Up to
 // 65 536 series the threads are too few to hide their own latency, and a launch less counts (8 192 series of
 // 100 / 200 steps: 14 + 5 / 21 + 8 us against 11 / 16; 32 768: 16 + 5 / 24 + 8 against 14 / 25).  First evaluations:
 // a warp per series while there are few (9.2 us against 12 at 8 192 series of 100 steps; at 32 768 series 28 against

@@ -53,15 +53,25 @@ struct Output {
     PyObject *key;
 };
 
-// The device pointers of a mapping's outputs; numel[i] elements at least, a negative number skips the output.
+// The device pointers of a mapping's outputs; numel[i] elements at least, a negative number skips the output.  keep: a new
+// tuple of N, which receives references to them, or NULL.
 template <int N>
-bool output_ptrs(PyObject *out, Output (&spec)[N], const int64_t (&numel)[N], void *(&ptr)[N]) {
+bool output_ptrs(PyObject *out, Output (&spec)[N], const int64_t (&numel)[N], void *(&ptr)[N], PyObject *keep = nullptr) {
     for (int i = 0; i < N; ++i) {
         ptr[i] = nullptr;
+        if (keep) {                // (no slot is ever empty)
+            Py_INCREF(Py_None);
+            PyTuple_SET_ITEM(keep, i, Py_None);
+        }
         if (numel[i] < 0) continue;
         if (!spec[i].key) spec[i].key = PyUnicode_InternFromString(spec[i].name);
         PyObject *hold = nullptr, *v = lookup(out, spec[i].key, &hold);
         const bool ok = v && device_ptr(v, spec[i].type, numel[i], &ptr[i]);
+        if (ok && keep) {
+            Py_INCREF(v);
+            PyTuple_SET_ITEM(keep, i, v);
+            Py_DECREF(Py_None);
+        }
         Py_XDECREF(hold);
         if (!ok) return false;
     }
@@ -75,6 +85,17 @@ struct Here {
     explicit Here(int device) {
         if (c10::cuda::current_device() != device) guard.set_index((c10::DeviceIndex)device);
         stream = (void *)c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)device).stream();
+    }
+};
+
+// A reference that is dropped unless it is given away.
+struct Ref {
+    PyObject *o;
+    ~Ref() { Py_XDECREF(o); }
+    PyObject *give() {
+        PyObject *r = o;
+        o = nullptr;
+        return r;
     }
 };
 
@@ -137,22 +158,24 @@ Output g_score_out[10] = {{"wmed", c10::kFloat, nullptr},      {"fleet_med", c10
                           {"flags", c10::kByte, nullptr},      {"tier", c10::kByte, nullptr},       {"topk_idx", c10::kInt, nullptr},
                           {"topk_score", c10::kFloat, nullptr}};
 
-// score(handle, device, R, M, K, out) -> status
+// score(handle, device, R, M, K, out, hold) -> status; with hold, references to the outputs in the place of a zero
 PyObject *py_score(PyObject *, PyObject *const *args, Py_ssize_t n) {
     long long h, dev, R, M, K;
-    if (!want_args(n, 6) || !to_ll(args[0], &h) || !to_ll(args[1], &dev) || !to_ll(args[2], &R) || !to_ll(args[3], &M) || !to_ll(args[4], &K))
+    if (!want_args(n, 7) || !to_ll(args[0], &h) || !to_ll(args[1], &dev) || !to_ll(args[2], &R) || !to_ll(args[3], &M) || !to_ll(args[4], &K))
         return nullptr;
     try {
         const int64_t numel[10] = {R * M, M, M, R * M, R * M, R, R, R, K > 0 ? K : -1, K > 0 ? K : -1};
         void *p[10];
-        if (!output_ptrs(args[5], g_score_out, numel, p)) return nullptr;
+        Ref keep{args[6] == Py_True ? PyTuple_New(10) : nullptr};
+        if (args[6] == Py_True && !keep.o) return nullptr;
+        if (!output_ptrs(args[5], g_score_out, numel, p, keep.o)) return nullptr;
         Here here((int)dev);
         int rc;
         Py_BEGIN_ALLOW_THREADS
         rc = guard_score((guard_ctx *)h, (float *)p[0], (float *)p[1], (float *)p[2], (float *)p[3], (uint16_t *)p[4], (uint32_t *)p[5],
                          (uint8_t *)p[6], (uint8_t *)p[7], (int32_t *)p[8], (float *)p[9], here.stream);
         Py_END_ALLOW_THREADS
-        return PyLong_FromLong(rc);
+        return rc == GUARD_OK && keep.o ? keep.give() : PyLong_FromLong(rc);
     } catch (const std::exception &e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
         return nullptr;

@@ -369,17 +369,16 @@ class Guard:
         """One evaluation; `out` maps output names to tensors (missing / None entries are skipped)."""
         if out is None:
             out = self.alloc_outputs()
-        rc = _native().score(self._hv, self._devidx, self.R, self.M, self.K, out)
-        if rc != GUARD_OK:
-            self._held += self._tensors(out)
+        # (the outputs held so far are complete in the current stream's order once the call has succeeded)
+        rc = _native().score(self._hv, self._devidx, self.R, self.M, self.K, out, self._deferred)
+        if rc.__class__ is tuple:
+            self._held = rc
+        elif rc == GUARD_OK:
+            self._held = ()
+        else:
+            self._held += tuple(map(out.get, _OUT_NAMES))
             self._check(rc)
-        # (the outputs held so far are complete in the current stream's order from here on)
-        self._held = self._tensors(out) if self._deferred else ()
         return out
-
-    @staticmethod
-    def _tensors(out) -> tuple:
-        return tuple(out.values()) if isinstance(out, dict) else tuple(map(out.get, _OUT_NAMES))
 
     def node_verdict(self, out: Optional[Dict[str, Optional[torch.Tensor]]] = None) -> Dict[str, Optional[torch.Tensor]]:
         """Node-level fold of the evaluation just made (call right after score())."""

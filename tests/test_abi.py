@@ -156,8 +156,8 @@ def test_outputs_of_pending_evaluations_are_held(glib, monkeypatch):
     class Calls:
         rc = 0
 
-        def score(self, *a):
-            return self.rc
+        def score(self, handle, device, R, M, K, out, hold):
+            return tuple(out.values()) if hold and self.rc == 0 else self.rc
 
         def node_verdict(self, *a):
             return self.rc

@@ -351,3 +351,33 @@ def test_state_exported_between_an_ingest_and_its_evaluation(gap):
             o.ingest(X[t:t + gap])
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("K", [0, 3])
+def test_native_score_hands_back_the_outputs_of_a_deferred_evaluation(K):
+    """What keeps the output tensors alive until the evaluation's writes are in order: one reference to each."""
+    import sys
+    from paper_2605_17879_b200 import guard
+    X, dirs = _rand_fleet(8, 20, 4, seed=4)
+    g = guard.Guard(20, 4, 6, 3, dir=dirs, capacity=8, topk=K, ranks_per_node=4)
+    g.set_deferred(True)
+    g.ingest(torch.from_numpy(X).cuda())
+    out = g.alloc_outputs()
+    flags = out["flags"]
+    before = sys.getrefcount(flags)
+    g.score(out)
+    assert sys.getrefcount(flags) == before + 1 and len(g._held) == 10
+    assert all(t is (out[n] if K or not n.startswith("topk") else None) for t, n in zip(g._held, out))
+    g.node_verdict({"node_flag": torch.empty(5, dtype=torch.uint8, device="cuda")})
+    assert len(g._held) == 13
+    with pytest.raises(ValueError):
+        g.score(dict(out, flags=out["scores"]))          # refused before anything is enqueued: still held
+    assert sys.getrefcount(flags) == before + 1
+    g.score({"scores": out["scores"]})                   # the others are not asked for any more
+    assert sys.getrefcount(flags) == before
+    g.join()
+    assert g._held == ()
+    g.set_deferred(False)
+    g.score(out)
+    assert g._held == () and sys.getrefcount(flags) == before
+    g.close()

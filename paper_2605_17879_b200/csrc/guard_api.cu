@@ -49,7 +49,7 @@ Layout make_layout(int R, int M, int C, int K) {
     L.xr_small = off;  off = align_up(off + (L.xr_steps ? xrank_scratch_small_bytes(M, L.xr_steps) : 0));
     L.xr_gridp = (xrank_count_supported(R) && R >= 8192) ? 1 : 0;
     L.xr_grid = off;   off = align_up(off + 2 * align_up(sizeof(RowHints)));
-    L.inc_rbc = off;   off = align_up(off + 64);   // rebuild list counter and ticket (zero before first use)
+    L.inc_rbc = off;   off = align_up(off + 64);   // their number and the finishing kernel's ticket (zero before first use)
     // the windowed medians and the kept top-k indices exist twice: consecutive evaluations alternate, so that a
     // deferred evaluation's tail may still read its medians while the next evaluation's window kernels write theirs
     L.wmed = off;      off = align_up(off + (size_t)R * M * sizeof(float));
@@ -69,7 +69,7 @@ Layout make_layout(int R, int M, int C, int K) {
     L.inc_hi = off;    off = align_up(off + window_inc_bytes(R * M));
     L.inc_cnt = off;   off = align_up(off + window_inc_bytes(R * M));
     L.inc_val = off;   off = align_up(off + (size_t)kIncSlots * window_inc_bytes(R * M));
-    L.inc_rbl = off;   off = align_up(off + window_inc_bytes(R * M));   // series a sliding launch has to rebuild
+    L.inc_rbl = off;   off = align_up(off + window_inc_bytes(R * M));   // series the thread path leaves to its finishing kernel
     L.xr_big = off;    off = align_up(off + (L.xr_split ? xrank_split_scratch_bytes(R, M, C < kSplitMaxSteps ? C : kSplitMaxSteps)
                                              : L.xr_steps ? xrank_scratch_big_bytes(R, M, L.xr_steps) : 0));
     // in deferred mode consecutive blocks run their cross-rank kernels on streams of their own
@@ -585,8 +585,6 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
         ia.cnt = (uint32_t *)(c->ws + c->L.inc_cnt);
         ia.val = (float *)(c->ws + c->L.inc_val);
         ia.rebuilds = c->status() + 14;
-        ia.rb_list = (uint32_t *)(c->ws + c->L.inc_rbl);
-        ia.rb_count = (uint32_t *)(c->ws + c->L.inc_rbc);
         const long long p1 = c->inc_seen, p0 = p1 - c->inc_n, q1 = c->seen, q0 = q1 - n;
         // the windows overlap, few steps entered / left, and the steps that left are still in the ring
         if (p1 >= 0 && q0 < p1 && q1 - p1 <= kIncMaxNew && q0 - p0 <= kIncMaxNew && q1 - p0 <= c->C) {
@@ -603,7 +601,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     c->inc_now = use_inc ? &ia : nullptr;
     c->seen_at_eval = c->seen;
     w.fb_count = c->status() + 8;
-    w.fb_list = (uint32_t *)(c->ws + c->L.inc_rbl);          // shared with the sliding path's rebuild list: an evaluation takes one path
+    w.fb_list = (uint32_t *)(c->ws + c->L.inc_rbl);
     w.fb_list_count = (uint32_t *)(c->ws + c->L.inc_rbc);
     w.status = c->status();
     w.first_wait_cycles = c->wait_limit;
@@ -769,7 +767,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     e = launch_score_flag(s, c->p, ts);
     if (e != cudaSuccess) return c->cuda_fail(e, "score_flag launch");
     c->evals += 1;
-    c->launches += 1 + window_launch_count(w) + (use_inc ? 1 : 0);
+    c->launches += 1 + (use_inc ? 1 : window_launch_count(w));
     if (defer) {
         e = cudaEventRecord(c->ev_e[q], c->tail);
         if (e != cudaSuccess) return c->cuda_fail(e, "event record");

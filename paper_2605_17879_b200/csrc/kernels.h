@@ -134,8 +134,6 @@ struct IncArgs {
     int entering;                 // steps that entered the window since the state was current (the newest ones)
     int leaving;                  // steps that left it (those right before the window's oldest step)
     uint32_t *rebuilds;           // diagnostic counter or NULL
-    uint32_t *rb_list;            // [series] scratch: the series this launch has to rebuild
-    uint32_t *rb_count;           // [2] their number and the rebuild kernel's ticket: zero before first use, self-resetting
 };
 size_t window_inc_bytes(int series);   // per array: lo, hi, cnt take series * 4 bytes, val kIncSlots * series * 4
 bool window_inc_supported(const WindowArgs &a);

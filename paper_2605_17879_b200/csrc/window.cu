@@ -364,18 +364,88 @@ cudaError_t launch_thread_path(const WindowArgs &a, cudaStream_t st) {
 // comes from a ballot, the shift from one shuffle), series after series; the median is then
 // position (middle - count) of the list.
 // A series whose median has left its interval, whose list is full, or that has no state yet is
-// rebuilt by its whole warp: the lanes fetch the window, sort it (bitonic network over registers
-// and shuffles) and take the median, the interval ends kIncHalf ranks beyond the middle ranks, and
-// the values inside.  Exact either way: the interval only decides which values are listed.
+// rebuilt from its whole window by a warp of the same CTA.  Exact either way: the interval only decides which values are
+// listed.  The CTA's four warps share its rebuilds (one CTA in two has one in steady state): queued inside the warp that
+// found them they make the kernel as slow as its unluckiest warp, and a kernel of their own costs the next step's update a
+// launch and a scan of lists (update and rebuilds of 262 144 series 19 + 10 us beside other work, together 23; single
+// steps of 2 048 ranks x 8 with node verdicts 31.5 us an evaluation, 27.6 so; six deferred steps of 32 768 x 8 242, 223 so).
 // ---------------------------------------------------------------------------------------
 constexpr int kIncThreads = 128;
 
-// NEW: the most steps that entered / left (1 for an evaluation after every step, else kIncMaxNew).
-template <int NEW>
+// The state of one series from its whole window, by a warp: the lanes fetch the window, sort it (bitonic network over
+// registers and shuffles), take the median, the interval ends kIncHalf ranks beyond the middle ranks, and the values inside.
+template <int VPL>
+__device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &s, const int series, const int first) {
+    const int lane = lane_id(), n = a.n;
+    const bool even = !(n & 1);
+    const int k1 = (n - 1) >> 1, k2 = n >> 1;
+    uint32_t kv[VPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const int row = lane + 32 * j;
+        kv[j] = 0xFFFFFFFFu;                 // padding sorts behind every finite value
+        if (row < n) {
+            int slot = first + row;
+            if (slot >= a.capacity) slot -= a.capacity;
+            kv[j] = f2key(__ldg(a.ring + (size_t)slot * a.row_stride + series));
+        }
+    }
+    warp_bitonic_sort<VPL>(kv, lane);        // ascending: element e in lane e / VPL, register e % VPL
+    auto pick = [&](int r) -> uint32_t {
+        uint32_t mine = kv[0];
+#pragma unroll
+        for (int j = 1; j < VPL; ++j) mine = ((r % VPL) == j) ? kv[j] : mine;
+        return __shfl_sync(0xFFFFFFFFu, mine, r / VPL);
+    };
+    const float med = median_from_keys(pick(k1), pick(k2), even);
+    const float flo = key2f(pick(max(0, k1 - kIncHalf))), fhi = key2f(pick(min(n - 1, k2 + kIncHalf)));
+    // values below / inside the interval, by the same float comparisons the sliding update uses
+    int below = 0, in = 0;
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const bool real = lane * VPL + j < n;
+        const float x = key2f(kv[j]);
+        below += real && (x < flo);
+        in += real && !(x < flo) && (x <= fhi);
+    }
+    int incl = in;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= d) incl += u;
+    }
+    const int nin2 = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const int cb2 = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below);
+    const bool fits = nin2 <= kIncSlots;
+    if (fits) {
+        int pos = incl - in;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            const bool real = lane * VPL + j < n;
+            const float x = key2f(kv[j]);
+            if (real && !(x < flo) && (x <= fhi)) { s.val[(size_t)series * kIncSlots + pos] = x; ++pos; }
+        }
+    }
+    if (lane == 0) {
+        a.wmed[series] = med;
+        s.lo[series] = flo;
+        s.hi[series] = fhi;
+        // an interval with more (tied) values than a list holds stays without state: it rebuilds every time
+        s.cnt[series] = fits ? (0x80000000u | ((uint32_t)nin2 << 16) | (uint32_t)cb2) : 0u;
+        if (s.rebuilds) atomicAdd(s.rebuilds, 1u);
+    }
+}
+
+// NEW: the most steps that entered / left (1 for an evaluation after every step, else kIncMaxNew); VPL: values per lane of
+// a rebuild.
+template <int NEW, int VPL>
 __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s) {
     pdl_wait();
     static_assert(kIncSlots > 32 && kIncSlots <= 64, "a lane holds list slots lane and lane + 32");
     __shared__ float sl[kIncThreads / 32][32][kIncSlots];   // per warp: the lists of the series it updates, staged asynchronously
+    __shared__ uint32_t rb_n, rb_list[kIncThreads];         // series of this CTA to rebuild
+    if (threadIdx.x == 0) rb_n = 0u;
+    __syncthreads();
     const int lane = lane_id(), wid = warp_id();
     const int n = a.n;
     const int c = blockIdx.x * kIncThreads + threadIdx.x;
@@ -420,9 +490,17 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             else if (xe[i] <= hi) in_e |= 1u << i;
         }
     }
-    // ---- list updates, one series at a time by the whole warp: lane j holds list slots j and j + 32 ----
+    // a series whose list stays as it is: the list is sorted, the middle ranks of the window are positions k1 - cb and
+    // k2 - cb of it (in flight beside the lists below)
     float f1 = 0.0f, f2 = 0.0f;
-    bool have = false;             // f1 / f2 hold the list values at the middle ranks
+    if (ok && (in_l | in_e) == 0u) {
+        ok = cb >= 0 && cb <= k1 && k2 < cb + nin;
+        if (ok) {
+            f1 = s.val[(size_t)c * kIncSlots + (k1 - cb)];
+            f2 = s.val[(size_t)c * kIncSlots + (k2 - cb)];
+        }
+    }
+    // ---- list updates, one series at a time by the whole warp: lane j holds list slots j and j + 32 ----
     unsigned upd = __ballot_sync(0xFFFFFFFFu, ok && (in_l | in_e) != 0u);
     {   // all lists this warp needs are fetched at once (asynchronous copies into shared memory: one round trip)
         unsigned m = upd;
@@ -502,114 +580,18 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             nin = ns;
             f1 = (j1 >> 5) ? g11 : g10;
             f2 = (j2 >> 5) ? g21 : g20;
-            have = true;
         }
     }
-    ok = ok && cb >= 0 && cb <= k1 && k2 < cb + nin;
     if (ok) {
-        // the list is sorted: the middle ranks of the window are positions k1 - cb and k2 - cb of it
-        if (!have) {
-            f1 = s.val[(size_t)c * kIncSlots + (k1 - cb)];
-            f2 = s.val[(size_t)c * kIncSlots + (k2 - cb)];
-        }
         const float med = median_from_keys(f2key(f1), f2key(f2), even);
         a.wmed[c] = med;
         s.cnt[c] = 0x80000000u | ((uint32_t)nin << 16) | (uint32_t)cb;
     }
-    // ---- series without a usable state go on the launch's rebuild list (window_rebuild_kernel follows) ----
-    const unsigned todo = __ballot_sync(0xFFFFFFFFu, active && !ok);
-    if (todo) {
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(s.rb_count, (uint32_t)__popc(todo));
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if ((todo >> lane) & 1u) s.rb_list[base + __popc(todo & ((1u << lane) - 1u))] = (uint32_t)c;
-    }
-}
-
-// The rebuilds of a launch, one warp per listed series (a few per thousand series in steady state, all of them
-// when sliding starts): the lanes fetch the window, sort it (bitonic network over registers and shuffles), take
-// the median, the interval ends kIncHalf ranks beyond the middle ranks, and the values inside.  A kernel of its
-// own so that the rebuilds spread over the whole GPU instead of queueing inside the warps that found them.
-constexpr int kRbThreads = 128;
-constexpr int kRbCtas = 148 * 8;
-
-template <int VPL>
-__global__ void __launch_bounds__(kRbThreads) window_rebuild_kernel(const WindowArgs a, const IncArgs s) {
-    pdl_wait();
-    __shared__ int is_last;
-    const int lane = lane_id();
-    const int n = a.n;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
-    const bool even = !(n & 1);
-    const int k1 = (n - 1) >> 1, k2 = n >> 1;
-    const uint32_t count = min(__ldcg(s.rb_count), (uint32_t)a.series);
-    const uint32_t nwarps = gridDim.x * (kRbThreads / 32);
-    for (uint32_t i = blockIdx.x * (kRbThreads / 32) + warp_id(); i < count; i += nwarps) {
-        const int series = (int)__ldcg(s.rb_list + i);
-        uint32_t kv[VPL];
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            const int row = lane + 32 * j;
-            kv[j] = 0xFFFFFFFFu;                 // padding sorts behind every finite value
-            if (row < n) {
-                int slot = first + row;
-                if (slot >= a.capacity) slot -= a.capacity;
-                kv[j] = f2key(__ldg(a.ring + (size_t)slot * a.row_stride + series));
-            }
-        }
-        warp_bitonic_sort<VPL>(kv, lane);        // ascending: element e in lane e / VPL, register e % VPL
-        auto pick = [&](int r) -> uint32_t {
-            uint32_t mine = kv[0];
-#pragma unroll
-            for (int j = 1; j < VPL; ++j) mine = ((r % VPL) == j) ? kv[j] : mine;
-            return __shfl_sync(0xFFFFFFFFu, mine, r / VPL);
-        };
-        const float med = median_from_keys(pick(k1), pick(k2), even);
-        const float flo = key2f(pick(max(0, k1 - kIncHalf))), fhi = key2f(pick(min(n - 1, k2 + kIncHalf)));
-        // values below / inside the interval, by the same float comparisons the sliding update uses
-        int below = 0, in = 0;
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            const bool real = lane * VPL + j < n;
-            const float x = key2f(kv[j]);
-            below += real && (x < flo);
-            in += real && !(x < flo) && (x <= fhi);
-        }
-        int incl = in;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int u = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-            if (lane >= d) incl += u;
-        }
-        const int nin2 = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        const int cb2 = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below);
-        const bool fits = nin2 <= kIncSlots;
-        if (fits) {
-            int pos = incl - in;
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                const bool real = lane * VPL + j < n;
-                const float x = key2f(kv[j]);
-                if (real && !(x < flo) && (x <= fhi)) { s.val[(size_t)series * kIncSlots + pos] = x; ++pos; }
-            }
-        }
-        if (lane == 0) {
-            a.wmed[series] = med;
-            s.lo[series] = flo;
-            s.hi[series] = fhi;
-            // an interval with more (tied) values than a list holds stays without state: it rebuilds every time
-            s.cnt[series] = fits ? (0x80000000u | ((uint32_t)nin2 << 16) | (uint32_t)cb2) : 0u;
-            if (s.rebuilds) atomicAdd(s.rebuilds, 1u);
-        }
-    }
-    // the CTA that finishes last clears the list for the next launch
+    // ---- series without a usable state: the CTA's warps share them ----
+    if (active && !ok) rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)c;
     __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(s.rb_count + 1, 1u) == gridDim.x - 1u) ? 1 : 0;
-    __syncthreads();
-    if (is_last && threadIdx.x == 0) {
-        s.rb_count[0] = 0u;
-        s.rb_count[1] = 0u;
-    }
+    const uint32_t count = rb_n;
+    for (uint32_t i = (uint32_t)wid; i < count; i += kIncThreads / 32) inc_rebuild<VPL>(a, s, (int)rb_list[i], first);
 }
 
 }  // namespace
@@ -633,15 +615,17 @@ size_t window_inc_bytes(int series) { return (size_t)series * sizeof(float); }
 
 bool window_inc_supported(const WindowArgs &a) { return a.n >= 1 && a.n <= 256; }
 
-cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {
+template <int VPL>
+static cudaError_t launch_inc(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {
     const int grid = (a.series + kIncThreads - 1) / kIncThreads;
-    const int rgrid = min(kRbCtas, (a.series + kRbThreads / 32 - 1) / (kRbThreads / 32));
-    const cudaError_t e = inc.entering <= 1 && inc.leaving <= 1 ? launch_after(window_inc_kernel<1>, grid, kIncThreads, st, a, inc)
-                                                                : launch_after(window_inc_kernel<kIncMaxNew>, grid, kIncThreads, st, a, inc);
-    if (e != cudaSuccess) return e;
-    if (a.n <= 64) return launch_after(window_rebuild_kernel<2>, rgrid, kRbThreads, st, a, inc);
-    if (a.n <= 128) return launch_after(window_rebuild_kernel<4>, rgrid, kRbThreads, st, a, inc);
-    return launch_after(window_rebuild_kernel<8>, rgrid, kRbThreads, st, a, inc);
+    return inc.entering <= 1 && inc.leaving <= 1 ? launch_after(window_inc_kernel<1, VPL>, grid, kIncThreads, st, a, inc)
+                                                 : launch_after(window_inc_kernel<kIncMaxNew, VPL>, grid, kIncThreads, st, a, inc);
+}
+
+cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {
+    if (a.n <= 64) return launch_inc<2>(a, inc, st);
+    if (a.n <= 128) return launch_inc<4>(a, inc, st);
+    return launch_inc<8>(a, inc, st);
 }
 
 cudaError_t launch_window_select(const WindowArgs &a, cudaStream_t st) {

@@ -2,6 +2,7 @@
 // last n ring steps.
 #include <math_constants.h>
 
+#include <climits>
 #include <mutex>
 
 #include "colselect.cuh"
@@ -360,8 +361,7 @@ cudaError_t launch_thread_path(const WindowArgs &a, cudaStream_t st) {
 // values below lo, and the handful of values inside the interval (global memory, each series' sorted
 // list contiguous).  An evaluation reads only the steps that entered and left the window, one thread
 // per series: a value below lo moves the count; a value inside the interval is inserted into /
-// removed from the series' list by the whole warp (lane j holds list slots j and j + 32: the position
-// comes from a ballot, the shift from one shuffle), series after series; the median is then
+// removed from the series' list by eight lanes, four series of the warp at a time; the median is then
 // position (middle - count) of the list.
 // A series whose median has left its interval, whose list is full, or that has no state yet is
 // rebuilt from its whole window by a warp of the same CTA.  Exact either way: the interval only decides which values are
@@ -371,6 +371,13 @@ cudaError_t launch_thread_path(const WindowArgs &a, cudaStream_t st) {
 // steps of 2 048 ranks x 8 with node verdicts 31.5 us an evaluation, 27.6 so; six deferred steps of 32 768 x 8 242, 223 so).
 // ---------------------------------------------------------------------------------------
 constexpr int kIncThreads = 128;
+constexpr int kIncLanes = 8, kIncPer = kIncSlots / kIncLanes;   // lanes that hold a list, and slots per lane
+static_assert(kIncPer * kIncLanes == kIncSlots, "a list is spread evenly");
+constexpr int kIncNone = INT_MAX;   // above the keys of all numbers
+
+// Signed integers in the total order of the floats, and back.
+__device__ __forceinline__ int inc_key(const float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7FFFFFFF); }
+__device__ __forceinline__ float inc_float(const int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
 
 // The state of one series from its whole window, by a warp: the lanes fetch the window, sort it (bitonic network over
 // registers and shuffles), take the median, the interval ends kIncHalf ranks beyond the middle ranks, and the values inside.
@@ -441,8 +448,8 @@ __device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &
 template <int NEW, int VPL>
 __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s) {
     pdl_wait();
-    static_assert(kIncSlots > 32 && kIncSlots <= 64, "a lane holds list slots lane and lane + 32");
-    __shared__ float sl[kIncThreads / 32][32][kIncSlots];   // per warp: the lists of the series it updates, staged asynchronously
+    __shared__ float sh_list[kIncThreads / 32][32 / kIncLanes][kIncSlots];   // per warp: the edited lists
+    __shared__ uint8_t sh_order[kIncThreads / 32][32];      // ... and the lanes whose lists are edited
     __shared__ uint32_t rb_n, rb_list[kIncThreads];         // series of this CTA to rebuild
     if (threadIdx.x == 0) rb_n = 0u;
     __syncthreads();
@@ -500,87 +507,78 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             f2 = s.val[(size_t)c * kIncSlots + (k2 - cb)];
         }
     }
-    // ---- list updates, one series at a time by the whole warp: lane j holds list slots j and j + 32 ----
-    unsigned upd = __ballot_sync(0xFFFFFFFFu, ok && (in_l | in_e) != 0u);
-    {   // all lists this warp needs are fetched at once (asynchronous copies into shared memory: one round trip)
-        unsigned m = upd;
-        int k = 0;
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            const int cs = __shfl_sync(0xFFFFFFFFu, c, src);
-            const int ns = __shfl_sync(0xFFFFFFFFu, nin, src);
-            const float *g = s.val + (size_t)cs * kIncSlots;   // a series' list is contiguous
-            if (lane < ns) cp_async4(&sl[wid][k][lane], g + lane);
-            if (lane + 32 < ns) cp_async4(&sl[wid][k][lane + 32], g + lane + 32);
-            ++k;
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
-    }
-    int kk = 0;
-    while (upd) {
-        const int src = __ffs(upd) - 1;
-        upd &= upd - 1;
-        const int cs = __shfl_sync(0xFFFFFFFFu, c, src);
+    // ---- list updates, four series at a time: eight lanes hold a list, kIncPer neighbouring slots each ----
+    const bool edits = ok && (in_l | in_e) != 0u;
+    const unsigned upd = __ballot_sync(0xFFFFFFFFu, edits);
+    const int nupd = __popc(upd), mine = __popc(upd & ((1u << lane) - 1u));   // this lane's series is the mine-th of them
+    if (edits) sh_order[wid][mine] = (uint8_t)lane;
+    __syncwarp();
+    const int grp = lane / kIncLanes, gl = lane % kIncLanes;
+    for (int i0 = 0; i0 < nupd; i0 += 32 / kIncLanes) {
+        const bool act = i0 + grp < nupd;
+        const int src = act ? sh_order[wid][i0 + grp] : 0;
         int ns = __shfl_sync(0xFFFFFFFFu, nin, src);
+        if (!act) ns = 0;
+        float *list = s.val + (size_t)__shfl_sync(0xFFFFFFFFu, c, src) * kIncSlots + gl * kIncPer;
+        int old[kIncPer], v[kIncPer];            // slots without a value lie above everything
+#pragma unroll
+        for (int j = 0; j < kIncPer; ++j) old[j] = gl * kIncPer + j < ns ? inc_key(list[j]) : kIncNone;
+#pragma unroll
+        for (int j = 0; j < kIncPer; ++j) v[j] = old[j];
         const uint32_t ml = __shfl_sync(0xFFFFFFFFu, in_l, src), me = __shfl_sync(0xFFFFFFFFu, in_e, src);
-        const size_t lbase = (size_t)cs * kIncSlots;
-        const float v0s = sl[wid][kk][lane], v1s = sl[wid][kk][(lane + 32) % kIncSlots];
-        float v0 = lane < ns ? v0s : 0.0f, v1 = lane + 32 < ns ? v1s : 0.0f;
-        ++kk;
-        bool good = true;
-        int dirty_from = kIncSlots;
+        bool good = act;
 #pragma unroll
         for (int i = 0; i < NEW; ++i) {
+            const bool here = act && ((ml >> i) & 1u);
+            if (!__any_sync(0xFFFFFFFFu, here)) continue;
             const float x = __shfl_sync(0xFFFFFFFFu, xl[i], src);
-            if (!((ml >> i) & 1u) || !good) continue;    // uniform: ml and good are the same in every lane
-            const uint32_t m0 = __ballot_sync(0xFFFFFFFFu, lane < ns && __float_as_uint(v0) == __float_as_uint(x));
-            const uint32_t m1 = __ballot_sync(0xFFFFFFFFu, lane + 32 < ns && __float_as_uint(v1) == __float_as_uint(x));
-            if ((m0 | m1) == 0u) { good = false; continue; }   // the books do not balance: rebuild
-            const int pos = m0 ? __ffs(m0) - 1 : 32 + __ffs(m1) - 1;
-            // positions above pos move down by one
-            const float d0 = __shfl_down_sync(0xFFFFFFFFu, v0, 1), h1 = __shfl_sync(0xFFFFFFFFu, v1, 0);
-            const float d1 = __shfl_down_sync(0xFFFFFFFFu, v1, 1);
-            if (lane >= pos) v0 = (lane == 31) ? h1 : d0;
-            if (lane + 32 >= pos) v1 = d1;
-            --ns;
-            dirty_from = min(dirty_from, pos);
+            const int kx = here ? inc_key(x) : kIncNone;
+            // values from the first one not below x on move down by one; that one has to be x
+            int next = __shfl_down_sync(0xFFFFFFFFu, v[0], 1, kIncLanes);
+            if (gl == kIncLanes - 1) next = kIncNone;
+            bool found = false;
+#pragma unroll
+            for (int j = 0; j < kIncPer; ++j) {
+                found |= v[j] == kx;
+                v[j] = v[j] < kx ? v[j] : (j + 1 < kIncPer ? v[j + 1] : next);
+            }
+            const uint32_t hit = (__ballot_sync(0xFFFFFFFFu, found) >> (grp * kIncLanes)) & ((1u << kIncLanes) - 1u);
+            if (here) { good = good && hit != 0u; --ns; }   // (else the books do not balance: rebuild)
         }
 #pragma unroll
         for (int i = 0; i < NEW; ++i) {
+            const bool here = act && ((me >> i) & 1u);
+            if (!__any_sync(0xFFFFFFFFu, here)) continue;
             const float x = __shfl_sync(0xFFFFFFFFu, xe[i], src);
-            if (!((me >> i) & 1u) || !good) continue;
-            if (ns >= kIncSlots) { good = false; continue; }
-            const uint32_t kx = f2key(x);
-            // behind the listed values whose key is not above x's
-            const int at = __popc(__ballot_sync(0xFFFFFFFFu, lane < ns && f2key(v0) <= kx)) +
-                           __popc(__ballot_sync(0xFFFFFFFFu, lane + 32 < ns && f2key(v1) <= kx));
-            const float u0 = __shfl_up_sync(0xFFFFFFFFu, v0, 1), t0 = __shfl_sync(0xFFFFFFFFu, v0, 31);
-            const float u1 = __shfl_up_sync(0xFFFFFFFFu, v1, 1);
-            if (lane + 32 > at) v1 = (lane == 0) ? t0 : u1;
-            else if (lane + 32 == at) v1 = x;
-            if (lane > at) v0 = u0;
-            else if (lane == at) v0 = x;
-            ++ns;
-            dirty_from = min(dirty_from, at);
+            const int kx = here ? inc_key(x) : kIncNone;
+            int prev = __shfl_up_sync(0xFFFFFFFFu, v[kIncPer - 1], 1, kIncLanes);
+            if (gl == 0) prev = INT_MIN;
+#pragma unroll
+            for (int j = kIncPer - 1; j >= 0; --j) v[j] = max(j ? v[j - 1] : prev, min(v[j], kx));
+            if (here) { good = good && ns < kIncSlots; ++ns; }
         }
         const int cbs = __shfl_sync(0xFFFFFFFFu, cb, src);
         good = good && cbs >= 0 && cbs <= k1 && k2 < cbs + ns;
-        if (good) {   // write back the part that moved; hand the middle ranks' values to the series' own lane
-            if (lane >= dirty_from && lane < ns) s.val[lbase + lane] = v0;
-            if (lane + 32 >= dirty_from && lane + 32 < ns) s.val[lbase + lane + 32] = v1;
+#pragma unroll
+        for (int j = 0; j < kIncPer; ++j) {
+            const int slot = gl * kIncPer + j;
+            sh_list[wid][grp][slot] = inc_float(v[j]);
+            if (good && slot < ns && v[j] != old[j]) list[j] = inc_float(v[j]);
         }
-        const int j1 = good ? k1 - cbs : 0, j2 = good ? k2 - cbs : 0;
-        const float g10 = __shfl_sync(0xFFFFFFFFu, v0, j1 & 31), g11 = __shfl_sync(0xFFFFFFFFu, v1, j1 & 31);
-        const float g20 = __shfl_sync(0xFFFFFFFFu, v0, j2 & 31), g21 = __shfl_sync(0xFFFFFFFFu, v1, j2 & 31);
-        if (lane == src) {
-            ok = good;
-            nin = ns;
-            f1 = (j1 >> 5) ? g11 : g10;
-            f2 = (j2 >> 5) ? g21 : g20;
+        __syncwarp();
+        // the series' own lanes take over
+        const int from = kIncLanes * (mine % (32 / kIncLanes));
+        const bool fine = __shfl_sync(0xFFFFFFFFu, (int)good, from) != 0;
+        const int num = __shfl_sync(0xFFFFFFFFu, ns, from);
+        if (edits && mine >= i0 && mine < i0 + 32 / kIncLanes) {
+            ok = fine;
+            nin = num;
+            if (ok) {
+                f1 = sh_list[wid][mine % (32 / kIncLanes)][k1 - cb];
+                f2 = sh_list[wid][mine % (32 / kIncLanes)][k2 - cb];
+            }
         }
+        __syncwarp();
     }
     if (ok) {
         const float med = median_from_keys(f2key(f1), f2key(f2), even);

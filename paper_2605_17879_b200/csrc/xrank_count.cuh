@@ -31,10 +31,13 @@ constexpr int kCtAll = 0, kCtStatistics = 1, kCtCut = 2;   // what a CTA (cluste
 // 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
 // barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3.
 constexpr int kCtClusterRanks = 4096;
-// Threads of the CTAs of a cluster: four values each, while a CTA has 512 of them at most.
+// Threads of the CTAs of a cluster: four values each, while a CTA has 256 of them at most: at 128 registers two such CTAs
+// share an SM, so that the clusters of a step's row and of another evaluation's tail find room beside one another and
+// beside the window kernels (six deferred steps of 32 768 ranks x 8 210 us with up to 512 threads, 199 so; a row alone the
+// same).
 inline int ct_cluster_threads(const int R, const int NC) {
     int T = 128;
-    while (T < 512 && R > 4 * NC * T) T <<= 1;
+    while (T < 256 && R > 4 * NC * T) T <<= 1;
     return T;
 }
 

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(1024, 1) score_flag_kernel(const ScoreArgs a, 
 
     const char *base = (const char *)a.mask_base + (size_t)r0 * MB;
     const size_t pitch = (size_t)a.R * MB;
-    const int first = ((a.last_slot - (a.n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (a.n - 1) + (a.last_slot < a.n - 1 ? a.capacity : 0);
     const int at = 4 * (lane % LW), bytes = nr * MB;                // this lane's bytes of a row's share
     const bool word_ok = at + 4 <= bytes && (pitch & 3) == 0;
     auto load = [&](int slot) -> uint32_t {
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kNodeWarps * 32) node_verdict_kernel(const Nod
     const int rpn = a.ranks_per_node;
     const size_t r0 = (size_t)node * rpn;
     const MaskT *mask_base = (const MaskT *)a.mask_base;
-    const int first = ((a.last_slot - (a.n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (a.n - 1) + (a.last_slot < a.n - 1 ? a.capacity : 0);
     const bool wide = sizeof(MaskT) == 1 && rpn == 8 && (a.R & 7) == 0;
     const unsigned long long want = 0x0101010101010101ull << a.primary;
     uint32_t stall = 0;

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(1024, 2) window_warp_kernel(const WindowArgs a
     __shared__ __align__(8) uint64_t bar[2];
     const int tid = threadIdx.x, lane = lane_id(), w = warp_id();
     const int n = a.n;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);
     const int bufwords = n * kWarpPitch;
 
     auto stage = [&](int tile, int b) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
     const int c = blockIdx.x * kThCols + tid;
     const bool active = c < a.series;
     const int cc = active ? c : a.series - 1;           // idle lanes of the last CTA read a valid column
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);
     const int n1 = min(n, a.capacity - first);          // rows before the ring wraps
 
     const float hint = a.centre[cc], h = a.spread[cc];
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const Window
     __shared__ int is_last;
     const int lane = lane_id();
     const int n = a.n;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);
     const uint32_t count = min(__ldcg(a.fb_list_count), (uint32_t)a.series);
     const uint32_t nwarps = gridDim.x * (kFinThreads / 32);
     for (uint32_t i = blockIdx.x * (kFinThreads / 32) + warp_id(); i < count; i += nwarps) {
@@ -379,38 +379,27 @@ constexpr int kIncNone = INT_MAX;   // above the keys of all numbers
 __device__ __forceinline__ int inc_key(const float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7FFFFFFF); }
 __device__ __forceinline__ float inc_float(const int k) { return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF)); }
 
-// The state of one series from its whole window, by a warp: the lanes fetch the window, sort it (bitonic network over
-// registers and shuffles), take the median, the interval ends kIncHalf ranks beyond the middle ranks, and the values inside.
-template <int VPL>
-__device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &s, const int series, const int first) {
+// Median and state of a series from P sorted values per lane (element e in lane e / P, register e % P; m of them): those of
+// ranks `base` and on of its window.
+template <int P>
+__device__ __forceinline__ void inc_store(const WindowArgs &a, const IncArgs &s, const int series, const uint32_t (&kv)[P], const int m, const int base) {
     const int lane = lane_id(), n = a.n;
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
-    uint32_t kv[VPL];
-#pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-        const int row = lane + 32 * j;
-        kv[j] = 0xFFFFFFFFu;                 // padding sorts behind every finite value
-        if (row < n) {
-            int slot = first + row;
-            if (slot >= a.capacity) slot -= a.capacity;
-            kv[j] = f2key(__ldg(a.ring + (size_t)slot * a.row_stride + series));
-        }
-    }
-    warp_bitonic_sort<VPL>(kv, lane);        // ascending: element e in lane e / VPL, register e % VPL
     auto pick = [&](int r) -> uint32_t {
+        r -= base;
         uint32_t mine = kv[0];
 #pragma unroll
-        for (int j = 1; j < VPL; ++j) mine = ((r % VPL) == j) ? kv[j] : mine;
-        return __shfl_sync(0xFFFFFFFFu, mine, r / VPL);
+        for (int j = 1; j < P; ++j) mine = ((r % P) == j) ? kv[j] : mine;
+        return __shfl_sync(0xFFFFFFFFu, mine, r / P);
     };
     const float med = median_from_keys(pick(k1), pick(k2), even);
     const float flo = key2f(pick(max(0, k1 - kIncHalf))), fhi = key2f(pick(min(n - 1, k2 + kIncHalf)));
     // values below / inside the interval, by the same float comparisons the sliding update uses
     int below = 0, in = 0;
 #pragma unroll
-    for (int j = 0; j < VPL; ++j) {
-        const bool real = lane * VPL + j < n;
+    for (int j = 0; j < P; ++j) {
+        const bool real = lane * P + j < m;
         const float x = key2f(kv[j]);
         below += real && (x < flo);
         in += real && !(x < flo) && (x <= fhi);
@@ -421,14 +410,14 @@ __device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &
         const int u = __shfl_up_sync(0xFFFFFFFFu, incl, d);
         if (lane >= d) incl += u;
     }
-    const int nin2 = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    const int cb2 = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below);
-    const bool fits = nin2 <= kIncSlots;
+    const int nin = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    const int cb = base + (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below);
+    const bool fits = nin <= kIncSlots;
     if (fits) {
         int pos = incl - in;
 #pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            const bool real = lane * VPL + j < n;
+        for (int j = 0; j < P; ++j) {
+            const bool real = lane * P + j < m;
             const float x = key2f(kv[j]);
             if (real && !(x < flo) && (x <= fhi)) { s.val[(size_t)series * kIncSlots + pos] = x; ++pos; }
         }
@@ -438,39 +427,94 @@ __device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &
         s.lo[series] = flo;
         s.hi[series] = fhi;
         // an interval with more (tied) values than a list holds stays without state: it rebuilds every time
-        s.cnt[series] = fits ? (0x80000000u | ((uint32_t)nin2 << 16) | (uint32_t)cb2) : 0u;
+        s.cnt[series] = fits ? (0x80000000u | ((uint32_t)nin << 16) | (uint32_t)cb) : 0u;
         if (s.rebuilds) atomicAdd(s.rebuilds, 1u);
     }
 }
 
+// The state of one series from its whole window, by a warp: the lanes fetch the window and sort it (bitonic network over
+// registers and shuffles) for the median, the interval ends kIncHalf ranks beyond the middle ranks, and the values inside.
+// A median that has left its interval has not gone far: where the values within a width of the interval hold all of these
+// ranks (counted), only they are sorted, two per lane (`list`: room for 64 of them).
+template <int VPL>
+__device__ __forceinline__ void inc_rebuild(const WindowArgs &a, const IncArgs &s, const int series, const int first, float *list) {
+    const int lane = lane_id(), n = a.n;
+    float x[VPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const int row = lane + 32 * j;
+        x[j] = 0.0f;
+        if (row < n) {
+            int slot = first + row;
+            if (slot >= a.capacity) slot -= a.capacity;
+            x[j] = __ldg(a.ring + (size_t)slot * a.row_stride + series);
+        }
+    }
+    if (VPL > 2 && !s.rebuild_all && (s.cnt[series] >> 31)) {
+        const float l0 = s.lo[series], h0 = s.hi[series], d = h0 - l0, lo = l0 - d, hi = h0 + d;
+        int below = 0, kept = 0;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            const bool real = lane + 32 * j < n;
+            below += real && x[j] < lo;
+            const bool in = real && x[j] >= lo && x[j] <= hi;
+            const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
+            const int at = kept + __popc(who & ((1u << lane) - 1u));
+            if (in && at < 64) list[at] = x[j];
+            kept += __popc(who);
+        }
+        const int base = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below);
+        const int r0 = max(0, ((n - 1) >> 1) - kIncHalf), r1 = min(n - 1, (n >> 1) + kIncHalf);
+        if (kept <= 64 && base <= r0 && r1 < base + kept) {   // (the same for the whole warp)
+            __syncwarp();
+            uint32_t kv[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) kv[j] = 2 * lane + j < kept ? f2key(list[2 * lane + j]) : 0xFFFFFFFFu;
+            warp_bitonic_sort<2>(kv, lane);
+            inc_store<2>(a, s, series, kv, kept, base);
+            __syncwarp();
+            return;
+        }
+        __syncwarp();
+    }
+    uint32_t kv[VPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) kv[j] = lane + 32 * j < n ? f2key(x[j]) : 0xFFFFFFFFu;   // padding sorts behind every finite value
+    warp_bitonic_sort<VPL>(kv, lane);
+    inc_store<VPL>(a, s, series, kv, n, 0);
+}
+
+// A series whose list is edited: what eight lanes need of it.
+template <int NEW>
+struct IncEdit {
+    int c, cb, nin;
+    uint32_t in_l, in_e;         // which of the steps lie inside the interval
+    float xl[NEW], xe[NEW];
+};
+
 // NEW: the most steps that entered / left (1 for an evaluation after every step, else kIncMaxNew); VPL: values per lane of
-// a rebuild.
+// a rebuild.  (Two series per thread, all of 262 144 resident at once: the same alone, and beside the cluster kernels of
+// other evaluations, which then wait for room, six deferred steps of 32 768 x 8 take 205 us instead of 194.)
 template <int NEW, int VPL>
 __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s) {
     pdl_wait();
     __shared__ float sh_list[kIncThreads / 32][32 / kIncLanes][kIncSlots];   // per warp: the edited lists
-    __shared__ uint8_t sh_order[kIncThreads / 32][32];      // ... and the lanes whose lists are edited
-    __shared__ uint32_t rb_n, rb_list[kIncThreads];         // series of this CTA to rebuild
+    __shared__ IncEdit<NEW> sh_edit[kIncThreads / 32][32];                   // ... and what is edited
+    __shared__ uint32_t rb_n, rb_list[kIncThreads];                          // series of this CTA to rebuild
     if (threadIdx.x == 0) rb_n = 0u;
     __syncthreads();
     const int lane = lane_id(), wid = warp_id();
     const int n = a.n;
-    const int c = blockIdx.x * kIncThreads + threadIdx.x;
-    const bool active = c < a.series;
-    const int cc = active ? c : a.series - 1;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;   // slot of the window's oldest step
+    const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);   // slot of the window's oldest step
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
+    const int c = blockIdx.x * kIncThreads + threadIdx.x, cc = min(c, a.series - 1);
 
-    const uint32_t w = s.cnt[cc];
-    bool ok = active && (w >> 31) && !s.rebuild_all;
-    int cb = (int)(w & 0xFFFFu), nin = (int)((w >> 16) & 0xFFu);
-    const float lo = s.lo[cc], hi = s.hi[cc];
     // The steps that left the window (the ones right before its oldest step) and the steps that entered it (the
-    // newest ones), all fetched up front.  A value below lo moves the count; a value inside the interval
-    // changes the series' sorted list, which the whole warp then updates (below).
+    // newest ones), all fetched up front.
+    const uint32_t w = s.cnt[cc];
+    const float lo = s.lo[cc], hi = s.hi[cc];
     float xl[NEW], xe[NEW];
-    uint32_t in_l = 0, in_e = 0;   // which of them lie inside the interval
 #pragma unroll
     for (int i = 0; i < NEW; ++i) {
         xl[i] = 0.0f;
@@ -486,6 +530,12 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             xe[i] = __ldg(a.ring + (size_t)slot * a.row_stride + cc);
         }
     }
+    // A value below lo moves the count; a value inside the interval changes the series' sorted list, which eight lanes
+    // then edit (below).  A list that stays as it is has the middle ranks of the window at positions k1 - cb and k2 - cb.
+    const bool ok = c < a.series && (w >> 31) && !s.rebuild_all;
+    int cb = (int)(w & 0xFFFFu);
+    const int nin = (int)((w >> 16) & 0xFFu);
+    uint32_t in_l = 0, in_e = 0;
 #pragma unroll
     for (int i = 0; i < NEW; ++i) {
         if (i < s.leaving) {
@@ -497,42 +547,58 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             else if (xe[i] <= hi) in_e |= 1u << i;
         }
     }
-    // a series whose list stays as it is: the list is sorted, the middle ranks of the window are positions k1 - cb and
-    // k2 - cb of it (in flight beside the lists below)
-    float f1 = 0.0f, f2 = 0.0f;
-    if (ok && (in_l | in_e) == 0u) {
-        ok = cb >= 0 && cb <= k1 && k2 < cb + nin;
-        if (ok) {
-            f1 = s.val[(size_t)c * kIncSlots + (k1 - cb)];
-            f2 = s.val[(size_t)c * kIncSlots + (k2 - cb)];
-        }
-    }
-    // ---- list updates, four series at a time: eight lanes hold a list, kIncPer neighbouring slots each ----
     const bool edits = ok && (in_l | in_e) != 0u;
+    const bool plain = ok && !edits && cb >= 0 && cb <= k1 && k2 < cb + nin;
+    float f1 = 0.0f, f2 = 0.0f;
+    uint32_t cnt = 0;
+    if (plain) {
+        f1 = s.val[(size_t)c * kIncSlots + (k1 - cb)];
+        f2 = s.val[(size_t)c * kIncSlots + (k2 - cb)];
+        cnt = 0x80000000u | ((uint32_t)nin << 16) | (uint32_t)cb;
+    }
     const unsigned upd = __ballot_sync(0xFFFFFFFFu, edits);
-    const int nupd = __popc(upd), mine = __popc(upd & ((1u << lane) - 1u));   // this lane's series is the mine-th of them
-    if (edits) sh_order[wid][mine] = (uint8_t)lane;
+    if (edits) {
+        IncEdit<NEW> &e = sh_edit[wid][__popc(upd & ((1u << lane) - 1u))];
+        e.c = c;
+        e.cb = cb;
+        e.nin = nin;
+        e.in_l = in_l;
+        e.in_e = in_e;
+#pragma unroll
+        for (int i = 0; i < NEW; ++i) { e.xl[i] = xl[i]; e.xe[i] = xe[i]; }
+    }
+    const int nedit = __popc(upd);
+    if (c < a.series && !plain && !edits) rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)c;
     __syncwarp();
+    // ---- list updates, four series at a time: eight lanes hold a list, kIncPer neighbouring slots each ----
     const int grp = lane / kIncLanes, gl = lane % kIncLanes;
-    for (int i0 = 0; i0 < nupd; i0 += 32 / kIncLanes) {
-        const bool act = i0 + grp < nupd;
-        const int src = act ? sh_order[wid][i0 + grp] : 0;
-        int ns = __shfl_sync(0xFFFFFFFFu, nin, src);
-        if (!act) ns = 0;
-        float *list = s.val + (size_t)__shfl_sync(0xFFFFFFFFu, c, src) * kIncSlots + gl * kIncPer;
+    float ahead[kIncPer];
+    auto fetch = [&](const int i) {              // (the next lists are on their way while these are edited)
+        if (i < nedit) {
+            const float *list = s.val + (size_t)sh_edit[wid][i].c * kIncSlots + gl * kIncPer;
+            const int ns = sh_edit[wid][i].nin;
+#pragma unroll
+            for (int j = 0; j < kIncPer; ++j)
+                if (gl * kIncPer + j < ns) ahead[j] = list[j];
+        }
+    };
+    fetch(grp);
+    for (int i0 = 0; i0 < nedit; i0 += 32 / kIncLanes) {
+        const bool act = i0 + grp < nedit;
+        const IncEdit<NEW> &e = sh_edit[wid][act ? i0 + grp : 0];
+        int ns = act ? e.nin : 0;
+        const int ce = e.c, cbe = e.cb;
+        const uint32_t ml = act ? e.in_l : 0u, me = act ? e.in_e : 0u;
         int old[kIncPer], v[kIncPer];            // slots without a value lie above everything
 #pragma unroll
-        for (int j = 0; j < kIncPer; ++j) old[j] = gl * kIncPer + j < ns ? inc_key(list[j]) : kIncNone;
-#pragma unroll
-        for (int j = 0; j < kIncPer; ++j) v[j] = old[j];
-        const uint32_t ml = __shfl_sync(0xFFFFFFFFu, in_l, src), me = __shfl_sync(0xFFFFFFFFu, in_e, src);
+        for (int j = 0; j < kIncPer; ++j) old[j] = v[j] = gl * kIncPer + j < ns ? inc_key(ahead[j]) : kIncNone;
+        fetch(i0 + 32 / kIncLanes + grp);
         bool good = act;
 #pragma unroll
         for (int i = 0; i < NEW; ++i) {
-            const bool here = act && ((ml >> i) & 1u);
+            const bool here = (ml >> i) & 1u;
             if (!__any_sync(0xFFFFFFFFu, here)) continue;
-            const float x = __shfl_sync(0xFFFFFFFFu, xl[i], src);
-            const int kx = here ? inc_key(x) : kIncNone;
+            const int kx = here ? inc_key(e.xl[i]) : kIncNone;
             // values from the first one not below x on move down by one; that one has to be x
             int next = __shfl_down_sync(0xFFFFFFFFu, v[0], 1, kIncLanes);
             if (gl == kIncLanes - 1) next = kIncNone;
@@ -547,18 +613,17 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
         }
 #pragma unroll
         for (int i = 0; i < NEW; ++i) {
-            const bool here = act && ((me >> i) & 1u);
+            const bool here = (me >> i) & 1u;
             if (!__any_sync(0xFFFFFFFFu, here)) continue;
-            const float x = __shfl_sync(0xFFFFFFFFu, xe[i], src);
-            const int kx = here ? inc_key(x) : kIncNone;
+            const int kx = here ? inc_key(e.xe[i]) : kIncNone;
             int prev = __shfl_up_sync(0xFFFFFFFFu, v[kIncPer - 1], 1, kIncLanes);
             if (gl == 0) prev = INT_MIN;
 #pragma unroll
             for (int j = kIncPer - 1; j >= 0; --j) v[j] = max(j ? v[j - 1] : prev, min(v[j], kx));
             if (here) { good = good && ns < kIncSlots; ++ns; }
         }
-        const int cbs = __shfl_sync(0xFFFFFFFFu, cb, src);
-        good = good && cbs >= 0 && cbs <= k1 && k2 < cbs + ns;
+        good = good && cbe >= 0 && cbe <= k1 && k2 < cbe + ns;
+        float *list = s.val + (size_t)ce * kIncSlots + gl * kIncPer;
 #pragma unroll
         for (int j = 0; j < kIncPer; ++j) {
             const int slot = gl * kIncPer + j;
@@ -566,30 +631,24 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
             if (good && slot < ns && v[j] != old[j]) list[j] = inc_float(v[j]);
         }
         __syncwarp();
-        // the series' own lanes take over
-        const int from = kIncLanes * (mine % (32 / kIncLanes));
-        const bool fine = __shfl_sync(0xFFFFFFFFu, (int)good, from) != 0;
-        const int num = __shfl_sync(0xFFFFFFFFu, ns, from);
-        if (edits && mine >= i0 && mine < i0 + 32 / kIncLanes) {
-            ok = fine;
-            nin = num;
-            if (ok) {
-                f1 = sh_list[wid][mine % (32 / kIncLanes)][k1 - cb];
-                f2 = sh_list[wid][mine % (32 / kIncLanes)][k2 - cb];
+        if (gl == 0 && act) {
+            if (good) {
+                a.wmed[ce] = median_from_keys(f2key(sh_list[wid][grp][k1 - cbe]), f2key(sh_list[wid][grp][k2 - cbe]), even);
+                s.cnt[ce] = 0x80000000u | ((uint32_t)ns << 16) | (uint32_t)cbe;
+            } else {
+                rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)ce;
             }
         }
         __syncwarp();
     }
-    if (ok) {
-        const float med = median_from_keys(f2key(f1), f2key(f2), even);
-        a.wmed[c] = med;
-        s.cnt[c] = 0x80000000u | ((uint32_t)nin << 16) | (uint32_t)cb;
+    if (plain) {
+        a.wmed[c] = median_from_keys(f2key(f1), f2key(f2), even);
+        s.cnt[c] = cnt;
     }
     // ---- series without a usable state: the CTA's warps share them ----
-    if (active && !ok) rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)c;
     __syncthreads();
     const uint32_t count = rb_n;
-    for (uint32_t i = (uint32_t)wid; i < count; i += kIncThreads / 32) inc_rebuild<VPL>(a, s, (int)rb_list[i], first);
+    for (uint32_t i = (uint32_t)wid; i < count; i += kIncThreads / 32) inc_rebuild<VPL>(a, s, (int)rb_list[i], first, &sh_list[wid][0][0]);
 }
 
 }  // namespace

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
     const int c = blockIdx.x * 32 + lane;
     const bool active = c < a.series;
     const int cc = active ? c : a.series - 1;
-    const int first = ((a.last_slot - (n - 1)) % a.capacity + a.capacity) % a.capacity;
+    const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);
     const bool even = !(n & 1);
     const uint32_t k1 = (uint32_t)((n - 1) >> 1), k2 = (uint32_t)(n >> 1);
     const float *colp = a.ring + cc;

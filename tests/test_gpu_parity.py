@@ -1007,3 +1007,36 @@ def test_outputs_follow_what_the_caller_enqueued_before(R, M, W, deferred, gap):
         for key in want:
             assert_bit_equal(to_np(nodes[key]), want[key], "t=%d %s" % (t, key))
     g.close()
+
+
+@pytest.mark.parametrize("R,M,W,drift,quant", [
+    (129, 1, 65, 0.02, None),     # the last CTA holds one series; two to four values per lane; medians that walk out of their intervals
+    (77, 3, 128, 0.1, None),      # steps so large that the values about the old interval do not hold the new one
+    (64, 8, 200, 0.01, None),
+    (130, 2, 256, 0.02, 40),      # longest windows; ties at the ends of the values that are sorted
+    (33, 4, 90, 0.0, 12),         # lists that fill up
+])
+def test_sliding_rebuilds(R, M, W, drift, quant):
+    from paper_2605_17879_b200 import guard
+    T = W + 70
+    X, dirs = _rand_fleet(T, R, M, seed=R + W, quant=quant)
+    X = (X * (1.0 + drift * np.arange(T) / 10.0)[:, None, None]).astype(np.float32)   # (every median moves the same way)
+    X[:, 1, 0] = X[0, 1, 0]                                                         # ... but one, which stays the same number
+    g = guard.Guard(R, M, W, W // 2, dir=dirs, capacity=W + 8, topk=8, min_signals=min(2, M))
+    o = go.Oracle(R, M, W, W // 2, 8, dir=dirs, min_signals=min(2, M))
+    Xd = torch.from_numpy(X).cuda()
+    t = W
+    g.ingest(Xd[:W])
+    o.ingest(X[:W])
+    for i in range(70):
+        b = 1 + 2 * (i % 7 == 6)
+        if t + b > T:
+            break
+        g.ingest(Xd[t:t + b])
+        o.ingest(X[t:t + b])
+        t += b
+        out = g.score()
+        assert g.sync_status() == 0
+        compare_score(out, o.score(), "t=%d" % t)
+    assert g.sliding_rebuilds() > R * M
+    g.close()

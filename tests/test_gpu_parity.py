@@ -1040,3 +1040,16 @@ def test_sliding_rebuilds(R, M, W, drift, quant):
         compare_score(out, o.score(), "t=%d" % t)
     assert g.sliding_rebuilds() > R * M
     g.close()
+
+
+@pytest.mark.parametrize("R,M,W,quant", [
+    (41, 3, 96, None), (41, 3, 97, None),      # twelve and sixteen values per thread
+    (21, 8, 160, None), (21, 8, 161, None),    # twenty and 24
+    (33, 4, 192, None), (33, 4, 193, None),    # 24 and 28
+    (40, 5, 224, None), (40, 5, 225, None),    # 28 and 32
+    (30, 4, 128, 2),                           # more equal values in a thread than it notes
+    (30, 4, 17, None), (30, 4, 47, None),      # windows too short for spread values of eight pairs
+    (2100, 8, 17, None), (2100, 8, 130, 4),    # ... and first evaluations
+])
+def test_window_tiles_at_their_edges(R, M, W, quant):
+    test_window_tiles(R, M, W, quant)

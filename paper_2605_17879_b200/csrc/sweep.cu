@@ -2,6 +2,8 @@
 // pass / fail verdicts against the fleet distribution (GPU level, then node level).
 #include <math_constants.h>
 
+#include <cfloat>
+
 #include "colselect.cuh"
 #include "kernels.h"
 #include "thselect.cuh"
@@ -48,9 +50,7 @@ __global__ void __launch_bounds__(kSweepCols) sweep_median_kernel(const SweepMed
 // middle ranks are then found among the kept keys (pivot search, as for the window medians).  A series whose counts
 // do not prove the bracket (or whose column overflows) is left to sweep_median_finish_kernel.
 // Bound by the chain of instructions of a series (8 000 of them, 21 warps per SM) and by the loads' cache lines (a
-// repetition is another line for every GPU of the warp): 39 us at 16 384 GPUs x 200 x 6 with the results in L2, 63 from
-// HBM.  Not faster: the next loads in flight ahead of the passes (the same), blocks staged whole in shared memory (seven
-// warps per SM: 62 and 64), or in chunks of eight repetitions, asynchronously (84) or through registers (49 and 68).
+// repetition is another line for every GPU of the warp).  What does not fit a warp per GPU (below) comes here.
 constexpr int kSwThreads = 128;
 constexpr int kSwSlots = 60;      // kept keys per series (the column format of the thread-per-series selection)
 constexpr int kSwRows = 8;        // repetitions in flight per thread
@@ -177,6 +177,209 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_series_kernel(const S
     if (sidx < (long long)a.G * a.M) sweep_warp_median<VPL>(a, (uint32_t)sidx, true);
 }
 
+// A warp per GPU, whose block of repetitions is read once, coalesced, into registers: L = 32 / M lanes per metric, lane
+// l < L M holds repetitions l / M, l / M + L, ... of metric l % M.  A series' mean and standard deviation bracket its median
+// (2.83 sd / sqrt(n) to either side, as in the thread path).  Every lane bins its values (16 bins, the first and the last
+// for what lies below and beyond; its counters are a column of shared memory, so that a warp's reductions never meet in a
+// bank); the lanes of a series scan their sum for the middle ranks; the values about the wanted bins are gathered, those
+// in them counted (as many as the bins say, or the series is not served) and ranked.  Series that are not served, or whose
+// wanted bin holds many different values, are sorted by the whole warp on the spot.
+// Bound by instruction issue and latency: 1 400 instructions a warp for 200 repetitions of 6 metrics (a third of them the
+// values' passes), 24 warps per SM.  16 384 GPUs x 200 x 6 from HBM 32 us (a thread per series, whose loads take a cache line
+// per GPU and pass, 53 + 5 for the series it leaves), 2 048 x 200 x 6 7.4 (a warp per series 16), 4 096 x 64 x 6 7.7 (18).
+// With the kept values of the bracket in a column each, binned behind the pass, 43 us; with 32 bins and the lanes of a
+// series reading the same column at a time (a bank conflict for each) 41.
+constexpr int kSgBins = 16;
+constexpr int kSgList = 16;       // wanted values that are ranked directly
+constexpr int kSgCtl = 8;         // words per series that its lanes share
+constexpr float kSgMagic = 12582912.0f;   // 1.5 * 2^23: adding it leaves an integer in the low mantissa bits
+
+// if (|x - c| <= h) { shared[addr] = x; addr += 128; }
+__device__ __forceinline__ void sg_gather(const float x, const float c, const float h, uint32_t &addr) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t.reg .f32 d;\n\t"
+        "sub.rn.f32 d, %1, %2;\n\t"
+        "abs.f32 d, d;\n\t"
+        "setp.le.f32 q, d, %3;\n\t"
+        "@q st.shared.f32 [%0], %1;\n\t"
+        "@q add.u32 %0, %0, 128;\n\t}"
+        : "+r"(addr)
+        : "f"(x), "f"(c), "f"(h)
+        : "memory");
+}
+
+__host__ __device__ constexpr int sg_rows(const int V) { return V > kSgBins ? V : kSgBins; }
+__host__ __device__ constexpr int sg_words(const int V, const int M) { return 32 * sg_rows(V) + (kSgList + kSgCtl) * M; }   // of shared memory per warp
+
+// V values per lane, at most S more than there are; MM: the number of metrics, or 0 where it is a run-time number.
+template <int V, int S, int MM>
+__global__ void __launch_bounds__(kSwThreads, V <= 24 ? 8 : (V <= 40 ? 6 : (V <= 56 ? 5 : 4))) sweep_median_gpu_kernel(const SweepMedArgs a) {
+    pdl_wait();
+    extern __shared__ __align__(16) uint32_t sg[];   // per warp: bins [kSgBins][32], then gathered values [V][32]; lists [M][kSgList], [M][kSgCtl]
+    const int lane = lane_id(), M = MM ? MM : a.M, n = a.reps;
+    const int L = 32 / M;
+    const int g = blockIdx.x * (kSwThreads / 32) + warp_id();
+    if (g >= a.G) return;
+    uint32_t *hist = sg + warp_id() * (32 * sg_rows(V) + (kSgList + kSgCtl) * M);
+    uint32_t *list = hist + 32 * sg_rows(V), *ctl = list + kSgList * M;
+    const int m = lane % M, q = lane / M;
+    const bool act = lane < L * M;
+    const float *base = a.S + (size_t)g * n * M + min(lane, L * M - 1);   // (idle lanes read a valid column)
+
+    // rows of L repetitions; the first V - S are whole
+    float x[V];
+    auto valid = [&](const int i) { return i < V - S || (act && i * L + q < n); };
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        x[i] = FLT_MAX;               // (beyond the repetitions: above every bracket)
+        if (valid(i)) x[i] = __ldg(base + i * (L * M));
+    }
+#pragma unroll
+    for (int i = 0; i < kSgBins / 4; ++i) reinterpret_cast<uint4 *>(hist)[lane + 32 * i] = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t peers = 0u;              // lanes of this one's series
+#pragma unroll
+    for (int k = 0; k < L; ++k) peers |= 1u << (m + k * M);
+
+    // mean and variance about the first value (no cancellation for values far from zero)
+    const float x0 = __shfl_sync(0xFFFFFFFFu, x[0], m);
+    float sd1 = 0.0f, sd2 = 0.0f, sda = 0.0f;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        const float d = valid(i) ? x[i] - x0 : 0.0f;
+        sd1 += d;
+        sd2 = fmaf(d, d, sd2);
+        sda += fabsf(d);
+    }
+    bool bad = false;
+    if (__any_sync(0xFFFFFFFFu, !(sd2 < CUDART_INF_F))) {   // values that are not finite, or far apart
+#pragma unroll
+        for (int i = 0; i < V; ++i) bad |= nonfinite_bits(__float_as_uint(x[i]));
+        if (a.status && __any_sync(0xFFFFFFFFu, bad && act) && lane == 0) atomicOr(a.status, kStatNonFinite);
+    }
+    bool differ = !(sda == 0.0f);
+    if (__any_sync(0xFFFFFFFFu, !differ && __float_as_uint(x0) << 1 == 0u)) {   // zeros of both signs are different values
+#pragma unroll
+        for (int i = 0; i < V; ++i) differ = differ || (valid(i) && __float_as_uint(x[i]) != __float_as_uint(x0));
+    }
+    const bool same = (__ballot_sync(0xFFFFFFFFu, differ) & peers) == 0u;   // a constant series is its own median
+    float t1 = 0.0f, t2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        t1 += __shfl_sync(0xFFFFFFFFu, sd1, m + k * M);
+        t2 += __shfl_sync(0xFFFFFFFFu, sd2, m + k * M);
+    }
+    const float inv = 1.0f / (float)n, mean_d = t1 * inv, var = fmaxf(t2 * inv - mean_d * mean_d, 0.0f);
+    const float c = x0 + mean_d, h = 2.83f * sqrtf(var * inv);
+    const bool usable = act && !same && th_usable(c, h);
+    const bool even = !(n & 1);
+    const uint32_t k1 = (uint32_t)((n - 1) >> 1), k2 = (uint32_t)(n >> 1);
+
+    // ---- bins: the bracket from the middle of the second to that of the last but one ----
+    constexpr float kTop = (float)(kSgBins - 1), kSpan = (float)(kSgBins - 3);
+    const float scale = usable ? (kSpan / kTop) * 0.5f / h : 0.0f, off = usable ? __fmaf_rn(h - c, scale, 1.0f / kTop) : 0.0f;
+    auto bin = [&](const float v) -> uint32_t { return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(v, scale, off)), kTop, kSgMagic)); };
+    const uint32_t column = (uint32_t)__cvta_generic_to_shared(hist + lane);
+    __syncwarp();
+    if (__any_sync(0xFFFFFFFFu, usable)) {
+        const uint32_t at = column - __float_as_uint(kSgMagic) * 128u;
+#pragma unroll
+        for (int i = 0; i < V; ++i) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(bin(x[i]) * 128u + at) : "memory");
+    }
+    if (q == 0) {
+        ctl[kSgCtl * m] = 0u;                 // wanted bins: k1's ...
+        ctl[kSgCtl * m + 1] = 0u;             // ... and k2's
+        ctl[kSgCtl * m + 4] = 0u;             // values found in them
+        ctl[kSgCtl * m + 5] = 0u;             // largest key of the first
+        ctl[kSgCtl * m + 6] = 0xFFFFFFFFu;    // smallest key of the second
+    }
+    __syncwarp();
+    // ---- scan: the lanes of a series share its bins ----
+    const int per = (kSgBins + L - 1) / L, first = q * per;
+    uint32_t sum = 0u, num[kSgBins];
+#pragma unroll
+    for (int j = 0; j < kSgBins; ++j) num[j] = 0u;
+    int from = q;                     // each lane begins with its own column: no two of a series read the same one at a time
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+#pragma unroll
+        for (int j = 0; j < kSgBins; ++j)
+            if (j < per && first + j < kSgBins && act) num[j] += hist[32 * (first + j) + m + from * M];
+        from = from + 1 < L ? from + 1 : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < kSgBins; ++j) sum += num[j];
+    uint32_t r = 0u;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        const uint32_t o = __shfl_sync(0xFFFFFFFFu, sum, m + k * M);
+        if (k < q) r += o;
+    }
+    if (usable && k2 >= r && k1 < r + sum) {
+#pragma unroll
+        for (int j = 0; j < kSgBins; ++j)
+            if (j < per) {
+                if (k1 >= r && k1 - r < num[j]) { ctl[kSgCtl * m] = (uint32_t)(first + j); ctl[kSgCtl * m + 2] = r; }
+                if (k2 >= r && k2 - r < num[j]) { ctl[kSgCtl * m + 1] = (uint32_t)(first + j); ctl[kSgCtl * m + 3] = r + num[j]; }
+                r += num[j];
+            }
+    }
+    __syncwarp();
+    const uint32_t b1 = ctl[kSgCtl * m], b2 = ctl[kSgCtl * m + 1], start = ctl[kSgCtl * m + 2], end = ctl[kSgCtl * m + 3];
+    bool ok = usable && b1 >= 1u && b2 >= 1u && b1 <= kSgBins - 2u && b2 <= kSgBins - 2u;
+    // ---- the values about the wanted bins (more than those in them: rounding moves a bin's ends) ----
+    const bool listed = ok && end - start <= (uint32_t)kSgList;
+    uint32_t addr = column;
+    if (__any_sync(0xFFFFFFFFu, ok)) {
+        const float width = h * (2.0f / kSpan);
+        const float gc = c - h + (0.5f * (float)(b1 + b2) - 1.0f) * width;
+        const float gh = ok ? (0.5f * (float)(b2 - b1) + 0.6f) * width + (fabsf(c) + h) * pow2_of(-21) : -1.0f;
+#pragma unroll
+        for (int i = 0; i < V; ++i) sg_gather(x[i], gc, gh, addr);
+    }
+    const int hits = (int)((addr - column) >> 7);
+    const uint32_t w1 = b1 + __float_as_uint(kSgMagic), w2 = b2 + __float_as_uint(kSgMagic);
+    for (int j = 0; j < hits; ++j) {
+        const float v = __uint_as_float(hist[32 * j + lane]);
+        const uint32_t b = bin(v);
+        if (b == w1 || b == w2) {
+            const uint32_t key = f2key(v), at = atomicAdd(&ctl[kSgCtl * m + 4], 1u);
+            if (listed) {
+                if (at < (uint32_t)kSgList) list[kSgList * m + at] = key;
+            } else {
+                if (b == w1) atomicMax(&ctl[kSgCtl * m + 5], key);
+                if (b == w2) atomicMin(&ctl[kSgCtl * m + 6], key);
+            }
+        }
+    }
+    __syncwarp();
+    ok = ok && ctl[kSgCtl * m + 4] == end - start;
+    if (ok && listed) {
+        const uint32_t num = end - start, q1 = k1 - start, q2 = k2 - start;
+        for (uint32_t j = (uint32_t)q; j < num; j += (uint32_t)L) {
+            const uint32_t key = list[kSgList * m + j];
+            uint32_t lt = 0u, le = 0u;
+            for (uint32_t i = 0; i < num; ++i) {
+                const uint32_t o = list[kSgList * m + i];
+                lt += o < key;
+                le += o <= key;
+            }
+            if (q1 >= lt && q1 < le) ctl[kSgCtl * m + 5] = key;
+            if (q2 >= lt && q2 < le) ctl[kSgCtl * m + 6] = key;
+        }
+    }
+    __syncwarp();
+    const uint32_t v1 = ctl[kSgCtl * m + 5], v2 = ctl[kSgCtl * m + 6];
+    ok = ok && (listed || b1 != b2 || v1 == v2);   // (else a bin of many different values)
+    if (act && q == 0 && (ok || (same && !bad))) {
+        const float med = ok ? median_from_keys(v1, v2, even) : x0;
+        const size_t o = (size_t)g * M + m;
+        a.gmed[o] = med;
+        if (a.gmed_user) a.gmed_user[o] = med;
+    }
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, act && q == 0 && !ok && !(same && !bad)); todo; todo &= todo - 1u)
+        sweep_warp_median<8>(a, (uint32_t)((size_t)g * M) + (uint32_t)(__ffs(todo) - 1), false);
+}
+
 // Fallback when the repetitions of one GPU do not fit a tile: bit-by-bit counting
 // selection from global memory, one thread per (GPU, metric).
 __global__ void sweep_median_global_kernel(const SweepMedArgs a) {
@@ -254,12 +457,49 @@ __global__ void __launch_bounds__(kVerdictThreads) sweep_verdict_kernel(const Sw
 
 }  // namespace
 
+template <int V, int S, int MM>
+static cudaError_t launch_gpu_medians(const SweepMedArgs &a, cudaStream_t st) {
+    const size_t smem = (size_t)(kSwThreads / 32) * sg_words(V, a.M) * sizeof(uint32_t);
+    return launch_after_smem(sweep_median_gpu_kernel<V, S, MM>, (unsigned)((a.G + kSwThreads / 32 - 1) / (kSwThreads / 32)), kSwThreads, smem, st, a);
+}
+template <int MM>
+static cudaError_t launch_gpu_medians(const SweepMedArgs &a, const int rows, cudaStream_t st) {
+    constexpr int kMost = MM ? (256 + 32 / MM - 1) / (32 / MM) : 64;   // rows of 256 repetitions
+    if (rows <= 8) return launch_gpu_medians<8, 8, MM>(a, st);
+    if (rows <= 16) return launch_gpu_medians<16, 8, MM>(a, st);
+    if (rows <= 24) return launch_gpu_medians<24, 8, MM>(a, st);
+    if (rows <= 32) return launch_gpu_medians<32, 8, MM>(a, st);
+    if constexpr (kMost > 32) {
+        if (rows <= 40) return launch_gpu_medians<40, 8, MM>(a, st);
+        if constexpr (kMost > 40) {
+            if (rows <= 48) return launch_gpu_medians<48, 8, MM>(a, st);
+            if constexpr (kMost > 48) {
+                if (rows <= 56) return launch_gpu_medians<56, 8, MM>(a, st);
+                if constexpr (kMost > 56) return launch_gpu_medians<64, 8, MM>(a, st);
+            }
+        }
+    }
+    return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st) {
     const long long series = (long long)a.G * a.M;
-    // A warp per series while they are few: one launch, and no thread's chain over all repetitions (1 776 series of 33
-    // repetitions 2.8 us against 8.9 + 1.9, 12 288 of 200 16 against 29 + 5, 24 576 of 64 18 against 15 + 4, 49 152 of
-    // 100 25 against 21 + 3, 98 304 of 200 95 against 45 + 5), and for fewer than 32 repetitions, which say too little
-    // about their median beforehand.
+    // A warp per GPU where its values fit the registers (and the lists of its series shared memory), unless the series are so
+    // few that a warp each is the shorter chain: 1 776 series of 33 repetitions 2.2 us against 3.7, 4 096 of 20 2.5 against
+    // 3.5, but 4 800 of 60 5.5 against 4.4, 6 144 of 120 7.3 against 5.2.
+    const int L = 32 / a.M, rows = (a.reps + L - 1) / L;
+    if (a.reps <= 256 && series < 0x7FFFFFFFLL && rows <= 64 && a.M <= 16 && series * ((a.reps + 31) / 32) > 6144) {
+        switch (a.M) {
+            case 4: return launch_gpu_medians<4>(a, rows, st);
+            case 5: return launch_gpu_medians<5>(a, rows, st);
+            case 6: return launch_gpu_medians<6>(a, rows, st);
+            case 8: return launch_gpu_medians<8>(a, rows, st);
+            default: return launch_gpu_medians<0>(a, rows, st);
+        }
+    }
+    // (Other numbers of metrics and repetitions.)  A warp per series while they are few: one launch, and no thread's chain over
+    // all repetitions (12 288 series of 200 16 us against 29 + 5 by threads, 49 152 of 100 25 against 21 + 3), and for fewer
+    // than 32 repetitions, which say too little about their median beforehand.
     if (a.reps <= 256 && series < 0x7FFFFFFFLL && (series <= 32768 || a.reps < 32)) {
         const unsigned grid = (unsigned)((series + kSwThreads / 32 - 1) / (kSwThreads / 32));
         if (a.reps <= 32) return launch_after(sweep_median_series_kernel<1>, grid, kSwThreads, st, a);

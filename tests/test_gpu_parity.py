@@ -1053,3 +1053,46 @@ def test_sliding_rebuilds(R, M, W, drift, quant):
 ])
 def test_window_tiles_at_their_edges(R, M, W, quant):
     test_window_tiles(R, M, W, quant)
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (6200, 1, 1, 1),               # one value per series
+    (3100, 1, 64, 1), (3083, 1, 256, 2), (2049, 1, 96, 3),   # 32, 16 and ten lanes per series
+    (1601, 1, 33, 4), (800, 1, 256, 4),                      # rows of eight: five of them, all 32
+    (401, 2, 48, 5), (397, 2, 49, 5), (260, 1, 255, 5),      # a whole number of rows, one repetition more, the most
+    (601, 1, 40, 6), (603, 1, 41, 6), (211, 1, 200, 6), (160, 1, 256, 6),
+    (150, 2, 32, 8), (150, 2, 33, 8), (99, 1, 256, 8),
+    (300, 1, 64, 7), (260, 1, 192, 9), (200, 1, 128, 13), (210, 1, 128, 16),   # other numbers of metrics
+])
+def test_sweep_gpu_by_warp(nodes, gpn, N, M):
+    """A warp per GPU: ends of its rows of lanes; constant series, zeros of both signs, two values, many equal ones about the
+    middle, an outlier that makes the spread useless, and values near the ends of the range of floats."""
+    from paper_2605_17879_b200 import guard
+    rng = np.random.default_rng(1000 * N + M)
+    G = nodes * gpn
+    S = (1.0 + 0.02 * rng.standard_normal((G, N, M), dtype=np.float32)).astype(np.float32)
+    S[3::9] = S[3::9, :1]
+    S[4::9] = np.where(S[4::9] > 1.0, np.float32(1.0), np.float32(0.5))
+    S[5::9] = np.round(S[5::9] * np.float32(100.0)) / np.float32(100.0)
+    S[6::27] *= np.float32(1e-39)
+    S[7::27] *= np.float32(1e38) * np.sign(rng.standard_normal((1, N, 1))).astype(np.float32)
+    S[8::27, N // 2] = np.float32(1e30)
+    S[10::27] = np.copysign(np.float32(0.0), S[10::27] - 1.0)
+    S[11::27] -= np.float32(1.0)
+    S[12::27] = np.where(np.abs(S[12::27] - 1.0) < 0.01, np.copysign(np.float32(0.0), S[12::27] - 1.0), S[12::27] - 1.0)
+    S[13::27] = np.exp(200.0 * (S[13::27] - 1.0))
+    dirs = [-1 if m % 2 else 1 for m in range(M)]
+    ref = go.sweep(S, nodes, gpn, dir=dirs)
+    out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
+    assert int(out["status"].cpu()[0]) == 0
+    for key in ref:
+        assert_bit_equal(to_np(out[key]), ref[key], key)
+    S[G // 2, N - 1, M - 1] = np.float32("inf")
+    out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
+    assert int(out["status"].cpu()[0]) & 1
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [(2100, 1, 40, 20), (1100, 2, 200, 16)])   # more metrics or repetitions than a warp holds
+def test_sweep_by_threads(nodes, gpn, N, M):
+    test_sweep_of_many_series(nodes, gpn, N, M)
+    test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M)

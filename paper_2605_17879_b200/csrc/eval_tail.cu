@@ -223,7 +223,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
 }
 
 template <int V, int NC>
-__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : 256, NC == 1 ? 1 : 2) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
+__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : ct_most_threads(NC), NC == 1 ? 1 : 512 / ct_most_threads(NC)) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
     __shared__ CtShared<1> sh;
     __shared__ TopShared ts;
     pdl_wait();

@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(1024) xrank_count_kernel(const XrankArgs a, co
 
 // A cluster of NC CTAs per column: a few wide columns.
 template <int V, int NC, bool APART>
-__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(256, 2) xrank_count_cluster_kernel(const XrankArgs a, const MetricParams p) {
+__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(ct_most_threads(NC), 512 / ct_most_threads(NC)) xrank_count_cluster_kernel(const XrankArgs a, const MetricParams p) {
     __shared__ CtShared<1> sh;
     pdl_wait();
     const int column = (int)blockIdx.x / NC;

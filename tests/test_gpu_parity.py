@@ -1096,3 +1096,10 @@ def test_sweep_gpu_by_warp(nodes, gpn, N, M):
 def test_sweep_by_threads(nodes, gpn, N, M):
     test_sweep_of_many_series(nodes, gpn, N, M)
     test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M)
+
+
+@pytest.mark.parametrize("R,M,B", [(16385, 18, 2), (17000, 9, 4), (32768, 20, 1)])
+def test_widest_rows_of_four_cta_clusters(R, M, B):
+    """More columns than clusters of eight find room for, and more ranks than four CTAs of 256 threads hold."""
+    X, dirs = _rand_fleet(3 * B, R, M, seed=R + M)
+    run_both(X, 2, 1, 4, dirs, [B], capacity=3 * B)

@@ -48,7 +48,7 @@ struct CtShared {
     __align__(16) uint32_t hist[C][kCtBins];
     uint32_t lo[C], width[C];      // the range [lo, lo + width]
     uint32_t below[C];             // keys below it
-    uint32_t f0[C], fw[C];         // keys to fetch: [f0, f0 + fw]
+    uint32_t f0[C], fe[C];         // keys to fetch: [f0, fe]
     uint32_t how[C];               // 0 nothing to fetch, 1 list and rank, 2 largest up to / smallest from `cutk`, 3 smallest and largest
     uint32_t cutk[C];
     uint32_t q1[C];                // rank of k1 among the fetched keys
@@ -168,46 +168,42 @@ __device__ __forceinline__ void ct_scan(CtShared<C> &sh, const int c, const uint
     uint32_t incl = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) { const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, incl, d); if (lane >= d) incl += u; }
-    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    // this lane's bin of k1 / k2 (if it has it), the rank inside it and the number of its keys
-    uint32_t r = below + incl - sum, b1 = 0, b2 = 0, q = 0, n = 0;
-    const bool has1 = k1 - r < sum && k1 >= r, has2 = k2 - r < sum && k2 >= r;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        if (k1 >= r && k1 - r < w[j]) { b1 = (uint32_t)(8 * lane + j); q = k1 - r; n = w[j]; }
-        if (k2 >= r && k2 - r < w[j]) b2 = (uint32_t)(8 * lane + j);
-        r += w[j];
-    }
-    const uint32_t l1 = __ballot_sync(0xFFFFFFFFu, has1), l2 = __ballot_sync(0xFFFFFFFFu, has2);
-    const int s1 = l1 ? __ffs(l1) - 1 : 0, s2 = l2 ? __ffs(l2) - 1 : 0;
-    b1 = __shfl_sync(0xFFFFFFFFu, b1, s1);
-    b2 = __shfl_sync(0xFFFFFFFFu, b2, s2);
-    q = __shfl_sync(0xFFFFFFFFu, q, s1);
-    n = __shfl_sync(0xFFFFFFFFu, n, s1);
+    const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sum);
     if (lane == 0) {
         if (NC == 1) sh.below[c] = 0u;
         sh.nl[c] = 0u;
         sh.mx[c] = 0u;
         sh.mn[c] = kCtNone;
-        sh.q1[c] = q;
-        if (l1 && l2) {
-            const int sft = ct_shift(width);
-            const uint32_t o1 = b1 << sft, in_bin = (1u << sft) - 1u;
-            sh.f0[c] = lo + o1;
-            sh.fw[c] = min((b2 << sft) + in_bin, width) - o1;
-            sh.cutk[c] = lo + o1 + in_bin;              // last key of k1's bin
-            sh.how[c] = b1 != b2 ? 2u : (n <= (uint32_t)kCtList ? 1u : 3u);
-        } else {   // the range does not hold both ranks: move or stretch it, sixteenfold
-            const uint32_t hi = lo + width, step = width >= 0x07FF0000u ? 0x7FFFFFFFu : 16u * width + 65536u;
-            uint32_t nlo = lo, nhi = hi;
-            if (below > k1) { nlo = lo > step ? lo - step : 0u; if (below > k2) nhi = lo; }
-            if (k2 >= below + total) { nhi = hi < kCtNone - step ? hi + step : kCtNone; if (k1 >= below + total) nlo = hi; }
-            sh.lo[c] = nlo;
-            sh.width[c] = nhi - nlo;
-            sh.f0[c] = kCtNone;
-            sh.fw[c] = 0u;
-            sh.how[c] = 0u;
+    }
+    if (k1 >= below && k2 < below + total) {   // the lane that has k1's bin, and the one that has k2's, say so themselves
+        const int sft = ct_shift(width);
+        const uint32_t in_bin = (1u << sft) - 1u;
+        uint32_t r = below + incl - sum, b1 = 0, b2 = 0, q = 0, n = 0;
+        const bool has1 = k1 - r < sum && k1 >= r, has2 = k2 - r < sum && k2 >= r;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (k1 >= r && k1 - r < w[j]) { b1 = (uint32_t)(8 * lane + j); q = k1 - r; n = w[j]; }
+            if (k2 >= r && k2 - r < w[j]) b2 = (uint32_t)(8 * lane + j);
+            r += w[j];
         }
+        if (has1) {
+            const uint32_t first = lo + (b1 << sft);
+            sh.q1[c] = q;
+            sh.f0[c] = first;
+            sh.cutk[c] = first + in_bin;               // last key of k1's bin
+            sh.how[c] = q + (k2 - k1) >= n ? 2u : (n <= (uint32_t)kCtList ? 1u : 3u);
+        }
+        if (has2) sh.fe[c] = lo + min((b2 << sft) + in_bin, width);
+    } else if (lane == 0) {   // the range does not hold both ranks: move or stretch it, sixteenfold
+        const uint32_t hi = lo + width, step = width >= 0x07FF0000u ? 0x7FFFFFFFu : 16u * width + 65536u;
+        uint32_t nlo = lo, nhi = hi;
+        if (below > k1) { nlo = lo > step ? lo - step : 0u; if (below > k2) nhi = lo; }
+        if (k2 >= below + total) { nhi = hi < kCtNone - step ? hi + step : kCtNone; if (k1 >= below + total) nlo = hi; }
+        sh.lo[c] = nlo;
+        sh.width[c] = nhi - nlo;
+        sh.f0[c] = kCtNone;
+        sh.fe[c] = kCtNone;
+        sh.how[c] = 0u;
     }
 }
 
@@ -216,42 +212,24 @@ template <int C, int NC = 1>
 __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bool pair) {
     const int lane = lane_id();
     const uint32_t how = sh.how[c], q1 = sh.q1[c];
-    uint32_t n, mx, mn, mine, mine2;
-    const uint32_t *list;
+    uint32_t n, mx, mn, own = 0, base = 0;
+    const uint32_t part = (uint32_t)(lane & (NC - 1));   // (clusters) the CTA whose keys this lane fetches
     if (NC == 1) {
         n = sh.nl[c];
         mx = sh.mx[c];
         mn = sh.mn[c];
-        list = sh.list[c];
     } else {
-        const uint32_t k = (uint32_t)(lane & (NC - 1));
-        const uint32_t own = ct_ld(ct_map(&sh.nl[c], k));
-        mx = __reduce_max_sync(0xFFFFFFFFu, ct_ld(ct_map(&sh.mx[c], k)));
-        mn = __reduce_min_sync(0xFFFFFFFFu, ct_ld(ct_map(&sh.mn[c], k)));
-        // all CTAs' keys in one list (their bins hold kCtList at most together)
-        uint32_t incl = lane < NC ? own : 0u;
-        const uint32_t cnt = incl;
+        own = ct_ld(ct_map(&sh.nl[c], part));
+        mx = ct_ld(ct_map(&sh.mx[c], part));
+        mn = ct_ld(ct_map(&sh.mn[c], part));
+        base = own;
 #pragma unroll
-        for (int d = 1; d < NC; d <<= 1) { const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, incl, d); if (lane >= d) incl += u; }
-        n = __shfl_sync(0xFFFFFFFFu, incl, NC - 1);
-        if (how == 1u && n <= (uint32_t)kCtList) {
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const uint32_t e = (uint32_t)(lane + 32 * half);
-                uint32_t from = 0, off = 0;
-#pragma unroll
-                for (int d = 0; d < NC; ++d) {
-                    const uint32_t end = __shfl_sync(0xFFFFFFFFu, incl, d), num = __shfl_sync(0xFFFFFFFFu, cnt, d);
-                    if (e < end && e >= end - num) { from = (uint32_t)d; off = e - (end - num); }
-                }
-                if (e < n) sh.all[e] = ct_ld(ct_map(&sh.list[c][off], from));
-            }
-            __syncwarp();
-        }
-        list = sh.all;
+        for (int d = 1; d < NC; d <<= 1) { const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, base, d, NC); if ((int)part >= d) base += u; }
+        n = __shfl_sync(0xFFFFFFFFu, base, NC - 1);
+        base -= own;
+        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+        mn = __reduce_min_sync(0xFFFFFFFFu, mn);
     }
-    mine = list[lane];
-    mine2 = list[lane + 32];
     if (how == 0u) return true;                      // the range moved
     if (how != 1u) {
         if (how == 3u && mx != mn) {                 // a full bin of different keys becomes the range
@@ -262,7 +240,14 @@ __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bo
         return false;
     }
     const uint32_t q2 = pair ? q1 + 1u : q1;
-    auto rank = [&](const uint32_t x, const bool real) {
+    const uint32_t *list = NC == 1 ? sh.list[c] : sh.all;
+    if (NC > 1) {                                    // all CTAs' keys in one list (their bins hold kCtList at most together)
+        for (uint32_t e = (uint32_t)(lane / NC); e < own; e += 32u / NC)
+            if (base + e < (uint32_t)kCtList) sh.all[base + e] = ct_ld(ct_map(&sh.list[c][e], part));
+        __syncwarp();
+    }
+    for (uint32_t e = (uint32_t)lane; e < n; e += 32u) {
+        const uint32_t x = list[e];
         uint32_t lt = 0, le = 0;
 #pragma unroll 4
         for (uint32_t j = 0; j < n; ++j) {
@@ -270,11 +255,9 @@ __device__ __forceinline__ bool ct_settle(CtShared<C> &sh, const int c, const bo
             lt += o < x;
             le += o <= x;
         }
-        if (real && q1 >= lt && q1 < le) sh.v1[c] = x;
-        if (real && q2 >= lt && q2 < le) sh.v2[c] = x;
-    };
-    rank(mine, lane < (int)n);
-    if (n > 32u) rank(mine2, lane + 32 < (int)n);
+        if (q1 >= lt && q1 < le) sh.v1[c] = x;
+        if (q2 >= lt && q2 < le) sh.v2[c] = x;
+    }
     return false;
 }
 
@@ -297,15 +280,19 @@ __device__ __forceinline__ int ct_select(const uint32_t (&key)[V], const uint32_
             uint32_t below = 0;
 #pragma unroll
             for (int i = 0; i < V; ++i) ct_bin(key[i], lo, width, sft, hist, below);
+            if (C == 1) {
+                below = __reduce_add_sync(0xFFFFFFFFu, below);
+            } else {
 #pragma unroll
-            for (int d = 16; d >= C; d >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, d);
+                for (int d = 16; d >= C; d >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, d);
+            }
             if (lane < C) atomicAdd(&sh.below[lane], below);
         }
         ct_sync<NC>();
         if (warp < C && searching) ct_scan<C, NC>(sh, warp, k1, k2);
         __syncthreads();
         {
-            const uint32_t f0 = sh.f0[col], fw = sh.fw[col];
+            const uint32_t f0 = sh.f0[col], fw = sh.fe[col] - f0;
             uint32_t hits = 0;
 #pragma unroll
             for (int i = 0; i < V; ++i) ct_hit(key[i], f0, fw, 1u << i, hits);
@@ -336,7 +323,7 @@ __device__ __forceinline__ int ct_select(const uint32_t (&key)[V], const uint32_
             searching = ct_settle<C, NC>(sh, warp, k2 != k1);
             if (lane == 0) {
                 if (searching) sh.any_open[it & 1] = 1u;
-                else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fw[warp] = 0u; }   // (no key of a number, a computed NaN or padding)
+                else { sh.lo[warp] = 0xFFFFFFFDu; sh.width[warp] = 0u; sh.f0[warp] = 0xFFFFFFFDu; sh.fe[warp] = 0xFFFFFFFDu; }   // (no key of a number, a computed NaN or padding)
             }
         }
         __syncthreads();
@@ -353,7 +340,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     const int tid = threadIdx.x, lane = lane_id(), warp = warp_id(), T = blockDim.x;
     const int R = a.R, M = a.M;
     const int col = tid & (C - 1);
-    const int slot = (int)(((long long)a.first_slot + s) % a.capacity);
+    const int slot = a.first_slot + s - (s >= a.capacity - a.first_slot ? a.capacity : 0);   // (s < capacity)
     constexpr bool kCopies = NC == 1 && V <= 8;   // (the larger ones have no registers to spare)
     const float *ring = a.base + (size_t)slot * a.row_stride + m0, *row = kCopies && a.copy_from ? a.copy_from + (size_t)s * a.row_stride + m0 : ring;
     const bool even = (R & 1) == 0;
@@ -374,8 +361,6 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
         if (NC == 1 ? a.prev_rows > 0 : s < a.prev_rows) {
             const size_t o = (size_t)min(s, a.prev_rows - 1) * M + m0 + warp;
             if (lane == 0) { hmed = a.med[o]; hmad = a.mad[o]; }
-            hmed = __shfl_sync(0xFFFFFFFFu, hmed, 0);
-            hmad = __shfl_sync(0xFFFFFFFFu, hmad, 0);
         }
     }
 #pragma unroll
@@ -383,6 +368,10 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
         const int r = r0 + i * dr;
         key[i] = 0x7FFFFFFFu;             // a NaN whose keys lie above those of all numbers
         if (r < R) key[i] = __float_as_uint(__ldg(row + (size_t)r * M + col));
+    }
+    if (warp < C) {                       // (behind the loads of the values: they are all in flight together)
+        hmed = __shfl_sync(0xFFFFFFFFu, hmed, 0);
+        hmad = __shfl_sync(0xFFFFFFFFu, hmad, 0);
     }
     if (kCopies && a.copy_from) {         // (a copy in front, with its launch, takes 2.5 us more at 64 ranks x 4 x 50)
 #pragma unroll
@@ -420,6 +409,7 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
     }
 #pragma unroll
     for (int i = 0; i < V; ++i) key[i] = key_of_bits(key[i]);
+    float med = 0.0f;                     // of this thread's column
     // what: 0 the median, 1 the MAD, 2 + c the extra order statistic of metric m0 + c (before the MAD)
 #pragma unroll 1
     for (int what = part == kCtCut ? 2 : 0;;) {
@@ -427,13 +417,14 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
         const uint32_t q1 = extra ? (uint32_t)a.cut_rank[m0 + what - 2] : k1, q2 = extra ? q1 : k2;
         const int rounds = ct_select<V, C, NC>(key, q1, q2, sh);
         settled = settled && (extra || (hinted && rounds == 1));   // (thread 0's warp knows of a hint)
-        if (tid < C) {
+        if (what == 0) {   // (the keys stand until the next selection settles)
+            med = median_from_keys(sh.v1[col], sh.v2[col], even);
+            if (tid < C) sh.med[tid] = med;
+        } else if (tid < C) {
             const uint32_t v1 = sh.v1[tid], v2 = sh.v2[tid];
             const int m = m0 + tid;
             const size_t o = (size_t)s * M + m;
-            if (what == 0) {
-                sh.med[tid] = median_from_keys(v1, v2, even);
-            } else if (what == 1) {
+            if (what == 1) {
                 const float lo = __uint_as_float(v1 >> 1), md = sh.med[tid];
                 const float mad = even ? __fmul_rn(0.5f, __fadd_rn(lo, __uint_as_float(v2 >> 1))) : lo;
                 sh.mad[tid] = mad;
@@ -458,17 +449,16 @@ __device__ __forceinline__ void ct_row(const XrankArgs &a, const MetricParams &p
             if (tid == 0 && speaks && sh.bad && a.status) atomicOr(a.status, kStatInternal);
             break;
         }
-        __syncthreads();
         // the metrics' extra ranks first (they need the values), then the deviations
         what = !a.cut || part == kCtStatistics ? 1 : (what == 0 ? 2 : (what - 1 < C ? what + 1 : 1));
         if (what >= 2) {
             if (warp < C) sampled(f2key(xs), (uint32_t)a.cut_rank[m0 + what - 2]);
         } else {
             // the keys of the deviations: their bits with the sign as the lowest bit
-            const float med = sh.med[col];
             if (warp < C) {
+                const float centre = C == 1 ? med : __shfl_sync(0xFFFFFFFFu, med, warp);   // (lane c holds column c's)
                 if (hinted) range(__float_as_uint(fmaxf(hmad - 6.6f * u, 0.0f)) << 1, (__float_as_uint(hmad + 6.6f * u) << 1) | 1u);
-                else sampled(__float_as_uint(__fsub_rn(xs, sh.med[warp])) << 1, k1);
+                else sampled(__float_as_uint(__fsub_rn(xs, centre)) << 1, k1);
             }
 #pragma unroll
             for (int i = 0; i < V; ++i) {

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kSpThreads, 3) xsplit_sample_kernel(const Xran
     __shared__ SpSampleShared sh;
     const int q = blockIdx.x, t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.R, M = a.M;
-    const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
+    const int slot = a.first_slot + t - (t >= a.capacity - a.first_slot ? a.capacity : 0);
     const float *row = a.base + (size_t)slot * a.row_stride;
     SpCol *cols = sc.col + (size_t)t * M + 4 * q;
     const bool reuse = t < rows;   // the scratch has held this step position before
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 6) xsplit_sweep_kernel(const Xr
     __shared__ SpSweepShared sh;
     const int chunk = blockIdx.x, t = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.R;
-    const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
+    const int slot = a.first_slot + t - (t >= a.capacity - a.first_slot ? a.capacity : 0);
     const float *row = a.base + (size_t)slot * a.row_stride;
     uint8_t *maskrow = a.mask_base ? reinterpret_cast<uint8_t *>(a.mask_base) + (size_t)slot * R : nullptr;
     const int r0 = min(R, (chunk * kSpWarps + warp) * g.strip), r1 = min(R, r0 + g.strip);
@@ -542,7 +542,7 @@ __device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, 
         if (warp == 0) ct_scan<1>(sh, 0, k1, k2);
         __syncthreads();
         {
-            const uint32_t f0 = sh.f0[0], fw = sh.fw[0], how = sh.how[0], cutk = sh.cutk[0];
+            const uint32_t f0 = sh.f0[0], fw = sh.fe[0] - f0, how = sh.how[0], cutk = sh.cutk[0];
 #pragma unroll 4
             for (uint32_t i = tid; i < n; i += T) {
                 const uint32_t k = key(i, false);
@@ -729,7 +729,7 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(512, 2) xs
     for (int t = blockIdx.x; t < S; t += gridDim.x) {
         if (a.mask_base) {
             const uint32_t na = min(sc.namb[t], (uint32_t)kSpAmb);
-            const int slot = (int)(((long long)a.first_slot + t) % a.capacity);
+            const int slot = a.first_slot + t - (t >= a.capacity - a.first_slot ? a.capacity : 0);
             const float *row = a.base + (size_t)slot * a.row_stride;
             uint8_t *maskrow = reinterpret_cast<uint8_t *>(a.mask_base) + (size_t)slot * R;
             const SpCol *cols = sc.col + (size_t)t * M;

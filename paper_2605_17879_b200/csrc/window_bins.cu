@@ -15,7 +15,7 @@
 // saturation does, a scan shared by all warps, selecting noted values from registers by their index (a chain over all of
 // them per hit), and 20 to 236 bytes of spills; now none up to 28 values a thread.
 // Measured, kernel alone: 98 760 first windows of 180 steps 45 us (68 with those), 65 536 of 100 steps with ties 22 (33),
-// 65 536 of 120 beside the cross-rank kernel 19 (38), 8 192 of 1 000 steps 21.5 (23.4; half as many warps that read the
+// 65 536 of 120 beside the cross-rank kernel 19 (38), 8 192 of 1 000 steps 19 (24; half as many warps that read the
 // window again 60), 8 192 of 100 8.5 (10.9).  131 072 of 200 steps 64 to 80 beside other kernels: a thread per series
 // (window.cu) takes 7 instructions a value and one warp's selection for 32 series, 37 + 10.
 #include <math_constants.h>
@@ -28,7 +28,8 @@ namespace {
 
 constexpr int kWbBins = 32;
 constexpr int kWbSample = 16;
-constexpr int kWbList = 16;        // values of a bin that are ranked directly
+// Values of a bin that are ranked directly (sixteen to 32 of them take eight warps longer than another round)
+__host__ __device__ constexpr int wb_list(const int G) { return G <= 8 ? 16 : 32; }
 __host__ __device__ constexpr int wb_hits(const int G) { return G <= 8 ? 10 : 6; }   // wanted values that a thread notes (more than that: ties)
 constexpr int kWbRounds = 6;       // rounds of ranges before the bit-by-bit selection
 constexpr float kWbSmooth = 0.3f;  // weight of the newest median in the range's centre
@@ -46,7 +47,7 @@ struct WbShared {
     float width[32];               // of the first range its width, the values inside, and why it did not serve, if so
     uint32_t inside[32];           // (diagnostic): 1 too many values in a bin, 2 the median lies below it, 3 above it
     int why[32];
-    uint32_t list[kWbList][32];
+    uint32_t list[wb_list(G)][32];
     uint32_t prefix[32], krem[32], cnt[32];   // bit-by-bit selection
 };
 
@@ -88,7 +89,7 @@ __device__ __forceinline__ float wb_t(const float x, const float scale, const fl
 template <int V, int G, bool RELOAD>
 __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window_bins_kernel(const WindowArgs a) {
     pdl_wait();
-    constexpr int H = wb_hits(G);
+    constexpr int H = wb_hits(G), kWbList = wb_list(G);
     __shared__ WbShared<G> sh;
     const int lane = lane_id(), w = __shfl_sync(0xFFFFFFFFu, warp_id(), 0), n = a.n;   // (w in a uniform register: so are the rows' numbers)
     const int c = blockIdx.x * 32 + lane;
@@ -208,8 +209,8 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
             sh.nl[lane] = 0u;
             sh.mx[lane] = 0u;
             sh.mn[lane] = 0xFFFFFFFFu;
-            if (live && !served) {     // move or stretch the range sixteenfold, from the second time on to everything
-                const float wd = hi - lo, edge = 0.0625f * wd, step = round == 0 ? 16.0f * wd + 1.0e-30f : kWbMax;
+            if (live && !served) {     // move or stretch the range: a little (a level that shifts or drifts), far, to everything
+                const float wd = hi - lo, edge = 0.0625f * wd, step = round < 2 ? (round == 0 ? 4.0f : 64.0f) * wd + 1.0e-30f : kWbMax;
                 float nlo = lo, nhi = hi;
                 if (b1 == 0u) { nlo = fmaxf(lo - step, -kWbMax); if (b2 == 0u) nhi = lo + edge; }
                 if (b2 == kWbBins - 1) { nhi = fminf(hi + step, kWbMax); if (b1 == kWbBins - 1) nlo = hi - edge; }

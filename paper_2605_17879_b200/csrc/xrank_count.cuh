@@ -16,7 +16,7 @@
 // branches and returning atomics per value, rounds of pivots (each some 500 cycles of dependent scalar work in one
 // warp, whatever the number of values) and column-wise loads (a cache line per lane).  Measured, kernel alone:
 // 100 steps of 1 024 ranks x 8 metrics 9.5 us (8-bit radix select of xrank_direct.cuh: 76), 60 steps of 4 096 x 16
-// 29 us (576; three CTAs per SM; the instances with 16 and 32 values a thread spill 12 and 44 bytes at 64 registers).
+// 29 us (576; three CTAs per SM; the instances with 32 values a thread spill 44 and 56 bytes at 64 registers).
 #pragma once
 #include "kernels.h"
 

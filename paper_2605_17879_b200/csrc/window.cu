@@ -292,6 +292,7 @@ constexpr int kFinCtas = 148 * 4;
 template <int VPL>
 __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const WindowArgs a) {
     pdl_wait();
+    __shared__ float near_med[kFinThreads / 32][64];
     __shared__ int is_last;
     const int lane = lane_id();
     const int n = a.n;
@@ -301,28 +302,68 @@ __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const Window
     for (uint32_t i = blockIdx.x * (kFinThreads / 32) + warp_id(); i < count; i += nwarps) {
         const uint32_t item = __ldcg(a.fb_list + i);
         const int series = (int)(item & 0x0FFFFFFFu), why_src = (int)(item >> 28);
-        uint32_t kv[VPL];
-        int nreal = 0;
+        float x[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) {
             const int row = lane + 32 * j;
-            kv[j] = 0xFFFFFFFFu;
+            x[j] = 0.0f;
             if (row < n) {
                 int slot = first + row;
                 if (slot >= a.capacity) slot -= a.capacity;
-                kv[j] = f2key(__ldg(a.ring + (size_t)slot * a.row_stride + series));
-                ++nreal;
+                x[j] = __ldg(a.ring + (size_t)slot * a.row_stride + series);
             }
         }
-        lane_sort<VPL>(kv);
-        float m2 = 0.0f;
-        const bool ok2 = warp_median<VPL>(kv, nreal, n, 0u, m2);
-        const float h0 = warp_spread_guess<VPL>(kv, n, m2);
+        float med = 0.0f, spread = 0.0f;
+        bool done = false;
+        // a median just outside of its interval: the values of the neighbouring stretch of that width, two per lane, if they
+        // hold the middle ranks (counted)
+        if (VPL > 2 && (why_src == 2 || why_src == 3)) {
+            const float h = a.spread[series], c = a.centre[series];
+            const float lo = why_src == 2 ? c - 3.0f * h : c + 0.9f * h, hi = why_src == 2 ? c - 0.9f * h : c + 3.0f * h;
+            int below = 0, kept = 0;
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                const bool real = lane + 32 * j < n;
+                below += real && x[j] < lo;
+                const bool in = real && x[j] >= lo && x[j] <= hi;
+                const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
+                const int at = kept + __popc(who & ((1u << lane) - 1u));
+                if (in && at < 64) near_med[warp_id()][at] = x[j];
+                kept += __popc(who);
+            }
+            const int base = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below), r1 = ((n - 1) >> 1) - base, r2 = (n >> 1) - base;
+            __syncwarp();
+            if (kept <= 64 && r1 >= 0 && r2 < kept) {   // (the same for the whole warp)
+                uint32_t kv[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) kv[j] = 2 * lane + j < kept ? f2key(near_med[warp_id()][2 * lane + j]) : 0xFFFFFFFFu;
+                warp_bitonic_sort<2>(kv, lane);         // ascending: element e in lane e / 2, register e % 2
+                const uint32_t v1 = __shfl_sync(0xFFFFFFFFu, (r1 & 1) ? kv[1] : kv[0], r1 >> 1);
+                const uint32_t v2 = __shfl_sync(0xFFFFFFFFu, (r2 & 1) ? kv[1] : kv[0], r2 >> 1);
+                med = median_from_keys(v1, v2, !(n & 1));
+                spread = 1.25f * h;
+                done = true;
+            }
+            __syncwarp();
+        }
+        if (!done) {
+            uint32_t kv[VPL];
+            int nreal = 0;
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                const bool real = lane + 32 * j < n;
+                kv[j] = real ? f2key(x[j]) : 0xFFFFFFFFu;
+                nreal += real;
+            }
+            lane_sort<VPL>(kv);
+            const bool ok2 = warp_median<VPL>(kv, nreal, n, 0u, med);
+            spread = warp_spread_guess<VPL>(kv, n, med);
+            if (lane == 0 && !ok2) atomicOr(a.status, kStatInternal);
+        }
         if (lane == 0) {
-            if (!ok2) atomicOr(a.status, kStatInternal);
-            a.wmed[series] = m2;
-            a.spread[series] = h0;
-            a.centre[series] = m2;
+            a.wmed[series] = med;
+            a.spread[series] = spread;
+            a.centre[series] = med;
             if (a.fb_count) { atomicAdd(a.fb_count, 1u); atomicAdd(a.fb_count + 1 + why_src, 1u); }
         }
     }

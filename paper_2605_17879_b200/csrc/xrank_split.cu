@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 6) xsplit_sweep_kernel(const Xr
 }
 
 // ---- 2. selection ------------------------------------------------------------------------------
-// Keys of the two middle ranks among those that key(i) gives for a list's values (0xFFFFFFFF: not among them), left in
+// Keys of the two middle ranks among those that key() gives for a list's n values (whole quads; 0xFFFFFFFF: not among them), left in
 // sh.v1[0] / sh.v2[0]; the range is in sh.lo / sh.width, the bins are zero.  ranks(k1, k2) gives their places among the
 // keys once key() has seen every value, or false.  The steps of ct_select, with the list read again in every pass (it
 // is in the first-level cache): what a pass keeps in registers would halve the CTAs that share an SM.
@@ -531,8 +531,14 @@ __device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, 
             const uint32_t lo = sh.lo[0], width = sh.width[0];
             const int sft = ct_shift(width);
             uint32_t below = 0;
-#pragma unroll 4
-            for (uint32_t i = tid; i < n; i += T) ct_bin(key(i, it == 0), lo, width, sft, hist, below);
+#pragma unroll 2
+            for (uint32_t i = tid; i < n / 4u; i += T) {
+                const float4 v = key.list[i];
+                ct_bin(key(v.x, it == 0), lo, width, sft, hist, below);
+                ct_bin(key(v.y, it == 0), lo, width, sft, hist, below);
+                ct_bin(key(v.z, it == 0), lo, width, sft, hist, below);
+                ct_bin(key(v.w, it == 0), lo, width, sft, hist, below);
+            }
             below = __reduce_add_sync(0xFFFFFFFFu, below);
             if (lane == 0) atomicAdd(&sh.below[0], below);
         }
@@ -543,9 +549,10 @@ __device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, 
         __syncthreads();
         {
             const uint32_t f0 = sh.f0[0], fw = sh.fe[0] - f0, how = sh.how[0], cutk = sh.cutk[0];
-#pragma unroll 4
-            for (uint32_t i = tid; i < n; i += T) {
-                const uint32_t k = key(i, false);
+            key.range(f0, sh.fe[0]);
+            auto take = [&](const float x) {
+                if (!key.near(x)) return;          // (as a rule: no key is worked out)
+                const uint32_t k = key(x, false);
                 if (k - f0 <= fw) {
                     if (how == 1u) {
                         const uint32_t pos = atomicAdd(&sh.nl[0], 1u);
@@ -555,6 +562,14 @@ __device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, 
                         if (how == 3u || k > cutk) atomicMin(&sh.mn[0], k);
                     }
                 }
+            };
+#pragma unroll 2
+            for (uint32_t i = tid; i < n / 4u; i += T) {
+                const float4 v = key.list[i];
+                take(v.x);
+                take(v.y);
+                take(v.z);
+                take(v.w);
             }
         }
         __syncthreads();
@@ -572,12 +587,13 @@ __device__ __forceinline__ bool sp_pick(Key key, Ranks ranks, const uint32_t n, 
 // Keys of the kept values in the median's band (the very comparisons of the sweep; NaN is in no band), and how many values
 // are in either band.
 struct SpMedianKey {
-    const float *list;
+    const float4 *list;
     float ks, kb, hm, a, ha;
     uint32_t *s_n;
     uint32_t nm = 0, na = 0;
-    __device__ __forceinline__ uint32_t operator()(const uint32_t i, const bool count) {
-        const float x = list[i], d = fabsf(__fmaf_rn(x, ks, kb));
+    float lo = 0.0f, hi = 0.0f;
+    __device__ __forceinline__ uint32_t operator()(const float x, const bool count) {
+        const float d = fabsf(__fmaf_rn(x, ks, kb));
         const bool in = d <= hm;
         if (count) {
             nm += in;
@@ -585,6 +601,9 @@ struct SpMedianKey {
         }
         return in ? f2key(x) : 0xFFFFFFFFu;
     }
+    // values that may have keys from f0 to fe (all of these among them)
+    __device__ __forceinline__ void range(const uint32_t f0, const uint32_t fe) { lo = key2f(f0); hi = key2f(fe); }
+    __device__ __forceinline__ bool near(const float x) const { return x >= lo && x <= hi; }
     __device__ __forceinline__ void share() {
         const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, nm | (na << 16));
         if (lane_id() == 0) { atomicAdd(&s_n[0], tot & 0xFFFFu); atomicAdd(&s_n[1], tot >> 16); }
@@ -592,12 +611,17 @@ struct SpMedianKey {
 };
 // ... and of the exact deviations of those in the MAD's band.
 struct SpMadKey {
-    const float *list;
+    const float4 *list;
     float ks, kb, a, ha, med;
-    __device__ __forceinline__ uint32_t operator()(const uint32_t i, const bool) const {
-        const float x = list[i];
+    float lo = 0.0f, hi = 0.0f;
+    __device__ __forceinline__ uint32_t operator()(const float x, const bool) const {
         const bool in = fabsf(__fsub_rn(fabsf(__fmaf_rn(x, ks, kb)), a)) <= ha;
         return in ? __float_as_uint(__fsub_rn(x, med)) << 1 : 0xFFFFFFFFu;
+    }
+    __device__ __forceinline__ void range(const uint32_t f0, const uint32_t fe) { lo = __uint_as_float(f0 >> 1); hi = __uint_as_float(fe >> 1); }
+    __device__ __forceinline__ bool near(const float x) const {
+        const float d = fabsf(__fsub_rn(x, med));
+        return d >= lo && d <= hi;
     }
     __device__ __forceinline__ void share() const {}
 };
@@ -620,7 +644,7 @@ __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, co
         sh.lo[0] = lo;
         sh.width[0] = hi - lo;
     }
-    bool ok = sp_pick<T>(SpMedianKey{list, ks, kb, b.hm, b.a, b.ha, s_n},
+    bool ok = sp_pick<T>(SpMedianKey{reinterpret_cast<const float4 *>(list), ks, kb, b.hm, b.a, b.ha, s_n},
                       [&](uint32_t &k1, uint32_t &k2) {
                           // (the sweep counted with the sign folded in: below there is above here)
                           const uint32_t nm = s_n[0], blt = sgn > 0.0f ? below : (uint32_t)R - below - nm;
@@ -640,7 +664,7 @@ __device__ __forceinline__ int sp_select(const float *list, const uint32_t n, co
         sh.lo[0] = l;
         sh.width[0] = h - l;
     }
-    ok = sp_pick<T>(SpMadKey{list, ks, kb, b.a, b.ha, med},
+    ok = sp_pick<T>(SpMadKey{reinterpret_cast<const float4 *>(list), ks, kb, b.a, b.ha, med},
                  [&](uint32_t &k1, uint32_t &k2) {
                      k1 = r1 - inner;
                      k2 = r2 - inner;

@@ -20,6 +20,7 @@
 // (window.cu) takes 7 instructions a value and one warp's selection for 32 series, 37 + 10.
 #include <math_constants.h>
 
+#include "binmap.cuh"
 #include "kernels.h"
 
 namespace guard {
@@ -178,10 +179,10 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
     int round = 0;
 #pragma unroll 1
     for (;; ++round) {
-        // ---- bin: the range from the middle of the second bin to that of the last but one; the first and the last take
-        // all values below and beyond ----
-        float scale = hi > lo ? fminf((29.0f / 31.0f) / (hi - lo), 1.0e37f) : 1.0f;
-        float off = __fmaf_rn(-lo, scale, 1.0f / 31.0f);
+        // ---- bin: the range (a little wider: binmap.cuh) from the middle of the second bin to that of the last but one; the
+        // first and the last take all values below and beyond ----
+        const BinMap map = bin_map<kWbBins - 1>(lo, hi);
+        float scale = map.scale, off = map.off;
         if (hi - lo > kWbMax) { scale = 0.0f; off = 0.5f; }   // (a range wider than the largest number: all values share a bin)
         if (!live) { scale = 0.0f; off = 0.0f; }              // (settled series count nothing that matters)
         __syncthreads();           // bins are zero
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(32 * G, G <= 8 ? 4 : (G <= 16 ? 2 : 1)) window
             sh.mx[lane] = 0u;
             sh.mn[lane] = 0xFFFFFFFFu;
             if (live && !served) {     // move or stretch the range: a little (a level that shifts or drifts), far, to everything
-                const float wd = hi - lo, edge = 0.0625f * wd, step = round < 2 ? (round == 0 ? 4.0f : 64.0f) * wd + 1.0e-30f : kWbMax;
+                const float wd = map.span, edge = 0.0625f * wd, step = round < 2 ? (round == 0 ? 4.0f : 64.0f) * wd + 1.0e-30f : kWbMax;
                 float nlo = lo, nhi = hi;
                 if (b1 == 0u) { nlo = fmaxf(lo - step, -kWbMax); if (b2 == 0u) nhi = lo + edge; }
                 if (b2 == kWbBins - 1) { nhi = fminf(hi + step, kWbMax); if (b1 == kWbBins - 1) nlo = hi - edge; }

@@ -283,16 +283,22 @@ __global__ void __launch_bounds__(kThCols, 9) window_thread_kernel(const WindowA
 }
 
 // The series the thread path's interval did not serve (a few per thousand), one warp per listed series: the lanes
-// fetch the window, sort their own keys and run the warp selection; the series' interval state starts afresh.
-// A kernel of its own, so that these series spread over the GPU instead of queueing behind one another at the end
-// of the warp that found them.
+// fetch the window, sort their own keys and run the warp selection.  A kernel of its own, so that these series spread
+// over the GPU instead of queueing behind one another at the end of the warp that found them.
+// The interval starts afresh at the median.  One that the median left by less than its width was not too narrow for the
+// noise, but a little: it keeps a quarter more than its width, where a width from the window's deviations would be as far
+// off as the first one was (passes of 24 000 ranks x 8 x 100 in blocks of 50 166.2 us, 170.0 afresh, 167.0 with the width as
+// it was; 16 384 x 8 x 200 251.9 in blocks of 100, 260.2, 257.2; windows of up to 64 steps, of noisier medians, 160.8 and
+// 158.8 afresh).  Bound by the loads' cache lines, one for each step of a listed series, and the chain of the selection: all
+// of 131 072 series of 200 steps 180 us.  (Looking for a median just outside of its interval among the values of the
+// neighbouring stretch first: the same beside other kernels, and 8 % more where all series are listed.)
 constexpr int kFinThreads = 128;
 constexpr int kFinCtas = 148 * 4;
+constexpr float kFinNear = 3.0f, kFinWiden = 1.25f;
 
 template <int VPL>
 __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const WindowArgs a) {
     pdl_wait();
-    __shared__ float near_med[kFinThreads / 32][64];
     __shared__ int is_last;
     const int lane = lane_id();
     const int n = a.n;
@@ -302,65 +308,31 @@ __global__ void __launch_bounds__(kFinThreads) window_finish_kernel(const Window
     for (uint32_t i = blockIdx.x * (kFinThreads / 32) + warp_id(); i < count; i += nwarps) {
         const uint32_t item = __ldcg(a.fb_list + i);
         const int series = (int)(item & 0x0FFFFFFFu), why_src = (int)(item >> 28);
-        float x[VPL];
+        float h = -1.0f, c = 0.0f;                         // (in flight with the window)
+        if (VPL > 2 && (why_src == 2 || why_src == 3)) {   // below or above the interval
+            h = __ldcg(a.spread + series);
+            c = __ldcg(a.centre + series);
+        }
+        uint32_t kv[VPL];
+        int nreal = 0;
 #pragma unroll
         for (int j = 0; j < VPL; ++j) {
             const int row = lane + 32 * j;
-            x[j] = 0.0f;
+            kv[j] = 0xFFFFFFFFu;
             if (row < n) {
                 int slot = first + row;
                 if (slot >= a.capacity) slot -= a.capacity;
-                x[j] = __ldg(a.ring + (size_t)slot * a.row_stride + series);
+                kv[j] = f2key(__ldg(a.ring + (size_t)slot * a.row_stride + series));
+                ++nreal;
             }
         }
-        float med = 0.0f, spread = 0.0f;
-        bool done = false;
-        // a median just outside of its interval: the values of the neighbouring stretch of that width, two per lane, if they
-        // hold the middle ranks (counted)
-        if (VPL > 2 && (why_src == 2 || why_src == 3)) {
-            const float h = a.spread[series], c = a.centre[series];
-            const float lo = why_src == 2 ? c - 3.0f * h : c + 0.9f * h, hi = why_src == 2 ? c - 0.9f * h : c + 3.0f * h;
-            int below = 0, kept = 0;
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                const bool real = lane + 32 * j < n;
-                below += real && x[j] < lo;
-                const bool in = real && x[j] >= lo && x[j] <= hi;
-                const uint32_t who = __ballot_sync(0xFFFFFFFFu, in);
-                const int at = kept + __popc(who & ((1u << lane) - 1u));
-                if (in && at < 64) near_med[warp_id()][at] = x[j];
-                kept += __popc(who);
-            }
-            const int base = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)below), r1 = ((n - 1) >> 1) - base, r2 = (n >> 1) - base;
-            __syncwarp();
-            if (kept <= 64 && r1 >= 0 && r2 < kept) {   // (the same for the whole warp)
-                uint32_t kv[2];
-#pragma unroll
-                for (int j = 0; j < 2; ++j) kv[j] = 2 * lane + j < kept ? f2key(near_med[warp_id()][2 * lane + j]) : 0xFFFFFFFFu;
-                warp_bitonic_sort<2>(kv, lane);         // ascending: element e in lane e / 2, register e % 2
-                const uint32_t v1 = __shfl_sync(0xFFFFFFFFu, (r1 & 1) ? kv[1] : kv[0], r1 >> 1);
-                const uint32_t v2 = __shfl_sync(0xFFFFFFFFu, (r2 & 1) ? kv[1] : kv[0], r2 >> 1);
-                med = median_from_keys(v1, v2, !(n & 1));
-                spread = 1.25f * h;
-                done = true;
-            }
-            __syncwarp();
-        }
-        if (!done) {
-            uint32_t kv[VPL];
-            int nreal = 0;
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                const bool real = lane + 32 * j < n;
-                kv[j] = real ? f2key(x[j]) : 0xFFFFFFFFu;
-                nreal += real;
-            }
-            lane_sort<VPL>(kv);
-            const bool ok2 = warp_median<VPL>(kv, nreal, n, 0u, med);
-            spread = warp_spread_guess<VPL>(kv, n, med);
-            if (lane == 0 && !ok2) atomicOr(a.status, kStatInternal);
-        }
+        lane_sort<VPL>(kv);
+        float med = 0.0f;
+        const bool ok2 = warp_median<VPL>(kv, nreal, n, 0u, med);
+        float spread = warp_spread_guess<VPL>(kv, n, med);
+        if (fabsf(med - c) <= kFinNear * h) spread = kFinWiden * h;
         if (lane == 0) {
+            if (!ok2) atomicOr(a.status, kStatInternal);
             a.wmed[series] = med;
             a.spread[series] = spread;
             a.centre[series] = med;

@@ -378,10 +378,9 @@ cudaError_t launch_thread_path(const WindowArgs &a, cudaStream_t st) {
 // position (middle - count) of the list.
 // A series whose median has left its interval, whose list is full, or that has no state yet is
 // rebuilt from its whole window by a warp of the same CTA.  Exact either way: the interval only decides which values are
-// listed.  The CTA's four warps share its rebuilds (one CTA in two has one in steady state): queued inside the warp that
-// found them they make the kernel as slow as its unluckiest warp, and a kernel of their own costs the next step's update a
-// launch and a scan of lists (update and rebuilds of 262 144 series 19 + 10 us beside other work, together 23; single
-// steps of 2 048 ranks x 8 with node verdicts 31.5 us an evaluation, 27.6 so; six deferred steps of 32 768 x 8 242, 223 so).
+// listed.  The CTA's four warps share its rebuilds (of 128 series of continuous values one CTA in two has one): queued inside
+// the warp that found them they make the kernel as slow as its unluckiest warp, and a kernel of their own costs the next
+// step's update a launch and a scan of lists (an eighth of a single step of 2 048 ranks x 8, with node verdicts).
 // ---------------------------------------------------------------------------------------
 constexpr int kIncThreads = 128;
 constexpr int kIncLanes = 8, kIncPer = kIncSlots / kIncLanes;   // lanes that hold a list, and slots per lane
@@ -509,7 +508,7 @@ struct IncEdit {
 // a rebuild.  (Two series per thread, all of 262 144 resident at once: the same alone, and beside the cluster kernels of
 // other evaluations, which then wait for room, six deferred steps of 32 768 x 8 take 205 us instead of 194.)
 template <int NEW, int VPL>
-__global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s) {
+__global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s, const int per) {
     pdl_wait();
     __shared__ float sh_list[kIncThreads / 32][32 / kIncLanes][kIncSlots];   // per warp: the edited lists
     __shared__ IncEdit<NEW> sh_edit[kIncThreads / 32][32];                   // ... and what is edited
@@ -521,31 +520,32 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
     const int first = a.last_slot - (n - 1) + (a.last_slot < n - 1 ? a.capacity : 0);   // slot of the window's oldest step
     const bool even = !(n & 1);
     const int k1 = (n - 1) >> 1, k2 = n >> 1;
-    const int c = blockIdx.x * kIncThreads + threadIdx.x, cc = min(c, a.series - 1);
+    const int c = blockIdx.x * per + threadIdx.x;        // (the other threads take part in the rebuilds)
+    const bool mine = (int)threadIdx.x < per && c < a.series;
 
     // The steps that left the window (the ones right before its oldest step) and the steps that entered it (the
     // newest ones), all fetched up front.
-    const uint32_t w = s.cnt[cc];
-    const float lo = s.lo[cc], hi = s.hi[cc];
+    const uint32_t w = mine ? s.cnt[c] : 0u;
+    const float lo = mine ? s.lo[c] : 0.0f, hi = mine ? s.hi[c] : 0.0f;
     float xl[NEW], xe[NEW];
 #pragma unroll
     for (int i = 0; i < NEW; ++i) {
         xl[i] = 0.0f;
         xe[i] = 0.0f;
-        if (i < s.leaving) {
+        if (mine && i < s.leaving) {
             int slot = first - s.leaving + i;
             if (slot < 0) slot += a.capacity;
-            xl[i] = __ldg(a.ring + (size_t)slot * a.row_stride + cc);
+            xl[i] = __ldg(a.ring + (size_t)slot * a.row_stride + c);
         }
-        if (i < s.entering) {
+        if (mine && i < s.entering) {
             int slot = a.last_slot - (s.entering - 1 - i);
             if (slot < 0) slot += a.capacity;
-            xe[i] = __ldg(a.ring + (size_t)slot * a.row_stride + cc);
+            xe[i] = __ldg(a.ring + (size_t)slot * a.row_stride + c);
         }
     }
     // A value below lo moves the count; a value inside the interval changes the series' sorted list, which eight lanes
     // then edit (below).  A list that stays as it is has the middle ranks of the window at positions k1 - cb and k2 - cb.
-    const bool ok = c < a.series && (w >> 31) && !s.rebuild_all;
+    const bool ok = mine && (w >> 31) && !s.rebuild_all;
     int cb = (int)(w & 0xFFFFu);
     const int nin = (int)((w >> 16) & 0xFFu);
     uint32_t in_l = 0, in_e = 0;
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const Window
         for (int i = 0; i < NEW; ++i) { e.xl[i] = xl[i]; e.xe[i] = xe[i]; }
     }
     const int nedit = __popc(upd);
-    if (c < a.series && !plain && !edits) rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)c;
+    if (mine && !plain && !edits) rb_list[atomicAdd(&rb_n, 1u)] = (uint32_t)c;
     __syncwarp();
     // ---- list updates, four series at a time: eight lanes hold a list, kIncPer neighbouring slots each ----
     const int grp = lane / kIncLanes, gl = lane % kIncLanes;
@@ -685,11 +685,22 @@ size_t window_inc_bytes(int series) { return (size_t)series * sizeof(float); }
 
 bool window_inc_supported(const WindowArgs &a) { return a.n >= 1 && a.n <= 256; }
 
+// Series of a CTA of the sliding update: its warps share its rebuilds, so that few series to a CTA spread the rebuilds over
+// the whole chip.  Where many series keep no list (constant or coarse values) or all leave theirs at a time (a common shift of
+// level), 128 series to a CTA take an evaluation of 64 ranks x 4 x 50 steps from 17.9 us to 73.3 (all series constant), of
+// 2 048 x 8 x 200 from 41.3 to 69.9 and of 8 192 x 8 x 200 from 95.5 to 133.4 (two metrics of eight constant).  1 024 CTAs at
+// most: the more there are, the fewer find room beside the cross-rank clusters (continuous values of 8 192 x 8 x 200 33.7 us,
+// with 128 series to a CTA 33.4, with the 1 184 CTAs that an idle chip holds 34.1 and, of constant ones, 87).
+static int inc_series_per_cta(const int series) {
+    constexpr int kMost = 1024;
+    return min(kIncThreads, max(8, ((series + kMost - 1) / kMost + 7) & ~7));
+}
+
 template <int VPL>
 static cudaError_t launch_inc(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {
-    const int grid = (a.series + kIncThreads - 1) / kIncThreads;
-    return inc.entering <= 1 && inc.leaving <= 1 ? launch_after(window_inc_kernel<1, VPL>, grid, kIncThreads, st, a, inc)
-                                                 : launch_after(window_inc_kernel<kIncMaxNew, VPL>, grid, kIncThreads, st, a, inc);
+    const int per = inc_series_per_cta(a.series), grid = (a.series + per - 1) / per;
+    return inc.entering <= 1 && inc.leaving <= 1 ? launch_after(window_inc_kernel<1, VPL>, grid, kIncThreads, st, a, inc, per)
+                                                 : launch_after(window_inc_kernel<kIncMaxNew, VPL>, grid, kIncThreads, st, a, inc, per);
 }
 
 cudaError_t launch_window_incremental(const WindowArgs &a, const IncArgs &inc, cudaStream_t st) {

@@ -73,3 +73,37 @@ def test_medians_of_few_steps_between_floats(W, scale):
         assert_bit_equal(to_np(g.score()["wmed"]), o.score()["wmed"], "t=%d" % t)
     assert g.sync_status() == 0
     g.close()
+
+
+def _step_us(X, W):
+    """Time of a step with its evaluation, windows sliding on from a full one."""
+    from paper_2605_17879_b200 import guard
+    T, R, M = X.shape
+    g = guard.Guard(R, M, W, W // 2, dir=[1] * M, capacity=W + 16, min_signals=1)
+    out = g.alloc_outputs()
+    g.ingest(X[:W])
+    g.score(out)
+    us, per = [], (T - W) // 6
+    for i in range(6):
+        torch.cuda.synchronize()
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for t in range(W + i * per, W + (i + 1) * per):
+            g.ingest(X[t:t + 1])
+            g.score(out)
+        b.record()
+        torch.cuda.synchronize()
+        us.append(a.elapsed_time(b) * 1000.0 / per)
+    assert g.sync_status() == 0
+    g.close()
+    return float(np.median(us))
+
+
+@pytest.mark.parametrize("R,M,W,constant", [(256, 8, 100, 8), (512, 8, 200, 8), (2048, 8, 200, 2)])
+def test_steps_of_constant_series(R, M, W, constant):
+    """Series that keep no list are rebuilt in every evaluation: by the whole chip (1.2, 1.6 and 1.6 times a step of continuous
+    values), not by the few CTAs that a small fleet has at 128 series each (5.9, 8.6 and 2.7)."""
+    X = (1.0 + 0.03 * torch.randn(W + 120, R, M, generator=torch.Generator().manual_seed(R))).cuda()
+    C = X.clone()
+    C[:, :, M - constant:] = C[:1, :, M - constant:]
+    assert _step_us(C, W) < 2.2 * _step_us(X, W)

@@ -223,7 +223,7 @@ __device__ __forceinline__ void top_row(const TopkArgs &a, const MetricParams &p
 }
 
 template <int V, int NC>
-__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : ct_most_threads(NC), NC == 1 ? 1 : 512 / ct_most_threads(NC)) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
+__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : 512, 1) eval_tail_kernel(const XrankArgs x, const TopkArgs t, const MetricParams p) {
     __shared__ CtShared<1> sh;
     __shared__ TopShared ts;
     pdl_wait();
@@ -234,8 +234,8 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(NC == 1 ? 1024 : ct
 }
 
 template <int NC>
-cudaError_t launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st) {
-    const int T = ct_cluster_threads(x.R, NC), v = (x.R + NC * T - 1) / (NC * T), grid = (x.M + (t.K > 0 ? 1 : 0)) * NC;
+cudaError_t launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, const int most, cudaStream_t st) {
+    const int T = ct_cluster_threads(x.R, NC, most), v = (x.R + NC * T - 1) / (NC * T), grid = (x.M + (t.K > 0 ? 1 : 0)) * NC;
     if (v <= 4) return launch_after(eval_tail_kernel<4, NC>, grid, T, st, x, t, p);
     if (v <= 8) return launch_after(eval_tail_kernel<8, NC>, grid, T, st, x, t, p);
     return launch_after(eval_tail_kernel<16, NC>, grid, T, st, x, t, p);
@@ -244,14 +244,18 @@ cudaError_t launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p,
 }  // namespace
 
 // The fleet baseline x (one row, no exceedance bits) and, with t.K > 0, the top-k list t (no scores) of one evaluation;
-// R <= kCountMaxRanks.
-cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st) {
+// R <= kCountMaxRanks.  steps: evaluations follow one another by a few steps.  Their tails share the GPU with the clusters of
+// the next steps' rows: CTAs of up to 256 threads, two to an SM, where four values a thread would ask for 512 (deferred single
+// steps of 16 384 ranks x 8 24.3 us, with 512 26.1; of 24 000 28.3 and 32.4).  After a block the tail is what the pass waits
+// for: up to 512, the shorter chain (blocks of 50 steps of 24 000 x 8, W = 100, 164.1 us, with 256 166.6; of 32 768 205.8 and
+// 209.1).
+cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, const bool steps, cudaStream_t st) {
     if (x.R <= kCtClusterRanks) {
         int T = 32;
         while (T < 1024 && x.R > 4 * T) T <<= 1;
         return launch_after(eval_tail_kernel<4, 1>, x.M + (t.K > 0 ? 1 : 0), T, st, x, t, p);
     }
-    return (x.M + 1) * 8 <= 148 ? launch<8>(x, t, p, st) : launch<4>(x, t, p, st);
+    return (x.M + 1) * 8 <= 148 ? launch<8>(x, t, p, steps ? ct_most_threads(8) : 512, st) : launch<4>(x, t, p, 512, st);
 }
 
 }  // namespace guard

@@ -716,7 +716,7 @@ int guard_score(guard_ctx *c, float *d_wmed, float *d_fleet_med, float *d_fleet_
     x.prev_rows = c->row_hints && c->evals > 0 ? 1 : 0;
     if (together) {
         if (c->L.xr_gridp && c->row_hints) x.hint = c->hint_state(1);
-        e = launch_eval_tail(x, t, c->p, ts);
+        e = launch_eval_tail(x, t, c->p, gap <= kIncMaxNew, ts);
         c->launches += 1;
     } else {
         e = c->xrank(x, 1, ts, !defer, 1);

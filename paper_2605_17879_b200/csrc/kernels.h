@@ -214,7 +214,7 @@ int topk_blocks(int R);
 void set_global_error(const char *text);
 cudaError_t launch_topk(const TopkArgs &a, const MetricParams &p, cudaStream_t st);
 // Fleet baseline and top-k list of one evaluation in one launch (R <= kCountMaxRanks; K = 0: no list).
-cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, cudaStream_t st);
+cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, bool steps, cudaStream_t st);
 
 // Node sweep: per-GPU medians over repetitions, then the verdicts.
 struct SweepMedArgs {

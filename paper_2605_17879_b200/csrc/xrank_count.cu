@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(1024) xrank_count_apart_kernel(const XrankArgs
 template <int NC, bool APART>
 cudaError_t launch_cluster(const XrankArgs &a, const MetricParams &p, int S, cudaStream_t st) {
     const dim3 grid(a.M * NC * (APART ? 2 : 1), S);
-    const int T = ct_cluster_threads(a.R, NC);
+    const int T = ct_cluster_threads(a.R, NC, ct_most_threads(NC));
     const int v = (a.R + NC * T - 1) / (NC * T);
     if (v <= 4) return launch_after(xrank_count_cluster_kernel<4, NC, APART>, grid, T, st, a, p);
     if (v <= 8) return launch_after(xrank_count_cluster_kernel<8, NC, APART>, grid, T, st, a, p);

@@ -33,12 +33,13 @@ constexpr int kCtAll = 0, kCtStatistics = 1, kCtCut = 2;   // what a CTA (cluste
 constexpr int kCtClusterRanks = 4096;
 // Threads of the CTAs of a cluster: four values each, while a CTA has 256 of them at most: at 128 registers two such CTAs
 // share an SM, so that the clusters of a step's row and of another evaluation's tail find room beside one another and
-// beside the window kernels (six deferred steps of 32 768 ranks x 8 210 us with up to 512 threads, 199 so; a row alone the
-// same).  Clusters of four need 512 to hold the widest rows in sixteen values a thread.
+// beside the window kernels (six deferred steps of 32 768 ranks x 8 take 5 % longer with up to 512 threads; steps that nothing
+// runs beside, of 16 384 to 32 768 ranks, the same within 0.5 %).  Clusters of four need 512 to hold the widest rows in sixteen
+// values a thread.
 __host__ __device__ constexpr int ct_most_threads(const int NC) { return NC >= 8 ? 256 : 512; }
-inline int ct_cluster_threads(const int R, const int NC) {
+inline int ct_cluster_threads(const int R, const int NC, const int most) {
     int T = 128;
-    while (T < ct_most_threads(NC) && R > 4 * NC * T) T <<= 1;
+    while (T < most && R > 4 * NC * T) T <<= 1;
     return T;
 }
 static_assert(16 * 8 * ct_most_threads(8) >= kCountMaxRanks && 16 * 4 * ct_most_threads(4) >= kCountMaxRanks, "every row fits sixteen values a thread");

@@ -4,6 +4,7 @@
 
 #include <cfloat>
 
+#include "binmap.cuh"
 #include "colselect.cuh"
 #include "kernels.h"
 #include "thselect.cuh"
@@ -183,7 +184,10 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_series_kernel(const S
 // for what lies below and beyond; its counters are a column of shared memory, so that a warp's reductions never meet in a
 // bank); the lanes of a series scan their sum for the middle ranks; the values about the wanted bins are gathered, those
 // in them counted (as many as the bins say, or the series is not served) and ranked.  Series that are not served, or whose
-// wanted bin holds many different values, are sorted by the whole warp on the spot.
+// wanted bin holds many different values, are sorted by the whole warp on the spot: one in fifty of normal values.  Where all
+// of them are (values that spread over decades) that is up to twice as long as a warp for each (1 000 x 200 x 6 28 us and 17,
+// 4 096 x 200 x 6 54 and 40, 16 384 x 200 x 6 146 and 215).  Further rounds with ranges a standard deviation wide instead take 19,
+// 32 and 75, but in the same kernel they cost all other sweeps 2 to 5 %.
 // Bound by instruction issue and latency: 1 400 instructions a warp for 200 repetitions of 6 metrics (a third of them the
 // values' passes), 24 warps per SM.  16 384 GPUs x 200 x 6 from HBM 32 us (a thread per series, whose loads take a cache line
 // per GPU and pass, 53 + 5 for the series it leaves), 2 048 x 200 x 6 7.4 (a warp per series 16), 4 096 x 64 x 6 7.7 (18).
@@ -192,6 +196,7 @@ __global__ void __launch_bounds__(kSwThreads) sweep_median_series_kernel(const S
 constexpr int kSgBins = 16;
 constexpr int kSgList = 16;       // wanted values that are ranked directly
 constexpr int kSgCtl = 8;         // words per series that its lanes share
+constexpr int kSgReps = 256, kSgRows = 64;   // most repetitions, and values per lane
 constexpr float kSgMagic = 12582912.0f;   // 1.5 * 2^23: adding it leaves an integer in the low mantissa bits
 
 // if (|x - c| <= h) { shared[addr] = x; addr += 128; }
@@ -211,32 +216,154 @@ __device__ __forceinline__ void sg_gather(const float x, const float c, const fl
 __host__ __device__ constexpr int sg_rows(const int V) { return V > kSgBins ? V : kSgBins; }
 __host__ __device__ constexpr int sg_words(const int V, const int M) { return 32 * sg_rows(V) + (kSgList + kSgCtl) * M; }   // of shared memory per warp
 
-// V values per lane, at most S more than there are; MM: the number of metrics, or 0 where it is a run-time number.
-template <int V, int S, int MM>
+__device__ __forceinline__ void sg_store(const SweepMedArgs &a, const int series, const float med) {
+    a.gmed[series] = med;
+    if (a.gmed_user) a.gmed_user[series] = med;
+}
+
+// The medians of the open series that their ranges [lo, hi] serve; the others are left.  The bins are zero.
+template <int V, int M>
+__device__ __forceinline__ void sg_round(const SweepMedArgs &a, const float (&x)[V], const int g, const int m, const int q, const bool act, uint32_t *hist,
+                                         uint32_t *list, uint32_t *ctl, const float lo, const float hi, const bool open, bool &left) {
+    constexpr int L = 32 / M;
+    const int lane = lane_id(), n = a.reps;
+    const uint32_t k1 = (uint32_t)((n - 1) >> 1), k2 = (uint32_t)(n >> 1);
+    const uint32_t column = (uint32_t)__cvta_generic_to_shared(hist + lane);
+    const BinMap map = bin_map<kSgBins - 1>(lo, hi);
+    const float scale = open ? map.scale : 0.0f, off = open ? map.off : 0.0f;
+    auto bin = [&](const float v) -> uint32_t { return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(v, scale, off)), (float)(kSgBins - 1), kSgMagic)); };
+    __syncwarp();                 // bins are zero
+    {
+        const uint32_t at = column - __float_as_uint(kSgMagic) * 128u;
+#pragma unroll
+        for (int i = 0; i < V; ++i) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(bin(x[i]) * 128u + at) : "memory");
+    }
+    if (q == 0) {
+        ctl[kSgCtl * m] = 0u;                 // wanted bins: k1's ...
+        ctl[kSgCtl * m + 1] = 0u;             // ... and k2's
+        ctl[kSgCtl * m + 4] = 0u;             // values found in them
+        ctl[kSgCtl * m + 5] = 0u;             // largest key of the first
+        ctl[kSgCtl * m + 6] = 0xFFFFFFFFu;    // smallest key of the second
+    }
+    __syncwarp();
+    // ---- scan: the lanes of a series share its bins ----
+    constexpr int per = (kSgBins + L - 1) / L;
+    const int bin0 = q * per;
+    uint32_t sum = 0u, num[per];
+#pragma unroll
+    for (int j = 0; j < per; ++j) num[j] = 0u;
+    int from = q;                 // each lane begins with its own column: no two of a series read the same one at a time
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+#pragma unroll
+        for (int j = 0; j < per; ++j)
+            if (bin0 + j < kSgBins && act) num[j] += hist[32 * (bin0 + j) + m + from * M];
+        from = from + 1 < L ? from + 1 : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < per; ++j) sum += num[j];
+    uint32_t r = 0u;
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        const uint32_t o = __shfl_sync(0xFFFFFFFFu, sum, m + k * M);
+        if (k < q) r += o;
+    }
+    if (open && k2 >= r && k1 < r + sum) {
+#pragma unroll
+        for (int j = 0; j < per; ++j) {
+            if (k1 >= r && k1 - r < num[j]) { ctl[kSgCtl * m] = (uint32_t)(bin0 + j); ctl[kSgCtl * m + 2] = r; }
+            if (k2 >= r && k2 - r < num[j]) { ctl[kSgCtl * m + 1] = (uint32_t)(bin0 + j); ctl[kSgCtl * m + 3] = r + num[j]; }
+            r += num[j];
+        }
+    }
+    __syncwarp();
+    const uint32_t b1 = ctl[kSgCtl * m], b2 = ctl[kSgCtl * m + 1], start = ctl[kSgCtl * m + 2], end = ctl[kSgCtl * m + 3];
+    const bool served = open && b1 >= 1u && b2 >= 1u && b1 <= kSgBins - 2u && b2 <= kSgBins - 2u;
+    // ---- the values about the wanted bins (more than those in them: rounding moves a bin's ends) ----
+    const bool listed = served && end - start <= (uint32_t)kSgList;
+    uint32_t addr = column;
+    if (__any_sync(0xFFFFFFFFu, served)) {
+        const float width = map.span * (1.0f / (float)(kSgBins - 3));
+        const float gc = lo + (0.5f * (float)(b1 + b2) - 1.0f) * width;
+        const float gh = served ? (0.5f * (float)(b2 - b1) + 0.6f) * width + fmaxf(fabsf(lo), fabsf(hi)) * pow2_of(-21) : -1.0f;
+#pragma unroll
+        for (int i = 0; i < V; ++i) sg_gather(x[i], gc, gh, addr);
+    }
+    const int hits = (int)((addr - column) >> 7);
+    const uint32_t w1 = b1 + __float_as_uint(kSgMagic), w2 = b2 + __float_as_uint(kSgMagic);
+    for (int j = 0; j < hits; ++j) {
+        const float v = __uint_as_float(hist[32 * j + lane]);
+        const uint32_t b = bin(v);
+        if (b == w1 || b == w2) {
+            const uint32_t key = f2key(v), at = atomicAdd(&ctl[kSgCtl * m + 4], 1u);
+            if (listed) {
+                if (at < (uint32_t)kSgList) list[kSgList * m + at] = key;
+            } else {
+                if (b == w1) atomicMax(&ctl[kSgCtl * m + 5], key);
+                if (b == w2) atomicMin(&ctl[kSgCtl * m + 6], key);
+            }
+        }
+    }
+    __syncwarp();
+    const bool counted = served && ctl[kSgCtl * m + 4] == end - start;
+    if (counted && listed) {
+        const uint32_t cnt = end - start, q1 = k1 - start, q2 = k2 - start;
+        for (uint32_t j = (uint32_t)q; j < cnt; j += (uint32_t)L) {
+            const uint32_t key = list[kSgList * m + j];
+            uint32_t lt = 0u, le = 0u;
+            for (uint32_t i = 0; i < cnt; ++i) {
+                const uint32_t o = list[kSgList * m + i];
+                lt += o < key;
+                le += o <= key;
+            }
+            if (q1 >= lt && q1 < le) ctl[kSgCtl * m + 5] = key;
+            if (q2 >= lt && q2 < le) ctl[kSgCtl * m + 6] = key;
+        }
+    }
+    __syncwarp();
+    const uint32_t u1 = ctl[kSgCtl * m + 5], u2 = ctl[kSgCtl * m + 6];
+    if (counted && (listed || b1 != b2 || u1 == u2)) {   // (the same for all lanes of a series)
+        if (q == 0) sg_store(a, g * M + m, median_from_keys(u1, u2, !(n & 1)));
+        left = false;
+    }
+}
+
+// Rows of L repetitions of a GPU's block; the first V - S are whole.
+template <int V, int S, int M>
+__device__ __forceinline__ bool sg_valid(const int i, const bool act, const int q, const int n) { return i < V - S || (act && i * (32 / M) + q < n); }
+template <int V, int S, int M>
+__device__ __forceinline__ void sg_load(float (&x)[V], const float *from, const bool act, const int q, const int n) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        x[i] = FLT_MAX;               // (beyond the repetitions: ranks are counted from below)
+        if (sg_valid<V, S, M>(i, act, q, n)) x[i] = __ldg(from + i * (32 / M * M));
+    }
+}
+__device__ __forceinline__ void sg_clear(uint32_t *hist) {
+#pragma unroll
+    for (int i = 0; i < kSgBins / 4; ++i) reinterpret_cast<uint4 *>(hist)[lane_id() + 32 * i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// V values per lane, at most S more than there are.
+template <int V, int S, int M>
 __global__ void __launch_bounds__(kSwThreads, V <= 24 ? 8 : (V <= 40 ? 6 : (V <= 56 ? 5 : 4))) sweep_median_gpu_kernel(const SweepMedArgs a) {
     pdl_wait();
     extern __shared__ __align__(16) uint32_t sg[];   // per warp: bins [kSgBins][32], then gathered values [V][32]; lists [M][kSgList], [M][kSgCtl]
-    const int lane = lane_id(), M = MM ? MM : a.M, n = a.reps;
-    const int L = 32 / M;
+    constexpr int L = 32 / M;
+    const int lane = lane_id(), n = a.reps;
     const int g = blockIdx.x * (kSwThreads / 32) + warp_id();
     if (g >= a.G) return;
-    uint32_t *hist = sg + warp_id() * (32 * sg_rows(V) + (kSgList + kSgCtl) * M);
+    uint32_t *hist = sg + warp_id() * sg_words(V, M);
     uint32_t *list = hist + 32 * sg_rows(V), *ctl = list + kSgList * M;
     const int m = lane % M, q = lane / M;
     const bool act = lane < L * M;
     const float *base = a.S + (size_t)g * n * M + min(lane, L * M - 1);   // (idle lanes read a valid column)
 
-    // rows of L repetitions; the first V - S are whole
+    auto valid = [&](const int i) { return sg_valid<V, S, M>(i, act, q, n); };
     float x[V];
-    auto valid = [&](const int i) { return i < V - S || (act && i * L + q < n); };
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        x[i] = FLT_MAX;               // (beyond the repetitions: above every bracket)
-        if (valid(i)) x[i] = __ldg(base + i * (L * M));
-    }
-#pragma unroll
-    for (int i = 0; i < kSgBins / 4; ++i) reinterpret_cast<uint4 *>(hist)[lane + 32 * i] = make_uint4(0u, 0u, 0u, 0u);
-    uint32_t peers = 0u;              // lanes of this one's series
+    sg_load<V, S, M>(x, base, act, q, n);
+    sg_clear(hist);
+    uint32_t peers = 0u;          // lanes of this one's series
 #pragma unroll
     for (int k = 0; k < L; ++k) peers |= 1u << (m + k * M);
 
@@ -270,114 +397,16 @@ __global__ void __launch_bounds__(kSwThreads, V <= 24 ? 8 : (V <= 40 ? 6 : (V <=
     }
     const float inv = 1.0f / (float)n, mean_d = t1 * inv, var = fmaxf(t2 * inv - mean_d * mean_d, 0.0f);
     const float c = x0 + mean_d, h = 2.83f * sqrtf(var * inv);
-    const bool usable = act && !same && th_usable(c, h);
-    const bool even = !(n & 1);
-    const uint32_t k1 = (uint32_t)((n - 1) >> 1), k2 = (uint32_t)(n >> 1);
-
-    // ---- bins: the bracket from the middle of the second to that of the last but one ----
-    constexpr float kTop = (float)(kSgBins - 1), kSpan = (float)(kSgBins - 3);
-    const float scale = usable ? (kSpan / kTop) * 0.5f / h : 0.0f, off = usable ? __fmaf_rn(h - c, scale, 1.0f / kTop) : 0.0f;
-    auto bin = [&](const float v) -> uint32_t { return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(v, scale, off)), kTop, kSgMagic)); };
-    const uint32_t column = (uint32_t)__cvta_generic_to_shared(hist + lane);
-    __syncwarp();
-    if (__any_sync(0xFFFFFFFFu, usable)) {
-        const uint32_t at = column - __float_as_uint(kSgMagic) * 128u;
-#pragma unroll
-        for (int i = 0; i < V; ++i) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(bin(x[i]) * 128u + at) : "memory");
+    const bool open = act && !same && th_usable(c, h);
+    bool left = act;                  // without a result
+    if (act && same && !bad) {
+        if (q == 0) sg_store(a, g * M + m, x0);
+        left = false;
     }
-    if (q == 0) {
-        ctl[kSgCtl * m] = 0u;                 // wanted bins: k1's ...
-        ctl[kSgCtl * m + 1] = 0u;             // ... and k2's
-        ctl[kSgCtl * m + 4] = 0u;             // values found in them
-        ctl[kSgCtl * m + 5] = 0u;             // largest key of the first
-        ctl[kSgCtl * m + 6] = 0xFFFFFFFFu;    // smallest key of the second
-    }
-    __syncwarp();
-    // ---- scan: the lanes of a series share its bins ----
-    const int per = (kSgBins + L - 1) / L, first = q * per;
-    uint32_t sum = 0u, num[kSgBins];
-#pragma unroll
-    for (int j = 0; j < kSgBins; ++j) num[j] = 0u;
-    int from = q;                     // each lane begins with its own column: no two of a series read the same one at a time
-#pragma unroll
-    for (int k = 0; k < L; ++k) {
-#pragma unroll
-        for (int j = 0; j < kSgBins; ++j)
-            if (j < per && first + j < kSgBins && act) num[j] += hist[32 * (first + j) + m + from * M];
-        from = from + 1 < L ? from + 1 : 0;
-    }
-#pragma unroll
-    for (int j = 0; j < kSgBins; ++j) sum += num[j];
-    uint32_t r = 0u;
-#pragma unroll
-    for (int k = 0; k < L; ++k) {
-        const uint32_t o = __shfl_sync(0xFFFFFFFFu, sum, m + k * M);
-        if (k < q) r += o;
-    }
-    if (usable && k2 >= r && k1 < r + sum) {
-#pragma unroll
-        for (int j = 0; j < kSgBins; ++j)
-            if (j < per) {
-                if (k1 >= r && k1 - r < num[j]) { ctl[kSgCtl * m] = (uint32_t)(first + j); ctl[kSgCtl * m + 2] = r; }
-                if (k2 >= r && k2 - r < num[j]) { ctl[kSgCtl * m + 1] = (uint32_t)(first + j); ctl[kSgCtl * m + 3] = r + num[j]; }
-                r += num[j];
-            }
-    }
-    __syncwarp();
-    const uint32_t b1 = ctl[kSgCtl * m], b2 = ctl[kSgCtl * m + 1], start = ctl[kSgCtl * m + 2], end = ctl[kSgCtl * m + 3];
-    bool ok = usable && b1 >= 1u && b2 >= 1u && b1 <= kSgBins - 2u && b2 <= kSgBins - 2u;
-    // ---- the values about the wanted bins (more than those in them: rounding moves a bin's ends) ----
-    const bool listed = ok && end - start <= (uint32_t)kSgList;
-    uint32_t addr = column;
-    if (__any_sync(0xFFFFFFFFu, ok)) {
-        const float width = h * (2.0f / kSpan);
-        const float gc = c - h + (0.5f * (float)(b1 + b2) - 1.0f) * width;
-        const float gh = ok ? (0.5f * (float)(b2 - b1) + 0.6f) * width + (fabsf(c) + h) * pow2_of(-21) : -1.0f;
-#pragma unroll
-        for (int i = 0; i < V; ++i) sg_gather(x[i], gc, gh, addr);
-    }
-    const int hits = (int)((addr - column) >> 7);
-    const uint32_t w1 = b1 + __float_as_uint(kSgMagic), w2 = b2 + __float_as_uint(kSgMagic);
-    for (int j = 0; j < hits; ++j) {
-        const float v = __uint_as_float(hist[32 * j + lane]);
-        const uint32_t b = bin(v);
-        if (b == w1 || b == w2) {
-            const uint32_t key = f2key(v), at = atomicAdd(&ctl[kSgCtl * m + 4], 1u);
-            if (listed) {
-                if (at < (uint32_t)kSgList) list[kSgList * m + at] = key;
-            } else {
-                if (b == w1) atomicMax(&ctl[kSgCtl * m + 5], key);
-                if (b == w2) atomicMin(&ctl[kSgCtl * m + 6], key);
-            }
-        }
-    }
-    __syncwarp();
-    ok = ok && ctl[kSgCtl * m + 4] == end - start;
-    if (ok && listed) {
-        const uint32_t num = end - start, q1 = k1 - start, q2 = k2 - start;
-        for (uint32_t j = (uint32_t)q; j < num; j += (uint32_t)L) {
-            const uint32_t key = list[kSgList * m + j];
-            uint32_t lt = 0u, le = 0u;
-            for (uint32_t i = 0; i < num; ++i) {
-                const uint32_t o = list[kSgList * m + i];
-                lt += o < key;
-                le += o <= key;
-            }
-            if (q1 >= lt && q1 < le) ctl[kSgCtl * m + 5] = key;
-            if (q2 >= lt && q2 < le) ctl[kSgCtl * m + 6] = key;
-        }
-    }
-    __syncwarp();
-    const uint32_t v1 = ctl[kSgCtl * m + 5], v2 = ctl[kSgCtl * m + 6];
-    ok = ok && (listed || b1 != b2 || v1 == v2);   // (else a bin of many different values)
-    if (act && q == 0 && (ok || (same && !bad))) {
-        const float med = ok ? median_from_keys(v1, v2, even) : x0;
-        const size_t o = (size_t)g * M + m;
-        a.gmed[o] = med;
-        if (a.gmed_user) a.gmed_user[o] = med;
-    }
-    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, act && q == 0 && !ok && !(same && !bad)); todo; todo &= todo - 1u)
-        sweep_warp_median<8>(a, (uint32_t)((size_t)g * M) + (uint32_t)(__ffs(todo) - 1), false);
+    if (__any_sync(0xFFFFFFFFu, open)) sg_round<V, M>(a, x, g, m, q, act, hist, list, ctl, c - h, c + h, open, left);
+    uint32_t todo = __ballot_sync(0xFFFFFFFFu, left && q == 0);
+    constexpr int VPL = V * L <= 64 ? 2 : (V * L <= 128 ? 4 : 8);
+    for (; todo; todo &= todo - 1u) sweep_warp_median<VPL>(a, (uint32_t)((size_t)g * M) + (uint32_t)(__ffs(todo) - 1), false);
 }
 
 // Fallback when the repetitions of one GPU do not fit a tile: bit-by-bit counting
@@ -457,44 +486,53 @@ __global__ void __launch_bounds__(kVerdictThreads) sweep_verdict_kernel(const Sw
 
 }  // namespace
 
-template <int V, int S, int MM>
+template <int V, int S, int M>
 static cudaError_t launch_gpu_medians(const SweepMedArgs &a, cudaStream_t st) {
-    const size_t smem = (size_t)(kSwThreads / 32) * sg_words(V, a.M) * sizeof(uint32_t);
-    return launch_after_smem(sweep_median_gpu_kernel<V, S, MM>, (unsigned)((a.G + kSwThreads / 32 - 1) / (kSwThreads / 32)), kSwThreads, smem, st, a);
+    constexpr size_t smem = (size_t)(kSwThreads / 32) * sg_words(V, M) * sizeof(uint32_t);
+    return launch_after_smem(sweep_median_gpu_kernel<V, S, M>, (unsigned)((a.G + kSwThreads / 32 - 1) / (kSwThreads / 32)), kSwThreads, smem, st, a);
 }
-template <int MM>
+// The instance for this many rows: V values per lane, in steps of eight, of sixteen where a metric has three lanes or fewer.
+template <int V, int M>
 static cudaError_t launch_gpu_medians(const SweepMedArgs &a, const int rows, cudaStream_t st) {
-    constexpr int kMost = MM ? (256 + 32 / MM - 1) / (32 / MM) : 64;   // rows of 256 repetitions
-    if (rows <= 8) return launch_gpu_medians<8, 8, MM>(a, st);
-    if (rows <= 16) return launch_gpu_medians<16, 8, MM>(a, st);
-    if (rows <= 24) return launch_gpu_medians<24, 8, MM>(a, st);
-    if (rows <= 32) return launch_gpu_medians<32, 8, MM>(a, st);
-    if constexpr (kMost > 32) {
-        if (rows <= 40) return launch_gpu_medians<40, 8, MM>(a, st);
-        if constexpr (kMost > 40) {
-            if (rows <= 48) return launch_gpu_medians<48, 8, MM>(a, st);
-            if constexpr (kMost > 48) {
-                if (rows <= 56) return launch_gpu_medians<56, 8, MM>(a, st);
-                if constexpr (kMost > 56) return launch_gpu_medians<64, 8, MM>(a, st);
-            }
-        }
+    constexpr int L = 32 / M, S = L > 3 ? 8 : 16, kWanted = (kSgReps + L - 1) / L, kMost = kWanted < kSgRows ? kWanted : kSgRows;
+    if constexpr (V < kMost) {
+        if (rows > V) return launch_gpu_medians<V + S, M>(a, rows, st);
     }
-    return cudaErrorInvalidValue;
+    return launch_gpu_medians<V, S, M>(a, st);
+}
+template <int M>
+static cudaError_t launch_gpu_medians(const SweepMedArgs &a, const int rows, cudaStream_t st) {
+    return launch_gpu_medians<(32 / M > 3 ? 8 : 16), M>(a, rows, st);
 }
 
 cudaError_t launch_sweep_medians(const SweepMedArgs &a, cudaStream_t st) {
     const long long series = (long long)a.G * a.M;
-    // A warp per GPU where its values fit the registers (and the lists of its series shared memory), unless the series are so
-    // few that a warp each is the shorter chain: 1 776 series of 33 repetitions 2.2 us against 3.7, 4 096 of 20 2.5 against
-    // 3.5, but 4 800 of 60 5.5 against 4.4, 6 144 of 120 7.3 against 5.2.
+    // A warp per GPU where its values fit the registers, with three to sixteen metrics (the lanes of a series share the scan of
+    // its bins: 16 384 GPUs x 64 x 1 take 87 us so, by threads 28; x 2 58 and 40), from as many values on as it is the shorter
+    // way.  Four to eight metrics: 230 000 (a sweep of 296 x 100 x 6 10.9 us, a warp per series 10.2; 1 000 x 33 x 4 10.6 and
+    // 10.1; but 592 x 64 x 8 11.4 and 12.7, 296 x 200 x 4 10.5 and 11.6).  Three, or two to three lanes to a series: 600 000
+    // (296 x 100 x 12 14.8 and 11.2, 592 x 100 x 12 13.5 and 13.1, 1 000 x 100 x 12 14.6 and 15.8).  Three metrics have too few
+    // repetitions to a lane below 64 (16 384 x 33 x 3 30.9, by threads 28.4; of 64 32 and 37).
     const int L = 32 / a.M, rows = (a.reps + L - 1) / L;
-    if (a.reps <= 256 && series < 0x7FFFFFFFLL && rows <= 64 && a.M <= 16 && series * ((a.reps + 31) / 32) > 6144) {
+    if (a.reps <= kSgReps && rows <= kSgRows && series < 0x7FFFFFFFLL && series * a.reps >= (a.M >= 4 && a.M <= 8 ? 230000 : 600000)) {
         switch (a.M) {
+            case 3:
+                if (a.reps >= 64) return launch_gpu_medians<3>(a, rows, st);
+                break;
             case 4: return launch_gpu_medians<4>(a, rows, st);
             case 5: return launch_gpu_medians<5>(a, rows, st);
             case 6: return launch_gpu_medians<6>(a, rows, st);
+            case 7: return launch_gpu_medians<7>(a, rows, st);
             case 8: return launch_gpu_medians<8>(a, rows, st);
-            default: return launch_gpu_medians<0>(a, rows, st);
+            case 9: return launch_gpu_medians<9>(a, rows, st);
+            case 10: return launch_gpu_medians<10>(a, rows, st);
+            case 11: return launch_gpu_medians<11>(a, rows, st);
+            case 12: return launch_gpu_medians<12>(a, rows, st);
+            case 13: return launch_gpu_medians<13>(a, rows, st);
+            case 14: return launch_gpu_medians<14>(a, rows, st);
+            case 15: return launch_gpu_medians<15>(a, rows, st);
+            case 16: return launch_gpu_medians<16>(a, rows, st);
+            default: break;
         }
     }
     // (Other numbers of metrics and repetitions.)  A warp per series while they are few: one launch, and no thread's chain over

@@ -586,11 +586,11 @@ def test_exceedance_counts(R, M, W):
 
 @pytest.mark.parametrize("nodes,gpn,N,M", [
     (6145, 8, 32, 1),              # the last warp has few series left
-    (2400, 7, 33, 3),              # one repetition in the last round
-    (1031, 8, 200, 6),             # a warp per series no longer; GPUs over two warps
+    (2400, 7, 33, 3),              # by threads: one repetition in the last round
+    (1031, 8, 200, 6),             # a warp per GPU
     (77, 130, 45, 5),              # more GPUs per node than a CTA has threads
     (400, 4, 256, 32),             # the most repetitions and metrics
-    (340, 8, 100, 12),             # a warp per series, the most of them
+    (340, 8, 100, 12),             # a warp per GPU, eight lanes of it idle
     (700, 8, 33, 12),              # fleet statistics by clusters of four, the cut beside them
     (600, 8, 20, 20),              # the same without room beside
 ])
@@ -908,9 +908,9 @@ def test_window_threads_serve_values_of_any_size(scale):
 
 
 @pytest.mark.parametrize("nodes,gpn,N,M", [
-    (10923, 1, 33, 3),             # quarters of words; one series in the last
-    (1300, 8, 64, 4),              # halves
-    (2500, 8, 40, 8),              # whole words, more than there are warps
+    (10923, 1, 33, 3),             # by threads and the finishing kernel: quarters of words; one series in the last
+    (1300, 8, 64, 4),              # by a warp per GPU, which sorts every series
+    (2500, 8, 40, 8),
 ])
 def test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M):
     """Results that spread over decades: the mean says nothing about the median, and next to no series is served by it."""
@@ -1056,8 +1056,8 @@ def test_window_tiles_at_their_edges(R, M, W, quant):
 
 
 @pytest.mark.parametrize("nodes,gpn,N,M", [
-    (6200, 1, 1, 1),               # one value per series
-    (3100, 1, 64, 1), (3083, 1, 256, 2), (2049, 1, 96, 3),   # 32, 16 and ten lanes per series
+    (6200, 1, 1, 1),               # one value per series (by a warp per series, as one and two metrics and the smaller ones below)
+    (3100, 1, 64, 1), (3083, 1, 256, 2), (2049, 1, 96, 3),
     (1601, 1, 33, 4), (800, 1, 256, 4),                      # rows of eight: five of them, all 32
     (401, 2, 48, 5), (397, 2, 49, 5), (260, 1, 255, 5),      # a whole number of rows, one repetition more, the most
     (601, 1, 40, 6), (603, 1, 41, 6), (211, 1, 200, 6), (160, 1, 256, 6),
@@ -1090,6 +1090,32 @@ def test_sweep_gpu_by_warp(nodes, gpn, N, M):
     S[G // 2, N - 1, M - 1] = np.float32("inf")
     out = guard.sweep_qualify(torch.from_numpy(S).cuda(), nodes, gpn, dir=dirs)
     assert int(out["status"].cpu()[0]) & 1
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (3200, 1, 64, 3), (800, 1, 256, 3),                      # ten lanes per series: eight and 32 values each
+    (2900, 1, 20, 4), (1800, 1, 33, 4), (240, 1, 256, 4),    # eight lanes: eight values, all 32
+    (401, 3, 48, 5), (480, 2, 49, 5), (260, 1, 255, 5),      # a whole number of rows of six, one repetition more, the most
+    (1001, 1, 40, 6), (1003, 1, 41, 6), (211, 1, 200, 6), (160, 1, 256, 6),
+    (600, 1, 64, 7), (150, 1, 256, 7),                       # 28 lanes in use
+    (1000, 1, 32, 8), (500, 2, 33, 8), (120, 1, 256, 8),
+    (4200, 1, 16, 9), (360, 1, 192, 9), (500, 1, 128, 10),   # three lanes: sixteen values at least, all 64
+    (860, 1, 64, 11), (1600, 1, 33, 12), (370, 1, 128, 13), (700, 1, 63, 14), (1300, 1, 31, 15), (1200, 1, 32, 16), (300, 1, 128, 16),
+])
+def test_sweep_gpu_by_warp_of_any_metrics(nodes, gpn, N, M):
+    """... at the ends of the instances, and enough values that a warp per GPU is taken."""
+    test_sweep_gpu_by_warp(nodes, gpn, N, M)
+
+
+@pytest.mark.parametrize("nodes,gpn,N,M", [
+    (10923, 1, 33, 3), (1000, 2, 33, 17),   # quarters of words
+    (1500, 2, 64, 20),                      # halves
+    (3000, 1, 100, 26),                     # whole words, up to 128 repetitions
+    (9100, 1, 33, 18),                      # ... more of them than there are warps
+])
+def test_sweep_finishing_kernel(nodes, gpn, N, M):
+    """Sweeps by threads, whose series a warp per GPU does not take."""
+    test_sweep_series_left_to_the_finishing_kernel(nodes, gpn, N, M)
 
 
 @pytest.mark.parametrize("nodes,gpn,N,M", [(2100, 1, 40, 20), (1100, 2, 200, 16)])   # more metrics or repetitions than a warp holds

@@ -49,7 +49,7 @@ Layout make_layout(int R, int M, int C, int K) {
     L.xr_small = off;  off = align_up(off + (L.xr_steps ? xrank_scratch_small_bytes(M, L.xr_steps) : 0));
     L.xr_gridp = (xrank_count_supported(R) && R >= 8192) ? 1 : 0;
     L.xr_grid = off;   off = align_up(off + 2 * align_up(sizeof(RowHints)));
-    L.inc_rbc = off;   off = align_up(off + 64);   // their number and the finishing kernel's ticket (zero before first use)
+    L.inc_rbc = off;   off = align_up(off + 64);   // number of series that the thread path leaves, and its finishing kernel's ticket (zero before first use)
     // the windowed medians and the kept top-k indices exist twice: consecutive evaluations alternate, so that a
     // deferred evaluation's tail may still read its medians while the next evaluation's window kernels write theirs
     L.wmed = off;      off = align_up(off + (size_t)R * M * sizeof(float));

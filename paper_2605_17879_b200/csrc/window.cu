@@ -506,7 +506,7 @@ struct IncEdit {
 
 // NEW: the most steps that entered / left (1 for an evaluation after every step, else kIncMaxNew); VPL: values per lane of
 // a rebuild.  (Two series per thread, all of 262 144 resident at once: the same alone, and beside the cluster kernels of
-// other evaluations, which then wait for room, six deferred steps of 32 768 x 8 take 205 us instead of 194.)
+// other evaluations, which then wait for room, six deferred steps of 32 768 x 8 take 6 % longer.)
 template <int NEW, int VPL>
 __global__ void __launch_bounds__(kIncThreads, 8) window_inc_kernel(const WindowArgs a, const IncArgs s, const int per) {
     pdl_wait();

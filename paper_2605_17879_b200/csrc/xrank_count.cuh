@@ -29,7 +29,8 @@ constexpr uint32_t kCtNone = 0xFFFFFFFFu;  // the largest key: a NaN's, and what
 constexpr int kCtAll = 0, kCtStatistics = 1, kCtCut = 2;   // what a CTA (cluster) computes: both, median and MAD, the extra order statistic
 // Single rows of 8 metrics, bracketed by the row before / not: one CTA of 1 024 threads per column takes 6.3 / 7.5 us at
 // 2 048 ranks, 7.9 / 9.6 at 4 096, 9.5 / 11.6 at 6 000 (and 12.9 / 17.5 at 16 384); a cluster of eight pays two cluster
-// barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3.
+// barriers and the gathering of bins a round and takes 8.8 / 10.2, 9.1 / 10.8, 9.2 / 11.6 and 10.4 / 15.3 (with up to 512
+// threads a CTA).
 constexpr int kCtClusterRanks = 4096;
 // Threads of the CTAs of a cluster: four values each, while a CTA has 256 of them at most: at 128 registers two such CTAs
 // share an SM, so that the clusters of a step's row and of another evaluation's tail find room beside one another and

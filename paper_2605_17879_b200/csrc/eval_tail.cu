@@ -246,16 +246,18 @@ cudaError_t launch(const XrankArgs &x, const TopkArgs &t, const MetricParams &p,
 // The fleet baseline x (one row, no exceedance bits) and, with t.K > 0, the top-k list t (no scores) of one evaluation;
 // R <= kCountMaxRanks.  steps: evaluations follow one another by a few steps.  Their tails share the GPU with the clusters of
 // the next steps' rows: CTAs of up to 256 threads, two to an SM, where four values a thread would ask for 512 (deferred single
-// steps of 16 384 ranks x 8 24.3 us, with 512 26.1; of 24 000 28.3 and 32.4).  After a block the tail is what the pass waits
-// for: up to 512, the shorter chain (blocks of 50 steps of 24 000 x 8, W = 100, 164.1 us, with 256 166.6; of 32 768 205.8 and
-// 209.1).
+// steps of 16 384 ranks x 8 24.3 us, with 512 26.1; of 24 000 28.3 and 32.4).  After a block up to 512 where 256 would hold sixteen
+// values a thread, a longer chain (blocks of 50 steps of 24 000 x 8, W = 100, 163.4 us, with 256 166.2; of 32 768 205.6 and
+// 208.9), but not with eight, where the next blocks' kernels need the room (a hundred blocks of 200 steps of 16 384 x 8, W =
+// 200, 10.48 ms, with 512 10.68).
 cudaError_t launch_eval_tail(const XrankArgs &x, const TopkArgs &t, const MetricParams &p, const bool steps, cudaStream_t st) {
     if (x.R <= kCtClusterRanks) {
         int T = 32;
         while (T < 1024 && x.R > 4 * T) T <<= 1;
         return launch_after(eval_tail_kernel<4, 1>, x.M + (t.K > 0 ? 1 : 0), T, st, x, t, p);
     }
-    return (x.M + 1) * 8 <= 148 ? launch<8>(x, t, p, steps ? ct_most_threads(8) : 512, st) : launch<4>(x, t, p, 512, st);
+    const bool few = steps || x.R <= 8 * 8 * ct_most_threads(8);
+    return (x.M + 1) * 8 <= 148 ? launch<8>(x, t, p, few ? ct_most_threads(8) : 512, st) : launch<4>(x, t, p, 512, st);
 }
 
 }  // namespace guard
